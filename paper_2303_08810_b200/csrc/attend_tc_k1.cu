@@ -23,6 +23,7 @@
 //   correlation of V from the halo tile), one bf16 store of O  ->  copy of the halo of tile n + 1.
 // Every wait (on an MMA, on a copy) is bounded.
 #include "attend_tc_common.cuh"
+#include "tma_map.h"
 
 namespace bra {
 
@@ -572,38 +573,6 @@ attend_tc_k1_kernel(const __grid_constant__ K1Maps maps, const int32_t* index,
 }
 
 // ------------------------------------------------------------------ host side
-namespace {
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-// The driver's encoder, looked up through the runtime (the library does not link against the driver).
-EncodeTiledFn encoder() {
-    static EncodeTiledFn fn = [] {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) != cudaSuccess ||
-            q != cudaDriverEntryPointSuccess)
-            p = nullptr;
-        return reinterpret_cast<EncodeTiledFn>(p);
-    }();
-    return fn;
-}
-
-// Tensor map over a [B,H,W,C] bf16 tensor of this GPU's memory; box = (bc channels, bx, by tokens, 1 image).
-bool make_map(CUtensorMap* m, const void* base, const Dims& d, int bc, int bx, int by, CUtensorMapSwizzle sw) {
-    EncodeTiledFn enc = encoder();
-    if (!enc) return false;
-    const cuuint64_t dims[4] = {(cuuint64_t)d.C, (cuuint64_t)d.W, (cuuint64_t)d.H, (cuuint64_t)d.B};
-    const cuuint64_t strides[3] = {(cuuint64_t)d.C * 2, (cuuint64_t)d.W * d.C * 2, (cuuint64_t)d.H * d.W * d.C * 2};
-    const cuuint32_t box[4] = {(cuuint32_t)bc, (cuuint32_t)bx, (cuuint32_t)by, 1};
-    const cuuint32_t es[4] = {1, 1, 1, 1};
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, es,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-}  // namespace
-
 static cudaError_t k1_attributes() {
     static PerDeviceOnce once;
     return once.run([]() -> cudaError_t {

@@ -20,11 +20,7 @@ WsLayout ws_layout(const Dims& d) {
     L.delta = off;    off += align256(sizeof(float) * (size_t)d.B * d.heads * d.N);
     L.inv_off = off;  off += align256(sizeof(int32_t) * (size_t)d.B * d.heads_i * (d.R + 1));
     L.inv_list = off; off += align256(sizeof(int32_t) * (size_t)d.B * d.heads_i * d.R * d.topk);
-    // one partial per (image, region row), capped so the scratch stays small
-    int blocks = d.B * d.S;
-    while (blocks > 1024 && blocks % 2 == 0) blocks /= 2;
-    L.dw_blocks = blocks;
-    L.dw_part = off;  off += align256(sizeof(float) * (size_t)blocks * d.C * 26);
+    L.dw_part = off;  off += align256(sizeof(float) * (size_t)lce_grad_partials(d) * d.C * 26);
     L.pad = L.pad_lse = off;
     L.pad_tensor = 0;
     if (d.H != d.H0 || d.W != d.W0) {

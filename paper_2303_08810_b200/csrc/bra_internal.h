@@ -40,13 +40,14 @@ struct WsLayout {
     size_t delta;       // fp32 [B,heads,N]  rowsum(P o dP) of the backward pass
     size_t inv_off;     // int32 [B,heads_i,R+1] CSR offsets of the inverse routing index
     size_t inv_list;    // int32 [B,heads_i,R*topk] query regions routed to each key region
-    size_t dw_part;     // fp32 [dw_blocks, C*26] partial LCE weight / bias gradients
+    size_t dw_part;     // fp32 [lce_grad_partials(d), 26*C] partial LCE weight / bias gradients
     size_t pad;         // padded maps only: seven [B,H,W,C] tensors of the padded size (Q, K, V, O / dO, dQ, dK, dV)
     size_t pad_lse;     // padded maps only: fp32 [B,heads,H*W] of the padded size
     size_t pad_tensor;  // bytes of one padded tensor
     size_t total;
-    int dw_blocks;
 };
+
+constexpr int kSMs = 148;      // B200
 
 WsLayout ws_layout(const Dims& d);
 
@@ -142,6 +143,11 @@ struct PerDeviceOnce {
 // order on the caller's stream).
 struct SideStream { cudaStream_t s; cudaEvent_t fork, join; };
 SideStream* side_stream();
+
+// Gradient of the LCE weights and bias from V and dO (part: lce_grad_partials(d) x 26 C floats of scratch).
+int lce_grad_partials(const Dims& d);
+cudaError_t launch_lce_grad(const Dims& d, int dtype, const void* V, const void* dO, float* part, float* d_lce_w, float* d_lce_b,
+                            int32_t* status, cudaStream_t st);
 
 bool backward_supported(const Dims& d);
 // impl: the bra_impl the caller asked for

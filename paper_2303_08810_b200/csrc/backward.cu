@@ -2,7 +2,7 @@
 // index (Eq. 7 with Eq. 1; the index of Eq. 5 is a constant), fp32 arithmetic
 // on CUDA cores.  Every sum has a fixed order: no atomics on the data path.
 //
-//   1. inverse index: for each key region, the list (in (query region, slot)
+//   1. inverse index (inverse_index.cuh): for each key region, the list (in (query region, slot)
 //      order) of query regions that routed to it, as CSR.
 //   2. dQ kernel, one thread per (query, head): delta = rowsum(P o dP), then
 //      dQ = scale * sum_j P_j (dP_j - delta) K_j; delta is kept for step 3.
@@ -10,58 +10,17 @@
 //      recomputes P from the saved log-sum-exp, accumulates dK, dV, then adds
 //      the LCE adjoint dV += sum_ij w[c,i,j] dO[y-i+2, x-j+2, c].
 //   4. d_lce_w / d_lce_b: lce_grad.cu.
-// Steps 2 and 3 run on the tensor cores instead (backward_mma.cu) for bf16 with head dim 32.
-#include "bra_internal.h"
+// Steps 1 to 3 run on the tensor cores instead (backward_img.cu, backward_direct.cu) for bf16 with head dim 32 or 64.
+#include "inverse_index.cuh"
 
 namespace bra {
 
 // ------------------------------------------------------------ inverse index
-// grid: B * heads_i CTAs of 256 threads.  The R * topk entries of the (image, head) are staged
-// in shared memory when they fit.  Warp w takes key regions w, w + 8, ...: it sweeps the entries
-// 32 at a time and finds its region's hits with a ballot, so the list of a key region comes out
-// in entry order (query region, then slot): a fixed order for the dK / dV sums.
 __global__ void __launch_bounds__(256)
 inverse_index_kernel(const int32_t* __restrict__ index, int32_t* __restrict__ inv_off,
-                     int32_t* __restrict__ inv_list, int staged, Dims dm) {
-    extern __shared__ int32_t sm[];   // counts[R + 1], then the staged entries
-    const int bh = blockIdx.x;
-    const int32_t* gidx = index + (size_t)bh * dm.R * dm.topk;
-    const int entries = dm.R * dm.topk;
-    int32_t* sidx = sm + dm.R + 1;
-    if (staged) {
-        for (int e = threadIdx.x; e < entries; e += blockDim.x) sidx[e] = gidx[e];
-        __syncthreads();
-    }
-    const int32_t* idx = staged ? sidx : gidx;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    for (int j = warp; j < dm.R; j += nwarps) {
-        int count = 0;
-        for (int e0 = 0; e0 < entries; e0 += 32) {
-            const int e = e0 + lane;
-            count += __popc(__ballot_sync(0xffffffffu, e < entries && idx[e] == j));
-        }
-        if (lane == 0) sm[j] = count;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int run = 0;
-        for (int r = 0; r < dm.R; ++r) { const int c = sm[r]; sm[r] = run; run += c; }
-        sm[dm.R] = run;
-    }
-    __syncthreads();
-    int32_t* off = inv_off + (size_t)bh * (dm.R + 1);
-    for (int j = threadIdx.x; j <= dm.R; j += blockDim.x) off[j] = sm[j];
-    for (int j = warp; j < dm.R; j += nwarps) {
-        int32_t* out = inv_list + (size_t)bh * entries + sm[j];
-        int pos = 0;
-        for (int e0 = 0; e0 < entries; e0 += 32) {
-            const int e = e0 + lane;
-            const bool hit = e < entries && idx[e] == j;
-            const unsigned m = __ballot_sync(0xffffffffu, hit);
-            if (hit) out[pos + __popc(m & ((1u << lane) - 1u))] = e / dm.topk;   // the query region of entry e
-            pos += __popc(m);
-        }
-    }
+                     int32_t* __restrict__ inv_list, bool use_bits, Dims dm) {
+    extern __shared__ int32_t sm[];
+    inverse_index_job(index, inv_off, inv_list, blockIdx.x, sm, use_bits, dm);
 }
 
 // ------------------------------------------------------------ dQ and delta
@@ -199,6 +158,19 @@ bool backward_supported(const Dims& d) {
     return (d.d == 16 || d.d == 32 || d.d == 64) && d.R <= 1000;
 }
 
+enum Family { FAMILY_SIMT, FAMILY_DIRECT, FAMILY_IMG };
+
+// bf16, head dim 32 or 64: tensor-core kernels.  Small maps with enough (image, head) pairs to fill the GPU keep a
+// whole slice resident (head dim 32); the rest take their operands straight from global memory.
+static Family choose_family(const Dims& d, int dtype, int impl) {
+    if (dtype != BRA_BF16 || impl == BRA_IMPL_SIMT) return FAMILY_SIMT;
+    if (backward_img_supported(d, dtype) &&
+        (impl == BRA_IMPL_IMG || (impl == BRA_IMPL_AUTO && (long long)d.B * d.heads >= 64)))
+        return FAMILY_IMG;
+    return backward_direct_supported(d, dtype) ? FAMILY_DIRECT : FAMILY_SIMT;
+}
+bool backward_any_map(const Dims& d, int dtype, int impl) { return choose_family(d, dtype, impl) == FAMILY_DIRECT; }
+
 // The LCE weight gradient needs only V and dO, the attention gradients need neither of its results: the two
 // run side by side (helper stream of bra_internal.h; everything stays on the caller's stream if there is none).
 template <typename T, int D>
@@ -230,29 +202,18 @@ static cudaError_t launch_bwd_t(const Dims& d, int impl, const void* Q, const vo
     }
     if (ss && cudaEventRecord(ss->join, ss->s) != cudaSuccess) return cudaErrorUnknown;
 
-    // bf16, head dim 32: tensor-core kernels.  Small maps with enough (image, head) pairs to fill the
-    // GPU keep a whole slice resident; the rest stream blocks through shared memory.
-    const bool img_ok = sizeof(T) == 2 && backward_img_supported(d, BRA_BF16);
-    const bool use_img = img_ok && (impl == BRA_IMPL_IMG ||
-                                    (impl == BRA_IMPL_AUTO && (long long)d.B * d.heads >= 64));
-    if (!use_img) {
-        const int thr = 256;
-        const size_t idx_bytes = sizeof(int32_t) * (size_t)d.R * d.topk;
-        const int staged = idx_bytes <= 40 * 1024;
-        inverse_index_kernel<<<d.B * d.heads_i, thr, sizeof(int32_t) * (d.R + 1) + (staged ? idx_bytes : 0), st>>>(
-            index, inv_off, inv_list, staged, d);
-        count_launch();
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    if (use_img) {
-        // the dQ kernel of this family also writes the inverse routing index
+    const Family family = choose_family(d, sizeof(T) == 2 ? BRA_BF16 : BRA_F32, impl);
+    if (family == FAMILY_IMG) {
+        // the dQ kernel of this family and of the next also writes the inverse routing index
         if ((e = launch_backward_img(d, Q, K, V, index, inv_off, inv_list, lce_w, lse, dO, dQ, dK, dV,
                                      delta, status, st)) != cudaSuccess) return e;
-    } else if (sizeof(T) == 2 && impl != BRA_IMPL_SIMT && backward_mma_supported(d, BRA_BF16)) {
-        // head dim 32, bf16: the two tensor-core kernels (dQ + delta, then dK / dV)
-        if ((e = launch_backward_mma(d, Q, K, V, index, inv_off, inv_list, lce_w, lse, dO, dQ, dK, dV,
-                                     delta, status, st)) != cudaSuccess) return e;
+    } else if (family == FAMILY_DIRECT) {
+        if ((e = launch_backward_direct(d, Q, K, V, index, inv_off, inv_list, lce_w, lse, dO, dQ, dK, dV,
+                                        delta, status, st)) != cudaSuccess) return e;
     } else {
+        inverse_index_kernel<<<d.B * d.heads_i, 256, inverse_smem(d), st>>>(index, inv_off, inv_list, inverse_uses_bits(d), d);
+        count_launch();
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
         const long long total = (long long)d.B * d.heads * d.R * d.n_r;
         const unsigned blocks = (unsigned)((total + 127) / 128);
         bwd_dq_kernel<T, D><<<blocks, 128, 0, st>>>(q, k, v, index, lse, go, static_cast<T*>(dQ), delta, status, d);

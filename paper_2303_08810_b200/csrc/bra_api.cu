@@ -97,6 +97,8 @@ SideStream* side_stream() {
 }
 
 static bool padded(const Dims& d) { return d.H != d.H0 || d.W != d.W0; }
+// the problem as seen by a kernel that works on the padded copies
+static Dims on_copies(const Dims& d) { Dims p = d; p.H0 = d.H; p.W0 = d.W; return p; }
 
 // The zero-padded copy of a caller's map in slot `slot` of the scratch buffer (or the map itself if S divides it).
 static const void* pad_in(const Dims& d, const WsLayout& L, char* w, int slot, const void* src, cudaStream_t st, bool* ok) {
@@ -114,12 +116,12 @@ static void crop_out(const Dims& d, const WsLayout& L, char* w, int slot, void* 
         *ok = false;
 }
 
-enum Path { PATH_NONE, PATH_SIMT, PATH_MMA, PATH_TC, PATH_TC_WIDE, PATH_IMG };
+enum Path { PATH_NONE, PATH_SIMT, PATH_DIRECT, PATH_TC, PATH_TC_WIDE, PATH_IMG };
 
 static Path choose_attend(const Dims& d, int dtype, int impl) {
     switch (impl) {
         case BRA_IMPL_SIMT: return attend_simt_supported(d) ? PATH_SIMT : PATH_NONE;
-        case BRA_IMPL_MMA:  return attend_mma_supported(d, dtype) ? PATH_MMA : PATH_NONE;
+        case BRA_IMPL_MMA:  return attend_direct_supported(d, dtype) ? PATH_DIRECT : PATH_NONE;
         case BRA_IMPL_TC_FUSED: return attend_tc_supported(d, dtype) ? PATH_TC : PATH_NONE;
         case BRA_IMPL_TC:   return attend_tc_supported(d, dtype) ? PATH_TC
                                  : attend_tc_wide_supported(d, dtype) ? PATH_TC_WIDE : PATH_NONE;
@@ -130,10 +132,13 @@ static Path choose_attend(const Dims& d, int dtype, int impl) {
     if (attend_tc_wide_supported(d, dtype)) return PATH_TC_WIDE;
     // one CTA per (image, head): worth it once those fill a good part of the GPU
     if (attend_img_supported(d, dtype) && (long long)d.B * d.heads >= 64) return PATH_IMG;
-    if (attend_mma_supported(d, dtype)) return PATH_MMA;
+    if (attend_direct_supported(d, dtype)) return PATH_DIRECT;
     if (attend_simt_supported(d)) return PATH_SIMT;
     return PATH_NONE;
 }
+
+// Paths whose kernels take a map that S does not divide as it is (the others get a zero-padded copy).
+static bool any_map(Path path) { return path == PATH_DIRECT; }
 
 static bra_status run_route(const Dims& d, int dtype, const void* Q, const void* K,
                             float* q_mean, float* k_mean, int32_t* index, cudaStream_t st) {
@@ -149,13 +154,41 @@ static bra_status run_attend(Path path, const Dims& d, int dtype, const void* Q,
     cudaError_t e = cudaErrorInvalidValue;
     switch (path) {
         case PATH_SIMT: e = launch_attend_simt(d, dtype, Q, K, V, index, lce_w, lce_b, O, lse, status, st); break;
-        case PATH_MMA:  e = launch_attend_mma(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel); break;
+        case PATH_DIRECT:  e = launch_attend_direct(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel); break;
         case PATH_TC:   e = launch_attend_tc(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel); break;
         case PATH_TC_WIDE: e = launch_attend_tc_wide(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel); break;
         case PATH_IMG:  e = launch_attend_img(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel); break;
         default: return BRA_ERR_UNSUPPORTED;
     }
     return e == cudaSuccess ? BRA_OK : BRA_ERR_CUDA;
+}
+
+// Runs `f` on the caller's map, or on zero-padded copies of Q, K, V with O and lse cropped back.
+template <typename F>
+static bra_status on_padded_map(const Dims& d, const WsLayout& L, const void* Q, const void* K, const void* V, void* O, float* lse,
+                                char* w, cudaStream_t st, F&& f) {
+    if (!padded(d)) return f(d, Q, K, V, O, lse);
+    bool ok = true;
+    Q = pad_in(d, L, w, 0, Q, st, &ok);
+    K = pad_in(d, L, w, 1, K, st, &ok);
+    V = pad_in(d, L, w, 2, V, st, &ok);
+    if (!ok) return BRA_ERR_CUDA;
+    float* lse_p = lse ? reinterpret_cast<float*>(w + L.pad_lse) : nullptr;
+    const bra_status s = f(on_copies(d), Q, K, V, pad_out(d, L, w, 3, O), lse_p);
+    if (s != BRA_OK) return s;
+    crop_out(d, L, w, 3, O, st, &ok);
+    if (lse && launch_pad_copy(lse_p, lse, (long long)d.B * d.heads, d.H0, d.W0, d.H, d.W, 4, false, st) != cudaSuccess) ok = false;
+    return ok ? BRA_OK : BRA_ERR_CUDA;
+}
+
+static bra_status attend_any_map(Path path, const Dims& d, const WsLayout& L, int dtype, const void* Q, const void* K, const void* V,
+                                 const int32_t* index, const float* lce_w, const float* lce_b, void* O, float* lse, char* w,
+                                 cudaStream_t st, bool after_own_kernel) {
+    int32_t* status = reinterpret_cast<int32_t*>(w + L.status);
+    if (any_map(path)) return run_attend(path, d, dtype, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel);
+    return on_padded_map(d, L, Q, K, V, O, lse, w, st, [&](const Dims& dp, const void* q, const void* k, const void* v, void* o, float* l) {
+        return run_attend(path, dp, dtype, q, k, v, index, lce_w, lce_b, o, l, status, st, after_own_kernel && !padded(d));
+    });
 }
 
 }  // namespace bra
@@ -186,12 +219,7 @@ bra_status bra_route(const bra_problem* p, const void* Q, const void* K,
     char* w = static_cast<char*>(ws);
     float* qm = q_mean ? q_mean : reinterpret_cast<float*>(w + L.q_mean);
     float* km = k_mean ? k_mean : reinterpret_cast<float*>(w + L.k_mean);
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    bool ok = true;
-    Q = pad_in(d, L, w, 0, Q, st, &ok);
-    K = pad_in(d, L, w, 1, K, st, &ok);
-    if (!ok) return BRA_ERR_CUDA;
-    return run_route(d, p->dtype, Q, K, qm, km, index, st);
+    return run_route(d, p->dtype, Q, K, qm, km, index, static_cast<cudaStream_t>(stream));
 }
 
 bra_status bra_attend(const bra_problem* p, const void* Q, const void* K, const void* V,
@@ -211,20 +239,7 @@ bra_status bra_attend(const bra_problem* p, const void* Q, const void* K, const 
     Path path = choose_attend(d, p->dtype, p->impl);
     if (path == PATH_NONE) return BRA_ERR_UNSUPPORTED;
     char* w = static_cast<char*>(ws);
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    bool ok = true;
-    Q = pad_in(d, L, w, 0, Q, st, &ok);
-    K = pad_in(d, L, w, 1, K, st, &ok);
-    V = pad_in(d, L, w, 2, V, st, &ok);
-    if (!ok) return BRA_ERR_CUDA;
-    float* lse_k = (lse && padded(d)) ? reinterpret_cast<float*>(w + L.pad_lse) : lse;
-    s = run_attend(path, d, p->dtype, Q, K, V, index, lce_w, lce_b, pad_out(d, L, w, 3, O), lse_k,
-                   reinterpret_cast<int32_t*>(w + L.status), st, false);
-    if (s != BRA_OK) return s;
-    crop_out(d, L, w, 3, O, st, &ok);
-    if (lse && padded(d) &&
-        launch_pad_copy(lse_k, lse, (long long)d.B * d.heads, d.H0, d.W0, d.H, d.W, 4, false, st) != cudaSuccess) ok = false;
-    return ok ? BRA_OK : BRA_ERR_CUDA;
+    return attend_any_map(path, d, L, p->dtype, Q, K, V, index, lce_w, lce_b, O, lse, w, static_cast<cudaStream_t>(stream), false);
 }
 
 bra_status bra_forward(const bra_problem* p, const void* Q, const void* K, const void* V,
@@ -250,33 +265,18 @@ bra_status bra_forward(const bra_problem* p, const void* Q, const void* K, const
     int32_t* status = reinterpret_cast<int32_t*>(w + L.status);
     float* qm = reinterpret_cast<float*>(w + L.q_mean);
     float* km = reinterpret_cast<float*>(w + L.k_mean);
-    bool ok = true;
-    Q = pad_in(d, L, w, 0, Q, st, &ok);
-    K = pad_in(d, L, w, 1, K, st, &ok);
-    V = pad_in(d, L, w, 2, V, st, &ok);
-    if (!ok) return BRA_ERR_CUDA;
-    void* O_user = O;
-    float* lse_user = lse;
-    O = pad_out(d, L, w, 3, O);
-    if (lse && padded(d)) lse = reinterpret_cast<float*>(w + L.pad_lse);
-    auto finish = [&](bra_status rs) -> bra_status {
-        if (rs != BRA_OK) return rs;
-        crop_out(d, L, w, 3, O_user, st, &ok);
-        if (lse_user && padded(d) &&
-            launch_pad_copy(lse, lse_user, (long long)d.B * d.heads, d.H0, d.W0, d.H, d.W, 4, false, st) != cudaSuccess) ok = false;
-        return ok ? BRA_OK : BRA_ERR_CUDA;
-    };
     // pooling, routing and attention in one launch
     static const bool one_launch = getenv("BRA_ONE_LAUNCH") != nullptr;     // tuning aid: also under BRA_IMPL_AUTO
     if (p->impl == BRA_IMPL_TC_FUSED && !forward_tc_supported(d, p->dtype)) return BRA_ERR_UNSUPPORTED;
     if (p->impl == BRA_IMPL_TC_FUSED ||
         (one_launch && p->impl == BRA_IMPL_AUTO && path == PATH_TC && forward_tc_supported(d, p->dtype))) {
-        const cudaError_t e = launch_forward_tc(d, Q, K, V, lce_w, lce_b, O, idx, lse, qm, km, status, p->inject, st);
-        return finish(e == cudaSuccess ? BRA_OK : BRA_ERR_CUDA);
+        return on_padded_map(d, L, Q, K, V, O, lse, w, st, [&](const Dims& dp, const void* q, const void* k, const void* v, void* o, float* l) {
+            return launch_forward_tc(dp, q, k, v, lce_w, lce_b, o, idx, l, qm, km, status, p->inject, st) == cudaSuccess ? BRA_OK : BRA_ERR_CUDA;
+        });
     }
     s = run_route(d, p->dtype, Q, K, qm, km, idx, st);
     if (s != BRA_OK) return s;
-    return finish(run_attend(path, d, p->dtype, Q, K, V, idx, lce_w, lce_b, O, lse, status, st, true));
+    return attend_any_map(path, d, L, p->dtype, Q, K, V, idx, lce_w, lce_b, O, lse, w, st, true);
 }
 
 bra_status bra_backward(const bra_problem* p, const void* Q, const void* K, const void* V,
@@ -299,18 +299,19 @@ bra_status bra_backward(const bra_problem* p, const void* Q, const void* K, cons
     if (!backward_supported(d)) return BRA_ERR_UNSUPPORTED;
     char* w = static_cast<char*>(ws);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (!padded(d) || backward_any_map(d, p->dtype, p->impl)) {
+        const cudaError_t e = launch_backward(d, p->dtype, p->impl, Q, K, V, index, lce_w, lse, dO, dQ, dK, dV, d_lce_w, d_lce_b, w, L, st);
+        return e == cudaSuccess ? BRA_OK : BRA_ERR_CUDA;
+    }
     bool ok = true;
     Q = pad_in(d, L, w, 0, Q, st, &ok);
     K = pad_in(d, L, w, 1, K, st, &ok);
     V = pad_in(d, L, w, 2, V, st, &ok);
     dO = pad_in(d, L, w, 3, dO, st, &ok);          // zero in the padding: padded queries contribute nothing
-    if (padded(d)) {                               // lse of the padded queries: 0 (their scores are 0, their P finite)
-        float* lp = reinterpret_cast<float*>(w + L.pad_lse);
-        if (launch_pad_copy(lse, lp, (long long)d.B * d.heads, d.H0, d.W0, d.H, d.W, 4, true, st) != cudaSuccess) ok = false;
-        lse = lp;
-    }
+    float* lp = reinterpret_cast<float*>(w + L.pad_lse);   // lse of the padded queries: 0 (their scores are 0, their P finite)
+    if (launch_pad_copy(lse, lp, (long long)d.B * d.heads, d.H0, d.W0, d.H, d.W, 4, true, st) != cudaSuccess) ok = false;
     if (!ok) return BRA_ERR_CUDA;
-    cudaError_t e = launch_backward(d, p->dtype, p->impl, Q, K, V, index, lce_w, lse, dO, pad_out(d, L, w, 4, dQ),
+    cudaError_t e = launch_backward(on_copies(d), p->dtype, p->impl, Q, K, V, index, lce_w, lp, dO, pad_out(d, L, w, 4, dQ),
                                     pad_out(d, L, w, 5, dK), pad_out(d, L, w, 6, dV), d_lce_w, d_lce_b, w, L, st);
     if (e != cudaSuccess) return BRA_ERR_CUDA;
     crop_out(d, L, w, 4, dQ, st, &ok);

@@ -25,8 +25,9 @@ struct Dims {
     int heads_i;  // heads of the routing index: heads, or 1 with shared routing
     int lce;      // 1: add LCE
     float scale;  // softmax scale (Eq. 1)
-    // When S does not divide the caller's map, H and W above are the padded sizes (next multiples of S: the
-    // kernels only ever see a divisible map) and these are the caller's; equal to H, W otherwise.
+    // When S does not divide the caller's map, H and W above are the padded sizes (next multiples of S) and these
+    // the sizes of the map in memory.  Kernels that take any map address it by H0, W0 and read zeros outside; the
+    // others are given a padded copy and H0 = H, W0 = W.
     int H0, W0;
     int esize;    // bytes per element of Q, K, V, O
 };
@@ -75,8 +76,8 @@ cudaError_t launch_attend_simt(const Dims& d, int dtype, const void* Q, const vo
                                const int32_t* index, const float* lce_w, const float* lce_b,
                                void* O, float* lse, int32_t* status, cudaStream_t st);
 
-bool attend_mma_supported(const Dims& d, int dtype);
-cudaError_t launch_attend_mma(const Dims& d, const void* Q, const void* K, const void* V,
+bool attend_direct_supported(const Dims& d, int dtype);
+cudaError_t launch_attend_direct(const Dims& d, const void* Q, const void* K, const void* V,
                               const int32_t* index, const float* lce_w, const float* lce_b,
                               void* O, float* lse, int32_t* status, cudaStream_t st, bool after_own_kernel);
 
@@ -102,9 +103,9 @@ cudaError_t launch_attend_tc_wide(const Dims& d, const void* Q, const void* K, c
                                   const int32_t* index, const float* lce_w, const float* lce_b,
                                   void* O, float* lse, int32_t* status, cudaStream_t st, bool after_own_kernel);
 
-bool backward_mma_supported(const Dims& d, int dtype);
-cudaError_t launch_backward_mma(const Dims& d, const void* Q, const void* K, const void* V,
-                                const int32_t* index, const int32_t* inv_off, const int32_t* inv_list,
+bool backward_direct_supported(const Dims& d, int dtype);
+cudaError_t launch_backward_direct(const Dims& d, const void* Q, const void* K, const void* V,
+                                const int32_t* index, int32_t* inv_off, int32_t* inv_list,
                                 const float* lce_w, const float* lse, const void* dO,
                                 void* dQ, void* dK, void* dV, float* delta, int32_t* status, cudaStream_t st);
 
@@ -150,6 +151,8 @@ cudaError_t launch_lce_grad(const Dims& d, int dtype, const void* V, const void*
                             int32_t* status, cudaStream_t st);
 
 bool backward_supported(const Dims& d);
+// true if the kernels launch_backward() takes for this problem work on maps that S does not divide
+bool backward_any_map(const Dims& d, int dtype, int impl);
 // impl: the bra_impl the caller asked for
 cudaError_t launch_backward(const Dims& d, int dtype, int impl, const void* Q, const void* K, const void* V,
                             const int32_t* index, const float* lce_w, const float* lse,

@@ -1,0 +1,100 @@
+// Inverse routing index of one (image, routing head): for each key region the query regions whose rows list it, in
+// entry order (query region, then slot) - the fixed order of the dK / dV sums - as CSR.
+#pragma once
+
+#include "bra_internal.h"
+
+namespace bra {
+
+constexpr int INVERSE_BITS_MAX = 40 * 1024;     // bytes of the bit matrix up to which it is used
+
+inline int inverse_words(const Dims& d) { return (d.R + 31) / 32; }
+inline bool inverse_uses_bits(const Dims& d) { return (size_t)d.R * inverse_words(d) * 4 <= INVERSE_BITS_MAX; }
+inline size_t inverse_smem(const Dims& d) {
+    return sizeof(int32_t) * ((size_t)d.R + 2 + (inverse_uses_bits(d) ? (size_t)d.R * inverse_words(d) : 0));
+}
+
+// One CTA.  A row of the index seldom names a region twice, so what has to be inverted is a bit matrix (key region x
+// query region): every entry sets a bit (atomics whose order does not matter), every key region counts and lists its
+// bits in ascending order: work proportional to the entries, where comparing every entry with every region took
+// 109 us at 256 regions, topk 4 and 41 us at 64 regions, topk 12.  A repeated entry (a caller's index may have them)
+// or a matrix that does not fit sends the CTA to the comparisons: warp w takes key regions w, w + nwarps, ..., sweeps
+// the entries 32 at a time and finds its region's hits with a ballot.  Entries outside [0, R) are in no list.
+__device__ __forceinline__ void inverse_index_job(const int32_t* __restrict__ index, int32_t* __restrict__ inv_off,
+                                                  int32_t* __restrict__ inv_list, int bh, int32_t* sm, bool use_bits, const Dims& dm) {
+    const int tid = threadIdx.x, nthreads = blockDim.x;
+    const int lane = tid & 31, warp = tid >> 5, nwarps = nthreads >> 5;
+    const int entries = dm.R * dm.topk, words = (dm.R + 31) >> 5;
+    const int32_t* idx = index + (size_t)bh * entries;
+    int32_t* off = inv_off + (size_t)bh * (dm.R + 1);
+    int32_t* list = inv_list + (size_t)bh * entries;
+    int32_t* count = sm;                                    // [R + 1]
+    uint32_t* bits = reinterpret_cast<uint32_t*>(sm + dm.R + 2);
+    int* repeated = sm + dm.R + 1;
+    bool by_bits = use_bits;
+    if (use_bits) {
+        for (int e = tid; e < dm.R * words; e += nthreads) bits[e] = 0u;
+        if (tid == 0) *repeated = 0;
+        __syncthreads();
+        for (int e = tid; e < entries; e += nthreads) {
+            const int j = idx[e], i = e / dm.topk;
+            if (j >= 0 && j < dm.R && (atomicOr(&bits[j * words + (i >> 5)], 1u << (i & 31)) >> (i & 31) & 1u)) *repeated = 1;
+        }
+        __syncthreads();
+        by_bits = *repeated == 0;
+    }
+    if (by_bits) {
+        for (int j = tid; j < dm.R; j += nthreads) {
+            int n = 0;
+            for (int w = 0; w < words; ++w) n += __popc(bits[j * words + w]);
+            count[j] = n;
+        }
+    } else {
+        for (int j = warp; j < dm.R; j += nwarps) {
+            int n = 0;
+            for (int e0 = 0; e0 < entries; e0 += 32) {
+                const int e = e0 + lane;
+                n += __popc(__ballot_sync(0xffffffffu, e < entries && idx[e] == j));
+            }
+            if (lane == 0) count[j] = n;
+        }
+    }
+    __syncthreads();
+    if (warp == 0) {                                        // exclusive prefix sum
+        int run = 0;
+        for (int j0 = 0; j0 < dm.R; j0 += 32) {
+            const int j = j0 + lane, n = j < dm.R ? count[j] : 0;
+            int incl = n;
+#pragma unroll
+            for (int s = 1; s < 32; s <<= 1) {
+                const int o = __shfl_up_sync(0xffffffffu, incl, s);
+                if (lane >= s) incl += o;
+            }
+            if (j < dm.R) count[j] = run + incl - n;
+            run += __shfl_sync(0xffffffffu, incl, 31);
+        }
+        if (lane == 0) count[dm.R] = run;
+    }
+    __syncthreads();
+    for (int j = tid; j <= dm.R; j += nthreads) off[j] = count[j];
+    if (by_bits) {
+        for (int j = tid; j < dm.R; j += nthreads) {
+            int32_t* out = list + count[j];
+            for (int w = 0; w < words; ++w)
+                for (uint32_t m = bits[j * words + w]; m; m &= m - 1) *out++ = w * 32 + __ffs(m) - 1;
+        }
+    } else {
+        for (int j = warp; j < dm.R; j += nwarps) {
+            int pos = count[j];
+            for (int e0 = 0; e0 < entries; e0 += 32) {
+                const int e = e0 + lane;
+                const bool hit = e < entries && idx[e] == j;
+                const unsigned m = __ballot_sync(0xffffffffu, hit);
+                if (hit) list[pos + __popc(m & ((1u << lane) - 1u))] = e / dm.topk;
+                pos += __popc(m);
+            }
+        }
+    }
+}
+
+}  // namespace bra

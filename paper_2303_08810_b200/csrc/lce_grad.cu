@@ -192,10 +192,10 @@ static LceGradGeom lce_grad_geom(const Dims& d) {
     LceGradGeom best = {};
     long long best_cost = -1;
     for (int tr = slots; tr <= 2 * slots; tr += slots) {
-        for (int nx = (d.W + 39) / 40; nx <= d.W; ++nx) {
+        for (int nx = (d.W0 + 39) / 40; nx <= d.W0; ++nx) {
             LceGradGeom g;
             g.tr = tr;
-            g.tc = (d.W + nx - 1) / nx;
+            g.tc = (d.W0 + nx - 1) / nx;
             // two rows per warp: an odd number of columns puts them on different banks
             g.vcols = slots > 4 ? (g.tc + 4) | 1 : g.tc + 4;
             g.gcols = slots > 4 ? g.tc | 1 : g.tc;
@@ -205,8 +205,8 @@ static LceGradGeom lce_grad_geom(const Dims& d) {
             if (g.off_bar < red) g.off_bar = (red + 127) / 128 * 128;
             g.smem_bytes = g.off_bar + 16;
             if (g.smem_bytes > lg::SMEM_LIMIT || g.vcols > 256) continue;
-            g.tiles_x = (d.W + g.tc - 1) / g.tc;
-            g.tiles_y = (d.H + g.tr - 1) / g.tr;
+            g.tiles_x = (d.W0 + g.tc - 1) / g.tc;
+            g.tiles_y = (d.H0 + g.tr - 1) / g.tr;
             g.tiles = d.B * g.tiles_y * g.tiles_x;
             const long long cost = (long long)((g.tiles + ctas - 1) / ctas) * (tr / slots * (g.tc + 6) + 10);
             if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = g; }

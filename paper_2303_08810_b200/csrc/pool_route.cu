@@ -2,6 +2,8 @@
 // region affinity A^r = Q^r (K^r)^T (Eq. 4) and row-wise top-k index (Eq. 5).
 #include "bra_internal.h"
 
+#include <type_traits>
+
 namespace bra {
 
 // ------------------------------------------------------------------ pooling
@@ -13,8 +15,13 @@ namespace bra {
 template <typename T> struct Vec;
 template <> struct Vec<float> { static constexpr int n = 4; };
 template <> struct Vec<__nv_bfloat16> { static constexpr int n = 8; };
+template <int n>
+__device__ __forceinline__ void zero_row(float* v) {
+#pragma unroll
+    for (int i = 0; i < n; ++i) v[i] = 0.f;
+}
 
-template <typename T>
+template <typename T, bool ANY_MAP>
 __global__ void __launch_bounds__(256)
 pool_kernel(const T* __restrict__ Q, const T* __restrict__ K,
             float* __restrict__ q_mean, float* __restrict__ k_mean, Dims dm) {
@@ -26,8 +33,11 @@ pool_kernel(const T* __restrict__ Q, const T* __restrict__ K,
     float* dst = blockIdx.z == 0 ? q_mean : k_mean;
     const int cvecs = dm.C / VEC;
     const int items = dm.ws * cvecs;                       // one token row of the region
-    const size_t row_elems = (size_t)dm.W * dm.C;
-    const T* reg = src + ((size_t)b * dm.H + (size_t)ry * dm.hs) * row_elems + (size_t)rx * dm.ws * dm.C;
+    const size_t row_elems = (size_t)dm.W0 * dm.C;
+    const T* reg = src + ((size_t)b * dm.H0 + (size_t)ry * dm.hs) * row_elems + (size_t)rx * dm.ws * dm.C;
+    // rows and columns of the region that lie on the map (the rest is zero padding: it adds nothing)
+    const int rows = ANY_MAP ? min(dm.hs, dm.H0 - ry * dm.hs) : dm.hs;
+    const int on_map = ANY_MAP ? min(dm.ws, dm.W0 - rx * dm.ws) * cvecs : items;
 
     for (int it = threadIdx.x; it < items; it += blockDim.x) {
         float acc[VEC];
@@ -35,7 +45,7 @@ pool_kernel(const T* __restrict__ Q, const T* __restrict__ K,
         for (int i = 0; i < VEC; ++i) acc[i] = 0.f;
         const T* p = reg + (size_t)it * VEC;               // (x, cvec) in row 0: the region's row is contiguous
         int y = 0;
-        for (; y + 8 <= dm.hs; y += 8) {                    // eight loads in flight
+        for (; (!ANY_MAP || it < on_map) && y + 8 <= rows; y += 8) {      // eight loads in flight
             float v[8][VEC];
 #pragma unroll
             for (int u = 0; u < 8; ++u) load_row<VEC>(p + (size_t)(y + u) * row_elems, v[u]);
@@ -44,7 +54,7 @@ pool_kernel(const T* __restrict__ Q, const T* __restrict__ K,
 #pragma unroll
                 for (int i = 0; i < VEC; ++i) acc[i] += v[u][i];
         }
-        for (; y < dm.hs; ++y) {
+        for (; (!ANY_MAP || it < on_map) && y < rows; ++y) {
             float v[VEC];
             load_row<VEC>(p + (size_t)y * row_elems, v);
 #pragma unroll
@@ -67,7 +77,7 @@ pool_kernel(const T* __restrict__ Q, const T* __restrict__ K,
 // Regions eight token rows high: two threads per (column, 16-byte vector), four rows each, so that a
 // region is summed by twice the threads with half the work each (short CTAs turn over faster, which
 // is what this latency-bound scan needs).  Row halves are added lower half first.
-template <typename T>
+template <typename T, bool ANY_MAP>
 __global__ void __launch_bounds__(256)
 pool_split_kernel(const T* __restrict__ Q, const T* __restrict__ K,
                   float* __restrict__ q_mean, float* __restrict__ k_mean, Dims dm) {
@@ -79,13 +89,16 @@ pool_split_kernel(const T* __restrict__ Q, const T* __restrict__ K,
     float* dst = blockIdx.z == 0 ? q_mean : k_mean;
     const int cvecs = dm.C / VEC;
     const int items = dm.ws * cvecs;
-    const size_t row_elems = (size_t)dm.W * dm.C;
+    const size_t row_elems = (size_t)dm.W0 * dm.C;
     const int wsC = dm.ws * dm.C;
     const int it = threadIdx.x % items, yh = threadIdx.x / items;        // blockDim.x == 2 * items
-    const T* p = src + ((size_t)b * dm.H + (size_t)ry * dm.hs + 4 * yh) * row_elems + (size_t)rx * dm.ws * dm.C + (size_t)it * VEC;
+    const T* p = src + ((size_t)b * dm.H0 + (size_t)ry * dm.hs + 4 * yh) * row_elems + (size_t)rx * dm.ws * dm.C + (size_t)it * VEC;
     float v[4][VEC];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) load_row<VEC>(p + (size_t)u * row_elems, v[u]);
+    for (int u = 0; u < 4; ++u) {
+        if (!ANY_MAP || (ry * dm.hs + 4 * yh + u < dm.H0 && rx * dm.ws + it / cvecs < dm.W0)) load_row<VEC>(p + (size_t)u * row_elems, v[u]);
+        else zero_row<VEC>(v[u]);
+    }
     float acc[VEC];
 #pragma unroll
     for (int i = 0; i < VEC; ++i) acc[i] = 0.f;
@@ -111,7 +124,7 @@ pool_split_kernel(const T* __restrict__ Q, const T* __restrict__ K,
 // in order, the columns in order: the sums of pool_kernel, bit for bit - so nothing goes through shared memory
 // and a CTA moves a whole row of regions.  (One CTA per region is 6 272 CTAs of 64 threads and 2 KB each at the
 // stage-3 shape: the launch rate of CTAs, not HBM, sets its time.)
-template <typename T, int HS, int WS>
+template <typename T, int HS, int WS, bool ANY_MAP>
 __global__ void __launch_bounds__(512)
 pool_rows_kernel(const T* __restrict__ Q, const T* __restrict__ K,
                  float* __restrict__ q_mean, float* __restrict__ k_mean, Dims dm) {
@@ -122,14 +135,17 @@ pool_rows_kernel(const T* __restrict__ Q, const T* __restrict__ K,
     const int cvecs = dm.C / VEC;
     const int rx = threadIdx.x / cvecs, cv = threadIdx.x - rx * cvecs;
     if (rx >= dm.S) return;
-    const size_t row_elems = (size_t)dm.W * dm.C;
-    const T* p = src + ((size_t)b * dm.H + (size_t)ry * HS) * row_elems + (size_t)rx * dm.ws * dm.C + (size_t)cv * VEC;
+    const size_t row_elems = (size_t)dm.W0 * dm.C;
+    const T* p = src + ((size_t)b * dm.H0 + (size_t)ry * HS) * row_elems + (size_t)rx * dm.ws * dm.C + (size_t)cv * VEC;
     // all HS x WS loads of the thread are issued before the first sum
     float v[WS][HS][VEC];
 #pragma unroll
     for (int x = 0; x < WS; ++x)
 #pragma unroll
-        for (int y = 0; y < HS; ++y) load_row<VEC>(p + (size_t)y * row_elems + (size_t)x * dm.C, v[x][y]);
+        for (int y = 0; y < HS; ++y) {
+            if (!ANY_MAP || (ry * HS + y < dm.H0 && rx * WS + x < dm.W0)) load_row<VEC>(p + (size_t)y * row_elems + (size_t)x * dm.C, v[x][y]);
+            else zero_row<VEC>(v[x][y]);
+        }
     // the next kernel may be set up from here on: this CTA's loads are out
     pdl_launch_dependents();
     float total[VEC];
@@ -153,18 +169,25 @@ pool_rows_kernel(const T* __restrict__ Q, const T* __restrict__ K,
     store_row<VEC>(dst + ((size_t)b * dm.R + (size_t)ry * dm.S + rx) * dm.C + (size_t)cv * VEC, total);
 }
 
-template <typename T>
-static cudaError_t launch_pool_rows(const Dims& d, const void* Q, const void* K, float* q_mean, float* k_mean,
+template <typename T, bool ANY_MAP>
+static cudaError_t launch_pool_rows_t(const Dims& d, const void* Q, const void* K, float* q_mean, float* k_mean,
                                     cudaStream_t st) {
     const int threads = (d.S * (d.C / Vec<T>::n) + 31) / 32 * 32;
     const dim3 grid(d.S, 2, d.B);
     const T* q = static_cast<const T*>(Q);
     const T* k = static_cast<const T*>(K);
-    if (d.hs == 1) pool_rows_kernel<T, 1, 1><<<grid, threads, 0, st>>>(q, k, q_mean, k_mean, d);
-    else if (d.hs == 2) pool_rows_kernel<T, 2, 2><<<grid, threads, 0, st>>>(q, k, q_mean, k_mean, d);
-    else pool_rows_kernel<T, 4, 4><<<grid, threads, 0, st>>>(q, k, q_mean, k_mean, d);
+    if (d.hs == 1) pool_rows_kernel<T, 1, 1, ANY_MAP><<<grid, threads, 0, st>>>(q, k, q_mean, k_mean, d);
+    else if (d.hs == 2) pool_rows_kernel<T, 2, 2, ANY_MAP><<<grid, threads, 0, st>>>(q, k, q_mean, k_mean, d);
+    else pool_rows_kernel<T, 4, 4, ANY_MAP><<<grid, threads, 0, st>>>(q, k, q_mean, k_mean, d);
     count_launch();
     return cudaGetLastError();
+}
+
+template <typename T>
+static cudaError_t launch_pool_rows(const Dims& d, const void* Q, const void* K, float* q_mean, float* k_mean,
+                                    cudaStream_t st) {
+    return d.H == d.H0 && d.W == d.W0 ? launch_pool_rows_t<T, false>(d, Q, K, q_mean, k_mean, st)
+                                      : launch_pool_rows_t<T, true>(d, Q, K, q_mean, k_mean, st);
 }
 
 cudaError_t launch_pool(const Dims& d, int dtype, const void* Q, const void* K,
@@ -178,32 +201,31 @@ cudaError_t launch_pool(const Dims& d, int dtype, const void* Q, const void* K,
     int threads = ((items < 256 ? items : 256) + 31) / 32 * 32;
     size_t smem = sizeof(float) * (size_t)d.ws * d.C;
     dim3 grid(d.R, d.B, 2);
-    cudaError_t e;
     if (d.hs == 8 && 2 * items <= 256 && 2 * smem <= 48 * 1024) {
-        if (dtype == BRA_BF16)
-            pool_split_kernel<__nv_bfloat16><<<grid, 2 * items, 2 * smem, st>>>(
-                static_cast<const __nv_bfloat16*>(Q), static_cast<const __nv_bfloat16*>(K), q_mean, k_mean, d);
-        else
-            pool_split_kernel<float><<<grid, 2 * items, 2 * smem, st>>>(
-                static_cast<const float*>(Q), static_cast<const float*>(K), q_mean, k_mean, d);
+        const bool any = d.H != d.H0 || d.W != d.W0;
+        auto go = [&](auto* q, auto* k) {
+            typedef typename std::remove_const<typename std::remove_pointer<decltype(q)>::type>::type T;
+            if (any) pool_split_kernel<T, true><<<grid, 2 * items, 2 * smem, st>>>(q, k, q_mean, k_mean, d);
+            else pool_split_kernel<T, false><<<grid, 2 * items, 2 * smem, st>>>(q, k, q_mean, k_mean, d);
+        };
+        if (dtype == BRA_BF16) go(static_cast<const __nv_bfloat16*>(Q), static_cast<const __nv_bfloat16*>(K));
+        else go(static_cast<const float*>(Q), static_cast<const float*>(K));
         count_launch();
         return cudaGetLastError();
     }
-    if (dtype == BRA_BF16) {
-        if (smem > 48 * 1024 &&
-            (e = cudaFuncSetAttribute(pool_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-            return e;
-        pool_kernel<__nv_bfloat16><<<grid, threads, smem, st>>>(
-            static_cast<const __nv_bfloat16*>(Q), static_cast<const __nv_bfloat16*>(K), q_mean, k_mean, d);
-    } else {
-        if (smem > 48 * 1024 &&
-            (e = cudaFuncSetAttribute(pool_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-            return e;
-        pool_kernel<float><<<grid, threads, smem, st>>>(
-            static_cast<const float*>(Q), static_cast<const float*>(K), q_mean, k_mean, d);
-    }
-    count_launch();
-    return cudaGetLastError();
+    auto go = [&](auto* q, auto* k) -> cudaError_t {
+        typedef typename std::remove_const<typename std::remove_pointer<decltype(q)>::type>::type T;
+        auto kernel = d.H != d.H0 || d.W != d.W0 ? pool_kernel<T, true> : pool_kernel<T, false>;
+        if (smem > 48 * 1024) {
+            const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+        }
+        kernel<<<grid, threads, smem, st>>>(q, k, q_mean, k_mean, d);
+        count_launch();
+        return cudaGetLastError();
+    };
+    return dtype == BRA_BF16 ? go(static_cast<const __nv_bfloat16*>(Q), static_cast<const __nv_bfloat16*>(K))
+                             : go(static_cast<const float*>(Q), static_cast<const float*>(K));
 }
 
 // ------------------------------------------------------------------ routing

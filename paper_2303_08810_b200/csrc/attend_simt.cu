@@ -1,152 +1,233 @@
-// Token-to-token attention over the routed regions plus LCE on CUDA cores
-// (Eq. 6, Eq. 7 with Eq. 1), fp32 arithmetic throughout.  This is the path of
-// fp32 problems (an fp32 result to 1e-5 rules out bf16/tf32 tensor-core inputs)
-// and the fallback for shapes the tensor-core kernels do not take.
-//
-// One thread per (query token, head).  The gathered keys K^g / values V^g are
-// never formed: the thread walks the k listed regions and reads their tokens'
-// rows in place (a warp whose lanes share head and region reads each row once,
-// as a broadcast).  Softmax is the one-pass running-max form, rescaled once per
-// chunk of 8 keys.
-#include "bra_internal.h"
+// Token-to-token attention over the routed regions plus LCE on CUDA cores (Eq. 6, Eq. 7 with Eq. 1), fp32 arithmetic
+// throughout (simt_common.cuh has the mapping).  K^g / V^g are never formed: the routing index picks the rows that are
+// copied to (or, with a resident slice, read from) shared memory.  Softmax is the one-pass running-max form in blocks of
+// four keys per lane.
+// Bound: the FMA pipe, 2 D FMAs per query and key (a packed FMA every two cycles and scheduler).
+#include "simt_common.cuh"
 
 namespace bra {
 
+using namespace ptx;
+
 template <typename T, int D>
-__global__ void __launch_bounds__(128)
-attend_simt_kernel(const T* __restrict__ Q, const T* __restrict__ K, const T* __restrict__ V,
-                   const int32_t* __restrict__ index, const float* __restrict__ lce_w,
-                   const float* __restrict__ lce_b, T* __restrict__ O, float* __restrict__ lse,
-                   int32_t* __restrict__ status, Dims dm) {
-    // flat thread id -> (b, h, region i, token t in region), t fastest
-    const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long total = (long long)dm.B * dm.heads * dm.R * dm.n_r;
-    if (gid >= total) return;
-    const int t = (int)(gid % dm.n_r);
-    const int i = (int)((gid / dm.n_r) % dm.R);
-    const int h = (int)((gid / ((long long)dm.n_r * dm.R)) % dm.heads);
-    const int b = (int)(gid / ((long long)dm.n_r * dm.R * dm.heads));
-    const int y = (i / dm.S) * dm.hs + t / dm.ws;
-    const int x = (i % dm.S) * dm.ws + t % dm.ws;
-    const size_t img = (size_t)b * dm.N * dm.C;
-    const size_t tok = img + ((size_t)y * dm.W + x) * dm.C + (size_t)h * D;
+__global__ void __launch_bounds__(sk::THREADS, D <= 16 ? 8 : D <= 32 ? 6 : D == 64 ? 4 : 2)
+attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* __restrict__ Vg, const int32_t* index,
+                   const float* __restrict__ lce_w, const float* __restrict__ lce_b, T* __restrict__ Og, float* __restrict__ lse,
+                   int32_t* __restrict__ status, Dims dm, SimtGeom gm) {
+    constexpr int QT = D <= 32 ? 2 : 1, U = 4;                        // simt_rows()
+    extern __shared__ __align__(128) uint8_t smem[];
+    const uint32_t sbase = smem_u32(smem);
+    const int tid = threadIdx.x;
+    const int h = blockIdx.y, b = blockIdx.z;
+    const SimtChunk chunk = simt_chunk(dm, gm, blockIdx.x % gm.chunks);
+    const int r0 = blockIdx.x / gm.chunks * gm.rpc;
+    const int nreg = min(gm.rpc, dm.R - r0);
+    const int N0 = dm.H0 * dm.W0;
+    const size_t head = (size_t)b * N0 * dm.C + (size_t)h * D;
+    const T* Q = Qg + head; const T* K = Kg + head; const T* V = Vg + head;
+    float* s_w = reinterpret_cast<float*>(smem + gm.off_w);
+    if (dm.lce) simt_load_weights(s_w, lce_w + (size_t)h * D * 25, 25 * D);
+    if (gm.resident) {
+        simt_copy_rows<T, D>(sbase + gm.off_a, sbase + gm.off_b, gm.row, K, V, dm.C, dm.N, [&](int row) {
+            const int r = fdiv(row, dm.n_r, gm.mul_nr);
+            return simt_token(dm, gm, r, row - r * dm.n_r);
+        });
+        cp_async_commit();
+    }
+    pdl_wait();          // in bra_forward the launch may overlap the tail of the routing kernel
 
-    float q[D], o[D];
-    load_row<D>(Q + tok, q);
-#pragma unroll
-    for (int c = 0; c < D; ++c) { q[c] *= dm.scale; o[c] = 0.f; }
-    float m_run = -INFINITY, l_run = 0.f;
-
+    // ---- routing entries: -1 if out of range ----
     const int hi = dm.heads_i == 1 ? 0 : h;
-    const int32_t* row = index + (((size_t)b * dm.heads_i + hi) * dm.R + i) * dm.topk;
-    for (int m = 0; m < dm.topk; ++m) {
-        const int r = row[m];
-        if (r < 0 || r >= dm.R) { record_error(status, BRA_ERR_INDEX, r); continue; }
-        const int y0 = (r / dm.S) * dm.hs, x0 = (r % dm.S) * dm.ws;
-        for (int j0 = 0; j0 < dm.n_r; j0 += 8) {
-            const int nj = dm.n_r - j0 < 8 ? dm.n_r - j0 : 8;
-            float s[8];
-            float cmax = -INFINITY;
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                s[u] = -INFINITY;
-                if (u < nj) {
-                    const int j = j0 + u;
-                    const size_t kt = img + ((size_t)(y0 + j / dm.ws) * dm.W + x0 + j % dm.ws) * dm.C + (size_t)h * D;
-                    float kr[D];
-                    load_row<D>(K + kt, kr);
-                    float acc = 0.f;
-#pragma unroll
-                    for (int c = 0; c < D; ++c) acc = fmaf(q[c], kr[c], acc);
-                    s[u] = acc;
-                    cmax = fmaxf(cmax, acc);
-                }
-            }
-            const float m_new = fmaxf(m_run, cmax);
-            const float corr = expf(m_run - m_new);      // 0 on the first chunk (m_run = -inf)
-            l_run *= corr;
-#pragma unroll
-            for (int c = 0; c < D; ++c) o[c] *= corr;
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                if (u < nj) {
-                    const int j = j0 + u;
-                    const size_t kt = img + ((size_t)(y0 + j / dm.ws) * dm.W + x0 + j % dm.ws) * dm.C + (size_t)h * D;
-                    const float p = expf(s[u] - m_new);
-                    l_run += p;
-                    float vr[D];
-                    load_row<D>(V + kt, vr);
-#pragma unroll
-                    for (int c = 0; c < D; ++c) o[c] = fmaf(p, vr[c], o[c]);
-                }
-            }
-            m_run = m_new;
-        }
-    }
-    const float inv = l_run > 0.f ? 1.0f / l_run : 0.f;
-#pragma unroll
-    for (int c = 0; c < D; ++c) o[c] *= inv;
-    if (lse) lse[((size_t)b * dm.heads + h) * dm.N + (size_t)y * dm.W + x] = m_run + logf(l_run);
+    const int32_t* irow = index + (((size_t)b * dm.heads_i + hi) * dm.R + r0) * dm.topk;
+    int32_t* s_idx = reinterpret_cast<int32_t*>(smem + gm.off_idx);
+    const bool idx_staged = gm.rpc * dm.topk <= sk::IDX_MAX;
+    auto checked = [&](int e) -> int {
+        const int r = __ldcg(irow + e);  // coherent load: the index may come from the kernel this one overlaps
+        if (r < 0 || r >= dm.R) { record_error(status, BRA_ERR_INDEX, r); return -1; }
+        return r;
+    };
+    bool bad = !idx_staged;                                           // some key may not count
+    if (idx_staged) for (int e = tid; e < nreg * dm.topk; e += blockDim.x) { s_idx[e] = checked(e); bad = bad || s_idx[e] < 0; }
+    auto entry = [&](int e) -> int { return idx_staged ? s_idx[e] : checked(e); };
+    bad = __syncthreads_or(bad);
+    bool weighted = false;
+    int32_t* cnt = reinterpret_cast<int32_t*>(smem + gm.off_cnt);
+    if (gm.dense)
+        weighted = !simt_counts(cnt, nreg, dm.R, nreg * dm.topk, [&](int e) { const int r = s_idx[e]; return r < 0 ? -1 : e / dm.topk * dm.R + r; });
 
-    if (dm.lce) {
-        // LCE(V)[y,x,c] = sum_ij w[c,i,j] V[y+i-2, x+j-2, c], zero outside the map
-        const float* wh = lce_w + (size_t)h * D * 25;
-        for (int ti = 0; ti < 5; ++ti) {
-            const int yy = y + ti - 2;
-            if (yy < 0 || yy >= dm.H) continue;
-            for (int tj = 0; tj < 5; ++tj) {
-                const int xx = x + tj - 2;
-                if (xx < 0 || xx >= dm.W) continue;
-                float vr[D];
-                load_row<D>(V + img + ((size_t)yy * dm.W + xx) * dm.C + (size_t)h * D, vr);
+    // ---- this lane's rows: QT queries of one region, a share of the keys ----
+    const int KS = 1 << gm.ksl, ks = tid & (KS - 1), slot = tid >> gm.ksl;
+    const int rl_raw = fdiv(slot, gm.spr, gm.mul_spr);
+    const bool active = rl_raw < nreg;
+    const int rl = active ? rl_raw : 0;
+    const int t0 = active ? QT * (slot - rl_raw * gm.spr) : 0;
+    float q[QT][D], o[QT][D], m_run[QT], l_run[QT];
+    int tok[QT];
 #pragma unroll
-                for (int c = 0; c < D; ++c) o[c] = fmaf(__ldg(wh + c * 25 + ti * 5 + tj), vr[c], o[c]);
+    for (int x = 0; x < QT; ++x) {
+        tok[x] = active ? simt_row(dm, gm, chunk, r0 + rl, t0 + x) : -1;
+        ldg_row<T, D>(q[x], Q + (size_t)(tok[x] < 0 ? 0 : tok[x]) * dm.C, tok[x] >= 0, dm.scale);
+        m_run[x] = -INFINITY; l_run[x] = 0.f;
+#pragma unroll
+        for (int i = 0; i < D; ++i) o[x][i] = 0.f;
+    }
+    const int total = dm.topk * dm.n_r;
+
+    // keys [k0, k1) of every region; row_of(kk, wt): row in shared memory (-1: the key does not count) and its weight
+    auto walk = [&](uint32_t abase, int k0, int k1, auto&& row_of) {
+        const int blocks = (k1 - k0 + U * KS - 1) / (U * KS);
+#pragma unroll 1
+        for (int blk = 0; blk < blocks; ++blk) {
+            uint32_t at[U];
+            int row[U];
+            float s[QT][U], wt[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int kk = k0 + (blk * U + u) * KS + ks;
+                wt[u] = 1.f;
+                row[u] = kk < k1 ? row_of(kk, wt[u]) : -1;
+                at[u] = abase + (row[u] < 0 ? 0 : row[u]) * gm.row;
+            }
+            dots<T, QT, U, D>(s, q, at, gm.off_a);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int x = 0; x < QT; ++x)
+                    if (row[u] < 0) s[x][u] = -INFINITY;
+#pragma unroll
+            for (int x = 0; x < QT; ++x) {
+                const float mx = fmaxf(fmaxf(s[x][0], s[x][1]), fmaxf(s[x][2], s[x][3]));
+                if (mx > m_run[x]) {
+                    const float corr = expf(m_run[x] - mx);           // 0 on the first block (m_run = -inf)
+                    m_run[x] = mx;
+                    l_run[x] *= corr;
+#pragma unroll
+                    for (int i = 0; i < D; ++i) o[x][i] *= corr;
+                }
+                const float mn = m_run[x] == -INFINITY ? 0.f : m_run[x];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    s[x][u] = expf(s[x][u] - mn);
+                    if (weighted) s[x][u] *= wt[u];
+                    l_run[x] += s[x][u];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                float v[D];
+                lds_row<T, D>(v, at[u] + gm.off_b);
+#pragma unroll
+                for (int x = 0; x < QT; ++x) axpy(o[x], s[x][u], v);
             }
         }
-        if (lce_b) {
-#pragma unroll
-            for (int c = 0; c < D; ++c) o[c] += __ldg(lce_b + h * D + c);
+    };
+    if (gm.resident) {
+        cp_async_wait<0>();
+        __syncthreads();
+        walk(sbase, 0, gm.dense ? dm.N : total, [&](int kk, float& wt) -> int {
+            if (gm.dense && !weighted) return kk;
+            const int m = fdiv(kk, dm.n_r, gm.mul_nr);
+            if (gm.dense) {
+                const int n = cnt[rl * dm.R + m];
+                wt = (float)n;
+                return n > 0 ? kk : -1;
+            }
+            const int r = entry(rl * dm.topk + m);
+            return r < 0 ? -1 : r * dm.n_r + kk - m * dm.n_r;
+        });
+    } else {
+        const int nst = (total + gm.kps - 1) / gm.kps;
+        auto load_stage = [&](int st) {
+            const uint32_t base = sbase + (st & 1) * gm.stage_bytes;
+            simt_copy_rows<T, D>(base + gm.off_a, base + gm.off_b, gm.row, K, V, dm.C, nreg * gm.kps, [&](int row) {
+                const int l = fdiv(row, gm.kps, gm.mul_kps), kk = st * gm.kps + row - l * gm.kps;
+                if (kk >= total) return -1;
+                const int m = fdiv(kk, dm.n_r, gm.mul_nr);
+                const int r = entry(l * dm.topk + m);
+                return r >= 0 ? simt_token(dm, gm, r, kk - m * dm.n_r) : -1;
+            });
+            cp_async_commit();
+        };
+        load_stage(0);
+        for (int st = 0; st < nst; ++st) {
+            if (st + 1 < nst) { load_stage(st + 1); cp_async_wait<1>(); } else cp_async_wait<0>();
+            __syncthreads();
+            const int k0 = st * gm.kps, k1 = min(total, k0 + gm.kps);
+            walk(sbase + (st & 1) * gm.stage_bytes, k0, k1, [&](int kk, float&) -> int {
+                if (bad && entry(rl * dm.topk + fdiv(kk, dm.n_r, gm.mul_nr)) < 0) return -1;
+                return rl * gm.kps + kk - k0;
+            });
+            __syncthreads();
         }
     }
-    store_row<D>(O + tok, o);
+
+    // ---- merge the key shares; normalise; stage; lse ----
+#pragma unroll
+    for (int x = 0; x < QT; ++x) {
+        float m = m_run[x];
+        for (int off = 1; off < KS; off <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+        float f = KS == 1 || m == -INFINITY ? 1.f : expf(m_run[x] - m), l = l_run[x] * f;
+        for (int off = 1; off < KS; off <<= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
+        f *= l > 0.f ? 1.0f / l : 0.f;
+#pragma unroll
+        for (int i = 0; i < D; ++i) o[x][i] *= f;
+        if (lse && tok[x] >= 0 && ks == 0) lse[((size_t)b * dm.heads + h) * N0 + tok[x]] = m + logf(l);
+    }
+    int first, held;
+    sum_shares<QT, D>(o, gm.ksl, ks, &first, &held);
+    __syncthreads();
+    float* st = reinterpret_cast<float*>(smem + gm.off_st);
+    if (active)
+        for_held<QT, D>(o, first, held, [&](int x, int c, const float4& v) {
+            *reinterpret_cast<float4*>(st + (rl * QT * gm.spr + t0 + x) * (D + 4) + c) = v;
+        });
+    __syncthreads();
+    const float* bias = dm.lce && lce_b ? lce_b + h * D : nullptr;
+    if (dm.hs <= 2) simt_lce<T, D, 2, false>(st, s_w, bias, V, Og + head, r0, nreg, QT * gm.spr, chunk, dm, gm);
+    else simt_lce<T, D, 4, false>(st, s_w, bias, V, Og + head, r0, nreg, QT * gm.spr, chunk, dm, gm);
 }
 
 bool attend_simt_supported(const Dims& d) {
-    return d.d == 16 || d.d == 32 || d.d == 64 || d.d == 128;
+    return (d.d == 16 || d.d == 32 || d.d == 64 || d.d == 128) && simt_fits(d, SIMT_ATTEND);
 }
 
 template <typename T, int D>
 static cudaError_t launch_t(const Dims& d, const void* Q, const void* K, const void* V,
                             const int32_t* index, const float* lce_w, const float* lce_b,
-                            void* O, float* lse, int32_t* status, cudaStream_t st) {
-    const long long total = (long long)d.B * d.heads * d.R * d.n_r;
-    const unsigned blocks = (unsigned)((total + 127) / 128);
-    attend_simt_kernel<T, D><<<blocks, 128, 0, st>>>(
-        static_cast<const T*>(Q), static_cast<const T*>(K), static_cast<const T*>(V), index,
-        lce_w, lce_b, static_cast<T*>(O), lse, status, d);
+                            void* O, float* lse, int32_t* status, cudaStream_t st, bool after_own_kernel) {
+    const SimtGeom g = simt_geom(d, SIMT_ATTEND);
+    static PerDeviceMax smem_set;
+    if (g.smem_bytes > 48 * 1024) {
+        const cudaError_t e = smem_set.ensure(g.smem_bytes, [&] {
+            return cudaFuncSetAttribute(attend_simt_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, g.smem_bytes);
+        });
+        if (e != cudaSuccess) return e;
+    }
     count_launch();
-    return cudaGetLastError();
+    return launch_kernel(attend_simt_kernel<T, D>, dim3(g.gpi, d.heads, d.B), dim3(g.threads), (size_t)g.smem_bytes, st, after_own_kernel,
+                         static_cast<const T*>(Q), static_cast<const T*>(K), static_cast<const T*>(V), index, lce_w, lce_b,
+                         static_cast<T*>(O), lse, status, d, g);
 }
 
 template <typename T>
 static cudaError_t launch_d(const Dims& d, const void* Q, const void* K, const void* V,
                             const int32_t* index, const float* lce_w, const float* lce_b,
-                            void* O, float* lse, int32_t* status, cudaStream_t st) {
+                            void* O, float* lse, int32_t* status, cudaStream_t st, bool after_own_kernel) {
     switch (d.d) {
-        case 16:  return launch_t<T, 16>(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st);
-        case 32:  return launch_t<T, 32>(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st);
-        case 64:  return launch_t<T, 64>(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st);
-        case 128: return launch_t<T, 128>(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st);
+        case 16:  return launch_t<T, 16>(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel);
+        case 32:  return launch_t<T, 32>(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel);
+        case 64:  return launch_t<T, 64>(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel);
+        case 128: return launch_t<T, 128>(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel);
     }
     return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_attend_simt(const Dims& d, int dtype, const void* Q, const void* K, const void* V,
                                const int32_t* index, const float* lce_w, const float* lce_b,
-                               void* O, float* lse, int32_t* status, cudaStream_t st) {
+                               void* O, float* lse, int32_t* status, cudaStream_t st, bool after_own_kernel) {
     if (dtype == BRA_BF16)
-        return launch_d<__nv_bfloat16>(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st);
-    return launch_d<float>(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st);
+        return launch_d<__nv_bfloat16>(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel);
+    return launch_d<float>(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel);
 }
 
 }  // namespace bra

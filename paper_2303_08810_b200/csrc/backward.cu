@@ -1,161 +1,349 @@
-// Gradients of O = softmax(scale Q K^g^T) V^g + LCE(V) for a fixed routing
-// index (Eq. 7 with Eq. 1; the index of Eq. 5 is a constant), fp32 arithmetic
-// on CUDA cores.  Every sum has a fixed order: no atomics on the data path.
+// Gradients of O = softmax(scale Q K^g^T) V^g + LCE(V) for a fixed routing index (Eq. 7 with Eq. 1; the index of Eq. 5 is
+// a constant): choice of the kernels, and the kernels with fp32 arithmetic on CUDA cores (simt_common.cuh has their
+// mapping).  Every sum has a fixed order: no atomics on the data path.
 //
-//   1. inverse index (inverse_index.cuh): for each key region, the list (in (query region, slot)
-//      order) of query regions that routed to it, as CSR.
-//   2. dQ kernel, one thread per (query, head): delta = rowsum(P o dP), then
-//      dQ = scale * sum_j P_j (dP_j - delta) K_j; delta is kept for step 3.
-//   3. dK/dV kernel, one thread per (key token, head): walks the inverse index,
-//      recomputes P from the saved log-sum-exp, accumulates dK, dV, then adds
-//      the LCE adjoint dV += sum_ij w[c,i,j] dO[y-i+2, x-j+2, c].
+//   1. inverse index (inverse_index.cuh): for each key region, the list (in (query region, slot) order) of query regions
+//      that routed to it, as CSR; built by extra CTAs of the dQ launch.
+//   2. dQ kernel: delta = rowsum(P o dP) in a first walk over the keys, dQ = scale * sum_j P_j (dP_j - delta) K_j in a
+//      second; delta is kept for step 3.
+//   3. dK/dV kernel: rows are keys, the walk goes over the queries of the regions on the key region's list; P from the
+//      saved log-sum-exp; then the LCE adjoint dV += sum_ij w[c,i,j] dO[y-i+2, x-j+2, c].
 //   4. d_lce_w / d_lce_b: lce_grad.cu.
 // Steps 1 to 3 run on the tensor cores instead (backward_img.cu, backward_direct.cu) for bf16 with head dim 32 or 64.
 #include "inverse_index.cuh"
+#include "simt_common.cuh"
 
 namespace bra {
 
-// ------------------------------------------------------------ inverse index
-__global__ void __launch_bounds__(256)
-inverse_index_kernel(const int32_t* __restrict__ index, int32_t* __restrict__ inv_off,
-                     int32_t* __restrict__ inv_list, bool use_bits, Dims dm) {
-    extern __shared__ int32_t sm[];
-    inverse_index_job(index, inv_off, inv_list, blockIdx.x, sm, use_bits, dm);
-}
+using namespace ptx;
 
 // ------------------------------------------------------------ dQ and delta
+// Grid row 0 builds the inverse index, row 1 + h is head h.
 template <typename T, int D>
-__global__ void __launch_bounds__(128)
-bwd_dq_kernel(const T* __restrict__ Q, const T* __restrict__ K, const T* __restrict__ V,
-              const int32_t* __restrict__ index, const float* __restrict__ lse,
-              const T* __restrict__ dO, T* __restrict__ dQ, float* __restrict__ delta,
-              int32_t* __restrict__ status, Dims dm) {
-    const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long total = (long long)dm.B * dm.heads * dm.R * dm.n_r;
-    if (gid >= total) return;
-    const int t = (int)(gid % dm.n_r);
-    const int i = (int)((gid / dm.n_r) % dm.R);
-    const int h = (int)((gid / ((long long)dm.n_r * dm.R)) % dm.heads);
-    const int b = (int)(gid / ((long long)dm.n_r * dm.R * dm.heads));
-    const int y = (i / dm.S) * dm.hs + t / dm.ws;
-    const int x = (i % dm.S) * dm.ws + t % dm.ws;
-    const size_t img = (size_t)b * dm.N * dm.C;
-    const size_t tok = img + ((size_t)y * dm.W + x) * dm.C + (size_t)h * D;
-    const size_t stat = ((size_t)b * dm.heads + h) * dm.N + (size_t)y * dm.W + x;
-
-    float q[D], go[D], acc[D];
-    load_row<D>(Q + tok, q);
-    load_row<D>(dO + tok, go);
-#pragma unroll
-    for (int c = 0; c < D; ++c) { q[c] *= dm.scale; acc[c] = 0.f; }
-    const float l = lse[stat];
+__global__ void __launch_bounds__(sk::THREADS, D <= 16 ? 6 : 4)
+bwd_dq_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* __restrict__ Vg, const int32_t* __restrict__ index,
+                   const float* __restrict__ lse, const T* __restrict__ dOg, T* __restrict__ dQg, float* __restrict__ delta,
+                   int32_t* __restrict__ inv_off, int32_t* __restrict__ inv_list, bool inv_bits,
+                   int32_t* __restrict__ status, Dims dm, SimtGeom gm) {
+    constexpr int QT = D <= 32 ? 2 : 1, U = 2;                        // simt_rows()
+    extern __shared__ __align__(128) uint8_t smem[];
+    if (blockIdx.y == 0) {
+        if ((int)blockIdx.x < dm.heads_i)
+            inverse_index_job(index, inv_off, inv_list, blockIdx.z * dm.heads_i + blockIdx.x, reinterpret_cast<int32_t*>(smem), inv_bits, dm);
+        return;
+    }
+    if ((int)blockIdx.x >= gm.gpi) return;
+    const uint32_t sbase = smem_u32(smem);
+    const int tid = threadIdx.x;
+    const int h = blockIdx.y - 1, b = blockIdx.z;
+    const SimtChunk chunk = simt_chunk(dm, gm, blockIdx.x % gm.chunks);
+    const int r0 = blockIdx.x / gm.chunks * gm.rpc;
+    const int nreg = min(gm.rpc, dm.R - r0);
+    const int N0 = dm.H0 * dm.W0;
+    const size_t head = (size_t)b * N0 * dm.C + (size_t)h * D;
+    const T* K = Kg + head; const T* V = Vg + head;
+    if (gm.resident) {
+        simt_copy_rows<T, D>(sbase + gm.off_a, sbase + gm.off_b, gm.row, K, V, dm.C, dm.N, [&](int row) {
+            const int r = fdiv(row, dm.n_r, gm.mul_nr);
+            return simt_token(dm, gm, r, row - r * dm.n_r);
+        });
+        cp_async_commit();
+    }
     const int hi = dm.heads_i == 1 ? 0 : h;
-    const int32_t* row = index + (((size_t)b * dm.heads_i + hi) * dm.R + i) * dm.topk;
+    const int32_t* irow = index + (((size_t)b * dm.heads_i + hi) * dm.R + r0) * dm.topk;
+    int32_t* s_idx = reinterpret_cast<int32_t*>(smem + gm.off_idx);
+    const bool idx_staged = gm.rpc * dm.topk <= sk::IDX_MAX;
+    auto checked = [&](int e) -> int {
+        const int r = __ldg(irow + e);
+        if (r < 0 || r >= dm.R) { record_error(status, BRA_ERR_INDEX, r); return -1; }
+        return r;
+    };
+    bool bad = !idx_staged;
+    if (idx_staged) for (int e = tid; e < nreg * dm.topk; e += blockDim.x) { s_idx[e] = checked(e); bad = bad || s_idx[e] < 0; }
+    auto entry = [&](int e) -> int { return idx_staged ? s_idx[e] : checked(e); };
+    bad = __syncthreads_or(bad);
+    bool weighted = false;
+    int32_t* cnt = reinterpret_cast<int32_t*>(smem + gm.off_cnt);
+    if (gm.dense)
+        weighted = !simt_counts(cnt, nreg, dm.R, nreg * dm.topk, [&](int e) { const int r = s_idx[e]; return r < 0 ? -1 : e / dm.topk * dm.R + r; });
 
-    float dsum = 0.f;
-    for (int pass = 0; pass < 2; ++pass) {
-        for (int m = 0; m < dm.topk; ++m) {
-            const int r = row[m];
-            if (r < 0 || r >= dm.R) { record_error(status, BRA_ERR_INDEX, r); continue; }
-            const int y0 = (r / dm.S) * dm.hs, x0 = (r % dm.S) * dm.ws;
-            for (int j = 0; j < dm.n_r; ++j) {
-                const size_t kt = img + ((size_t)(y0 + j / dm.ws) * dm.W + x0 + j % dm.ws) * dm.C + (size_t)h * D;
-                float kr[D], vr[D];
-                load_row<D>(K + kt, kr);
-                load_row<D>(V + kt, vr);
-                float s = 0.f, dp = 0.f;
+    const int KS = 1 << gm.ksl, ks = tid & (KS - 1), slot = tid >> gm.ksl;
+    const int rl_raw = fdiv(slot, gm.spr, gm.mul_spr);
+    const bool active = rl_raw < nreg;
+    const int rl = active ? rl_raw : 0;
+    const int t0 = active ? QT * (slot - rl_raw * gm.spr) : 0;
+    float q[QT][D], go[QT][D], acc[QT][D], l[QT], dsum[QT];
+    int tok[QT];
+    const float* lse_h = lse + ((size_t)b * dm.heads + h) * N0;
 #pragma unroll
-                for (int c = 0; c < D; ++c) { s = fmaf(q[c], kr[c], s); dp = fmaf(go[c], vr[c], dp); }
-                const float p = expf(s - l);
-                if (pass == 0) {
-                    dsum = fmaf(p, dp, dsum);
-                } else {
-                    const float ds = p * (dp - dsum);
+    for (int x = 0; x < QT; ++x) {
+        tok[x] = active ? simt_row(dm, gm, chunk, r0 + rl, t0 + x) : -1;
+        const size_t at = head + (size_t)(tok[x] < 0 ? 0 : tok[x]) * dm.C;
+        ldg_row<T, D>(q[x], Qg + at, tok[x] >= 0, dm.scale);
+        ldg_row<T, D>(go[x], dOg + at, tok[x] >= 0, 1.f);
+        l[x] = tok[x] >= 0 ? __ldg(lse_h + tok[x]) : 0.f;
+        dsum[x] = 0.f;
 #pragma unroll
-                    for (int c = 0; c < D; ++c) acc[c] = fmaf(ds, kr[c], acc[c]);
+        for (int i = 0; i < D; ++i) acc[x][i] = 0.f;
+    }
+    const int total = dm.topk * dm.n_r;
+    auto walk = [&](uint32_t abase, int k0, int k1, bool second, auto&& row_of) {
+        const int blocks = (k1 - k0 + U * KS - 1) / (U * KS);
+#pragma unroll 1
+        for (int blk = 0; blk < blocks; ++blk) {
+uint32_t at[U];
+            int row[U];
+            float s[QT][U], dp[QT][U], wt[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int kk = k0 + (blk * U + u) * KS + ks;
+                wt[u] = 1.f;
+                row[u] = kk < k1 ? row_of(kk, wt[u]) : -1;
+                at[u] = abase + (row[u] < 0 ? 0 : row[u]) * gm.row;
+            }
+            dots<T, QT, U, D>(s, q, at, gm.off_a);
+            dots<T, QT, U, D>(dp, go, at, gm.off_b);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int x = 0; x < QT; ++x) {
+                    s[x][u] = row[u] < 0 ? 0.f : expf(s[x][u] - l[x]);
+                    if (weighted) s[x][u] *= wt[u];
+                    if (!second) dsum[x] = fmaf(s[x][u], dp[x][u], dsum[x]);
+                    else s[x][u] *= dp[x][u] - dsum[x];
                 }
+            if (!second) continue;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                float k[D];
+                lds_row<T, D>(k, at[u] + gm.off_a);
+#pragma unroll
+                for (int x = 0; x < QT; ++x) axpy(acc[x], s[x][u], k);
             }
         }
-    }
-    delta[stat] = dsum;
+    };
+    auto end_of_first = [&]() {
+        for (int off = 1; off < KS; off <<= 1)
 #pragma unroll
-    for (int c = 0; c < D; ++c) acc[c] *= dm.scale;
-    store_row<D>(dQ + tok, acc);
+            for (int x = 0; x < QT; ++x) dsum[x] += __shfl_xor_sync(0xffffffffu, dsum[x], off);
+    };
+    if (gm.resident) {
+        cp_async_wait<0>();
+        __syncthreads();
+#pragma unroll 1
+        for (int sweep = 0; sweep < 2; ++sweep) {
+            walk(sbase, 0, gm.dense ? dm.N : total, sweep == 1, [&](int kk, float& wt) -> int {
+                if (gm.dense && !weighted) return kk;
+                const int m = fdiv(kk, dm.n_r, gm.mul_nr);
+                if (gm.dense) {
+                    const int n = cnt[rl * dm.R + m];
+                    wt = (float)n;
+                    return n > 0 ? kk : -1;
+                }
+                const int r = entry(rl * dm.topk + m);
+                return r < 0 ? -1 : r * dm.n_r + kk - m * dm.n_r;
+            });
+            if (sweep == 0) end_of_first();
+        }
+    } else {
+        const int nst = (total + gm.kps - 1) / gm.kps;
+        auto load_stage = [&](int it) {
+            const int st = it < nst ? it : it - nst;
+            const uint32_t base = sbase + (it & 1) * gm.stage_bytes;
+            simt_copy_rows<T, D>(base + gm.off_a, base + gm.off_b, gm.row, K, V, dm.C, nreg * gm.kps, [&](int row) {
+                const int lr = fdiv(row, gm.kps, gm.mul_kps), kk = st * gm.kps + row - lr * gm.kps;
+                if (kk >= total) return -1;
+                const int m = fdiv(kk, dm.n_r, gm.mul_nr);
+                const int r = entry(lr * dm.topk + m);
+                return r >= 0 ? simt_token(dm, gm, r, kk - m * dm.n_r) : -1;
+            });
+            cp_async_commit();
+        };
+        load_stage(0);
+        for (int it = 0; it < 2 * nst; ++it) {
+            if (it + 1 < 2 * nst) { load_stage(it + 1); cp_async_wait<1>(); } else cp_async_wait<0>();
+            __syncthreads();
+            const int k0 = (it < nst ? it : it - nst) * gm.kps, k1 = min(total, k0 + gm.kps);
+            walk(sbase + (it & 1) * gm.stage_bytes, k0, k1, it >= nst, [&](int kk, float&) -> int {
+                if (bad && entry(rl * dm.topk + fdiv(kk, dm.n_r, gm.mul_nr)) < 0) return -1;
+                return rl * gm.kps + kk - k0;
+            });
+            if (it == nst - 1) end_of_first();
+            __syncthreads();
+        }
+    }
+    int first, held;
+    sum_shares<QT, D>(acc, gm.ksl, ks, &first, &held);
+    pdl_launch_dependents();
+    if (!active) return;
+    for_held<QT, D>(acc, first, held, [&](int x, int c, const float4& v) {
+        const int tk = QT == 2 && x == 1 ? tok[QT - 1] : tok[0];
+        if (tk >= 0) store4(dQg + head + (size_t)tk * dm.C + c, make_float4(v.x * dm.scale, v.y * dm.scale, v.z * dm.scale, v.w * dm.scale));
+    });
+#pragma unroll
+    for (int x = 0; x < QT; ++x)
+        if (tok[x] >= 0 && ks == 0) delta[((size_t)b * dm.heads + h) * N0 + tok[x]] = dsum[x];
 }
 
 // ------------------------------------------------------------ dK, dV
 template <typename T, int D>
-__global__ void __launch_bounds__(128)
-bwd_dkv_kernel(const T* __restrict__ Q, const T* __restrict__ K, const T* __restrict__ V,
-               const int32_t* __restrict__ inv_off, const int32_t* __restrict__ inv_list,
-               const float* __restrict__ lse, const float* __restrict__ delta,
-               const T* __restrict__ dO, const float* __restrict__ lce_w,
-               T* __restrict__ dK, T* __restrict__ dV, Dims dm) {
-    const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long total = (long long)dm.B * dm.heads * dm.R * dm.n_r;
-    if (gid >= total) return;
-    const int t = (int)(gid % dm.n_r);
-    const int jr = (int)((gid / dm.n_r) % dm.R);          // key region
-    const int h = (int)((gid / ((long long)dm.n_r * dm.R)) % dm.heads);
-    const int b = (int)(gid / ((long long)dm.n_r * dm.R * dm.heads));
-    const int y = (jr / dm.S) * dm.hs + t / dm.ws;
-    const int x = (jr % dm.S) * dm.ws + t % dm.ws;
-    const size_t img = (size_t)b * dm.N * dm.C;
-    const size_t tok = img + ((size_t)y * dm.W + x) * dm.C + (size_t)h * D;
-
-    float kr[D], vr[D], gk[D], gv[D];
-    load_row<D>(K + tok, kr);
-    load_row<D>(V + tok, vr);
-#pragma unroll
-    for (int c = 0; c < D; ++c) { kr[c] *= dm.scale; gk[c] = 0.f; gv[c] = 0.f; }
+__global__ void __launch_bounds__(sk::THREADS, D <= 16 ? 6 : 4)
+bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* __restrict__ Vg, const int32_t* inv_off,
+                    const int32_t* inv_list, const float* __restrict__ lse, const float* delta, const T* __restrict__ dOg,
+                    const float* __restrict__ lce_w, T* __restrict__ dKg, T* __restrict__ dVg, Dims dm, SimtGeom gm) {
+    constexpr int U = 2;
+    extern __shared__ __align__(128) uint8_t smem[];
+    const uint32_t sbase = smem_u32(smem);
+    const int tid = threadIdx.x;
+    const int h = blockIdx.y, b = blockIdx.z;
+    const SimtChunk chunk = simt_chunk(dm, gm, blockIdx.x % gm.chunks);
+    const int r0 = blockIdx.x / gm.chunks * gm.rpc;
+    const int nreg = min(gm.rpc, dm.R - r0);
+    const int N0 = dm.H0 * dm.W0;
+    const size_t head = (size_t)b * N0 * dm.C + (size_t)h * D;
+    const T* Q = Qg + head; const T* dO = dOg + head;
+    float* s_w = reinterpret_cast<float*>(smem + gm.off_w);
+    if (dm.lce) simt_load_weights(s_w, lce_w + (size_t)h * D * 25, 25 * D);
+    if (gm.resident) {
+        simt_copy_rows<T, D>(sbase + gm.off_a, sbase + gm.off_b, gm.row, Q, dO, dm.C, dm.N, [&](int row) {
+            const int r = fdiv(row, dm.n_r, gm.mul_nr);
+            return simt_token(dm, gm, r, row - r * dm.n_r);
+        });
+        cp_async_commit();
+    }
+    pdl_wait();          // delta and the inverse index come from the dQ kernel
 
     const int hi = dm.heads_i == 1 ? 0 : h;
-    const size_t bh = (size_t)b * dm.heads_i + hi;
-    const int32_t* off = inv_off + bh * (dm.R + 1);
-    const int32_t* list = inv_list + bh * dm.R * dm.topk;
-    const size_t stat0 = ((size_t)b * dm.heads + h) * dm.N;
-    for (int e = off[jr]; e < off[jr + 1]; ++e) {
-        const int i = list[e];                            // a query region that lists jr
-        const int y0 = (i / dm.S) * dm.hs, x0 = (i % dm.S) * dm.ws;
-        for (int tq = 0; tq < dm.n_r; ++tq) {
-            const int yq = y0 + tq / dm.ws, xq = x0 + tq % dm.ws;
-            const size_t qt = img + ((size_t)yq * dm.W + xq) * dm.C + (size_t)h * D;
-            float qr[D], go[D];
-            load_row<D>(Q + qt, qr);
-            load_row<D>(dO + qt, go);
-            float s = 0.f, dp = 0.f;
-#pragma unroll
-            for (int c = 0; c < D; ++c) { s = fmaf(qr[c], kr[c], s); dp = fmaf(go[c], vr[c], dp); }
-            const size_t st = stat0 + (size_t)yq * dm.W + xq;
-            const float p = expf(s - lse[st]);
-            const float ds = p * (dp - delta[st]);
-#pragma unroll
-            for (int c = 0; c < D; ++c) { gk[c] = fmaf(ds, qr[c], gk[c]); gv[c] = fmaf(p, go[c], gv[c]); }
-        }
+    const size_t bhi = (size_t)b * dm.heads_i + hi;
+    const int32_t* offs = inv_off + bhi * (dm.R + 1) + r0;           // [nreg + 1]
+    const int32_t* list = inv_list + bhi * dm.R * dm.topk;
+    const float* lse_h = lse + ((size_t)b * dm.heads + h) * N0;
+    const float* delta_h = delta + ((size_t)b * dm.heads + h) * N0;
+    const int KS = 1 << gm.ksl, ks = tid & (KS - 1), slot = tid >> gm.ksl;
+    const int rl_raw = fdiv(slot, gm.spr, gm.mul_spr);
+    const bool active = rl_raw < nreg;
+    const int rl = active ? rl_raw : 0;
+    const int e0 = __ldcg(offs + rl), mine = (__ldcg(offs + rl + 1) - e0) * dm.n_r;     // queries of this lane's key region
+    const int warp_total = __reduce_max_sync(0xffffffffu, mine);
+    bool weighted = false;
+    int32_t* cnt = reinterpret_cast<int32_t*>(smem + gm.off_cnt);
+    if (gm.dense) {
+        __syncthreads();
+        const int first = __ldcg(offs), n = __ldcg(offs + nreg) - first;
+        weighted = !simt_counts(cnt, nreg, dm.R, n, [&](int e) {
+            int l = 0;
+            while (l + 1 < nreg && __ldcg(offs + l + 1) - first <= e) ++l;
+            return l * dm.R + __ldcg(list + first + e);
+        });
     }
+    const int t0 = active ? slot - rl_raw * gm.spr : 0;
+    const int tok = active ? simt_row(dm, gm, chunk, r0 + rl, t0) : -1;
+    float kr[D], vr[D], gk[1][D], gv[1][D];
+    {
+        const size_t at = head + (size_t)(tok < 0 ? 0 : tok) * dm.C;
+        ldg_row<T, D>(kr, Kg + at, tok >= 0, dm.scale);
+        ldg_row<T, D>(vr, Vg + at, tok >= 0, 1.f);
 #pragma unroll
-    for (int c = 0; c < D; ++c) gk[c] *= dm.scale;
-    if (dm.lce) {
-        const float* wh = lce_w + (size_t)h * D * 25;
-        for (int ti = 0; ti < 5; ++ti) {
-            const int yy = y - ti + 2;
-            if (yy < 0 || yy >= dm.H) continue;
-            for (int tj = 0; tj < 5; ++tj) {
-                const int xx = x - tj + 2;
-                if (xx < 0 || xx >= dm.W) continue;
-                float go[D];
-                load_row<D>(dO + img + ((size_t)yy * dm.W + xx) * dm.C + (size_t)h * D, go);
+        for (int i = 0; i < D; ++i) gk[0][i] = gv[0][i] = 0.f;
+    }
+    // statistics of a row: lse and delta; a row that does not count has lse = inf (P = 0); a row of the zero padding has
+    // zero Q and dO and lse = delta = 0 and adds nothing
+    auto walk = [&](int stage, int k0, int k1, auto&& row_of) {
+        const uint32_t abase = sbase + stage * gm.stage_bytes;
+        const int blocks = (k1 - k0 + U * KS - 1) / (U * KS);
+#pragma unroll 1
+        for (int blk = 0; blk < blocks; ++blk) {
 #pragma unroll
-                for (int c = 0; c < D; ++c) gv[c] = fmaf(__ldg(wh + c * 25 + ti * 5 + tj), go[c], gv[c]);
+            for (int u = 0; u < U; ++u) {
+                const int kk = k0 + (blk * U + u) * KS + ks;
+                float wt = 1.f;
+                const int row = kk < k1 ? row_of(kk, wt) : -1;
+                const int rr = row < 0 ? 0 : row;
+                const uint32_t at = abase + rr * gm.row;
+                const float2 stat = lds_f32x2(abase + gm.off_stat + rr * 8);
+                float g[D], qv[D];
+                lds_row<T, D>(g, at + gm.off_b);
+                const float dp = dot4(vr, g);
+                lds_row<T, D>(qv, at + gm.off_a);
+                float p = row < 0 ? 0.f : expf(dot(qv, kr) - stat.x);
+                if (weighted) p *= wt;
+                axpy(gk[0], p * (dp - stat.y), qv);
+                axpy(gv[0], p, g);
             }
         }
+    };
+    if (gm.resident) {
+        float2* stat = reinterpret_cast<float2*>(smem + gm.off_stat);
+        for (int row = tid; row < dm.N; row += blockDim.x) {
+            const int r = fdiv(row, dm.n_r, gm.mul_nr);
+            const int tk = simt_token(dm, gm, r, row - r * dm.n_r);
+            stat[row] = tk >= 0 ? make_float2(__ldg(lse_h + tk), __ldcg(delta_h + tk)) : make_float2(0.f, 0.f);
+        }
+        cp_async_wait<0>();
+        __syncthreads();
+        walk(0, 0, gm.dense ? dm.N : warp_total, [&](int kk, float& wt) -> int {
+            if (gm.dense && !weighted) return kk;
+            const int m = fdiv(kk, dm.n_r, gm.mul_nr);
+            if (gm.dense) {
+                const int n = cnt[rl * dm.R + m];
+                wt = (float)n;
+                return n > 0 ? kk : -1;
+            }
+            return kk < mine ? __ldcg(list + e0 + m) * dm.n_r + kk - m * dm.n_r : -1;
+        });
+    } else {
+        int most = 0;
+        for (int l = 0; l < nreg; ++l) most = max(most, __ldcg(offs + l + 1) - __ldcg(offs + l));
+        most *= dm.n_r;
+        const int nst = (most + gm.kps - 1) / gm.kps;
+        auto load_stage = [&](int st) {
+            const uint32_t base = sbase + (st & 1) * gm.stage_bytes;
+            float2* stat = reinterpret_cast<float2*>(smem + (st & 1) * gm.stage_bytes + gm.off_stat);
+            simt_copy_rows<T, D>(base + gm.off_a, base + gm.off_b, gm.row, Q, dO, dm.C, nreg * gm.kps, [&](int row) {
+                const int lr = fdiv(row, gm.kps, gm.mul_kps), kk = st * gm.kps + row - lr * gm.kps;
+                const int s0 = __ldcg(offs + lr);
+                const int m = fdiv(kk, dm.n_r, gm.mul_nr);
+                int tk = -1;
+                float2 v = make_float2(INFINITY, 0.f);
+                if (s0 + m < __ldcg(offs + lr + 1)) {
+                    tk = simt_token(dm, gm, __ldcg(list + s0 + m), kk - m * dm.n_r);
+                    v = tk >= 0 ? make_float2(__ldg(lse_h + tk), __ldcg(delta_h + tk)) : make_float2(0.f, 0.f);
+                }
+                if ((threadIdx.x & 3) == 0) stat[row] = v;
+                return tk;
+            });
+            cp_async_commit();
+        };
+        if (nst > 0) load_stage(0);
+        for (int st = 0; st < nst; ++st) {
+            if (st + 1 < nst) { load_stage(st + 1); cp_async_wait<1>(); } else cp_async_wait<0>();
+            __syncthreads();
+            const int k0 = st * gm.kps, k1 = min(warp_total, k0 + gm.kps);
+            if (k0 < k1) walk(st & 1, k0, k1, [&](int kk, float&) -> int { return rl * gm.kps + kk - k0; });
+            __syncthreads();
+        }
     }
-    store_row<D>(dK + tok, gk);
-    store_row<D>(dV + tok, gv);
+    int first, held;
+    sum_shares<1, D>(gk, gm.ksl, ks, &first, &held);
+    sum_shares<1, D>(gv, gm.ksl, ks, &first, &held);
+    cp_async_wait<0>();
+    __syncthreads();
+    float* st = reinterpret_cast<float*>(smem + gm.off_st);
+    if (tok >= 0) {
+        for_held<1, D>(gk, first, held, [&](int, int c, const float4& v) {
+            store4(dKg + head + (size_t)tok * dm.C + c, make_float4(v.x * dm.scale, v.y * dm.scale, v.z * dm.scale, v.w * dm.scale));
+        });
+        for_held<1, D>(gv, first, held, [&](int, int c, const float4& v) {
+            *reinterpret_cast<float4*>(st + (rl * gm.spr + t0) * (D + 4) + c) = v;
+        });
+    }
+    __syncthreads();
+    if (dm.hs <= 2) simt_lce<T, D, 2, true>(st, s_w, nullptr, dO, dVg + head, r0, nreg, gm.spr, chunk, dm, gm);
+    else simt_lce<T, D, 4, true>(st, s_w, nullptr, dO, dVg + head, r0, nreg, gm.spr, chunk, dm, gm);
 }
 
 bool backward_supported(const Dims& d) {
-    return (d.d == 16 || d.d == 32 || d.d == 64) && d.R <= 1000;
+    return (d.d == 16 || d.d == 32 || d.d == 64) && d.R <= 1000 && simt_fits(d, SIMT_DQ) && simt_fits(d, SIMT_DKV);
 }
 
 enum Family { FAMILY_SIMT, FAMILY_DIRECT, FAMILY_IMG };
@@ -169,7 +357,7 @@ static Family choose_family(const Dims& d, int dtype, int impl) {
         return FAMILY_IMG;
     return backward_direct_supported(d, dtype) ? FAMILY_DIRECT : FAMILY_SIMT;
 }
-bool backward_any_map(const Dims& d, int dtype, int impl) { return choose_family(d, dtype, impl) == FAMILY_DIRECT; }
+bool backward_any_map(const Dims& d, int dtype, int impl) { return choose_family(d, dtype, impl) != FAMILY_IMG; }
 
 // The LCE weight gradient needs only V and dO, the attention gradients need neither of its results: the two
 // run side by side (helper stream of bra_internal.h; everything stays on the caller's stream if there is none).
@@ -211,19 +399,29 @@ static cudaError_t launch_bwd_t(const Dims& d, int impl, const void* Q, const vo
         if ((e = launch_backward_direct(d, Q, K, V, index, inv_off, inv_list, lce_w, lse, dO, dQ, dK, dV,
                                         delta, status, st)) != cudaSuccess) return e;
     } else {
-        inverse_index_kernel<<<d.B * d.heads_i, 256, inverse_smem(d), st>>>(index, inv_off, inv_list, inverse_uses_bits(d), d);
+        SimtGeom g = simt_geom(d, SIMT_DQ);
+        const int inv = (int)inverse_smem(d);
+        if (g.smem_bytes < inv) g.smem_bytes = inv;
+        static PerDeviceMax set_q, set_kv;
+        if (g.smem_bytes > 48 * 1024 && (e = set_q.ensure(g.smem_bytes, [&] {
+                return cudaFuncSetAttribute(bwd_dq_simt_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, g.smem_bytes);
+            })) != cudaSuccess)
+            return e;
+        e = launch_kernel(bwd_dq_simt_kernel<T, D>, dim3(g.gpi > d.heads_i ? g.gpi : d.heads_i, d.heads + 1, d.B), dim3(g.threads),
+                          (size_t)g.smem_bytes, st, false, q, k, v, index, lse, go, static_cast<T*>(dQ), delta, inv_off, inv_list,
+                          inverse_uses_bits(d), status, d, g);
         count_launch();
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        const long long total = (long long)d.B * d.heads * d.R * d.n_r;
-        const unsigned blocks = (unsigned)((total + 127) / 128);
-        bwd_dq_kernel<T, D><<<blocks, 128, 0, st>>>(q, k, v, index, lse, go, static_cast<T*>(dQ), delta, status, d);
+        if (e != cudaSuccess) return e;
+        const SimtGeom gk = simt_geom(d, SIMT_DKV);
+        if (gk.smem_bytes > 48 * 1024 && (e = set_kv.ensure(gk.smem_bytes, [&] {
+                return cudaFuncSetAttribute(bwd_dkv_simt_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, gk.smem_bytes);
+            })) != cudaSuccess)
+            return e;
+        e = launch_kernel(bwd_dkv_simt_kernel<T, D>, dim3(gk.gpi, d.heads, d.B), dim3(gk.threads), (size_t)gk.smem_bytes, st, true,
+                          q, k, v, static_cast<const int32_t*>(inv_off), static_cast<const int32_t*>(inv_list), lse,
+                          static_cast<const float*>(delta), go, lce_w, static_cast<T*>(dK), static_cast<T*>(dV), d, gk);
         count_launch();
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-
-        bwd_dkv_kernel<T, D><<<blocks, 128, 0, st>>>(q, k, v, inv_off, inv_list, lse, delta, go, lce_w,
-                                                     static_cast<T*>(dK), static_cast<T*>(dV), d);
-        count_launch();
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if (e != cudaSuccess) return e;
     }
 
     if (ss && cudaStreamWaitEvent(st, ss->join, 0) != cudaSuccess) return cudaErrorUnknown;

@@ -138,7 +138,7 @@ static Path choose_attend(const Dims& d, int dtype, int impl) {
 }
 
 // Paths whose kernels take a map that S does not divide as it is (the others get a zero-padded copy).
-static bool any_map(Path path) { return path == PATH_DIRECT; }
+static bool any_map(Path path) { return path == PATH_DIRECT || path == PATH_SIMT; }
 
 static bra_status run_route(const Dims& d, int dtype, const void* Q, const void* K,
                             float* q_mean, float* k_mean, int32_t* index, cudaStream_t st) {
@@ -153,7 +153,7 @@ static bra_status run_attend(Path path, const Dims& d, int dtype, const void* Q,
                              cudaStream_t st, bool after_own_kernel) {
     cudaError_t e = cudaErrorInvalidValue;
     switch (path) {
-        case PATH_SIMT: e = launch_attend_simt(d, dtype, Q, K, V, index, lce_w, lce_b, O, lse, status, st); break;
+        case PATH_SIMT: e = launch_attend_simt(d, dtype, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel); break;
         case PATH_DIRECT:  e = launch_attend_direct(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel); break;
         case PATH_TC:   e = launch_attend_tc(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel); break;
         case PATH_TC_WIDE: e = launch_attend_tc_wide(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel); break;

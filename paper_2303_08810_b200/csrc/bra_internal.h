@@ -74,7 +74,7 @@ bool route_supported(const Dims& d);
 bool attend_simt_supported(const Dims& d);
 cudaError_t launch_attend_simt(const Dims& d, int dtype, const void* Q, const void* K, const void* V,
                                const int32_t* index, const float* lce_w, const float* lce_b,
-                               void* O, float* lse, int32_t* status, cudaStream_t st);
+                               void* O, float* lse, int32_t* status, cudaStream_t st, bool after_own_kernel);
 
 bool attend_direct_supported(const Dims& d, int dtype);
 cudaError_t launch_attend_direct(const Dims& d, const void* Q, const void* K, const void* V,

@@ -1,0 +1,359 @@
+// Shared by the fp32-arithmetic kernels on CUDA cores (attend_simt.cu, backward.cu): fp32 problems (a result to 1e-5 and
+// the precision of fp32 sums rule out bf16 / tf32 matrix instructions) and the shapes the tensor-core kernels do not take.
+//
+// Mapping.  A lane owns QT rows of this side (queries; keys in the dK / dV kernel) with all their channels and walks the
+// rows of the other side, which all lanes of a region read from shared memory at once (a 16-byte read that several lanes
+// share costs the SM two cycles: with QT = 1 those reads, not the FMA pipe, set the time of S and P V; with QT = 2 the two
+// are level).  Dot products are single chains over the channels in increasing order.  Where a call has too few rows to
+// fill the GPU, 2, 4 or 8 lanes share their rows and split the other side between them (`ksl`).
+//
+// The other side's rows reach shared memory by asynchronous copies: the whole (image, head) slice where it is small
+// (`resident`: every routed row would otherwise be copied once per region that lists it), else a block of rows per region
+// of the CTA, double-buffered.  Rows are padded by 16 bytes, so that the rows of eight regions read at once start on
+// different banks.
+#pragma once
+
+#include "mma_common.cuh"
+
+namespace bra {
+
+namespace sk {
+constexpr int THREADS = 64;             // short CTAs: several per SM, an even tail
+constexpr int RESIDENT_MAX = 100 * 1024;
+constexpr int IDX_MAX = 4096;           // routing entries kept in shared memory per CTA
+}  // namespace sk
+
+struct SimtGeom {
+    int hb, cw;            // rows and columns of a chunk of a region (the whole region unless it is large)
+    int cx, chunks;        // chunks per row of chunks, chunks per region
+    int rpc, spr;          // regions per CTA; lane groups (QT rows each) per region (of a full chunk)
+    int ksl;               // log2 of the lanes that share rows
+    int threads, gpi;      // the grid is (gpi, heads, images)
+    int resident, dense;   // dense: topk == R, walk every region and weigh it by how often the list names it
+    int kps, stages;       // rows of the other side per region and stage
+    uint32_t mul_nr, mul_ws, mul_s, mul_spr, mul_kps, mul_cw;
+    int row;               // bytes of a row of one tensor in shared memory
+    int off_a, off_b, off_stat, off_idx, off_cnt, off_w, off_st, stage_bytes, smem_bytes;
+};
+
+enum SimtKind { SIMT_ATTEND, SIMT_DQ, SIMT_DKV };
+
+// rows per lane: two where registers allow it (the dK / dV kernel keeps four rows of channels per key)
+inline int simt_rows(int head_dim, SimtKind kind) { return kind != SIMT_DKV && head_dim <= 32 ? 2 : 1; }
+
+inline SimtGeom simt_geom(const Dims& d, SimtKind kind) {
+    SimtGeom g;
+    const int qt = simt_rows(d.d, kind);
+    g.row = d.d * d.esize + 16;
+    g.mul_nr = recip32(d.n_r); g.mul_ws = recip32(d.ws); g.mul_s = recip32(d.S);
+    // lanes of this call against the lanes the GPU holds at once (12 warps per SM)
+    const long long lanes = (long long)d.B * d.heads * d.R * ((d.n_r + qt - 1) / qt);
+    g.ksl = 0;
+    while (g.ksl < 3 && (lanes << g.ksl) < kSMs * 256 && (qt * d.d >> (g.ksl + 1)) >= 4) ++g.ksl;    // sum_shares: whole float4s
+    const int most = sk::THREADS >> g.ksl;                            // lane groups of a CTA
+    g.hb = d.hs; g.cw = d.ws;
+    if ((d.n_r + qt - 1) / qt > most) {
+        if (g.cw > qt * most) g.cw = qt * most;
+        g.hb = qt * most / g.cw;
+        if (g.hb > d.hs) g.hb = d.hs;
+    }
+    g.cx = (d.ws + g.cw - 1) / g.cw;
+    g.chunks = (d.hs + g.hb - 1) / g.hb * g.cx;
+    g.mul_cw = recip32(g.cw);
+    g.spr = (g.hb * g.cw + qt - 1) / qt;
+    g.rpc = g.chunks > 1 ? 1 : most / g.spr;
+    if (g.rpc < 1) g.rpc = 1;
+    if (g.rpc > d.R) g.rpc = d.R;
+    if ((long long)g.rpc * d.topk > sk::IDX_MAX) g.rpc = sk::IDX_MAX / d.topk > 0 ? sk::IDX_MAX / d.topk : 1;
+    const int ctas = (d.R + g.rpc - 1) / g.rpc;                       // even out the regions over them
+    g.rpc = (d.R + ctas - 1) / ctas;
+    g.mul_spr = recip32(g.spr);
+    g.threads = ((g.rpc * g.spr << g.ksl) + 31) / 32 * 32;
+    g.gpi = ctas * g.chunks;
+    const long long slice = 2ll * d.N * g.row;
+    // copies of the slice against copies of the listed rows (a key region is listed topk times on average)
+    g.resident = slice <= sk::RESIDENT_MAX && (long long)g.rpc * d.topk * d.n_r >= d.N;
+    g.dense = g.resident && d.topk == d.R && d.R <= 64;
+    // about 64 rows of two tensors per stage (18 KB at D = 32, fp32), in whole blocks of four per lane
+    const int block = 4 << g.ksl;
+    g.kps = 64 / g.rpc / block * block;
+    if (g.kps < block) g.kps = block;
+    if (g.kps > 32) g.kps = 32;
+    g.mul_kps = recip32(g.kps);
+    g.stages = g.resident ? 1 : 2;
+    const int rows = g.resident ? d.N : g.rpc * g.kps;                // of one stage
+    int off = 0;
+    g.off_a = off;    off += rows * g.row;
+    g.off_b = off;    off += rows * g.row;
+    g.off_stat = off; off += kind == SIMT_DKV ? (rows * 8 + 15) / 16 * 16 : 0;     // lse, delta
+    g.stage_bytes = off;
+    off *= g.stages;
+    g.off_idx = off;                                                  // (dK / dV: the lists are read through L1)
+    if (kind != SIMT_DKV && (long long)g.rpc * d.topk <= sk::IDX_MAX) off += g.rpc * d.topk * 4;
+    g.off_cnt = off;  off += g.dense ? g.rpc * d.R * 4 : 0;
+    g.off_w = off;    off += kind != SIMT_DQ && d.lce ? 25 * d.d * 4 : 0;
+    off = (off + 15) / 16 * 16;
+    g.off_st = 0;                                                     // over the rows, once they have been read
+    const int st = kind != SIMT_DQ ? g.rpc * qt * g.spr * (d.d + 4) * 4 : 0;
+    if (st > g.stages * g.stage_bytes) { g.off_st = off; off += st; }
+    g.smem_bytes = off;
+    return g;
+}
+inline bool simt_fits(const Dims& d, SimtKind kind) {
+    return (long long)d.topk * d.n_r * d.n_r < (1ll << 32) && (long long)d.R * d.n_r * d.n_r < (1ll << 32) && d.B <= 65535 &&
+           d.heads <= 65534 && (long long)d.H * d.W < (1ll << 30) && simt_geom(d, kind).smem_bytes <= 220 * 1024;
+}
+
+// Token (row-major in the caller's map) of token t of region r; -1 in the zero padding.
+__device__ __forceinline__ int simt_token(const Dims& dm, const SimtGeom& gm, int r, int t) {
+    const int ry = fdiv(r, dm.S, gm.mul_s), rx = r - ry * dm.S;
+    const int ty = fdiv(t, dm.ws, gm.mul_ws), tx = t - ty * dm.ws;
+    const int y = ry * dm.hs + ty, x = rx * dm.ws + tx;
+    return y < dm.H0 && x < dm.W0 ? y * dm.W0 + x : -1;
+}
+
+// Chunk ck of a region: first row and column in the region, extent.
+struct SimtChunk { int y, x, rows, cols; };
+__device__ __forceinline__ SimtChunk simt_chunk(const Dims& dm, const SimtGeom& gm, int ck) {
+    SimtChunk c;
+    const int cy = ck / gm.cx;
+    c.y = cy * gm.hb; c.x = (ck - cy * gm.cx) * gm.cw;
+    c.rows = min(gm.hb, dm.hs - c.y); c.cols = min(gm.cw, dm.ws - c.x);
+    return c;
+}
+// Token of row t of a chunk (gm.cw rows of this side per line) of region r; -1 outside the chunk or the map.
+__device__ __forceinline__ int simt_row(const Dims& dm, const SimtGeom& gm, const SimtChunk& c, int r, int t) {
+    const int ly = fdiv(t, gm.cw, gm.mul_cw), lx = t - ly * gm.cw;
+    if (ly >= c.rows || lx >= c.cols) return -1;
+    const int ry = fdiv(r, dm.S, gm.mul_s), rx = r - ry * dm.S;
+    const int y = ry * dm.hs + c.y + ly, x = rx * dm.ws + c.x + lx;
+    return y < dm.H0 && x < dm.W0 ? y * dm.W0 + x : -1;
+}
+
+// N channels of a row
+template <typename T, int N>
+__device__ __forceinline__ void lds_row(float (&v)[N], uint32_t a) {
+    if (sizeof(T) == 4) {
+#pragma unroll
+        for (int i = 0; i < N / 4; ++i) {
+            const float4 f = ptx::lds_f32x4(a + 16 * i);
+            v[4 * i] = f.x; v[4 * i + 1] = f.y; v[4 * i + 2] = f.z; v[4 * i + 3] = f.w;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < N / 8; ++i) {
+            const float4 f = ptx::lds_f32x4(a + 16 * i);
+            const uint32_t w[4] = {__float_as_uint(f.x), __float_as_uint(f.y), __float_as_uint(f.z), __float_as_uint(f.w)};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) { v[8 * i + 2 * j] = __uint_as_float(w[j] << 16); v[8 * i + 2 * j + 1] = __uint_as_float(w[j] & 0xffff0000u); }
+        }
+    }
+}
+template <typename T, int N>
+__device__ __forceinline__ void ldg_row(float (&v)[N], const T* p, bool ok, float f) {
+    if (ok) {
+        load_row<N>(p, v);
+#pragma unroll
+        for (int i = 0; i < N; ++i) v[i] *= f;
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; ++i) v[i] = 0.f;
+    }
+}
+// s[x][u] = q[x] . row at[u]: one chain each over the channels in increasing order, all chains interleaved (an FMA waits
+// four cycles for the one before it in its chain)
+template <typename T, int QT, int U, int N>
+__device__ __forceinline__ void dots(float (&s)[QT][U], const float (&q)[QT][N], const uint32_t (&at)[U], int off) {
+    constexpr int CH = 16 / (int)sizeof(T);
+#pragma unroll
+    for (int x = 0; x < QT; ++x)
+#pragma unroll
+        for (int u = 0; u < U; ++u) s[x][u] = 0.f;
+#pragma unroll
+    for (int c = 0; c < N; c += CH) {
+        float k[U][CH];
+#pragma unroll
+        for (int u = 0; u < U; ++u) lds_row<T, CH>(k[u], at[u] + off + c * (int)sizeof(T));
+#pragma unroll
+        for (int i = 0; i < CH; ++i)
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int x = 0; x < QT; ++x) s[x][u] = fmaf(q[x][c + i], k[u][i], s[x][u]);
+    }
+}
+template <int N>
+__device__ __forceinline__ float dot(const float (&a)[N], const float (&b)[N]) {
+    float s = 0.f;
+#pragma unroll
+    for (int i = 0; i < N; ++i) s = fmaf(a[i], b[i], s);
+    return s;
+}
+// the same in four chains
+template <int N>
+__device__ __forceinline__ float dot4(const float (&a)[N], const float (&b)[N]) {
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < N; ++i) s[i & 3] = fmaf(a[i], b[i], s[i & 3]);
+    return (s[0] + s[1]) + (s[2] + s[3]);
+}
+template <int N>
+__device__ __forceinline__ void axpy(float (&acc)[N], float f, const float (&b)[N]) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) acc[i] = fmaf(f, b[i], acc[i]);
+}
+// Sums QT rows of N channels over 2^ksl neighbouring lanes, lane ks of them weighing its share by f[x]: every round a lane
+// hands half of what it still holds to its partner and keeps the other half.  Afterwards the lane holds `held` consecutive
+// values from `first` on of the QT x N values (row-major), at least four.
+template <int QT, int N>
+__device__ __forceinline__ void sum_shares(float (&v)[QT][N], int ksl, int ks, int* first, int* held) {
+    float* w = &v[0][0];
+    int at = 0, n = QT * N;
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        constexpr int ALL = QT * N;
+        const int half = ALL >> (r + 1);
+        if (r < ksl) {
+            const bool up = (ks >> r) & 1;
+#pragma unroll
+            for (int i = 0; i < ALL / 2; ++i) {
+                if (i < half) {
+                    const float give = up ? w[i] : w[i + half], keep = up ? w[i + half] : w[i];
+                    w[i] = keep + __shfl_xor_sync(0xffffffffu, give, 1 << r);
+                }
+            }
+            n = half;
+            at += up ? half : 0;
+        }
+    }
+    *first = at; *held = n;
+}
+// values 4 i .. 4 i + 3 of what sum_shares left, for all of them: f(x, channel, float4)
+template <int QT, int N, typename F>
+__device__ __forceinline__ void for_held(const float (&v)[QT][N], int first, int held, F&& f) {
+    const float* w = &v[0][0];
+#pragma unroll
+    for (int i = 0; i < QT * N; i += 4) {
+        if (i < held) {
+            const int at = first + i;
+            f(at / N, at % N, make_float4(w[i], w[i + 1], w[i + 2], w[i + 3]));
+        }
+    }
+}
+__device__ __forceinline__ void store4(float* p, const float4& v) { *reinterpret_cast<float4*>(p) = v; }
+__device__ __forceinline__ void store4(__nv_bfloat16* p, const float4& v) {
+    *reinterpret_cast<uint2*>(p) = make_uint2(pack2_bf16(v.x, v.y), pack2_bf16(v.z, v.w));
+}
+
+// Rows 0 .. n - 1 of two tensors into shared memory; tok_at(row): token, -1 for a row of zeros.
+template <typename T, int D, typename TokAt>
+__device__ __forceinline__ void simt_copy_rows(uint32_t dst_a, uint32_t dst_b, int row_bytes, const T* A, const T* B, int C, int n, TokAt&& tok_at) {
+    constexpr int CH = D * (int)sizeof(T) / 16;
+    for (int e = threadIdx.x; e < n * 4; e += blockDim.x) {
+        const int row = e >> 2;
+        const int tok = tok_at(row);
+        const size_t off = (size_t)(tok < 0 ? 0 : tok) * C;
+        const uint32_t bytes = tok < 0 ? 0u : 16u;
+#pragma unroll
+        for (int c0 = 0; c0 < CH; c0 += 4) {
+            const int c = c0 + (e & 3);
+            if (CH % 4 == 0 || c < CH) {
+                ptx::cp_async_16(dst_a + row * row_bytes + c * 16, A + off + c * (16 / sizeof(T)), bytes);
+                ptx::cp_async_16(dst_b + row * row_bytes + c * 16, B + off + c * (16 / sizeof(T)), bytes);
+            }
+        }
+    }
+}
+
+// LCE weights of a head as they lie in memory: [D channels][25] (odd stride: lane = channel reads without conflicts)
+__device__ __forceinline__ void simt_load_weights(float* s_w, const float* lce_w, int n) {
+    for (int e = threadIdx.x; e < n; e += blockDim.x) s_w[e] = __ldg(lce_w + e);
+}
+
+__device__ __forceinline__ float simt_ld(const float* p) { return __ldg(p); }
+__device__ __forceinline__ float simt_ld(const __nv_bfloat16* p) { return __bfloat162float(__ldg(p)); }
+__device__ __forceinline__ void simt_st(float* p, float v) { *p = v; }
+__device__ __forceinline__ void simt_st(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
+
+// Adds the 5 x 5 depthwise correlation of `in` (FLIP: with the flipped filter) to the staged rows of the CTA's regions and
+// stores them.  Lane = channel (32 at a time), TS x TS positions per pass: every input value is read once per tile.
+template <typename T, int D, int TS, bool FLIP>
+__device__ __forceinline__ void simt_lce(const float* st, const float* s_w, const float* bias, const T* in, T* out, int r0, int nreg, int rows_per_region,
+                                         const SimtChunk& c,                                         const Dims& dm, const SimtGeom& gm) {
+    constexpr int LANES = D < 32 ? D : 32, GROUPS = D / LANES, SUB = 32 / LANES;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int nty = (c.rows + TS - 1) / TS, ntx = (c.cols + TS - 1) / TS, tiles = nty * ntx;
+    const int items = nreg * tiles * GROUPS;
+    float w[25], b = 0.f;
+    int loaded = -1;
+    for (int it = warp * SUB + lane / LANES; it < items; it += nwarps * SUB) {
+        const int cg = it % GROUPS, q = it / GROUPS;                  // GROUPS is a constant
+        const int rl = q / tiles, tile = q - rl * tiles;
+        const int ty = tile / ntx, tx = tile - ty * ntx;
+        const int ch = cg * LANES + lane % LANES;
+        if (cg != loaded) {
+            loaded = cg;
+#pragma unroll
+            for (int k = 0; k < 25; ++k) w[k] = dm.lce ? s_w[ch * 25 + k] : 0.f;
+            b = bias ? __ldg(bias + ch) : 0.f;
+        }
+        const int r = r0 + rl;
+        const int ry = fdiv(r, dm.S, gm.mul_s), rx = r - ry * dm.S;
+        const int ly0 = ty * TS, lx0 = tx * TS;                       // within the chunk
+        const int y0 = ry * dm.hs + c.y + ly0, x0 = rx * dm.ws + c.x + lx0;
+        float acc[TS][TS];
+#pragma unroll
+        for (int yy = 0; yy < TS; ++yy)
+#pragma unroll
+            for (int xx = 0; xx < TS; ++xx) acc[yy][xx] = b;
+        if (dm.lce) {
+bool in_x[TS + 4];
+#pragma unroll
+            for (int cc = 0; cc < TS + 4; ++cc) in_x[cc] = (unsigned)(x0 + cc - 2) < (unsigned)dm.W0;
+            const T* p = in + (ptrdiff_t)((y0 - 2) * dm.W0 + x0 - 2) * dm.C + ch;
+#pragma unroll
+            for (int rr = 0; rr < TS + 4; ++rr) {
+                const bool in_y = (unsigned)(y0 + rr - 2) < (unsigned)dm.H0;
+                float v[TS + 4];
+#pragma unroll
+                for (int cc = 0; cc < TS + 4; ++cc) v[cc] = in_y && in_x[cc] ? simt_ld(p + cc * dm.C) : 0.f;
+                p += (ptrdiff_t)dm.W0 * dm.C;
+#pragma unroll
+                for (int yy = 0; yy < TS; ++yy) {
+                    const int ti = rr - yy;
+                    if (ti < 0 || ti > 4) continue;
+#pragma unroll
+                    for (int tj = 0; tj < 5; ++tj)
+#pragma unroll
+                        for (int xx = 0; xx < TS; ++xx) acc[yy][xx] = fmaf(w[FLIP ? 24 - (ti * 5 + tj) : ti * 5 + tj], v[xx + tj], acc[yy][xx]);
+                }
+            }
+        }
+#pragma unroll
+        for (int yy = 0; yy < TS; ++yy)
+#pragma unroll
+            for (int xx = 0; xx < TS; ++xx)
+                if (ly0 + yy < c.rows && lx0 + xx < c.cols && y0 + yy < dm.H0 && x0 + xx < dm.W0) {
+                    const float a = st[(rl * rows_per_region + (ly0 + yy) * gm.cw + lx0 + xx) * (D + 4) + ch];
+                    simt_st(out + (ptrdiff_t)((y0 + yy) * dm.W0 + x0 + xx) * dm.C + ch, a + acc[yy][xx]);
+                }
+    }
+}
+
+// How often each region is named by the list of each region of the CTA: cnt[rl][R]; true if every count is one.
+// entry_at(e): rl * R + region, -1 for no region.
+template <typename EntryAt>
+__device__ __forceinline__ bool simt_counts(int32_t* cnt, int nreg, int R, int entries, EntryAt&& entry_at) {
+    for (int e = threadIdx.x; e < nreg * R; e += blockDim.x) cnt[e] = 0;
+    __syncthreads();
+    for (int e = threadIdx.x; e < entries; e += blockDim.x) {
+        const int at = entry_at(e);
+        if (at >= 0) atomicAdd(cnt + at, 1);
+    }
+    __syncthreads();
+    bool ones = true;
+    for (int e = threadIdx.x; e < nreg * R; e += blockDim.x) ones = ones && cnt[e] == 1;
+    return __syncthreads_and(ones);
+}
+
+}  // namespace bra

@@ -5,12 +5,14 @@
 // Bound: the FMA pipe, 2 D FMAs per query and key (a packed FMA every two cycles and scheduler).
 #include "simt_common.cuh"
 
+#include <type_traits>
+
 namespace bra {
 
 using namespace ptx;
 
 template <typename T, int D>
-__global__ void __launch_bounds__(sk::THREADS, D <= 16 ? 8 : D <= 32 ? 6 : D == 64 ? 4 : 2)
+__global__ void __launch_bounds__(sk::THREADS, D <= 16 ? 8 : 4)
 attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* __restrict__ Vg, const int32_t* index,
                    const float* __restrict__ lce_w, const float* __restrict__ lce_b, T* __restrict__ Og, float* __restrict__ lse,
                    int32_t* __restrict__ status, Dims dm, SimtGeom gm) {
@@ -28,8 +30,9 @@ attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
     float* s_w = reinterpret_cast<float*>(smem + gm.off_w);
     if (dm.lce) simt_load_weights(s_w, lce_w + (size_t)h * D * 25, 25 * D);
     if (gm.resident) {
-        simt_copy_rows<T, D>(sbase + gm.off_a, sbase + gm.off_b, gm.row, K, V, dm.C, dm.N, [&](int row) {
+        simt_copy_rows<T, D>(sbase + gm.off_a, sbase + gm.off_b, K, V, dm.C, dm.N, [&](int row, uint32_t& at) {
             const int r = fdiv(row, dm.n_r, gm.mul_nr);
+            at = row * gm.row;
             return simt_token(dm, gm, r, row - r * dm.n_r);
         });
         cp_async_commit();
@@ -73,32 +76,41 @@ attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
     }
     const int total = dm.topk * dm.n_r;
 
-    // keys [k0, k1) of every region; row_of(kk, wt): row in shared memory (-1: the key does not count) and its weight
-    auto walk = [&](uint32_t abase, int k0, int k1, auto&& row_of) {
+    // keys [k0, k1): rows from offset at0 on, in order (PLAIN), or row_of(kk, wt): offset of the row in shared memory (-1: the
+    // key does not count) and its weight.  The reference maximum follows the scores only when one lies 16 above it (P and its sums
+    // are fp32: any reference gives the same relative precision), so that the sums are seldom rescaled.
+    auto walk = [&](auto plain, uint32_t abase, uint32_t at0, int k0, int k1, auto&& row_of) {
+        constexpr bool PLAIN = decltype(plain)::value;
         const int blocks = (k1 - k0 + U * KS - 1) / (U * KS);
+        uint32_t next = abase + at0 + ks * gm.row;
 #pragma unroll 1
         for (int blk = 0; blk < blocks; ++blk) {
             uint32_t at[U];
-            int row[U];
+            bool dead[U];
             float s[QT][U], wt[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int kk = k0 + (blk * U + u) * KS + ks;
-                wt[u] = 1.f;
-                row[u] = kk < k1 ? row_of(kk, wt[u]) : -1;
-                at[u] = abase + (row[u] < 0 ? 0 : row[u]) * gm.row;
+                dead[u] = kk >= k1;
+                if constexpr (PLAIN) {
+                    at[u] = dead[u] ? abase : next;
+                    next += KS * gm.row;
+                } else {
+                    wt[u] = 1.f;
+                    const int row = dead[u] ? -1 : row_of(kk, wt[u]);
+                    dead[u] = row < 0;
+                    at[u] = abase + (dead[u] ? 0 : row);
+                }
             }
             dots<T, QT, U, D>(s, q, at, gm.off_a);
 #pragma unroll
-            for (int u = 0; u < U; ++u)
-#pragma unroll
-                for (int x = 0; x < QT; ++x)
-                    if (row[u] < 0) s[x][u] = -INFINITY;
-#pragma unroll
             for (int x = 0; x < QT; ++x) {
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (dead[u]) s[x][u] = -INFINITY;
                 const float mx = fmaxf(fmaxf(s[x][0], s[x][1]), fmaxf(s[x][2], s[x][3]));
-                if (mx > m_run[x]) {
-                    const float corr = expf(m_run[x] - mx);           // 0 on the first block (m_run = -inf)
+                if (mx > m_run[x] + 16.f) {                           // always for the first keys that count
+                    const float corr = expf(m_run[x] - mx);           // 0 then (m_run = -inf)
                     m_run[x] = mx;
                     l_run[x] *= corr;
 #pragma unroll
@@ -108,7 +120,7 @@ attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     s[x][u] = expf(s[x][u] - mn);
-                    if (weighted) s[x][u] *= wt[u];
+                    if (!PLAIN && weighted) s[x][u] *= wt[u];
                     l_run[x] += s[x][u];
                 }
             }
@@ -121,44 +133,39 @@ attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
             }
         }
     };
-    if (gm.resident) {
-        cp_async_wait<0>();
-        __syncthreads();
-        walk(sbase, 0, gm.dense ? dm.N : total, [&](int kk, float& wt) -> int {
-            if (gm.dense && !weighted) return kk;
+    const int nst = gm.resident ? 1 : (total + gm.kps - 1) / gm.kps;
+    auto load_stage = [&](int st) {
+        const uint32_t base = sbase + (st & 1) * gm.stage_bytes;
+        simt_copy_rows<T, D>(base + gm.off_a, base + gm.off_b, K, V, dm.C, nreg * gm.kps, [&](int row, uint32_t& at) {
+            const int l = fdiv(row, gm.kps, gm.mul_kps), kk = st * gm.kps + row - l * gm.kps;
+            at = l * gm.reg + (row - l * gm.kps) * gm.row;
+            if (kk >= total) return -1;
             const int m = fdiv(kk, dm.n_r, gm.mul_nr);
-            if (gm.dense) {
-                const int n = cnt[rl * dm.R + m];
-                wt = (float)n;
-                return n > 0 ? kk : -1;
-            }
-            const int r = entry(rl * dm.topk + m);
-            return r < 0 ? -1 : r * dm.n_r + kk - m * dm.n_r;
+            const int r = entry(l * dm.topk + m);
+            return r >= 0 ? simt_token(dm, gm, r, kk - m * dm.n_r) : -1;
         });
-    } else {
-        const int nst = (total + gm.kps - 1) / gm.kps;
-        auto load_stage = [&](int st) {
-            const uint32_t base = sbase + (st & 1) * gm.stage_bytes;
-            simt_copy_rows<T, D>(base + gm.off_a, base + gm.off_b, gm.row, K, V, dm.C, nreg * gm.kps, [&](int row) {
-                const int l = fdiv(row, gm.kps, gm.mul_kps), kk = st * gm.kps + row - l * gm.kps;
-                if (kk >= total) return -1;
+        cp_async_commit();
+    };
+    if (!gm.resident) load_stage(0);
+    for (int st = 0; st < nst; ++st) {
+        if (st + 1 < nst) { load_stage(st + 1); cp_async_wait<1>(); } else cp_async_wait<0>();
+        __syncthreads();
+        const uint32_t abase = sbase + (st & 1) * gm.stage_bytes;
+        const int k0 = gm.resident ? 0 : st * gm.kps;
+        if (gm.resident ? gm.dense && !weighted : !bad)
+            walk(std::true_type(), abase, gm.resident ? 0 : rl * gm.reg, k0, gm.resident ? dm.N : min(total, k0 + gm.kps), 0);
+        else
+            walk(std::false_type(), abase, 0, k0, gm.dense ? dm.N : gm.resident ? total : min(total, k0 + gm.kps), [&](int kk, float& wt) -> int {
                 const int m = fdiv(kk, dm.n_r, gm.mul_nr);
-                const int r = entry(l * dm.topk + m);
-                return r >= 0 ? simt_token(dm, gm, r, kk - m * dm.n_r) : -1;
+                if (gm.dense) {
+                    const int n = cnt[rl * dm.R + m];
+                    wt = (float)n;
+                    return n > 0 ? kk * gm.row : -1;
+                }
+                const int r = entry(rl * dm.topk + m);
+                return r < 0 ? -1 : gm.resident ? (r * dm.n_r + kk - m * dm.n_r) * gm.row : rl * gm.reg + (kk - k0) * gm.row;
             });
-            cp_async_commit();
-        };
-        load_stage(0);
-        for (int st = 0; st < nst; ++st) {
-            if (st + 1 < nst) { load_stage(st + 1); cp_async_wait<1>(); } else cp_async_wait<0>();
-            __syncthreads();
-            const int k0 = st * gm.kps, k1 = min(total, k0 + gm.kps);
-            walk(sbase + (st & 1) * gm.stage_bytes, k0, k1, [&](int kk, float&) -> int {
-                if (bad && entry(rl * dm.topk + fdiv(kk, dm.n_r, gm.mul_nr)) < 0) return -1;
-                return rl * gm.kps + kk - k0;
-            });
-            __syncthreads();
-        }
+        __syncthreads();
     }
 
     // ---- merge the key shares; normalise; stage; lse ----

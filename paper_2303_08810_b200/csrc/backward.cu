@@ -13,6 +13,8 @@
 #include "inverse_index.cuh"
 #include "simt_common.cuh"
 
+#include <type_traits>
+
 namespace bra {
 
 using namespace ptx;
@@ -43,8 +45,9 @@ bwd_dq_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
     const size_t head = (size_t)b * N0 * dm.C + (size_t)h * D;
     const T* K = Kg + head; const T* V = Vg + head;
     if (gm.resident) {
-        simt_copy_rows<T, D>(sbase + gm.off_a, sbase + gm.off_b, gm.row, K, V, dm.C, dm.N, [&](int row) {
+        simt_copy_rows<T, D>(sbase + gm.off_a, sbase + gm.off_b, K, V, dm.C, dm.N, [&](int row, uint32_t& at) {
             const int r = fdiv(row, dm.n_r, gm.mul_nr);
+            at = row * gm.row;
             return simt_token(dm, gm, r, row - r * dm.n_r);
         });
         cp_async_commit();
@@ -87,19 +90,28 @@ bwd_dq_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
         for (int i = 0; i < D; ++i) acc[x][i] = 0.f;
     }
     const int total = dm.topk * dm.n_r;
-    auto walk = [&](uint32_t abase, int k0, int k1, bool second, auto&& row_of) {
+    auto walk = [&](auto plain, uint32_t abase, uint32_t at0, int k0, int k1, bool second, auto&& row_of) {
+        constexpr bool PLAIN = decltype(plain)::value;
         const int blocks = (k1 - k0 + U * KS - 1) / (U * KS);
+        uint32_t next = abase + at0 + ks * gm.row;
 #pragma unroll 1
         for (int blk = 0; blk < blocks; ++blk) {
-uint32_t at[U];
-            int row[U];
+            uint32_t at[U];
+            bool dead[U];
             float s[QT][U], dp[QT][U], wt[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int kk = k0 + (blk * U + u) * KS + ks;
-                wt[u] = 1.f;
-                row[u] = kk < k1 ? row_of(kk, wt[u]) : -1;
-                at[u] = abase + (row[u] < 0 ? 0 : row[u]) * gm.row;
+                dead[u] = kk >= k1;
+                if constexpr (PLAIN) {
+                    at[u] = dead[u] ? abase : next;
+                    next += KS * gm.row;
+                } else {
+                    wt[u] = 1.f;
+                    const int row = dead[u] ? -1 : row_of(kk, wt[u]);
+                    dead[u] = row < 0;
+                    at[u] = abase + (dead[u] ? 0 : row);
+                }
             }
             dots<T, QT, U, D>(s, q, at, gm.off_a);
             dots<T, QT, U, D>(dp, go, at, gm.off_b);
@@ -107,8 +119,8 @@ uint32_t at[U];
             for (int u = 0; u < U; ++u)
 #pragma unroll
                 for (int x = 0; x < QT; ++x) {
-                    s[x][u] = row[u] < 0 ? 0.f : expf(s[x][u] - l[x]);
-                    if (weighted) s[x][u] *= wt[u];
+                    s[x][u] = dead[u] ? 0.f : expf(s[x][u] - l[x]);
+                    if (!PLAIN && weighted) s[x][u] *= wt[u];
                     if (!second) dsum[x] = fmaf(s[x][u], dp[x][u], dsum[x]);
                     else s[x][u] *= dp[x][u] - dsum[x];
                 }
@@ -127,50 +139,41 @@ uint32_t at[U];
 #pragma unroll
             for (int x = 0; x < QT; ++x) dsum[x] += __shfl_xor_sync(0xffffffffu, dsum[x], off);
     };
-    if (gm.resident) {
-        cp_async_wait<0>();
+    const int nst = gm.resident ? 1 : (total + gm.kps - 1) / gm.kps;
+    auto load_stage = [&](int it) {
+        const int st = it < nst ? it : it - nst;
+        const uint32_t base = sbase + (it & 1) * gm.stage_bytes;
+        simt_copy_rows<T, D>(base + gm.off_a, base + gm.off_b, K, V, dm.C, nreg * gm.kps, [&](int row, uint32_t& at) {
+            const int lr = fdiv(row, gm.kps, gm.mul_kps), kk = st * gm.kps + row - lr * gm.kps;
+            at = lr * gm.reg + (row - lr * gm.kps) * gm.row;
+            if (kk >= total) return -1;
+            const int m = fdiv(kk, dm.n_r, gm.mul_nr);
+            const int r = entry(lr * dm.topk + m);
+            return r >= 0 ? simt_token(dm, gm, r, kk - m * dm.n_r) : -1;
+        });
+        cp_async_commit();
+    };
+    if (!gm.resident) load_stage(0);
+    for (int it = 0; it < 2 * nst; ++it) {
+        if (!gm.resident && it + 1 < 2 * nst) { load_stage(it + 1); cp_async_wait<1>(); } else cp_async_wait<0>();
         __syncthreads();
-#pragma unroll 1
-        for (int sweep = 0; sweep < 2; ++sweep) {
-            walk(sbase, 0, gm.dense ? dm.N : total, sweep == 1, [&](int kk, float& wt) -> int {
-                if (gm.dense && !weighted) return kk;
+        const int k0 = gm.resident ? 0 : (it < nst ? it : it - nst) * gm.kps;
+        const uint32_t abase = sbase + (gm.resident ? 0 : it & 1) * gm.stage_bytes;
+        if (gm.resident ? gm.dense && !weighted : !bad)
+            walk(std::true_type(), abase, gm.resident ? 0 : rl * gm.reg, k0, gm.resident ? dm.N : min(total, k0 + gm.kps), it >= nst, 0);
+        else
+            walk(std::false_type(), abase, 0, k0, gm.dense ? dm.N : gm.resident ? total : min(total, k0 + gm.kps), it >= nst, [&](int kk, float& wt) -> int {
                 const int m = fdiv(kk, dm.n_r, gm.mul_nr);
                 if (gm.dense) {
                     const int n = cnt[rl * dm.R + m];
                     wt = (float)n;
-                    return n > 0 ? kk : -1;
+                    return n > 0 ? kk * gm.row : -1;
                 }
                 const int r = entry(rl * dm.topk + m);
-                return r < 0 ? -1 : r * dm.n_r + kk - m * dm.n_r;
+                return r < 0 ? -1 : gm.resident ? (r * dm.n_r + kk - m * dm.n_r) * gm.row : rl * gm.reg + (kk - k0) * gm.row;
             });
-            if (sweep == 0) end_of_first();
-        }
-    } else {
-        const int nst = (total + gm.kps - 1) / gm.kps;
-        auto load_stage = [&](int it) {
-            const int st = it < nst ? it : it - nst;
-            const uint32_t base = sbase + (it & 1) * gm.stage_bytes;
-            simt_copy_rows<T, D>(base + gm.off_a, base + gm.off_b, gm.row, K, V, dm.C, nreg * gm.kps, [&](int row) {
-                const int lr = fdiv(row, gm.kps, gm.mul_kps), kk = st * gm.kps + row - lr * gm.kps;
-                if (kk >= total) return -1;
-                const int m = fdiv(kk, dm.n_r, gm.mul_nr);
-                const int r = entry(lr * dm.topk + m);
-                return r >= 0 ? simt_token(dm, gm, r, kk - m * dm.n_r) : -1;
-            });
-            cp_async_commit();
-        };
-        load_stage(0);
-        for (int it = 0; it < 2 * nst; ++it) {
-            if (it + 1 < 2 * nst) { load_stage(it + 1); cp_async_wait<1>(); } else cp_async_wait<0>();
-            __syncthreads();
-            const int k0 = (it < nst ? it : it - nst) * gm.kps, k1 = min(total, k0 + gm.kps);
-            walk(sbase + (it & 1) * gm.stage_bytes, k0, k1, it >= nst, [&](int kk, float&) -> int {
-                if (bad && entry(rl * dm.topk + fdiv(kk, dm.n_r, gm.mul_nr)) < 0) return -1;
-                return rl * gm.kps + kk - k0;
-            });
-            if (it == nst - 1) end_of_first();
-            __syncthreads();
-        }
+        if (it == nst - 1) end_of_first();
+        __syncthreads();
     }
     int first, held;
     sum_shares<QT, D>(acc, gm.ksl, ks, &first, &held);
@@ -191,7 +194,6 @@ __global__ void __launch_bounds__(sk::THREADS, D <= 16 ? 6 : 4)
 bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* __restrict__ Vg, const int32_t* inv_off,
                     const int32_t* inv_list, const float* __restrict__ lse, const float* delta, const T* __restrict__ dOg,
                     const float* __restrict__ lce_w, T* __restrict__ dKg, T* __restrict__ dVg, Dims dm, SimtGeom gm) {
-    constexpr int U = 2;
     extern __shared__ __align__(128) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
     const int tid = threadIdx.x;
@@ -205,8 +207,9 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
     float* s_w = reinterpret_cast<float*>(smem + gm.off_w);
     if (dm.lce) simt_load_weights(s_w, lce_w + (size_t)h * D * 25, 25 * D);
     if (gm.resident) {
-        simt_copy_rows<T, D>(sbase + gm.off_a, sbase + gm.off_b, gm.row, Q, dO, dm.C, dm.N, [&](int row) {
+        simt_copy_rows<T, D>(sbase + gm.off_a, sbase + gm.off_b, Q, dO, dm.C, dm.N, [&](int row, uint32_t& at) {
             const int r = fdiv(row, dm.n_r, gm.mul_nr);
+            at = row * gm.row;
             return simt_token(dm, gm, r, row - r * dm.n_r);
         });
         cp_async_commit();
@@ -248,30 +251,39 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
     }
     // statistics of a row: lse and delta; a row that does not count has lse = inf (P = 0); a row of the zero padding has
     // zero Q and dO and lse = delta = 0 and adds nothing
-    auto walk = [&](int stage, int k0, int k1, auto&& row_of) {
-        const uint32_t abase = sbase + stage * gm.stage_bytes;
-        const int blocks = (k1 - k0 + U * KS - 1) / (U * KS);
+    auto walk = [&](auto plain, uint32_t abase, uint32_t at0, int row0, int k0, int k1, auto&& row_of) {
+        constexpr bool PLAIN = decltype(plain)::value;
+        uint32_t next = abase + at0 + ks * gm.row, next_stat = abase + gm.off_stat + (row0 + ks) * 8;
 #pragma unroll 1
-        for (int blk = 0; blk < blocks; ++blk) {
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int kk = k0 + (blk * U + u) * KS + ks;
-                float wt = 1.f;
-                const int row = kk < k1 ? row_of(kk, wt) : -1;
-                const int rr = row < 0 ? 0 : row;
-                const uint32_t at = abase + rr * gm.row;
-                const float2 stat = lds_f32x2(abase + gm.off_stat + rr * 8);
-                float g[D], qv[D];
-                lds_row<T, D>(g, at + gm.off_b);
-                const float dp = dot4(vr, g);
-                lds_row<T, D>(qv, at + gm.off_a);
-                float p = row < 0 ? 0.f : expf(dot(qv, kr) - stat.x);
-                if (weighted) p *= wt;
-                axpy(gk[0], p * (dp - stat.y), qv);
-                axpy(gv[0], p, g);
+        for (int kb = k0; kb < k1; kb += KS) {
+            const int kk = kb + ks;
+            uint32_t at = next, at_stat = next_stat;
+            bool dead = kk >= k1;
+            float wt = 1.f;
+            if constexpr (PLAIN) {
+                if (dead) { at = abase; at_stat = abase + gm.off_stat; }
+                next += KS * gm.row;
+                next_stat += KS * 8;
+            } else {
+                const int row = dead ? -1 : row_of(kk, wt);
+                dead = row < 0;
+                at = abase + (dead ? 0 : row) * gm.row;               // (resident: row number)
+                at_stat = abase + gm.off_stat + (dead ? 0 : row) * 8;
             }
+            const float2 stat = lds_f32x2(at_stat);
+            float g[D], qv[D];
+            lds_row<T, D>(qv, at + gm.off_a);
+            lds_row<T, D>(g, at + gm.off_b);
+            const float dp = dot4(vr, g);
+            float p = expf(dot(qv, kr) - stat.x);
+            if (!PLAIN && weighted) p *= wt;
+            float ds = p * (dp - stat.y);
+            if (dead) p = ds = 0.f;
+            axpy(gk[0], ds, qv);
+            axpy(gv[0], p, g);
         }
     };
+    int most = warp_total;                                            // longest list of the CTA's regions
     if (gm.resident) {
         float2* stat = reinterpret_cast<float2*>(smem + gm.off_stat);
         for (int row = tid; row < dm.N; row += blockDim.x) {
@@ -279,49 +291,51 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
             const int tk = simt_token(dm, gm, r, row - r * dm.n_r);
             stat[row] = tk >= 0 ? make_float2(__ldg(lse_h + tk), __ldcg(delta_h + tk)) : make_float2(0.f, 0.f);
         }
-        cp_async_wait<0>();
-        __syncthreads();
-        walk(0, 0, gm.dense ? dm.N : warp_total, [&](int kk, float& wt) -> int {
-            if (gm.dense && !weighted) return kk;
-            const int m = fdiv(kk, dm.n_r, gm.mul_nr);
-            if (gm.dense) {
-                const int n = cnt[rl * dm.R + m];
-                wt = (float)n;
-                return n > 0 ? kk : -1;
-            }
-            return kk < mine ? __ldcg(list + e0 + m) * dm.n_r + kk - m * dm.n_r : -1;
-        });
     } else {
-        int most = 0;
-        for (int l = 0; l < nreg; ++l) most = max(most, __ldcg(offs + l + 1) - __ldcg(offs + l));
-        most *= dm.n_r;
-        const int nst = (most + gm.kps - 1) / gm.kps;
-        auto load_stage = [&](int st) {
-            const uint32_t base = sbase + (st & 1) * gm.stage_bytes;
-            float2* stat = reinterpret_cast<float2*>(smem + (st & 1) * gm.stage_bytes + gm.off_stat);
-            simt_copy_rows<T, D>(base + gm.off_a, base + gm.off_b, gm.row, Q, dO, dm.C, nreg * gm.kps, [&](int row) {
-                const int lr = fdiv(row, gm.kps, gm.mul_kps), kk = st * gm.kps + row - lr * gm.kps;
-                const int s0 = __ldcg(offs + lr);
+        for (int l = 0; l < nreg; ++l) most = max(most, (__ldcg(offs + l + 1) - __ldcg(offs + l)) * dm.n_r);
+    }
+    const int nst = gm.resident ? 1 : (most + gm.kps - 1) / gm.kps;
+    auto load_stage = [&](int st) {
+        const uint32_t base = sbase + (st & 1) * gm.stage_bytes;
+        float2* stat = reinterpret_cast<float2*>(smem + (st & 1) * gm.stage_bytes + gm.off_stat);
+        simt_copy_rows<T, D>(base + gm.off_a, base + gm.off_b, Q, dO, dm.C, nreg * gm.kps, [&](int row, uint32_t& at) {
+            const int lr = fdiv(row, gm.kps, gm.mul_kps), kk = st * gm.kps + row - lr * gm.kps;
+            at = lr * gm.reg + (row - lr * gm.kps) * gm.row;
+            const int s0 = __ldcg(offs + lr);
+            const int m = fdiv(kk, dm.n_r, gm.mul_nr);
+            int tk = -1;
+            float2 v = make_float2(INFINITY, 0.f);
+            if (s0 + m < __ldcg(offs + lr + 1)) {
+                tk = simt_token(dm, gm, __ldcg(list + s0 + m), kk - m * dm.n_r);
+                v = tk >= 0 ? make_float2(__ldg(lse_h + tk), __ldcg(delta_h + tk)) : make_float2(0.f, 0.f);
+            }
+            if ((threadIdx.x & 3) == 0) stat[row] = v;
+            return tk;
+        });
+        cp_async_commit();
+    };
+    if (!gm.resident && nst > 0) load_stage(0);
+    for (int st = 0; st < nst; ++st) {
+        if (st + 1 < nst) { load_stage(st + 1); cp_async_wait<1>(); } else cp_async_wait<0>();
+        __syncthreads();
+        const int k0 = gm.resident ? 0 : st * gm.kps;
+        const uint32_t abase = sbase + (st & 1) * gm.stage_bytes;
+        if (!gm.resident) {
+            if (k0 < warp_total) walk(std::true_type(), abase, rl * gm.reg, rl * gm.kps, k0, min(warp_total, k0 + gm.kps), 0);
+        } else if (gm.dense && !weighted) {
+            walk(std::true_type(), abase, 0, 0, 0, dm.N, 0);
+        } else {
+            walk(std::false_type(), abase, 0, 0, 0, gm.dense ? dm.N : warp_total, [&](int kk, float& wt) -> int {
                 const int m = fdiv(kk, dm.n_r, gm.mul_nr);
-                int tk = -1;
-                float2 v = make_float2(INFINITY, 0.f);
-                if (s0 + m < __ldcg(offs + lr + 1)) {
-                    tk = simt_token(dm, gm, __ldcg(list + s0 + m), kk - m * dm.n_r);
-                    v = tk >= 0 ? make_float2(__ldg(lse_h + tk), __ldcg(delta_h + tk)) : make_float2(0.f, 0.f);
+                if (gm.dense) {
+                    const int n = cnt[rl * dm.R + m];
+                    wt = (float)n;
+                    return n > 0 ? kk : -1;
                 }
-                if ((threadIdx.x & 3) == 0) stat[row] = v;
-                return tk;
+                return kk < mine ? __ldcg(list + e0 + m) * dm.n_r + kk - m * dm.n_r : -1;
             });
-            cp_async_commit();
-        };
-        if (nst > 0) load_stage(0);
-        for (int st = 0; st < nst; ++st) {
-            if (st + 1 < nst) { load_stage(st + 1); cp_async_wait<1>(); } else cp_async_wait<0>();
-            __syncthreads();
-            const int k0 = st * gm.kps, k1 = min(warp_total, k0 + gm.kps);
-            if (k0 < k1) walk(st & 1, k0, k1, [&](int kk, float&) -> int { return rl * gm.kps + kk - k0; });
-            __syncthreads();
         }
+        __syncthreads();
     }
     int first, held;
     sum_shares<1, D>(gk, gm.ksl, ks, &first, &held);

@@ -9,8 +9,8 @@
 //
 // The other side's rows reach shared memory by asynchronous copies: the whole (image, head) slice where it is small
 // (`resident`: every routed row would otherwise be copied once per region that lists it), else a block of rows per region
-// of the CTA, double-buffered.  Rows are padded by 16 bytes, so that the rows of eight regions read at once start on
-// different banks.
+// of the CTA, double-buffered.  Rows are padded by 16 bytes and so are the blocks of the regions, so that rows read at
+// once (of several regions, or of several key shares) start on different banks.
 #pragma once
 
 #include "mma_common.cuh"
@@ -33,6 +33,7 @@ struct SimtGeom {
     int kps, stages;       // rows of the other side per region and stage
     uint32_t mul_nr, mul_ws, mul_s, mul_spr, mul_kps, mul_cw;
     int row;               // bytes of a row of one tensor in shared memory
+    int reg;               // bytes from one region's rows of a stage to the next region's
     int off_a, off_b, off_stat, off_idx, off_cnt, off_w, off_st, stage_bytes, smem_bytes;
 };
 
@@ -74,17 +75,18 @@ inline SimtGeom simt_geom(const Dims& d, SimtKind kind) {
     // copies of the slice against copies of the listed rows (a key region is listed topk times on average)
     g.resident = slice <= sk::RESIDENT_MAX && (long long)g.rpc * d.topk * d.n_r >= d.N;
     g.dense = g.resident && d.topk == d.R && d.R <= 64;
-    // about 64 rows of two tensors per stage (18 KB at D = 32, fp32), in whole blocks of four per lane
     const int block = 4 << g.ksl;
+    // about 64 rows of two tensors per stage (18 KB at D = 32, fp32), in whole blocks of four per lane
     g.kps = 64 / g.rpc / block * block;
     if (g.kps < block) g.kps = block;
     if (g.kps > 32) g.kps = 32;
     g.mul_kps = recip32(g.kps);
     g.stages = g.resident ? 1 : 2;
     const int rows = g.resident ? d.N : g.rpc * g.kps;                // of one stage
+    g.reg = (g.kps * g.row + 111) / 128 * 128 + 16;                   // 16 modulo 128
     int off = 0;
-    g.off_a = off;    off += rows * g.row;
-    g.off_b = off;    off += rows * g.row;
+    g.off_a = off;    off += g.resident ? rows * g.row : g.rpc * g.reg;
+    g.off_b = off;    off += g.resident ? rows * g.row : g.rpc * g.reg;
     g.off_stat = off; off += kind == SIMT_DKV ? (rows * 8 + 15) / 16 * 16 : 0;     // lse, delta
     g.stage_bytes = off;
     off *= g.stages;
@@ -197,10 +199,15 @@ __device__ __forceinline__ float dot4(const float (&a)[N], const float (&b)[N]) 
     for (int i = 0; i < N; ++i) s[i & 3] = fmaf(a[i], b[i], s[i & 3]);
     return (s[0] + s[1]) + (s[2] + s[3]);
 }
+// acc += f b, two channels per instruction
 template <int N>
 __device__ __forceinline__ void axpy(float (&acc)[N], float f, const float (&b)[N]) {
+    const float2 f2 = make_float2(f, f);
 #pragma unroll
-    for (int i = 0; i < N; ++i) acc[i] = fmaf(f, b[i], acc[i]);
+    for (int i = 0; i < N; i += 2) {
+        const float2 r = __ffma2_rn(f2, make_float2(b[i], b[i + 1]), make_float2(acc[i], acc[i + 1]));
+        acc[i] = r.x; acc[i + 1] = r.y;
+    }
 }
 // Sums QT rows of N channels over 2^ksl neighbouring lanes, lane ks of them weighing its share by f[x]: every round a lane
 // hands half of what it still holds to its partner and keeps the other half.  Afterwards the lane holds `held` consecutive
@@ -245,21 +252,23 @@ __device__ __forceinline__ void store4(__nv_bfloat16* p, const float4& v) {
     *reinterpret_cast<uint2*>(p) = make_uint2(pack2_bf16(v.x, v.y), pack2_bf16(v.z, v.w));
 }
 
-// Rows 0 .. n - 1 of two tensors into shared memory; tok_at(row): token, -1 for a row of zeros.
+// Rows 0 .. n - 1 of two tensors into shared memory; tok_at(row, at): token (-1 for a row of zeros) and the byte offset
+// of the row from the start of its tensor's rows.
 template <typename T, int D, typename TokAt>
-__device__ __forceinline__ void simt_copy_rows(uint32_t dst_a, uint32_t dst_b, int row_bytes, const T* A, const T* B, int C, int n, TokAt&& tok_at) {
+__device__ __forceinline__ void simt_copy_rows(uint32_t dst_a, uint32_t dst_b, const T* A, const T* B, int C, int n, TokAt&& tok_at) {
     constexpr int CH = D * (int)sizeof(T) / 16;
     for (int e = threadIdx.x; e < n * 4; e += blockDim.x) {
         const int row = e >> 2;
-        const int tok = tok_at(row);
+        uint32_t at;
+        const int tok = tok_at(row, at);
         const size_t off = (size_t)(tok < 0 ? 0 : tok) * C;
         const uint32_t bytes = tok < 0 ? 0u : 16u;
 #pragma unroll
         for (int c0 = 0; c0 < CH; c0 += 4) {
             const int c = c0 + (e & 3);
             if (CH % 4 == 0 || c < CH) {
-                ptx::cp_async_16(dst_a + row * row_bytes + c * 16, A + off + c * (16 / sizeof(T)), bytes);
-                ptx::cp_async_16(dst_b + row * row_bytes + c * 16, B + off + c * (16 / sizeof(T)), bytes);
+                ptx::cp_async_16(dst_a + at + c * 16, A + off + c * (16 / sizeof(T)), bytes);
+                ptx::cp_async_16(dst_b + at + c * 16, B + off + c * (16 / sizeof(T)), bytes);
             }
         }
     }

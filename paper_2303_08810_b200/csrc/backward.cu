@@ -360,14 +360,15 @@ bool backward_supported(const Dims& d) {
     return (d.d == 16 || d.d == 32 || d.d == 64) && d.R <= 1000 && simt_fits(d, SIMT_DQ) && simt_fits(d, SIMT_DKV);
 }
 
-enum Family { FAMILY_SIMT, FAMILY_DIRECT, FAMILY_IMG };
+enum Family { FAMILY_SIMT, FAMILY_DIRECT, FAMILY_IMG, FAMILY_DENSE };
 
 // bf16, head dim 32 or 64: tensor-core kernels.  Small maps with enough (image, head) pairs to fill the GPU keep a
 // whole slice resident (head dim 32); the rest take their operands straight from global memory.
 static Family choose_family(const Dims& d, int dtype, int impl) {
     if (dtype != BRA_BF16 || impl == BRA_IMPL_SIMT) return FAMILY_SIMT;
+    if (impl == BRA_IMPL_AUTO && backward_dense_supported(d, dtype) && dense_pays(d, 2 * kSMs)) return FAMILY_DENSE;
     if (backward_img_supported(d, dtype) &&
-        (impl == BRA_IMPL_IMG || (impl == BRA_IMPL_AUTO && (long long)d.B * d.heads >= 64)))
+        (impl == BRA_IMPL_IMG || (impl == BRA_IMPL_AUTO && img_pays(d))))
         return FAMILY_IMG;
     return backward_direct_supported(d, dtype) ? FAMILY_DIRECT : FAMILY_SIMT;
 }
@@ -409,6 +410,8 @@ static cudaError_t launch_bwd_t(const Dims& d, int impl, const void* Q, const vo
         // the dQ kernel of this family and of the next also writes the inverse routing index
         if ((e = launch_backward_img(d, Q, K, V, index, inv_off, inv_list, lce_w, lse, dO, dQ, dK, dV,
                                      delta, status, st)) != cudaSuccess) return e;
+    } else if (family == FAMILY_DENSE) {
+        if ((e = launch_backward_dense(d, Q, K, V, index, lce_w, lse, dO, dQ, dK, dV, status, st)) != cudaSuccess) return e;
     } else if (family == FAMILY_DIRECT) {
         if ((e = launch_backward_direct(d, Q, K, V, index, inv_off, inv_list, lce_w, lse, dO, dQ, dK, dV,
                                         delta, status, st)) != cudaSuccess) return e;

@@ -1,0 +1,260 @@
+// Gradients of the routed attention for a fixed routing index on small maps with every token on the other side
+// (dense_common.cuh), bf16, head dim 32: one launch, CTA = (image, head), the slices of Q, K, V and dO resident.
+//   1. warp = 16 queries: delta = rowsum(P o dP) in a first walk over the keys, dQ = scale dS K in a second
+//   2. warp = 16 keys: dK = scale dS^T Q and dV = P^T dO in one walk over the queries; dV + LCE adjoint
+// P from the saved log-sum-exp, dP = dO V^T, dS = P o (dP - delta).  Who is routed where is the count table, so no inverse
+// index is needed.  Every sum has a fixed order.
+#include "dense_common.cuh"
+
+namespace bra {
+
+using namespace ptx;
+
+template <int TX, int NR>
+__global__ void __launch_bounds__(256, 2)
+bwd_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __restrict__ Kg, const __nv_bfloat16* __restrict__ Vg,
+                 const int32_t* __restrict__ index, const float* __restrict__ lse, const __nv_bfloat16* __restrict__ dOg,
+                 const float* __restrict__ lce_w, __nv_bfloat16* __restrict__ dQg, __nv_bfloat16* __restrict__ dKg,
+                 __nv_bfloat16* __restrict__ dVg, int32_t* __restrict__ status, Dims dm, DenseGeom gm) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    const uint32_t sbase = smem_u32(smem);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nthreads = blockDim.x;
+    const int g = lane >> 2, t4 = lane & 3;
+    const int h = blockIdx.y, b = blockIdx.z;
+    const int N0 = dm.H0 * dm.W0;
+    const size_t head_off = (size_t)b * N0 * dm.C * 2 + (size_t)h * 64;
+    const uint8_t* Gh = reinterpret_cast<const uint8_t*>(dOg) + head_off;
+    const uint32_t qs = sbase + gm.off_a, ks = sbase + gm.off_b, vs = sbase + gm.off_c, gs = sbase + gm.off_d;
+    Dims map = dm;
+    map.ws = dm.W;
+
+    dense_load_slices<4>({qs, ks, vs, gs}, {reinterpret_cast<const uint8_t*>(Qg) + head_off, reinterpret_cast<const uint8_t*>(Kg) + head_off,
+                                            reinterpret_cast<const uint8_t*>(Vg) + head_off, Gh}, dm, gm, tid, nthreads);
+    cp_async_commit();
+    float* s_w = reinterpret_cast<float*>(smem + gm.g.off_w);
+    if (dm.lce) {
+        load_lce_weights(s_w, lce_w, h, 32 * 25, tid, nthreads);
+        load_halo<1>(sbase + gm.g.off_halo, Gh, 0, 0, dm.H, map, gm.g, tid, nthreads);
+    }
+    cp_async_commit();
+    // lse * log2(e) and delta per token; a token behind the last has lse = inf (P = 0); one of the zero padding has zero rows
+    // of Q and dO and lse = delta = 0: as a query it adds nothing
+    float* s_l2 = reinterpret_cast<float*>(smem + gm.off_stat);
+    float* s_dl = s_l2 + gm.rows;
+    const float* lse_h = lse + ((size_t)b * dm.heads + h) * N0;
+    for (int t = tid; t < gm.rows; t += nthreads) {
+        const int2 at = dense_pos(dm, gm, t);
+        s_l2[t] = t >= dm.N ? INFINITY : at.y < dm.H0 && at.x < dm.W0 ? __ldg(lse_h + at.y * dm.W0 + at.x) * 1.4426950408889634f : 0.f;
+        s_dl[t] = 0.f;
+    }
+    uint8_t* reg = smem + gm.off_reg;
+    float* bias = reinterpret_cast<float*>(smem + gm.off_bias);
+    dense_regions(reg, dm, gm, tid, nthreads);
+    const int hi = dm.heads_i == 1 ? 0 : h;
+    unsigned long long* mask = reinterpret_cast<unsigned long long*>(smem + gm.off_mask);
+    const DenseRoutes routes = dense_routes(mask, bias, index + ((size_t)b * dm.heads_i + hi) * dm.R * dm.topk, status, dm, gm, tid, nthreads);
+    cp_async_wait<1>();
+    __syncthreads();
+
+    const float sl2 = dm.scale * 1.4426950408889634f;
+    const int steps = (dm.N + 15) / 16;
+    // token t in the caller's map, -1 in the padding
+    auto token = [&](int t) -> int {
+        const int2 at = dense_pos(dm, gm, t);
+        return t < dm.N && at.y < dm.H0 && at.x < dm.W0 ? at.y * dm.W0 + at.x : -1;
+    };
+
+    // ---- queries: delta, dQ ----
+#pragma unroll 1
+    for (int tile = warp; tile < steps; tile += gm.nw) {
+        const int r0 = tile * 16;
+        uint32_t qa[1][2][4], ga[1][2][4];
+        dense_a(qa, qs, r0, g, t4);
+        dense_a(ga, gs, r0, g, t4);
+        const float l0 = s_l2[r0 + g], l1 = s_l2[r0 + 8 + g];
+        const int i0 = min((int)reg[r0 + g], dm.R - 1), i1 = min((int)reg[r0 + 8 + g], dm.R - 1);
+        const unsigned long long m0 = mask[i0], m1 = mask[i1];
+        float delta[2] = {0.f, 0.f}, dq[1][4][4];
+#pragma unroll
+        for (int n = 0; n < 4; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) dq[0][n][e] = 0.f;
+#pragma unroll 1
+        for (int sweep = 0; sweep < 2; ++sweep) {
+#pragma unroll 2
+            for (int kb = 0; kb < dm.N; kb += 16) {
+                float c[2][4], dp[2][4];
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const uint4 kr[1] = {dense_row(ks, kb + 8 * j + g, t4)}, vr[1] = {dense_row(vs, kb + 8 * j + g, t4)};
+                    mma_rows<1>(c[j], qa, kr);
+                    mma_rows<1>(dp[j], ga, vr);
+                    float a0 = -l0, a1 = -l0, a2 = -l1, a3 = -l1;
+                    const int k = kb + 8 * j + 2 * t4;
+                    if (routes.weighted) {
+                        const uchar2 kg = *reinterpret_cast<const uchar2*>(reg + k);
+                        const float* b0 = bias + i0 * dm.R;
+                        const float* b1 = bias + i1 * dm.R;
+                        if (kg.x < 64) { a0 += b0[kg.x]; a2 += b1[kg.x]; }
+                        if (kg.y < 64) { a1 += b0[kg.y]; a3 += b1[kg.y]; }
+                    }
+                    c[j][0] = ex2_approx(fmaf(c[j][0], sl2, a0));
+                    c[j][1] = ex2_approx(fmaf(c[j][1], sl2, a1));
+                    c[j][2] = ex2_approx(fmaf(c[j][2], sl2, a2));
+                    c[j][3] = ex2_approx(fmaf(c[j][3], sl2, a3));
+                }
+                if (routes.masked || kb + 16 > dm.N) dense_mask<NR, 2>(c, m0, m1, kb, t4, reg, 0.f);
+                if (sweep == 0) {
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        delta[0] = fmaf(c[j][0], dp[j][0], fmaf(c[j][1], dp[j][1], delta[0]));
+                        delta[1] = fmaf(c[j][2], dp[j][2], fmaf(c[j][3], dp[j][3], delta[1]));
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        c[j][0] *= dp[j][0] - delta[0]; c[j][1] *= dp[j][1] - delta[0];
+                        c[j][2] *= dp[j][2] - delta[1]; c[j][3] *= dp[j][3] - delta[1];
+                    }
+                    uint32_t sa[1][4];
+                    frag_hi(sa[0], c[0], c[1]);
+                    dense_mma_tokens<1>(dq, sa, ks, kb, lane);
+                }
+            }
+            if (sweep == 0) {
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    delta[r] += __shfl_xor_sync(0xffffffffu, delta[r], 1);
+                    delta[r] += __shfl_xor_sync(0xffffffffu, delta[r], 2);
+                }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int t = r0 + g + 8 * r, tok = token(t);
+            if (tok < 0) continue;                                    // delta of a padding row stays 0
+            if (t4 == 0) s_dl[t] = delta[r];
+            uint32_t* o = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(dQg) + head_off) + (size_t)(uint32_t)tok * (dm.C / 2) + t4;
+#pragma unroll
+            for (int n = 0; n < 4; ++n) o[4 * n] = pack2_bf16(dq[0][n][2 * r] * dm.scale, dq[0][n][2 * r + 1] * dm.scale);
+        }
+    }
+    __syncthreads();
+
+    // ---- keys: dK, dV (a warp has at most two tiles; dV is staged once all warps have read the slices) ----
+    float dv[2][4][4];
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        const int r0 = (warp + x * gm.nw) * 16;
+        if (r0 >= steps * 16) continue;
+        uint32_t ka[1][2][4], va[1][2][4];
+        dense_a(ka, ks, r0, g, t4);
+        dense_a(va, vs, r0, g, t4);
+        const int k0 = min((int)reg[r0 + g], dm.R - 1), k1 = min((int)reg[r0 + 8 + g], dm.R - 1);
+        const unsigned long long m0 = mask[64 + k0], m1 = mask[64 + k1];
+        float dk[1][4][4];
+#pragma unroll
+        for (int n = 0; n < 4; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) dk[0][n][e] = dv[x][n][e] = 0.f;
+#pragma unroll 2
+        for (int qb = 0; qb < dm.N; qb += 16) {
+            float c[2][4], dp[2][4];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const uint4 qr[1] = {dense_row(qs, qb + 8 * j + g, t4)}, gr[1] = {dense_row(gs, qb + 8 * j + g, t4)};
+                mma_rows<1>(c[j], ka, qr);
+                mma_rows<1>(dp[j], va, gr);
+                const int q = qb + 8 * j + 2 * t4;
+                const float2 l2 = *reinterpret_cast<const float2*>(s_l2 + q), dl = *reinterpret_cast<const float2*>(s_dl + q);
+                float a0 = -l2.x, a1 = -l2.y, a2 = -l2.x, a3 = -l2.y;
+                if (routes.weighted) {
+                    const uchar2 qg = *reinterpret_cast<const uchar2*>(reg + q);
+                    if (qg.x < 64) { a0 += bias[qg.x * dm.R + k0]; a2 += bias[qg.x * dm.R + k1]; }
+                    if (qg.y < 64) { a1 += bias[qg.y * dm.R + k0]; a3 += bias[qg.y * dm.R + k1]; }
+                }
+                c[j][0] = ex2_approx(fmaf(c[j][0], sl2, a0));
+                c[j][1] = ex2_approx(fmaf(c[j][1], sl2, a1));
+                c[j][2] = ex2_approx(fmaf(c[j][2], sl2, a2));
+                c[j][3] = ex2_approx(fmaf(c[j][3], sl2, a3));
+                dp[j][0] -= dl.x; dp[j][1] -= dl.y; dp[j][2] -= dl.x; dp[j][3] -= dl.y;
+            }
+            if (routes.masked) dense_mask<NR, 2>(c, m0, m1, qb, t4, reg, 0.f);
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) dp[j][e] *= c[j][e];
+            uint32_t a[1][4];
+            frag_hi(a[0], dp[0], dp[1]);
+            dense_mma_tokens<1>(dk, a, qs, qb, lane);
+            frag_hi(a[0], c[0], c[1]);
+            dense_mma_tokens<1>(dv + x, a, gs, qb, lane);
+        }
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int tok = token(r0 + g + 8 * r);
+            if (tok < 0) continue;
+            uint32_t* o = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(dKg) + head_off) + (size_t)(uint32_t)tok * (dm.C / 2) + t4;
+#pragma unroll
+            for (int n = 0; n < 4; ++n) o[4 * n] = pack2_bf16(dk[0][n][2 * r] * dm.scale, dk[0][n][2 * r + 1] * dm.scale);
+        }
+    }
+    cp_async_wait<0>();
+    __syncthreads();
+    float* st = reinterpret_cast<float*>(smem + gm.g.off_st);
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        const int r0 = (warp + x * gm.nw) * 16;
+        if (r0 >= steps * 16) continue;
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int t = r0 + g + 8 * r;
+            if (t >= dm.N) continue;
+            const int2 at = dense_pos(dm, gm, t);
+            float* dst = st + (at.y * dm.W + at.x) * dn::ST + 2 * t4;
+#pragma unroll
+            for (int n = 0; n < 4; ++n) *reinterpret_cast<float2*>(dst + 8 * n) = make_float2(dv[x][n][2 * r], dv[x][n][2 * r + 1]);
+        }
+    }
+    __syncthreads();
+    // ---- LCE adjoint + store of dV: correlation of dO with the flipped filter ----
+    lce_chunk<1, 4, TX, true, dn::ST>(st, sbase + gm.g.off_halo, s_w, nullptr, dm.lce, dVg + head_off / 2, 0, 0, dm.H, map, gm.g, warp, gm.nw, lane);
+}
+
+// ------------------------------------------------------------------ host side
+bool backward_dense_supported(const Dims& d, int dtype) {
+    return dense_supported(d, dtype) && dense_geom(d, 4, d.S).smem_bytes <= 200 * 1024;
+}
+
+template <int TX, int NR>
+static cudaError_t launch_t(const Dims& d, const DenseGeom& g, const void* Q, const void* K, const void* V, const int32_t* index,
+                            const float* lce_w, const float* lse, const void* dO, void* dQ, void* dK, void* dV, int32_t* status, cudaStream_t st) {
+    auto kernel = bwd_dense_kernel<TX, NR>;
+    static PerDeviceMax smem_set;
+    if (g.smem_bytes > 48 * 1024) {
+        const cudaError_t e = smem_set.ensure(g.smem_bytes, [&] {
+            return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, g.smem_bytes);
+        });
+        if (e != cudaSuccess) return e;
+    }
+    typedef __nv_bfloat16 bf;
+    count_launch();
+    return launch_kernel(kernel, dim3(1, d.heads, d.B), dim3(g.nw * 32), (size_t)g.smem_bytes, st, false,
+                         static_cast<const bf*>(Q), static_cast<const bf*>(K), static_cast<const bf*>(V), index, lse, static_cast<const bf*>(dO),
+                         lce_w, static_cast<bf*>(dQ), static_cast<bf*>(dK), static_cast<bf*>(dV), status, d, g);
+}
+
+cudaError_t launch_backward_dense(const Dims& d, const void* Q, const void* K, const void* V, const int32_t* index, const float* lce_w,
+                                  const float* lse, const void* dO, void* dQ, void* dK, void* dV, int32_t* status, cudaStream_t st) {
+    const DenseGeom g = dense_geom(d, 4, d.S);
+    Dims map = d;
+    map.ws = d.W;
+    const bool narrow = lce_tile_width(g.g, map) == 2;
+#define BRA_GO(TX, NR) return launch_t<TX, NR>(d, g, Q, K, V, index, lce_w, lse, dO, dQ, dK, dV, status, st)
+    if (d.n_r == 4) { if (narrow) BRA_GO(2, 4); BRA_GO(4, 4); }
+    if (narrow) BRA_GO(2, 0);
+    BRA_GO(4, 0);
+#undef BRA_GO
+}
+
+}  // namespace bra

@@ -116,7 +116,7 @@ static void crop_out(const Dims& d, const WsLayout& L, char* w, int slot, void* 
         *ok = false;
 }
 
-enum Path { PATH_NONE, PATH_SIMT, PATH_DIRECT, PATH_TC, PATH_TC_WIDE, PATH_IMG };
+enum Path { PATH_NONE, PATH_SIMT, PATH_DIRECT, PATH_TC, PATH_TC_WIDE, PATH_IMG, PATH_DENSE };
 
 static Path choose_attend(const Dims& d, int dtype, int impl) {
     switch (impl) {
@@ -130,15 +130,15 @@ static Path choose_attend(const Dims& d, int dtype, int impl) {
     }
     if (attend_tc_supported(d, dtype)) return PATH_TC;
     if (attend_tc_wide_supported(d, dtype)) return PATH_TC_WIDE;
-    // one CTA per (image, head): worth it once those fill a good part of the GPU
-    if (attend_img_supported(d, dtype) && (long long)d.B * d.heads >= 64) return PATH_IMG;
+    if (attend_dense_supported(d, dtype) && dense_pays(d, 64)) return PATH_DENSE;
+    if (attend_img_supported(d, dtype) && img_pays(d)) return PATH_IMG;
     if (attend_direct_supported(d, dtype)) return PATH_DIRECT;
     if (attend_simt_supported(d)) return PATH_SIMT;
     return PATH_NONE;
 }
 
 // Paths whose kernels take a map that S does not divide as it is (the others get a zero-padded copy).
-static bool any_map(Path path) { return path == PATH_DIRECT || path == PATH_SIMT; }
+static bool any_map(Path path) { return path == PATH_DIRECT || path == PATH_SIMT || path == PATH_DENSE; }
 
 static bra_status run_route(const Dims& d, int dtype, const void* Q, const void* K,
                             float* q_mean, float* k_mean, int32_t* index, cudaStream_t st) {
@@ -158,6 +158,7 @@ static bra_status run_attend(Path path, const Dims& d, int dtype, const void* Q,
         case PATH_TC:   e = launch_attend_tc(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel); break;
         case PATH_TC_WIDE: e = launch_attend_tc_wide(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel); break;
         case PATH_IMG:  e = launch_attend_img(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel); break;
+        case PATH_DENSE: e = launch_attend_dense(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel); break;
         default: return BRA_ERR_UNSUPPORTED;
     }
     return e == cudaSuccess ? BRA_OK : BRA_ERR_CUDA;
@@ -274,9 +275,14 @@ bra_status bra_forward(const bra_problem* p, const void* Q, const void* K, const
             return launch_forward_tc(dp, q, k, v, lce_w, lce_b, o, idx, l, qm, km, status, p->inject, st) == cudaSuccess ? BRA_OK : BRA_ERR_CUDA;
         });
     }
+    // every region is routed to and the caller does not ask in which order: nothing to route
+    if (path == PATH_DENSE && d.topk == d.R && !index)
+        return attend_any_map(path, d, L, p->dtype, Q, K, V, nullptr, lce_w, lce_b, O, lse, w, st, false);
     s = run_route(d, p->dtype, Q, K, qm, km, idx, st);
     if (s != BRA_OK) return s;
-    return attend_any_map(path, d, L, p->dtype, Q, K, V, idx, lce_w, lce_b, O, lse, w, st, true);
+    // with every region routed to, the attention need not look at the order
+    const int32_t* seen = path == PATH_DENSE && d.topk == d.R ? nullptr : idx;
+    return attend_any_map(path, d, L, p->dtype, Q, K, V, seen, lce_w, lce_b, O, lse, w, st, true);
 }
 
 bra_status bra_backward(const bra_problem* p, const void* Q, const void* K, const void* V,

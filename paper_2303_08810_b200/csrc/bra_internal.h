@@ -98,6 +98,27 @@ bool attend_img_supported(const Dims& d, int dtype);
 cudaError_t launch_attend_img(const Dims& d, const void* Q, const void* K, const void* V,
                               const int32_t* index, const float* lce_w, const float* lce_b,
                               void* O, float* lse, int32_t* status, cudaStream_t st, bool after_own_kernel);
+// Small maps, every token a key (index NULL: every query attends to every region once)
+bool attend_dense_supported(const Dims& d, int dtype);
+cudaError_t launch_attend_dense(const Dims& d, const void* Q, const void* K, const void* V,
+                                const int32_t* index, const float* lce_w, const float* lce_b,
+                                void* O, float* lse, int32_t* status, cudaStream_t st, bool after_own_kernel);
+// true if the dense kernels are the faster ones: they walk all tokens of the map for 16 queries at a time, the routed ones
+// topk regions for a tile of one region, n_r of whose 16 rows are used.  With more than 64 tokens a CTA's walk is long and
+// wants `pairs` (image, head) pairs to fill the GPU.  Measured (B200, us, dense against the best other kernel), attention /
+// gradients, 14 x 14 map, 49 regions, topk 16, 8 heads: 512 pairs 44 / 103 against 44 / 156, 128 pairs 17 / 53 against
+// 25 / 47, 32 pairs 14 / 36 against 11 / 28; 7 x 7 map, topk 49, 16 heads: 1024 pairs 27 / 41 against 120 / 282, 16 pairs
+// 17 / 25 against 11 / 28.
+inline bool dense_pays(const Dims& d, int pairs) {
+    return (long long)d.N < (long long)d.topk * ((d.n_r + 15) / 16 * 16) && (d.N <= 64 || (long long)d.B * d.heads >= pairs);
+}
+// true if there are enough (image, head) pairs for the kernels with one CTA each.  Measured, 28 x 28 map, 4 heads, topk 4,
+// attention / gradients against the kernels with a CTA per region: 256 pairs 43 / 103 against 50 / 112, 64 pairs 31 / 50
+// against 19 / 36.
+inline bool img_pays(const Dims& d) { return (long long)d.B * d.heads >= kSMs; }
+bool backward_dense_supported(const Dims& d, int dtype);
+cudaError_t launch_backward_dense(const Dims& d, const void* Q, const void* K, const void* V, const int32_t* index, const float* lce_w,
+                                  const float* lse, const void* dO, void* dQ, void* dK, void* dV, int32_t* status, cudaStream_t st);
 bool attend_tc_wide_supported(const Dims& d, int dtype);
 cudaError_t launch_attend_tc_wide(const Dims& d, const void* Q, const void* K, const void* V,
                                   const int32_t* index, const float* lce_w, const float* lce_b,

@@ -240,7 +240,7 @@ __device__ __forceinline__ void lce_tile(float2 (&acc)[TY][TX], uint32_t halo, i
 }
 // The LCE of a chunk (rows x ws tokens at (y0, x0)) by `gwarps` warps, added to the staged attention term
 // (fp32 [token][32 PL channels]) and stored as bf16.
-template <int PL, int TY, int TX, bool FLIP>
+template <int PL, int TY, int TX, bool FLIP, int ST = 32 * PL>       // ST: floats per staged token
 __device__ __forceinline__ void lce_chunk(const float* st, uint32_t halo, const float* s_w, const float* bias, bool lce, __nv_bfloat16* out_head,
                                           int y0, int x0, int rows, const Dims& dm, const DirGeom& gm, int gwarp, int gwarps, int lane) {
     const int cp = PL == 2 ? lane : lane & 15, sub = PL == 2 ? 0 : lane >> 4;
@@ -265,7 +265,7 @@ __device__ __forceinline__ void lce_chunk(const float* st, uint32_t halo, const 
 #pragma unroll
             for (int xx = 0; xx < TX; ++xx) acc[yy][xx] = b2;
         if (lce) lce_tile<PL, TY, TX, FLIP>(acc, halo + ty * TY * gm.halo_row + tx * TX * 64 * PL + cp * 4, gm.halo_row, wv);
-        const float* src = st + (ty * TY * dm.ws + tx * TX) * 32 * PL + 2 * cp;
+        const float* src = st + (ty * TY * dm.ws + tx * TX) * ST + 2 * cp;
         __nv_bfloat16* dst = out_head + (size_t)(uint32_t)((y0 + ty * TY) * dm.W0 + x0 + tx * TX) * dm.C + 2 * cp;
         const int ny = min(rows - ty * TY, dm.H0 - y0 - ty * TY), nx = min(dm.ws - tx * TX, dm.W0 - x0 - tx * TX);
 #pragma unroll
@@ -274,11 +274,11 @@ __device__ __forceinline__ void lce_chunk(const float* st, uint32_t halo, const 
 #pragma unroll
             for (int xx = 0; xx < TX; ++xx) {
                 if (xx >= nx) break;
-                const float2 a = *reinterpret_cast<const float2*>(src + xx * 32 * PL);
+                const float2 a = *reinterpret_cast<const float2*>(src + xx * ST);
                 const float2 o = __fadd2_rn(a, acc[yy][xx]);
                 *reinterpret_cast<uint32_t*>(dst + (size_t)xx * dm.C) = pack2_bf16(o.x, o.y);
             }
-            src += dm.ws * 32 * PL;
+            src += dm.ws * ST;
             dst += (size_t)dm.W0 * dm.C;
         }
     }

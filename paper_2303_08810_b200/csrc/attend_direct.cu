@@ -15,14 +15,12 @@
 // the routed keys (every group reads topk * n_r of them).
 #include "direct_common.cuh"
 
-#include <type_traits>
-
 namespace bra {
 
 using namespace ptx;
 
-template <int PL, bool EXACT, bool ZEROS, int TY, int TX>
-__global__ void __launch_bounds__(PL == 2 ? 128 : 256, PL == 2 ? 3 : 2)
+template <int PL, bool EXACT, int RT, int TY, int TX>
+__global__ void __launch_bounds__((PL == 2 ? 128 : 256) / RT, RT == 2 ? (PL == 2 ? 4 : 3) : PL == 2 ? 3 : 2)
 attend_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __restrict__ Kg,
                      const __nv_bfloat16* __restrict__ Vg, const int32_t* index,
                      const float* __restrict__ lce_w, const float* __restrict__ lce_b,
@@ -63,6 +61,10 @@ attend_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* 
         if (live) load_halo<PL>(sbase + gm.off_halo + grp * gm.halo_bytes, Vh, y0, x0, rows, dm, gm, glane, glanes);
     }
     cp_async_commit();
+    uint32_t* tab = reinterpret_cast<uint32_t*>(smem + gm.off_tab + grp * gm.tab_bytes);
+    uint32_t* dead = tab + gm.tab;
+    int* zeros = reinterpret_cast<int*>(dead + gm.tab / 32);          // keys of the zero padding
+    if (glane == 0) *zeros = 0;
     __syncthreads();                                                  // weights
     pdl_wait();          // in bra_forward the launch may overlap the tail of the routing kernel
     if (!live) return;                                                // a whole warp (one_warp) and no barrier of the CTA follows
@@ -70,120 +72,144 @@ attend_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* 
     const int hi = dm.heads_i == 1 ? 0 : h;
     const int32_t* irow = index + (((size_t)b * dm.heads_i + hi) * dm.R + i) * dm.topk;
     const int total = dm.topk * dm.n_r;
-    uint32_t* tab = reinterpret_cast<uint32_t*>(smem + gm.off_tab) + grp * gm.tab;
     float* st = reinterpret_cast<float*>(smem + gm.off_st + grp * gm.st_bytes);
     const float sl2 = dm.scale * 1.4426950408889634f;
     const int passes = (total + gm.tab - 1) / gm.tab;
-    bool any_bad = false;
-
-    for (int tile = gwarp; tile - gwarp < gm.tpc; tile += gwarps) {   // every warp of the group takes the same number of rounds
+    for (int tile = gwarp * RT; tile - gwarp * RT < gm.tpc; tile += gwarps * RT) {    // every warp of the group takes the same number of rounds
         const bool has = tile * 16 < ntok;
-        uint32_t qa[PL][2][4];
-        {
-            uint4 lo[PL], hi4[PL];
-            const int ta = tile * 16 + g, tb = ta + 8;
-            ld_row<PL>(lo, Qb, ta < ntok ? token_of(dm, gm, i, ck * gm.hb * dm.ws + ta) : -1, tok_bytes);
-            ld_row<PL>(hi4, Qb, tb < ntok ? token_of(dm, gm, i, ck * gm.hb * dm.ws + tb) : -1, tok_bytes);
-            rows_to_a<PL>(qa, lo, hi4);
+        const bool first_round = tile == gwarp * RT;
+        uint32_t qa[RT][PL][2][4];
+        int tok[RT][2];
+#pragma unroll
+        for (int x = 0; x < RT; ++x) {
+            uint4 v[2][PL];
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const int t = (tile + x) * 16 + g + 8 * r;
+                tok[x][r] = t < ntok ? token_of(dm, gm, i, ck * gm.hb * dm.ws + t) : -1;
+                ld_row<PL>(v[r], Qb, tok[x][r], tok_bytes);
+            }
+            rows_to_a<PL>(qa[x], v[0], v[1]);
         }
-        float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
-        float o[PL][4][4];
+        float m_run[RT][2], l_run[RT][2], o[RT][PL][4][4];
 #pragma unroll
-        for (int p = 0; p < PL; ++p)
+        for (int x = 0; x < RT; ++x) {
+            m_run[x][0] = m_run[x][1] = -INFINITY;
+            l_run[x][0] = l_run[x][1] = 0.f;
 #pragma unroll
-            for (int n = 0; n < 4; ++n)
+            for (int p = 0; p < PL; ++p)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) o[p][n][e] = 0.f;
+                for (int n = 0; n < 4; ++n)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) o[x][p][n][e] = 0.f;
+        }
 
         for (int pass = 0; pass < passes; ++pass) {
             const int k0 = pass * gm.tab;
             const int nk = min(gm.tab, (total - k0 + 31) / 32 * 32);
-            if (passes > 1 || tile == gwarp) {
-                if (pass > 0 || tile != gwarp) group_sync();          // the table before has been read
-                const bool bad = fill_keys(tab, irow, i, k0, nk, total, glane, glanes, status, dm, gm);
-                any_bad = (one_warp ? __any_sync(0xffffffffu, bad) : __syncthreads_or(bad)) || any_bad;
-                if (one_warp) __syncwarp();
+            if (passes > 1 || first_round) {
+                if (pass > 0 || !first_round) group_sync();           // the table before has been read
+                int z = fill_keys(tab, dead, irow, k0, nk, total, glane, glanes, status, dm, gm);
+                if (first_round) {
+                    z = __reduce_add_sync(0xffffffffu, z);
+                    if (lane == 0 && z) atomicAdd(zeros, z);
+                }
+                group_sync();
             }
             if (!has) continue;
             uint4 kr[2][2][PL], vr[2][2][PL];                         // [16-key step][rows g, g + 8]
 #pragma unroll
             for (int s = 0; s < 2; ++s)
 #pragma unroll
-                for (int e = 0; e < 2; ++e) ld_token<PL, ZEROS>(kr[s][e], Kb, tab[16 * s + 8 * e + g]);
+                for (int e = 0; e < 2; ++e) ld_token<PL>(kr[s][e], Kb, tab[16 * s + 8 * e + g]);
             for (int kb = 0; kb < nk; kb += 32) {
-                float c[4][4];
+                float c[RT][4][4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) mma_rows<PL>(c[j], qa, kr[j >> 1][j & 1]);
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int x = 0; x < RT; ++x) mma_rows<PL>(c[x][j], qa[x], kr[j >> 1][j & 1]);
 #pragma unroll
                 for (int s = 0; s < 2; ++s)
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
-                        ld_token<PL, ZEROS>(vr[s][e], Vb, tab[kb + 16 * s + 8 * e + g]);
-                        if (kb + 32 < nk) ld_token<PL, ZEROS>(kr[s][e], Kb, tab[kb + 32 + 16 * s + 8 * e + g]);
+                        ld_token<PL>(vr[s][e], Vb, tab[kb + 16 * s + 8 * e + g]);
+                        if (kb + 32 < nk) ld_token<PL>(kr[s][e], Kb, tab[kb + 32 + 16 * s + 8 * e + g]);
                     }
-                if (any_bad || k0 + kb + 32 > total) {                // keys that do not count
+                const uint32_t bits = dead[kb >> 5];
+                if (bits) mask_columns<RT, 4>(c, bits, t4, -INFINITY);
+                float mx[RT][2];
+                bool up = false;
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const int kk = k0 + kb + 8 * j + 2 * t4;
-                        if (dead_key(kk, total, any_bad, irow, dm, gm)) { c[j][0] = -INFINITY; c[j][2] = -INFINITY; }
-                        if (dead_key(kk + 1, total, any_bad, irow, dm, gm)) { c[j][1] = -INFINITY; c[j][3] = -INFINITY; }
-                    }
-                }
-                float mx[2];
-#pragma unroll
-                for (int r = 0; r < 2; ++r)
-                    mx[r] = fmaxf(fmax3(fmax3(c[0][2 * r], c[0][2 * r + 1], c[1][2 * r]), c[1][2 * r + 1], c[2][2 * r]),
-                                  fmax3(c[2][2 * r + 1], c[3][2 * r], c[3][2 * r + 1])) * sl2;
-                if (__any_sync(0xffffffffu, mx[0] > m_run[0] || mx[1] > m_run[1])) {
+                for (int x = 0; x < RT; ++x)
 #pragma unroll
                     for (int r = 0; r < 2; ++r) {
-                        mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 1));
-                        mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 2));
-                        const float mnew = fmaxf(m_run[r], mx[r]);
-                        const float corr = mnew == -INFINITY ? 1.f : ex2_approx(m_run[r] - mnew);
-                        m_run[r] = mnew;
-                        l_run[r] *= corr;
+                        mx[x][r] = fmaxf(fmax3(fmax3(c[x][0][2 * r], c[x][0][2 * r + 1], c[x][1][2 * r]), c[x][1][2 * r + 1], c[x][2][2 * r]),
+                                         fmax3(c[x][2][2 * r + 1], c[x][3][2 * r], c[x][3][2 * r + 1])) * sl2;
+                        up = up || mx[x][r] > m_run[x][r];
+                    }
+                if (__any_sync(0xffffffffu, up)) {
 #pragma unroll
-                        for (int p = 0; p < PL; ++p)
+                    for (int x = 0; x < RT; ++x)
 #pragma unroll
-                            for (int n = 0; n < 4; ++n) { o[p][n][2 * r] *= corr; o[p][n][2 * r + 1] *= corr; }
+                        for (int r = 0; r < 2; ++r) {
+                            mx[x][r] = fmaxf(mx[x][r], __shfl_xor_sync(0xffffffffu, mx[x][r], 1));
+                            mx[x][r] = fmaxf(mx[x][r], __shfl_xor_sync(0xffffffffu, mx[x][r], 2));
+                            const float mnew = fmaxf(m_run[x][r], mx[x][r]);
+                            const float corr = mnew == -INFINITY ? 1.f : ex2_approx(m_run[x][r] - mnew);
+                            m_run[x][r] = mnew;
+                            l_run[x][r] *= corr;
+#pragma unroll
+                            for (int p = 0; p < PL; ++p)
+#pragma unroll
+                                for (int n = 0; n < 4; ++n) { o[x][p][n][2 * r] *= corr; o[x][p][n][2 * r + 1] *= corr; }
+                        }
+                }
+#pragma unroll
+                for (int x = 0; x < RT; ++x) {
+                    const float mn0 = m_run[x][0] == -INFINITY ? 0.f : -m_run[x][0], mn1 = m_run[x][1] == -INFINITY ? 0.f : -m_run[x][1];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        c[x][j][0] = ex2_approx(fmaf(c[x][j][0], sl2, mn0));
+                        c[x][j][1] = ex2_approx(fmaf(c[x][j][1], sl2, mn0));
+                        c[x][j][2] = ex2_approx(fmaf(c[x][j][2], sl2, mn1));
+                        c[x][j][3] = ex2_approx(fmaf(c[x][j][3], sl2, mn1));
+                        l_run[x][0] += c[x][j][0] + c[x][j][1];
+                        l_run[x][1] += c[x][j][2] + c[x][j][3];
                     }
                 }
-                const float mn0 = m_run[0] == -INFINITY ? 0.f : -m_run[0], mn1 = m_run[1] == -INFINITY ? 0.f : -m_run[1];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    c[j][0] = ex2_approx(fmaf(c[j][0], sl2, mn0));
-                    c[j][1] = ex2_approx(fmaf(c[j][1], sl2, mn0));
-                    c[j][2] = ex2_approx(fmaf(c[j][2], sl2, mn1));
-                    c[j][3] = ex2_approx(fmaf(c[j][3], sl2, mn1));
-                    l_run[0] += c[j][0] + c[j][1];
-                    l_run[1] += c[j][2] + c[j][3];
-                }
-#pragma unroll
-                for (int s = 0; s < 2; ++s) mma_tokens<PL, EXACT>(o, c[2 * s], c[2 * s + 1], vr[s][0], vr[s][1]);
+                for (int s = 0; s < 2; ++s) mma_tokens<PL, EXACT>(o, c, 2 * s, vr[s][0], vr[s][1]);
             }
         }
-        // ---- normalise; O^att to the staging tile; lse ----
+        // ---- keys of the zero padding; normalise; O^att to the staging tile; lse ----
+        const int nz = *zeros;
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            l_run[r] += __shfl_xor_sync(0xffffffffu, l_run[r], 1);
-            l_run[r] += __shfl_xor_sync(0xffffffffu, l_run[r], 2);
-            const int tk = tile * 16 + g + 8 * r;
-            if (has && tk < ntok) {
-                const float inv = l_run[r] > 0.f ? 1.f / l_run[r] : 0.f;
-                float* dst = st + tk * 32 * PL + t4 * 8;
+        for (int x = 0; x < RT; ++x)
 #pragma unroll
-                for (int p = 0; p < PL; ++p)
+            for (int r = 0; r < 2; ++r) {
+                float l = l_run[x][r], m = m_run[x][r], f = 1.f;
+                l += __shfl_xor_sync(0xffffffffu, l, 1);
+                l += __shfl_xor_sync(0xffffffffu, l, 2);
+                if (nz) {                                             // nz scores of 0
+                    const float mnew = fmaxf(m, 0.f);
+                    f = ex2_approx(m - mnew);
+                    l = l * f + (float)nz * ex2_approx(-mnew);
+                    m = mnew;
+                }
+                const int tk = (tile + x) * 16 + g + 8 * r;
+                if (tk < ntok) {
+                    const float inv = l > 0.f ? f / l : 0.f;
+                    float* dst = st + tk * 32 * PL + t4 * 8;
 #pragma unroll
-                    for (int q = 0; q < 2; ++q)
-                        *reinterpret_cast<float4*>(dst + p * 32 + 4 * q) =
-                            make_float4(o[p][2 * q][2 * r] * inv, o[p][2 * q][2 * r + 1] * inv, o[p][2 * q + 1][2 * r] * inv, o[p][2 * q + 1][2 * r + 1] * inv);
-                if (lse && t4 == 0) {
-                    const int tok = token_of(dm, gm, i, ck * gm.hb * dm.ws + tk);
-                    if (tok >= 0) lse[((size_t)b * dm.heads + h) * N0 + tok] = (m_run[r] + log2f(l_run[r])) * 0.6931471805599453f;
+                    for (int p = 0; p < PL; ++p)
+#pragma unroll
+                        for (int q = 0; q < 2; ++q)
+                            *reinterpret_cast<float4*>(dst + p * 32 + 4 * q) =
+                                make_float4(o[x][p][2 * q][2 * r] * inv, o[x][p][2 * q][2 * r + 1] * inv, o[x][p][2 * q + 1][2 * r] * inv,
+                                            o[x][p][2 * q + 1][2 * r + 1] * inv);
+                    if (lse && t4 == 0 && tok[x][r] >= 0) lse[((size_t)b * dm.heads + h) * N0 + tok[x][r]] = (m + log2f(l)) * 0.6931471805599453f;
                 }
             }
-        }
     }
     cp_async_wait<0>();
     group_sync();
@@ -196,13 +222,13 @@ bool attend_direct_supported(const Dims& d, int dtype) {
     if (dtype != BRA_BF16 || (d.d != 32 && d.d != 64)) return false;
     if (d.ws > 128 || d.R > 65535 || (long long)d.topk * d.n_r * d.n_r >= (1ll << 32)) return false;   // fast division by n_r
     if ((long long)d.H0 * d.W0 * d.C / 8 >= (1ll << 31) || d.heads > 65535 || d.B > 65535) return false;
-    return direct_geom(d, d.lce, 4).smem_bytes <= 200 * 1024;
+    return direct_geom(d, d.lce, 4, 1).smem_bytes <= 200 * 1024;
 }
 
-template <int PL, bool EXACT, bool ZEROS, int TY, int TX>
+template <int PL, bool EXACT, int RT, int TY, int TX>
 static cudaError_t launch_t(const Dims& d, const DirGeom& g, const void* Q, const void* K, const void* V, const int32_t* index,
                             const float* lce_w, const float* lce_b, void* O, float* lse, int32_t* status, cudaStream_t st, bool after_own_kernel) {
-    auto kernel = attend_direct_kernel<PL, EXACT, ZEROS, TY, TX>;
+    auto kernel = attend_direct_kernel<PL, EXACT, RT, TY, TX>;
     static PerDeviceMax smem_set;
     if (g.smem_bytes > 48 * 1024) {
         const cudaError_t e = smem_set.ensure(g.smem_bytes, [&] {
@@ -219,22 +245,22 @@ static cudaError_t launch_t(const Dims& d, const DirGeom& g, const void* Q, cons
 cudaError_t launch_attend_direct(const Dims& d, const void* Q, const void* K, const void* V,
                                  const int32_t* index, const float* lce_w, const float* lce_b,
                                  void* O, float* lse, int32_t* status, cudaStream_t st, bool after_own_kernel) {
-    const DirGeom g = direct_geom(d, d.lce, 4);
-    const bool zeros = d.H != d.H0 || d.W != d.W0;
-    auto go = [&](auto z) -> cudaError_t {
-        constexpr bool Z = decltype(z)::value;
-#define BRA_GO(PL, EX, TY, TX) return launch_t<PL, EX, Z, TY, TX>(d, g, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel)
-        if (d.hs <= 2) { if (g.planes == 2) BRA_GO(2, false, 2, 2); BRA_GO(1, false, 2, 2); }
-        if (g.planes == 2) BRA_GO(2, false, 4, 4);
-        if (direct_exact(d)) BRA_GO(1, true, 4, 3);
-        switch (lce_tile_width(g, d)) {
-            case 2: BRA_GO(1, false, 4, 2);
-            case 3: BRA_GO(1, false, 4, 3);
-            default: BRA_GO(1, false, 4, 4);
-        }
+    const int rt = direct_rt(d);
+    const DirGeom g = direct_geom(d, d.lce, 4, rt);
+#define BRA_GO(PL, EX, RT, TY, TX) return launch_t<PL, EX, RT, TY, TX>(d, g, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel)
+    if (g.planes == 2) {
+        if (rt == 2) BRA_GO(2, false, 2, 4, 4);
+        if (d.hs <= 2) BRA_GO(2, false, 1, 2, 2);
+        BRA_GO(2, false, 1, 4, 4);
+    }
+    if (direct_exact(d)) { if (rt == 2) BRA_GO(1, true, 2, 4, 4); BRA_GO(1, true, 1, 4, 4); }
+    const int tx = lce_tile_width(g, d);
+    if (rt == 2) { if (tx == 2) BRA_GO(1, false, 2, 4, 2); if (tx == 3) BRA_GO(1, false, 2, 4, 3); BRA_GO(1, false, 2, 4, 4); }
+    if (d.hs <= 2) BRA_GO(1, false, 1, 2, 2);
+    if (tx == 2) BRA_GO(1, false, 1, 4, 2);
+    if (tx == 3) BRA_GO(1, false, 1, 4, 3);
+    BRA_GO(1, false, 1, 4, 4);
 #undef BRA_GO
-    };
-    return zeros ? go(std::true_type()) : go(std::false_type());
 }
 
 }  // namespace bra

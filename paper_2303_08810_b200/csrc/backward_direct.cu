@@ -9,7 +9,8 @@
 // memory straight into MMA fragments, a table of token numbers per group, no barriers in the streaming loop.  A row
 // that was loaded serves both products it takes part in: as loaded where the contraction runs over channels, through
 // movmatrix where it runs over tokens.  No atomics: every sum has a fixed order, results are bit-identical from run
-// to run.
+// to run.  (Two tiles per warp, which pay in the forward kernel, do not here: 8 warps per SM at 168 registers,
+// dQ 140 -> 170 us and dK / dV 274 -> 331 us at 2 x 100 x 167, S = 16.)
 #include "direct_common.cuh"
 #include "inverse_index.cuh"
 
@@ -21,7 +22,7 @@ using namespace ptx;
 // The CTAs of grid row 0 build the inverse routing index for the dK / dV kernel instead.
 // SINGLE: all keys of a group (at most 64) in one block, S and dP computed once; otherwise one sweep for delta and
 // one for dQ.
-template <int PL, bool EXACT, bool SINGLE, bool ZEROS>
+template <int PL, bool EXACT, bool SINGLE>
 __global__ void __launch_bounds__(PL == 2 ? 128 : 256, PL == 2 ? 3 : 2)
 bwd_dq_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __restrict__ Kg,
                      const __nv_bfloat16* __restrict__ Vg, const int32_t* __restrict__ index,
@@ -29,7 +30,7 @@ bwd_dq_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* 
                      __nv_bfloat16* __restrict__ dQg, float* __restrict__ delta_out,
                      int32_t* __restrict__ inv_off, int32_t* __restrict__ inv_list, bool inv_bits,
                      int32_t* __restrict__ status, Dims dm, DirGeom gm) {
-    constexpr int KS = SINGLE ? 4 : 2;                                // 16-key steps per block
+    constexpr int RT = 1, KS = SINGLE ? 4 : 2;                        // tiles per warp, 16-key steps per block
     extern __shared__ __align__(128) uint8_t smem[];
     // blockIdx.y = 0: the inverse index (one CTA per (image, routing head)); else head blockIdx.y - 1
     if (blockIdx.y == 0) {
@@ -63,37 +64,39 @@ bwd_dq_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* 
     const int hi = dm.heads_i == 1 ? 0 : h;
     const int32_t* irow = index + (((size_t)b * dm.heads_i + hi) * dm.R + i) * dm.topk;
     const int total = dm.topk * dm.n_r;
-    uint32_t* tab = reinterpret_cast<uint32_t*>(smem + gm.off_tab) + grp * gm.tab;
+    uint32_t* tab = reinterpret_cast<uint32_t*>(smem + gm.off_tab + grp * gm.tab_bytes);
+    uint32_t* dead = tab + gm.tab;
     const float sl2 = dm.scale * 1.4426950408889634f;
     const int passes = (total + gm.tab - 1) / gm.tab;
-    bool any_bad = false, filled = false;
+    bool filled = false;
 
-    for (int tile = gwarp; tile - gwarp < gm.tpc; tile += gwarps) {
+    for (int tile = gwarp * RT; tile - gwarp * RT < gm.tpc; tile += gwarps * RT) {
         const bool has = tile * 16 < ntok;
-        int tok[2];
-        float lse2[2];
-        uint32_t qa[PL][2][4], ga[PL][2][4];
+        int tok[RT][2];
+        float lse2[RT][2], delta[RT][2];
+        uint32_t qa[RT][PL][2][4], ga[RT][PL][2][4];
+        float dq[RT][PL][4][4];
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            const int tk = tile * 16 + g + 8 * r;
-            tok[r] = tk < ntok ? token_of(dm, gm, i, c0 + tk) : -1;
-            lse2[r] = tok[r] >= 0 ? __ldg(lse + stat0 + tok[r]) * 1.4426950408889634f : 0.f;
+        for (int x = 0; x < RT; ++x) {
+            uint4 q[2][PL], go[2][PL];
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const int tk = (tile + x) * 16 + g + 8 * r;
+                tok[x][r] = tk < ntok ? token_of(dm, gm, i, c0 + tk) : -1;
+                lse2[x][r] = tok[x][r] >= 0 ? __ldg(lse + stat0 + tok[x][r]) * 1.4426950408889634f : 0.f;
+                delta[x][r] = 0.f;
+                ld_row<PL>(q[r], Qb, tok[x][r], tok_bytes);
+                ld_row<PL>(go[r], Gb, tok[x][r], tok_bytes);
+            }
+            rows_to_a<PL>(qa[x], q[0], q[1]);
+            rows_to_a<PL>(ga[x], go[0], go[1]);
+#pragma unroll
+            for (int p = 0; p < PL; ++p)
+#pragma unroll
+                for (int n = 0; n < 4; ++n)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) dq[x][p][n][e] = 0.f;
         }
-        {
-            uint4 lo[PL], up[PL];
-            ld_row<PL>(lo, Qb, tok[0], tok_bytes); ld_row<PL>(up, Qb, tok[1], tok_bytes);
-            rows_to_a<PL>(qa, lo, up);
-            ld_row<PL>(lo, Gb, tok[0], tok_bytes); ld_row<PL>(up, Gb, tok[1], tok_bytes);
-            rows_to_a<PL>(ga, lo, up);
-        }
-        float delta[2] = {0.f, 0.f};
-        float dq[PL][4][4];
-#pragma unroll
-        for (int p = 0; p < PL; ++p)
-#pragma unroll
-            for (int n = 0; n < 4; ++n)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) dq[p][n][e] = 0.f;
 
 #pragma unroll 1
         for (int it = 0; it < (SINGLE ? 1 : 2 * passes); ++it) {
@@ -102,83 +105,102 @@ bwd_dq_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* 
             const int nk = SINGLE ? 16 * KS : min(gm.tab, (total - k0 + 31) / 32 * 32);
             if (passes > 1 || !filled) {
                 if (filled) group_sync();
-                const bool bad = fill_keys(tab, irow, i, k0, nk, total, glane, glanes, status, dm, gm);
-                any_bad = (one_warp ? __any_sync(0xffffffffu, bad) : __syncthreads_or(bad)) || any_bad;
-                if (one_warp) __syncwarp();
+                fill_keys(tab, dead, irow, k0, nk, total, glane, glanes, status, dm, gm);
+                group_sync();
                 filled = true;
             }
             if (!has) continue;
 #pragma unroll 1
             for (int kb = 0; kb < nk; kb += 16 * KS) {
                 uint4 kr[KS][2][PL];
-                float c[2 * KS][4], dp[2 * KS][4];
+                float c[RT][2 * KS][4], dp[RT][2 * KS][4];
 #pragma unroll
                 for (int s = 0; s < KS; ++s)
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
                         const uint32_t kt = tab[kb + 16 * s + 8 * e + g];
                         uint4 vr[PL];
-                        ld_token<PL, ZEROS>(kr[s][e], Kb, kt);
-                        ld_token<PL, ZEROS>(vr, Vb, kt);
-                        mma_rows<PL>(c[2 * s + e], qa, kr[s][e]);
-                        mma_rows<PL>(dp[2 * s + e], ga, vr);
-                    }
-                const bool mask = any_bad || k0 + kb + 16 * KS > total;
+                        ld_token<PL>(kr[s][e], Kb, kt);
+                        ld_token<PL>(vr, Vb, kt);
 #pragma unroll
-                for (int j = 0; j < 2 * KS; ++j) {
-                    c[j][0] = ex2_approx(fmaf(c[j][0], sl2, -lse2[0]));
-                    c[j][1] = ex2_approx(fmaf(c[j][1], sl2, -lse2[0]));
-                    c[j][2] = ex2_approx(fmaf(c[j][2], sl2, -lse2[1]));
-                    c[j][3] = ex2_approx(fmaf(c[j][3], sl2, -lse2[1]));
-                }
-                if (mask) {
+                        for (int x = 0; x < RT; ++x) {
+                            mma_rows<PL>(c[x][2 * s + e], qa[x], kr[s][e]);
+                            mma_rows<PL>(dp[x][2 * s + e], ga[x], vr);
+                        }
+                    }
+#pragma unroll
+                for (int x = 0; x < RT; ++x)
 #pragma unroll
                     for (int j = 0; j < 2 * KS; ++j) {
-                        const int kk = k0 + kb + 8 * j + 2 * t4;
-                        if (dead_key(kk, total, any_bad, irow, dm, gm)) { c[j][0] = 0.f; c[j][2] = 0.f; }
-                        if (dead_key(kk + 1, total, any_bad, irow, dm, gm)) { c[j][1] = 0.f; c[j][3] = 0.f; }
+                        c[x][j][0] = ex2_approx(fmaf(c[x][j][0], sl2, -lse2[x][0]));
+                        c[x][j][1] = ex2_approx(fmaf(c[x][j][1], sl2, -lse2[x][0]));
+                        c[x][j][2] = ex2_approx(fmaf(c[x][j][2], sl2, -lse2[x][1]));
+                        c[x][j][3] = ex2_approx(fmaf(c[x][j][3], sl2, -lse2[x][1]));
                     }
+                // (keys of the zero padding add nothing to delta or dQ)
+                if (SINGLE) {
+                    const uint32_t b0 = dead[0], b1 = dead[1];
+                    if (b0 | b1) {
+                        const uint32_t w[2] = {b0 >> (2 * t4), b1 >> (2 * t4)};
+#pragma unroll
+                        for (int j = 0; j < 2 * KS; ++j)
+#pragma unroll
+                            for (int x = 0; x < RT; ++x) {
+                                if (w[j >> 2] >> (8 * (j & 3)) & 1) c[x][j][0] = c[x][j][2] = 0.f;
+                                if (w[j >> 2] >> (8 * (j & 3) + 1) & 1) c[x][j][1] = c[x][j][3] = 0.f;
+                            }
+                    }
+                } else {
+                    const uint32_t bits = dead[kb >> 5] >> (kb & 31);
+                    if (bits) mask_columns<RT, 2 * KS>(c, bits, t4, 0.f);
                 }
                 if (SINGLE || sweep == 0) {
 #pragma unroll
-                    for (int j = 0; j < 2 * KS; ++j) {
-                        delta[0] = fmaf(c[j][0], dp[j][0], fmaf(c[j][1], dp[j][1], delta[0]));
-                        delta[1] = fmaf(c[j][2], dp[j][2], fmaf(c[j][3], dp[j][3], delta[1]));
-                    }
-                    if (SINGLE || (pass == passes - 1 && kb + 16 * KS >= nk)) {
+                    for (int x = 0; x < RT; ++x) {
 #pragma unroll
-                        for (int r = 0; r < 2; ++r) {
-                            delta[r] += __shfl_xor_sync(0xffffffffu, delta[r], 1);
-                            delta[r] += __shfl_xor_sync(0xffffffffu, delta[r], 2);
+                        for (int j = 0; j < 2 * KS; ++j) {
+                            delta[x][0] = fmaf(c[x][j][0], dp[x][j][0], fmaf(c[x][j][1], dp[x][j][1], delta[x][0]));
+                            delta[x][1] = fmaf(c[x][j][2], dp[x][j][2], fmaf(c[x][j][3], dp[x][j][3], delta[x][1]));
+                        }
+                        if (SINGLE || (pass == passes - 1 && kb + 16 * KS >= nk)) {
+#pragma unroll
+                            for (int r = 0; r < 2; ++r) {
+                                delta[x][r] += __shfl_xor_sync(0xffffffffu, delta[x][r], 1);
+                                delta[x][r] += __shfl_xor_sync(0xffffffffu, delta[x][r], 2);
+                            }
                         }
                     }
                 }
                 if (SINGLE || sweep == 1) {
 #pragma unroll
-                    for (int j = 0; j < 2 * KS; ++j) {
-                        c[j][0] *= dp[j][0] - delta[0]; c[j][1] *= dp[j][1] - delta[0];
-                        c[j][2] *= dp[j][2] - delta[1]; c[j][3] *= dp[j][3] - delta[1];
-                    }
+                    for (int x = 0; x < RT; ++x)
 #pragma unroll
-                    for (int s = 0; s < KS; ++s) mma_tokens<PL, EXACT>(dq, c[2 * s], c[2 * s + 1], kr[s][0], kr[s][1]);
+                        for (int j = 0; j < 2 * KS; ++j) {
+                            c[x][j][0] *= dp[x][j][0] - delta[x][0]; c[x][j][1] *= dp[x][j][1] - delta[x][0];
+                            c[x][j][2] *= dp[x][j][2] - delta[x][1]; c[x][j][3] *= dp[x][j][3] - delta[x][1];
+                        }
+#pragma unroll
+                    for (int s = 0; s < KS; ++s) mma_tokens<PL, EXACT>(dq, c, 2 * s, kr[s][0], kr[s][1]);
                 }
             }
         }
         // ---- dQ = scale * acc, delta kept for the dK/dV kernel ----
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            if (tok[r] < 0) continue;
-            uint8_t* o = dQb + (size_t)(uint32_t)tok[r] * tok_bytes;
+        for (int x = 0; x < RT; ++x)
 #pragma unroll
-            for (int p = 0; p < PL; ++p) *reinterpret_cast<uint4*>(o + p * 64) = pack_row(dq[p], r, dm.scale);
-            if (t4 == 0) delta_out[stat0 + tok[r]] = delta[r];
-        }
+            for (int r = 0; r < 2; ++r) {
+                if (tok[x][r] < 0) continue;
+                uint8_t* o = dQb + (size_t)(uint32_t)tok[x][r] * tok_bytes;
+#pragma unroll
+                for (int p = 0; p < PL; ++p) *reinterpret_cast<uint4*>(o + p * 64) = pack_row(dq[x][p], r, dm.scale);
+                if (t4 == 0) delta_out[stat0 + tok[x][r]] = delta[x][r];
+            }
     }
     pdl_launch_dependents();
 }
 
 // ------------------------------------------------------------------ dK, dV
-template <int PL, bool EXACT, bool ZEROS, int TY, int TX>
+template <int PL, bool EXACT, int TY, int TX>
 __global__ void __launch_bounds__(PL == 2 ? 128 : 256, PL == 2 ? 3 : 2)
 bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __restrict__ Kg,
                       const __nv_bfloat16* __restrict__ Vg, const int32_t* inv_off,
@@ -186,7 +208,7 @@ bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16*
                       const float* delta, const __nv_bfloat16* __restrict__ dOg,
                       const float* __restrict__ lce_w, __nv_bfloat16* __restrict__ dKg,
                       __nv_bfloat16* __restrict__ dVg, Dims dm, DirGeom gm) {
-    constexpr int KS = PL == 2 ? 1 : 2;                               // 16-query steps per block
+    constexpr int RT = 1, KS = PL == 2 ? 1 : 2;                       // tiles per warp, 16-query steps per block
     extern __shared__ __align__(128) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -233,49 +255,50 @@ bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16*
     const int total = (e1 - e0) * dm.n_r;
     const float* lse_h = lse + ((size_t)b * dm.heads + h) * N0;
     const float* delta_h = delta + ((size_t)b * dm.heads + h) * N0;
-    uint32_t* tab = reinterpret_cast<uint32_t*>(smem + gm.off_tab) + grp * 3 * gm.tab;   // row offsets, lse * log2(e), delta
+    uint32_t* tab = reinterpret_cast<uint32_t*>(smem + gm.off_tab + grp * gm.tab_bytes);   // row offsets, lse * log2(e), delta
     float* s_l2 = reinterpret_cast<float*>(tab + gm.tab);
     float* s_dl = s_l2 + gm.tab;
     float* st = reinterpret_cast<float*>(smem + gm.off_st + grp * gm.st_bytes);
     const float sl2 = dm.scale * 1.4426950408889634f;
     const int passes = (total + gm.tab - 1) / gm.tab;
-    // A query beyond the list repeats the last one with lse = inf: its P is zero.  One in the zero padding has zero rows
-    // of Q and dO and lse = delta = 0: it adds nothing.
+    // A query beyond the list, or of the zero padding (zero rows of Q and dO: it adds nothing), names some readable row with
+    // lse = inf: its P is zero.
     auto fill_queries = [&](int k0, int n) {
         for (int e = glane; e < n; e += glanes) {
             const int kk = min(k0 + e, total - 1);
             const int m = fdiv(kk, dm.n_r, gm.mul_nr);
-            const int tk = token_of(dm, gm, __ldcg(list + m), kk - m * dm.n_r);
-            tab[e] = tk >= 0 ? (uint32_t)tk * (uint32_t)(dm.C >> 3) : dk::ZERO;
-            s_l2[e] = k0 + e >= total ? INFINITY : tk >= 0 ? __ldg(lse_h + tk) * 1.4426950408889634f : 0.f;
-            s_dl[e] = tk >= 0 ? __ldcg(delta_h + tk) : 0.f;
+            const int tk = token_of(dm, gm, __ldcg(list + m), kk - m * dm.n_r), at = max(tk, 0);
+            tab[e] = (uint32_t)at * (uint32_t)(dm.C >> 3);
+            s_l2[e] = k0 + e >= total || tk < 0 ? INFINITY : __ldg(lse_h + at) * 1.4426950408889634f;
+            s_dl[e] = __ldcg(delta_h + at);
         }
     };
     bool filled = false;
 
-    for (int tile = gwarp; tile - gwarp < gm.tpc; tile += gwarps) {
+    for (int tile = gwarp * RT; tile - gwarp * RT < gm.tpc; tile += gwarps * RT) {
         const bool has = tile * 16 < ntok;
-        int tok[2];
-        uint32_t ka[PL][2][4], va[PL][2][4];
+        int tok[RT][2];
+        uint32_t ka[RT][PL][2][4], va[RT][PL][2][4];
+        float dkx[RT][PL][4][4], dvx[RT][PL][4][4];
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            const int tk = tile * 16 + g + 8 * r;
-            tok[r] = tk < ntok ? token_of(dm, gm, jr, c0 + tk) : -1;
+        for (int x = 0; x < RT; ++x) {
+            uint4 k[2][PL], v[2][PL];
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const int tk = (tile + x) * 16 + g + 8 * r;
+                tok[x][r] = tk < ntok ? token_of(dm, gm, jr, c0 + tk) : -1;
+                ld_row<PL>(k[r], Kb, tok[x][r], tok_bytes);
+                ld_row<PL>(v[r], Vb, tok[x][r], tok_bytes);
+            }
+            rows_to_a<PL>(ka[x], k[0], k[1]);
+            rows_to_a<PL>(va[x], v[0], v[1]);
+#pragma unroll
+            for (int p = 0; p < PL; ++p)
+#pragma unroll
+                for (int n = 0; n < 4; ++n)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) { dkx[x][p][n][e] = 0.f; dvx[x][p][n][e] = 0.f; }
         }
-        {
-            uint4 lo[PL], up[PL];
-            ld_row<PL>(lo, Kb, tok[0], tok_bytes); ld_row<PL>(up, Kb, tok[1], tok_bytes);
-            rows_to_a<PL>(ka, lo, up);
-            ld_row<PL>(lo, Vb, tok[0], tok_bytes); ld_row<PL>(up, Vb, tok[1], tok_bytes);
-            rows_to_a<PL>(va, lo, up);
-        }
-        float dkx[PL][4][4], dvx[PL][4][4];
-#pragma unroll
-        for (int p = 0; p < PL; ++p)
-#pragma unroll
-            for (int n = 0; n < 4; ++n)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) { dkx[p][n][e] = 0.f; dvx[p][n][e] = 0.f; }
 
 #pragma unroll 1
         for (int pass = 0; pass < passes; ++pass) {
@@ -291,60 +314,67 @@ bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16*
 #pragma unroll 1
             for (int kb = 0; kb < nk; kb += 16 * KS) {
                 uint4 qr[KS][2][PL], gr[KS][2][PL];
-                float c[2 * KS][4], dp[2 * KS][4];
+                float c[RT][2 * KS][4], dp[RT][2 * KS][4];
 #pragma unroll
                 for (int s = 0; s < KS; ++s)
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
                         const uint32_t qt = tab[kb + 16 * s + 8 * e + g];
-                        ld_token<PL, ZEROS>(qr[s][e], Qb, qt);
-                        ld_token<PL, ZEROS>(gr[s][e], Gb, qt);
+                        ld_token<PL>(qr[s][e], Qb, qt);
+                        ld_token<PL>(gr[s][e], Gb, qt);
                     }
 #pragma unroll
                 for (int s = 0; s < KS; ++s)
 #pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        mma_rows<PL>(c[2 * s + e], ka, qr[s][e]);     // S^T = K Q^T
-                        mma_rows<PL>(dp[2 * s + e], va, gr[s][e]);    // dP^T = V dO^T
-                    }
+                    for (int e = 0; e < 2; ++e)
+#pragma unroll
+                        for (int x = 0; x < RT; ++x) {
+                            mma_rows<PL>(c[x][2 * s + e], ka[x], qr[s][e]);       // S^T = K Q^T
+                            mma_rows<PL>(dp[x][2 * s + e], va[x], gr[s][e]);      // dP^T = V dO^T
+                        }
 #pragma unroll
                 for (int j = 0; j < 2 * KS; ++j) {
                     const float2 l2 = *reinterpret_cast<const float2*>(s_l2 + kb + 8 * j + 2 * t4);
                     const float2 dl = *reinterpret_cast<const float2*>(s_dl + kb + 8 * j + 2 * t4);
-                    c[j][0] = ex2_approx(fmaf(c[j][0], sl2, -l2.x));
-                    c[j][1] = ex2_approx(fmaf(c[j][1], sl2, -l2.y));
-                    c[j][2] = ex2_approx(fmaf(c[j][2], sl2, -l2.x));
-                    c[j][3] = ex2_approx(fmaf(c[j][3], sl2, -l2.y));
-                    dp[j][0] = c[j][0] * (dp[j][0] - dl.x);
-                    dp[j][1] = c[j][1] * (dp[j][1] - dl.y);
-                    dp[j][2] = c[j][2] * (dp[j][2] - dl.x);
-                    dp[j][3] = c[j][3] * (dp[j][3] - dl.y);
+#pragma unroll
+                    for (int x = 0; x < RT; ++x) {
+                        c[x][j][0] = ex2_approx(fmaf(c[x][j][0], sl2, -l2.x));
+                        c[x][j][1] = ex2_approx(fmaf(c[x][j][1], sl2, -l2.y));
+                        c[x][j][2] = ex2_approx(fmaf(c[x][j][2], sl2, -l2.x));
+                        c[x][j][3] = ex2_approx(fmaf(c[x][j][3], sl2, -l2.y));
+                        dp[x][j][0] = c[x][j][0] * (dp[x][j][0] - dl.x);
+                        dp[x][j][1] = c[x][j][1] * (dp[x][j][1] - dl.y);
+                        dp[x][j][2] = c[x][j][2] * (dp[x][j][2] - dl.x);
+                        dp[x][j][3] = c[x][j][3] * (dp[x][j][3] - dl.y);
+                    }
                 }
 #pragma unroll
                 for (int s = 0; s < KS; ++s) {
-                    mma_tokens<PL, EXACT>(dkx, dp[2 * s], dp[2 * s + 1], qr[s][0], qr[s][1]);   // dK += dS^T Q
-                    mma_tokens<PL, EXACT>(dvx, c[2 * s], c[2 * s + 1], gr[s][0], gr[s][1]);     // dV += P^T dO
+                    mma_tokens<PL, EXACT>(dkx, dp, 2 * s, qr[s][0], qr[s][1]);    // dK += dS^T Q
+                    mma_tokens<PL, EXACT>(dvx, c, 2 * s, gr[s][0], gr[s][1]);     // dV += P^T dO
                 }
             }
         }
         // ---- dK = scale * acc; dV to the staging tile ----
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            const int tk = tile * 16 + g + 8 * r;
-            if (tk >= ntok) continue;
-            if (tok[r] >= 0) {
-                uint8_t* o = dKb + (size_t)(uint32_t)tok[r] * tok_bytes;
+        for (int x = 0; x < RT; ++x)
 #pragma unroll
-                for (int p = 0; p < PL; ++p) *reinterpret_cast<uint4*>(o + p * 64) = pack_row(dkx[p], r, dm.scale);
+            for (int r = 0; r < 2; ++r) {
+                const int tk = (tile + x) * 16 + g + 8 * r;
+                if (tk >= ntok) continue;
+                if (tok[x][r] >= 0) {
+                    uint8_t* o = dKb + (size_t)(uint32_t)tok[x][r] * tok_bytes;
+#pragma unroll
+                    for (int p = 0; p < PL; ++p) *reinterpret_cast<uint4*>(o + p * 64) = pack_row(dkx[x][p], r, dm.scale);
+                }
+                float* dst = st + tk * 32 * PL + t4 * 8;
+#pragma unroll
+                for (int p = 0; p < PL; ++p)
+#pragma unroll
+                    for (int q = 0; q < 2; ++q)
+                        *reinterpret_cast<float4*>(dst + p * 32 + 4 * q) = make_float4(dvx[x][p][2 * q][2 * r], dvx[x][p][2 * q][2 * r + 1],
+                                                                                       dvx[x][p][2 * q + 1][2 * r], dvx[x][p][2 * q + 1][2 * r + 1]);
             }
-            float* dst = st + tk * 32 * PL + t4 * 8;
-#pragma unroll
-            for (int p = 0; p < PL; ++p)
-#pragma unroll
-                for (int q = 0; q < 2; ++q)
-                    *reinterpret_cast<float4*>(dst + p * 32 + 4 * q) =
-                        make_float4(dvx[p][2 * q][2 * r], dvx[p][2 * q][2 * r + 1], dvx[p][2 * q + 1][2 * r], dvx[p][2 * q + 1][2 * r + 1]);
-        }
     }
     cp_async_wait<0>();
     group_sync();
@@ -354,10 +384,12 @@ bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16*
 }
 
 // ------------------------------------------------------------------ host side
+static bool dq_single(const Dims& d) { return d.d == 32 && d.topk * d.n_r <= 64 && !direct_exact(d); }
 static DirGeom dq_geom(const Dims& d) {
-    DirGeom g = direct_geom(d, false, 4);
-    if (d.topk * d.n_r <= 64) g.tab = 64;                            // one block of 64 keys
-    g.smem_bytes = g.off_tab + g.gpc * g.tab * 4;                    // the table only
+    Dims k = d;
+    if (dq_single(d)) k.topk = (64 + d.n_r - 1) / d.n_r;             // one block of 64 keys
+    DirGeom g = direct_geom(k, false, 4, 1);
+    g.smem_bytes = g.off_tab + g.gpc * g.tab_bytes;                  // the table only
     const int inv = (int)inverse_smem(d);
     if (g.smem_bytes < inv) g.smem_bytes = inv;
     return g;
@@ -365,7 +397,7 @@ static DirGeom dq_geom(const Dims& d) {
 static DirGeom dkv_geom(const Dims& d) {
     Dims full = d;
     full.topk = d.R;                                                 // a key region may be on every query region's list
-    return direct_geom(full, d.lce, 12);
+    return direct_geom(full, d.lce, 12, 1);
 }
 
 bool backward_direct_supported(const Dims& d, int dtype) {
@@ -393,10 +425,10 @@ struct BwdArgs {
 };
 }  // namespace
 
-template <int PL, bool EXACT, bool SINGLE, bool ZEROS>
+template <int PL, bool EXACT, bool SINGLE>
 static cudaError_t launch_dq(const Dims& d, const BwdArgs& a) {
     const DirGeom g = dq_geom(d);
-    auto kernel = bwd_dq_direct_kernel<PL, EXACT, SINGLE, ZEROS>;
+    auto kernel = bwd_dq_direct_kernel<PL, EXACT, SINGLE>;
     static PerDeviceMax set;
     const cudaError_t e = allow_smem(set, kernel, g.smem_bytes);
     if (e != cudaSuccess) return e;
@@ -405,10 +437,10 @@ static cudaError_t launch_dq(const Dims& d, const BwdArgs& a) {
                          a.q, a.k, a.v, a.index, a.lse, a.go, a.dq, a.delta, a.inv_off, a.inv_list, inverse_uses_bits(d), a.status, d, g);
 }
 
-template <int PL, bool EXACT, bool ZEROS, int TY, int TX>
+template <int PL, bool EXACT, int TY, int TX>
 static cudaError_t launch_dkv(const Dims& d, const BwdArgs& a) {
     const DirGeom g = dkv_geom(d);
-    auto kernel = bwd_dkv_direct_kernel<PL, EXACT, ZEROS, TY, TX>;
+    auto kernel = bwd_dkv_direct_kernel<PL, EXACT, TY, TX>;
     static PerDeviceMax set;
     const cudaError_t e = allow_smem(set, kernel, g.smem_bytes);
     if (e != cudaSuccess) return e;
@@ -417,21 +449,20 @@ static cudaError_t launch_dkv(const Dims& d, const BwdArgs& a) {
                          a.q, a.k, a.v, a.inv_off, a.inv_list, a.lse, a.delta, a.go, a.lce_w, a.dk, a.dv, d, g);
 }
 
-template <bool ZEROS>
 static cudaError_t launch_both(const Dims& d, const BwdArgs& a) {
-    const bool single = d.topk * d.n_r <= 64, exact = direct_exact(d);
-    const cudaError_t e = d.d == 64 ? launch_dq<2, true, false, ZEROS>(d, a)
-                        : exact     ? launch_dq<1, true, false, ZEROS>(d, a)
-                        : single    ? launch_dq<1, false, true, ZEROS>(d, a)
-                                    : launch_dq<1, false, false, ZEROS>(d, a);
+    const bool exact = direct_exact(d);
+    const cudaError_t e = d.d == 64      ? launch_dq<2, true, false>(d, a)
+                        : exact          ? launch_dq<1, true, false>(d, a)
+                        : dq_single(d)   ? launch_dq<1, false, true>(d, a)
+                                         : launch_dq<1, false, false>(d, a);
     if (e != cudaSuccess) return e;
-    if (d.hs <= 2) return d.d == 64 ? launch_dkv<2, true, ZEROS, 2, 2>(d, a) : launch_dkv<1, false, ZEROS, 2, 2>(d, a);
-    if (d.d == 64) return launch_dkv<2, true, ZEROS, 4, 4>(d, a);
-    if (exact) return launch_dkv<1, true, ZEROS, 4, 3>(d, a);
+    if (d.hs <= 2) return d.d == 64 ? launch_dkv<2, true, 2, 2>(d, a) : launch_dkv<1, false, 2, 2>(d, a);
+    if (d.d == 64) return launch_dkv<2, true, 4, 4>(d, a);
+    if (exact) return launch_dkv<1, true, 4, 4>(d, a);
     switch (lce_tile_width(dkv_geom(d), d)) {
-        case 2: return launch_dkv<1, false, ZEROS, 4, 2>(d, a);
-        case 3: return launch_dkv<1, false, ZEROS, 4, 3>(d, a);
-        default: return launch_dkv<1, false, ZEROS, 4, 4>(d, a);
+        case 2: return launch_dkv<1, false, 4, 2>(d, a);
+        case 3: return launch_dkv<1, false, 4, 3>(d, a);
+        default: return launch_dkv<1, false, 4, 4>(d, a);
     }
 }
 
@@ -442,7 +473,7 @@ cudaError_t launch_backward_direct(const Dims& d, const void* Q, const void* K, 
     typedef __nv_bfloat16 bf;
     const BwdArgs a = {static_cast<const bf*>(Q), static_cast<const bf*>(K), static_cast<const bf*>(V), static_cast<const bf*>(dO), index,
                        inv_off, inv_list, lce_w, lse, static_cast<bf*>(dQ), static_cast<bf*>(dK), static_cast<bf*>(dV), delta, status, st};
-    return d.H != d.H0 || d.W != d.W0 ? launch_both<true>(d, a) : launch_both<false>(d, a);
+    return launch_both(d, a);
 }
 
 }  // namespace bra

@@ -278,6 +278,11 @@ bra_status bra_forward(const bra_problem* p, const void* Q, const void* K, const
     // every region is routed to and the caller does not ask in which order: nothing to route
     if (path == PATH_DENSE && d.topk == d.R && !index)
         return attend_any_map(path, d, L, p->dtype, Q, K, V, nullptr, lce_w, lce_b, O, lse, w, st, false);
+    if (!any_map(path))                             // padded copies (if any) first, then the chain, whose kernels overlap at their ends
+        return on_padded_map(d, L, Q, K, V, O, lse, w, st, [&](const Dims& dp, const void* q, const void* k, const void* v, void* o, float* l) {
+            const bra_status rs = run_route(dp, p->dtype, q, k, qm, km, idx, st);
+            return rs != BRA_OK ? rs : run_attend(path, dp, p->dtype, q, k, v, idx, lce_w, lce_b, o, l, status, st, true);
+        });
     s = run_route(d, p->dtype, Q, K, qm, km, idx, st);
     if (s != BRA_OK) return s;
     // with every region routed to, the attention need not look at the order

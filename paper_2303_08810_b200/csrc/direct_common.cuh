@@ -18,23 +18,22 @@ namespace bra {
 namespace dk {
 constexpr int TAB = 512;            // tokens a table holds (per group)
 constexpr int TAB_WARP = 256;       // the same where a group is one warp
-constexpr uint32_t ZERO = 0xffffffffu;   // table entry of a token of the zero padding: all channels zero
 }  // namespace dk
 
 struct DirGeom {
     int planes;
     int hb, chunks;        // region rows per chunk, chunks per region
     int tpc;               // 16-token tiles of a (full) chunk
-    int nw, gpc;           // warps per CTA; groups (regions) per CTA: 4 when a region is one tile, else 1
+    int nw, gpc;           // warps per CTA; groups (regions) per CTA: several when a region is one warp's work, else 1
     int gpi;               // CTAs per (image, head): the grid is (gpi, heads, images)
     int halo_w, halo_row;  // tokens and bytes of a halo row
     uint32_t mul_nr, mul_ws, mul_s, mul_hw;
     int off_tab, off_w, off_halo, off_st, smem_bytes;
-    int tab, halo_bytes, st_bytes;     // per group
+    int tab, tab_bytes, halo_bytes, st_bytes;     // per group; tab: entries
 };
 
-// entry_bytes: bytes of a table entry
-inline DirGeom direct_geom(const Dims& d, bool with_lce, int entry_bytes) {
+// entry_bytes: bytes of a table entry; rt: 16-token tiles of a warp
+inline DirGeom direct_geom(const Dims& d, bool with_lce, int entry_bytes, int rt) {
     DirGeom g;
     g.planes = d.d / 32;
     g.hb = d.hs; g.chunks = 1;
@@ -46,8 +45,9 @@ inline DirGeom direct_geom(const Dims& d, bool with_lce, int entry_bytes) {
         g.chunks = (d.hs + g.hb - 1) / g.hb;
     }
     g.tpc = (g.hb * d.ws + 15) / 16;
-    if (g.tpc == 1 && g.chunks == 1) { g.gpc = 4; g.nw = 4; }
-    else { g.gpc = 1; const int most = g.planes == 2 ? 4 : 8; g.nw = g.tpc < most ? g.tpc : most; }
+    const int most = (g.planes == 2 ? 4 : 8) / rt, want = (g.tpc + rt - 1) / rt;
+    if (want == 1 && g.chunks == 1) g.gpc = g.nw = most < 4 ? most : 4;
+    else { g.gpc = 1; g.nw = want < most ? want : most; }
     g.gpi = (d.R + g.gpc - 1) / g.gpc * g.chunks;
     g.halo_w = d.ws + 4;
     g.halo_row = g.halo_w * 64 * g.planes + 16;        // tiles four rows apart start on different banks
@@ -56,12 +56,13 @@ inline DirGeom direct_geom(const Dims& d, bool with_lce, int entry_bytes) {
     const int need = (d.topk * d.n_r + 31) / 32 * 32;
     if (need < g.tab) g.tab = need;
     int off = 0;
-    g.off_tab = off;  off += g.gpc * g.tab * entry_bytes;
+    g.tab_bytes = (g.tab * entry_bytes + g.tab / 8 + 4 + 15) / 16 * 16;     // entries, a bit per entry, a counter
+    g.off_tab = off;  off += g.gpc * g.tab_bytes;
     g.off_w = off;    off += with_lce ? 32 * g.planes * 25 * 4 : 0;
     off = (off + 15) / 16 * 16;
     g.halo_bytes = with_lce ? (g.hb + 4) * g.halo_row : 0;
     g.off_halo = off; off += g.gpc * g.halo_bytes;
-    g.st_bytes = g.tpc * 16 * 128 * g.planes;
+    g.st_bytes = (g.tpc + rt - 1) / rt * rt * 16 * 128 * g.planes;
     g.off_st = off;   off += g.gpc * g.st_bytes;
     // LCE tiles that stick out of a chunk read (and discard) up to three halo rows behind it
     const int reach = g.off_halo + g.gpc * g.halo_bytes + (with_lce ? 3 * g.halo_row + 1024 : 0);
@@ -72,6 +73,13 @@ inline DirGeom direct_geom(const Dims& d, bool with_lce, int entry_bytes) {
 // Head dim 32, regions of more than 128 tokens whose rows do not divide 128: these shapes used to run in fp32 on the
 // CUDA cores, so the probabilities keep 16 bits of mantissa here (two MMAs).  Head dim 64: the same in the gradients.
 inline bool direct_exact(const Dims& d) { return d.n_r > 128 && 128 % d.ws != 0; }
+
+// Tiles per warp in the forward kernel: two share every row that is loaded (and transposed) where regions have two and enough
+// warps remain.  Measured: 2 x 100 x 167 tokens, S = 16, topk 4, 6 heads 124 -> 114 us; 2 x 112 x 112, S = 8: 98 -> 88 us.
+inline int direct_rt(const Dims& d) {
+    const long long warps = (long long)d.B * d.heads * d.R * ((d.n_r + 31) / 32);
+    return d.n_r > 16 && warps >= 8 * kSMs ? 2 : 1;
+}
 
 // ------------------------------------------------------------------ loads
 // 16 bytes of the read-only input tensors; zero where `ok` is false (nothing is read)
@@ -84,12 +92,12 @@ __device__ __forceinline__ uint4 ld16_or_zero(const uint8_t* p, bool ok) {
     return v;
 }
 __device__ __forceinline__ uint4 ld16(const uint8_t* p) { return __ldg(reinterpret_cast<const uint4*>(p)); }
-// A lane's chunks of the token whose row starts off16 * 16 bytes behind base.  ZEROS: the map has zero padding.
-template <int PL, bool ZEROS>
+// A lane's chunks of the token whose row starts off16 * 16 bytes behind base.
+template <int PL>
 __device__ __forceinline__ void ld_token(uint4 (&v)[PL], const uint8_t* base, uint32_t off16) {
     const uint8_t* p = base + (size_t)off16 * 16;
 #pragma unroll
-    for (int q = 0; q < PL; ++q) v[q] = ZEROS ? ld16_or_zero(p + q * 64, off16 != dk::ZERO) : ld16(p + q * 64);
+    for (int q = 0; q < PL; ++q) v[q] = ld16(p + q * 64);
 }
 // the same for a row that may not exist
 template <int PL>
@@ -136,21 +144,26 @@ __device__ __forceinline__ void frag_lo(uint32_t (&l)[4], const uint32_t (&a)[4]
     l[0] = left_over(a[0], c0[0], c0[1]); l[1] = left_over(a[1], c0[2], c0[3]);
     l[2] = left_over(a[2], c1[0], c1[1]); l[3] = left_over(a[3], c1[2], c1[3]);
 }
-// acc (16 x 32 PL) += A (16 x 16) * the 16 token rows lo (0-7), hi (8-15)
+// acc[x] (16 x 32 PL) += A[x] (16 x 16, fragments c[x][j0], c[x][j0 + 1]) * the 16 token rows lo (0-7), hi (8-15)
 // EXACT: A = hi + lo parts (16 bits of mantissa), for problems whose products were fp32 before they had these kernels
-template <int PL, bool EXACT>
-__device__ __forceinline__ void mma_tokens(float (&acc)[PL][4][4], const float (&c0)[4], const float (&c1)[4],
-                                           const uint4 (&lo)[PL], const uint4 (&hi)[PL]) {
-    uint32_t a[4], l[4];
-    frag_hi(a, c0, c1);
-    if (EXACT) frag_lo(l, a, c0, c1);
+template <int PL, bool EXACT, int RT, int J>
+__device__ __forceinline__ void mma_tokens(float (&acc)[RT][PL][4][4], const float (&c)[RT][J][4], int j0, const uint4 (&lo)[PL], const uint4 (&hi)[PL]) {
+    uint32_t a[RT][4], l[RT][4];
+#pragma unroll
+    for (int x = 0; x < RT; ++x) {
+        frag_hi(a[x], c[x][j0], c[x][j0 + 1]);
+        if (EXACT) frag_lo(l[x], a[x], c[x][j0], c[x][j0 + 1]);
+    }
 #pragma unroll
     for (int p = 0; p < PL; ++p)
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const uint32_t b0 = movm(reg_of(lo[p], i)), b1 = movm(reg_of(hi[p], i));
-            mma_bf16(acc[p][i], a, b0, b1);
-            if (EXACT) mma_bf16(acc[p][i], l, b0, b1);
+#pragma unroll
+            for (int x = 0; x < RT; ++x) {
+                mma_bf16(acc[x][p][i], a[x], b0, b1);
+                if (EXACT) mma_bf16(acc[x][p][i], l[x], b0, b1);
+            }
         }
 }
 // eight consecutive channels of one row (n-tiles 0..3, elements 2r, 2r + 1) times f, as bf16
@@ -168,28 +181,43 @@ __device__ __forceinline__ int token_of(const Dims& dm, const DirGeom& gm, int r
     return y < dm.H0 && x < dm.W0 ? y * dm.W0 + x : -1;
 }
 // Table of the keys [k0, k0 + n) of a group: key kk is token kk % n_r of region irow[kk / n_r].  An entry is the
-// offset of the token's row from the head's first byte, in units of 16 bytes.  Entries beyond `total` repeat the last
-// key and entries of a bad routing entry name the group's own region `self`: readable rows whose probabilities the
-// caller sets to zero.  Returns true if a bad routing entry was met.
-__device__ __forceinline__ bool fill_keys(uint32_t* tab, const int32_t* irow, int self, int k0, int n, int total, int lane0, int lanes,
-                                          int32_t* status, const Dims& dm, const DirGeom& gm) {
-    bool bad = false;
-    for (int e = lane0; e < n; e += lanes) {
+// offset of the token's row from the head's first byte, in units of 16 bytes.  Keys that are not rows of the map - entries
+// beyond `total`, of a bad routing entry, of the zero padding - name some readable row and have their bit set in `dead`:
+// the caller gives them the probability zero.  (A key of the zero padding has the score 0 and the value 0: all it does is
+// count in the softmax's denominator.)  Returns how many keys of the zero padding this lane met.
+__device__ __forceinline__ int fill_keys(uint32_t* tab, uint32_t* dead, const int32_t* irow, int k0, int n, int total, int lane0, int lanes,
+                                         int32_t* status, const Dims& dm, const DirGeom& gm) {
+    int zeros = 0;
+    for (int e = lane0; e < n; e += lanes) {                         // whole warps: n and lanes are multiples of 32
         const int kk = min(k0 + e, total - 1);
         const int m = fdiv(kk, dm.n_r, gm.mul_nr);
-        int r = __ldcg(irow + m);        // coherent load: the index may come from the kernel this one overlaps
-        if (r < 0 || r >= dm.R) { record_error(status, BRA_ERR_INDEX, r); bad = true; r = self; }
-        const int tok = token_of(dm, gm, r, kk - m * dm.n_r);
-        tab[e] = tok >= 0 ? (uint32_t)tok * (uint32_t)(dm.C >> 3) : dk::ZERO;
+        const int r = __ldcg(irow + m);  // coherent load: the index may come from the kernel this one overlaps
+        bool ok = k0 + e < total;
+        int tok = 0;
+        if (r < 0 || r >= dm.R) {
+            record_error(status, BRA_ERR_INDEX, r);
+            ok = false;
+        } else {
+            tok = token_of(dm, gm, r, kk - m * dm.n_r);
+            if (tok < 0) { zeros += ok; ok = false; tok = 0; }
+        }
+        tab[e] = (uint32_t)tok * (uint32_t)(dm.C >> 3);
+        const uint32_t word = __ballot_sync(0xffffffffu, !ok);
+        if ((e & 31) == 0) dead[e >> 5] = word;
     }
-    return bad;
+    return zeros;
 }
-// true if key kk of the group does not count
-__device__ __forceinline__ bool dead_key(int kk, int total, bool any_bad, const int32_t* irow, const Dims& dm, const DirGeom& gm) {
-    if (kk >= total) return true;
-    if (!any_bad) return false;
-    const int r = __ldcg(irow + fdiv(kk, dm.n_r, gm.mul_nr));
-    return r < 0 || r >= dm.R;
+// columns 8 j + 2 t4, + 1 (j = 0 .. J - 1) of the rows c[x] whose bits are set: value v
+template <int RT, int J>
+__device__ __forceinline__ void mask_columns(float (&c)[RT][J][4], uint32_t bits, int t4, float v) {
+    bits >>= 2 * t4;
+#pragma unroll
+    for (int j = 0; j < J; ++j)
+#pragma unroll
+        for (int x = 0; x < RT; ++x) {
+            if (bits >> (8 * j) & 1) c[x][j][0] = c[x][j][2] = v;
+            if (bits >> (8 * j + 1) & 1) c[x][j][1] = c[x][j][3] = v;
+        }
 }
 
 // ------------------------------------------------------------------ LCE

@@ -12,7 +12,7 @@ namespace bra {
 using namespace ptx;
 
 template <typename T, int D>
-__global__ void __launch_bounds__(sk::THREADS, D <= 16 ? 8 : 4)
+__global__ void __launch_bounds__(sk::THREADS, D <= 16 ? 2 : 1)
 attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* __restrict__ Vg, const int32_t* index,
                    const float* __restrict__ lce_w, const float* __restrict__ lce_b, T* __restrict__ Og, float* __restrict__ lse,
                    int32_t* __restrict__ status, Dims dm, SimtGeom gm) {
@@ -190,8 +190,8 @@ attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
         });
     __syncthreads();
     const float* bias = dm.lce && lce_b ? lce_b + h * D : nullptr;
-    if (dm.hs <= 2) simt_lce<T, D, 2, false>(st, s_w, bias, V, Og + head, r0, nreg, QT * gm.spr, chunk, dm, gm);
-    else simt_lce<T, D, 4, false>(st, s_w, bias, V, Og + head, r0, nreg, QT * gm.spr, chunk, dm, gm);
+    if (dm.hs <= 2) simt_lce<T, D, 2, false>(st, s_w, bias, V, Og + head, SimtFrom{r0}, nreg, QT * gm.spr, chunk, dm, gm);
+    else simt_lce<T, D, 4, false>(st, s_w, bias, V, Og + head, SimtFrom{r0}, nreg, QT * gm.spr, chunk, dm, gm);
 }
 
 bool attend_simt_supported(const Dims& d) {

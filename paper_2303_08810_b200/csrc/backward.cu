@@ -22,16 +22,16 @@ using namespace ptx;
 // ------------------------------------------------------------ dQ and delta
 // Grid row 0 builds the inverse index, row 1 + h is head h.
 template <typename T, int D>
-__global__ void __launch_bounds__(sk::THREADS, D <= 16 ? 6 : 4)
+__global__ void __launch_bounds__(sk::THREADS, 1)
 bwd_dq_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* __restrict__ Vg, const int32_t* __restrict__ index,
                    const float* __restrict__ lse, const T* __restrict__ dOg, T* __restrict__ dQg, float* __restrict__ delta,
-                   int32_t* __restrict__ inv_off, int32_t* __restrict__ inv_list, bool inv_bits,
+                   int32_t* __restrict__ inv_off, int32_t* __restrict__ inv_list, int32_t* __restrict__ inv_order, bool inv_bits,
                    int32_t* __restrict__ status, Dims dm, SimtGeom gm) {
     constexpr int QT = D <= 32 ? 2 : 1, U = 2;                        // simt_rows()
     extern __shared__ __align__(128) uint8_t smem[];
     if (blockIdx.y == 0) {
         if ((int)blockIdx.x < dm.heads_i)
-            inverse_index_job(index, inv_off, inv_list, blockIdx.z * dm.heads_i + blockIdx.x, reinterpret_cast<int32_t*>(smem), inv_bits, dm);
+            inverse_index_job(index, inv_off, inv_list, inv_order, blockIdx.z * dm.heads_i + blockIdx.x, reinterpret_cast<int32_t*>(smem), inv_bits, dm);
         return;
     }
     if ((int)blockIdx.x >= gm.gpi) return;
@@ -190,16 +190,16 @@ bwd_dq_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
 
 // ------------------------------------------------------------ dK, dV
 template <typename T, int D>
-__global__ void __launch_bounds__(sk::THREADS, D <= 16 ? 6 : 4)
+__global__ void __launch_bounds__(sk::THREADS, 1)
 bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* __restrict__ Vg, const int32_t* inv_off,
-                    const int32_t* inv_list, const float* __restrict__ lse, const float* delta, const T* __restrict__ dOg,
+                    const int32_t* inv_list, const int32_t* inv_order, const float* __restrict__ lse, const float* delta, const T* __restrict__ dOg,
                     const float* __restrict__ lce_w, T* __restrict__ dKg, T* __restrict__ dVg, Dims dm, SimtGeom gm) {
     extern __shared__ __align__(128) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
     const int tid = threadIdx.x;
-    const int h = blockIdx.y, b = blockIdx.z;
-    const SimtChunk chunk = simt_chunk(dm, gm, blockIdx.x % gm.chunks);
-    const int r0 = blockIdx.x / gm.chunks * gm.rpc;
+    const int h = blockIdx.x, b = blockIdx.y;                         // longest lists of all (image, head) pairs first
+    const SimtChunk chunk = simt_chunk(dm, gm, blockIdx.z % gm.chunks);
+    const int r0 = blockIdx.z / gm.chunks * gm.rpc;                   // regions r0 .. of the order
     const int nreg = min(gm.rpc, dm.R - r0);
     const int N0 = dm.H0 * dm.W0;
     const size_t head = (size_t)b * N0 * dm.C + (size_t)h * D;
@@ -218,7 +218,8 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
 
     const int hi = dm.heads_i == 1 ? 0 : h;
     const size_t bhi = (size_t)b * dm.heads_i + hi;
-    const int32_t* offs = inv_off + bhi * (dm.R + 1) + r0;           // [nreg + 1]
+    const int32_t* offs = inv_off + bhi * (dm.R + 1);
+    const int32_t* order = inv_order + bhi * dm.R + r0;              // the CTA's key regions
     const int32_t* list = inv_list + bhi * dm.R * dm.topk;
     const float* lse_h = lse + ((size_t)b * dm.heads + h) * N0;
     const float* delta_h = delta + ((size_t)b * dm.heads + h) * N0;
@@ -226,21 +227,20 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
     const int rl_raw = fdiv(slot, gm.spr, gm.mul_spr);
     const bool active = rl_raw < nreg;
     const int rl = active ? rl_raw : 0;
-    const int e0 = __ldcg(offs + rl), mine = (__ldcg(offs + rl + 1) - e0) * dm.n_r;     // queries of this lane's key region
+    const int jr = __ldcg(order + rl);                                // this lane's key region
+    const int e0 = __ldcg(offs + jr), mine = (__ldcg(offs + jr + 1) - e0) * dm.n_r;     // its queries
     const int warp_total = __reduce_max_sync(0xffffffffu, mine);
     bool weighted = false;
     int32_t* cnt = reinterpret_cast<int32_t*>(smem + gm.off_cnt);
     if (gm.dense) {
         __syncthreads();
-        const int first = __ldcg(offs), n = __ldcg(offs + nreg) - first;
-        weighted = !simt_counts(cnt, nreg, dm.R, n, [&](int e) {
-            int l = 0;
-            while (l + 1 < nreg && __ldcg(offs + l + 1) - first <= e) ++l;
-            return l * dm.R + __ldcg(list + first + e);
+        weighted = !simt_counts(cnt, nreg, dm.R, nreg * dm.R * dm.topk, [&](int e) {     // (topk == R: few entries)
+            const int l = e / (dm.R * dm.topk), j = __ldcg(order + l), at = __ldcg(offs + j) + e - l * dm.R * dm.topk;
+            return at < __ldcg(offs + j + 1) ? l * dm.R + __ldcg(list + at) : -1;
         });
     }
     const int t0 = active ? slot - rl_raw * gm.spr : 0;
-    const int tok = active ? simt_row(dm, gm, chunk, r0 + rl, t0) : -1;
+    const int tok = active ? simt_row(dm, gm, chunk, jr, t0) : -1;
     float kr[D], vr[D], gk[1][D], gv[1][D];
     {
         const size_t at = head + (size_t)(tok < 0 ? 0 : tok) * dm.C;
@@ -292,7 +292,8 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
             stat[row] = tk >= 0 ? make_float2(__ldg(lse_h + tk), __ldcg(delta_h + tk)) : make_float2(0.f, 0.f);
         }
     } else {
-        for (int l = 0; l < nreg; ++l) most = max(most, (__ldcg(offs + l + 1) - __ldcg(offs + l)) * dm.n_r);
+        const int j = __ldcg(order);                                  // the first has the longest list
+        most = (__ldcg(offs + j + 1) - __ldcg(offs + j)) * dm.n_r;
     }
     const int nst = gm.resident ? 1 : (most + gm.kps - 1) / gm.kps;
     auto load_stage = [&](int st) {
@@ -301,11 +302,11 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
         simt_copy_rows<T, D>(base + gm.off_a, base + gm.off_b, Q, dO, dm.C, nreg * gm.kps, [&](int row, uint32_t& at) {
             const int lr = fdiv(row, gm.kps, gm.mul_kps), kk = st * gm.kps + row - lr * gm.kps;
             at = lr * gm.reg + (row - lr * gm.kps) * gm.row;
-            const int s0 = __ldcg(offs + lr);
+            const int j = __ldcg(order + lr), s0 = __ldcg(offs + j);
             const int m = fdiv(kk, dm.n_r, gm.mul_nr);
             int tk = -1;
             float2 v = make_float2(INFINITY, 0.f);
-            if (s0 + m < __ldcg(offs + lr + 1)) {
+            if (s0 + m < __ldcg(offs + j + 1)) {
                 tk = simt_token(dm, gm, __ldcg(list + s0 + m), kk - m * dm.n_r);
                 v = tk >= 0 ? make_float2(__ldg(lse_h + tk), __ldcg(delta_h + tk)) : make_float2(0.f, 0.f);
             }
@@ -352,8 +353,8 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
         });
     }
     __syncthreads();
-    if (dm.hs <= 2) simt_lce<T, D, 2, true>(st, s_w, nullptr, dO, dVg + head, r0, nreg, gm.spr, chunk, dm, gm);
-    else simt_lce<T, D, 4, true>(st, s_w, nullptr, dO, dVg + head, r0, nreg, gm.spr, chunk, dm, gm);
+    if (dm.hs <= 2) simt_lce<T, D, 2, true>(st, s_w, nullptr, dO, dVg + head, order, nreg, gm.spr, chunk, dm, gm);
+    else simt_lce<T, D, 4, true>(st, s_w, nullptr, dO, dVg + head, order, nreg, gm.spr, chunk, dm, gm);
 }
 
 bool backward_supported(const Dims& d) {
@@ -386,6 +387,7 @@ static cudaError_t launch_bwd_t(const Dims& d, int impl, const void* Q, const vo
     float* delta = reinterpret_cast<float*>(ws + L.delta);
     int32_t* inv_off = reinterpret_cast<int32_t*>(ws + L.inv_off);
     int32_t* inv_list = reinterpret_cast<int32_t*>(ws + L.inv_list);
+    int32_t* inv_order = reinterpret_cast<int32_t*>(ws + L.inv_order);
     float* part = reinterpret_cast<float*>(ws + L.dw_part);
     const T* q = static_cast<const T*>(Q); const T* k = static_cast<const T*>(K);
     const T* v = static_cast<const T*>(V); const T* go = static_cast<const T*>(dO);
@@ -413,7 +415,7 @@ static cudaError_t launch_bwd_t(const Dims& d, int impl, const void* Q, const vo
     } else if (family == FAMILY_DENSE) {
         if ((e = launch_backward_dense(d, Q, K, V, index, lce_w, lse, dO, dQ, dK, dV, status, st)) != cudaSuccess) return e;
     } else if (family == FAMILY_DIRECT) {
-        if ((e = launch_backward_direct(d, Q, K, V, index, inv_off, inv_list, lce_w, lse, dO, dQ, dK, dV,
+        if ((e = launch_backward_direct(d, Q, K, V, index, inv_off, inv_list, inv_order, lce_w, lse, dO, dQ, dK, dV,
                                         delta, status, st)) != cudaSuccess) return e;
     } else {
         SimtGeom g = simt_geom(d, SIMT_DQ);
@@ -425,7 +427,7 @@ static cudaError_t launch_bwd_t(const Dims& d, int impl, const void* Q, const vo
             })) != cudaSuccess)
             return e;
         e = launch_kernel(bwd_dq_simt_kernel<T, D>, dim3(g.gpi > d.heads_i ? g.gpi : d.heads_i, d.heads + 1, d.B), dim3(g.threads),
-                          (size_t)g.smem_bytes, st, false, q, k, v, index, lse, go, static_cast<T*>(dQ), delta, inv_off, inv_list,
+                          (size_t)g.smem_bytes, st, false, q, k, v, index, lse, go, static_cast<T*>(dQ), delta, inv_off, inv_list, inv_order,
                           inverse_uses_bits(d), status, d, g);
         count_launch();
         if (e != cudaSuccess) return e;
@@ -434,8 +436,8 @@ static cudaError_t launch_bwd_t(const Dims& d, int impl, const void* Q, const vo
                 return cudaFuncSetAttribute(bwd_dkv_simt_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, gk.smem_bytes);
             })) != cudaSuccess)
             return e;
-        e = launch_kernel(bwd_dkv_simt_kernel<T, D>, dim3(gk.gpi, d.heads, d.B), dim3(gk.threads), (size_t)gk.smem_bytes, st, true,
-                          q, k, v, static_cast<const int32_t*>(inv_off), static_cast<const int32_t*>(inv_list), lse,
+        e = launch_kernel(bwd_dkv_simt_kernel<T, D>, dim3(d.heads, d.B, gk.gpi), dim3(gk.threads), (size_t)gk.smem_bytes, st, true,
+                          q, k, v, static_cast<const int32_t*>(inv_off), static_cast<const int32_t*>(inv_list), static_cast<const int32_t*>(inv_order), lse,
                           static_cast<const float*>(delta), go, lce_w, static_cast<T*>(dK), static_cast<T*>(dV), d, gk);
         count_launch();
         if (e != cudaSuccess) return e;

@@ -28,14 +28,14 @@ bwd_dq_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* 
                      const __nv_bfloat16* __restrict__ Vg, const int32_t* __restrict__ index,
                      const float* __restrict__ lse, const __nv_bfloat16* __restrict__ dOg,
                      __nv_bfloat16* __restrict__ dQg, float* __restrict__ delta_out,
-                     int32_t* __restrict__ inv_off, int32_t* __restrict__ inv_list, bool inv_bits,
+                     int32_t* __restrict__ inv_off, int32_t* __restrict__ inv_list, int32_t* __restrict__ inv_order, bool inv_bits,
                      int32_t* __restrict__ status, Dims dm, DirGeom gm) {
     constexpr int RT = 1, KS = SINGLE ? 4 : 2;                        // tiles per warp, 16-key steps per block
     extern __shared__ __align__(128) uint8_t smem[];
     // blockIdx.y = 0: the inverse index (one CTA per (image, routing head)); else head blockIdx.y - 1
     if (blockIdx.y == 0) {
         if ((int)blockIdx.x < dm.heads_i)
-            inverse_index_job(index, inv_off, inv_list, blockIdx.z * dm.heads_i + blockIdx.x, reinterpret_cast<int32_t*>(smem), inv_bits, dm);
+            inverse_index_job(index, inv_off, inv_list, inv_order, blockIdx.z * dm.heads_i + blockIdx.x, reinterpret_cast<int32_t*>(smem), inv_bits, dm);
         return;
     }
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -204,7 +204,7 @@ template <int PL, bool EXACT, int TY, int TX>
 __global__ void __launch_bounds__(PL == 2 ? 128 : 256, PL == 2 ? 3 : 2)
 bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __restrict__ Kg,
                       const __nv_bfloat16* __restrict__ Vg, const int32_t* inv_off,
-                      const int32_t* inv_list, const float* __restrict__ lse,
+                      const int32_t* inv_list, const int32_t* inv_order, const float* __restrict__ lse,
                       const float* delta, const __nv_bfloat16* __restrict__ dOg,
                       const float* __restrict__ lce_w, __nv_bfloat16* __restrict__ dKg,
                       __nv_bfloat16* __restrict__ dVg, Dims dm, DirGeom gm) {
@@ -214,18 +214,15 @@ bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16*
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = lane >> 2, t4 = lane & 3;
     const bool one_warp = gm.gpc > 1;
-    const int rest = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
+    const int rest = blockIdx.z, h = blockIdx.x, b = blockIdx.y;      // longest lists of all (image, head) pairs first
     const int grp = one_warp ? warp : 0;
     const int ck = one_warp ? 0 : rest % gm.chunks;
-    const int jr = one_warp ? rest * gm.gpc + warp : rest / gm.chunks;   // key region
+    const int nth = one_warp ? rest * gm.gpc + warp : rest / gm.chunks;  // by falling length of the list
     const int gwarp = one_warp ? 0 : warp, gwarps = one_warp ? 1 : gm.nw;
     const int glane = one_warp ? lane : tid, glanes = gwarps * 32;
-    const bool live = jr < dm.R;
+    const bool live = nth < dm.R;
     auto group_sync = [&]() { if (one_warp) __syncwarp(); else __syncthreads(); };
 
-    const int rj = live ? jr : 0;
-    const int ry = fdiv(rj, dm.S, gm.mul_s), rx = rj - ry * dm.S;
-    const int y0 = ry * dm.hs + ck * gm.hb, x0 = rx * dm.ws;
     const int rows = min(gm.hb, dm.hs - ck * gm.hb);
     const int ntok = rows * dm.ws, c0 = ck * gm.hb * dm.ws;
     const uint32_t tok_bytes = (uint32_t)dm.C * 2;
@@ -239,17 +236,18 @@ bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16*
     uint8_t* dKb = reinterpret_cast<uint8_t*>(dKg) + head_off + t4 * 16;
 
     float* s_w = reinterpret_cast<float*>(smem + gm.off_w);
-    if (dm.lce) {
-        load_lce_weights(s_w, lce_w, h, 32 * PL * 25, tid, gm.nw * 32);
-        if (live) load_halo<PL>(sbase + gm.off_halo + grp * gm.halo_bytes, Gh, y0, x0, rows, dm, gm, glane, glanes);
-    }
-    cp_async_commit();
+    if (dm.lce) load_lce_weights(s_w, lce_w, h, 32 * PL * 25, tid, gm.nw * 32);
     __syncthreads();                                                  // weights
-    pdl_wait();          // delta and the inverse index come from the dQ kernel
+    pdl_wait();          // delta, the inverse index and the order of the regions come from the dQ kernel
     if (!live) return;
 
     const int hi = dm.heads_i == 1 ? 0 : h;
     const size_t bhi = (size_t)b * dm.heads_i + hi;
+    const int jr = __ldcg(inv_order + bhi * dm.R + nth);              // key region
+    const int ry = fdiv(jr, dm.S, gm.mul_s), rx = jr - ry * dm.S;
+    const int y0 = ry * dm.hs + ck * gm.hb, x0 = rx * dm.ws;
+    if (dm.lce) load_halo<PL>(sbase + gm.off_halo + grp * gm.halo_bytes, Gh, y0, x0, rows, dm, gm, glane, glanes);
+    cp_async_commit();
     const int e0 = __ldcg(inv_off + bhi * (dm.R + 1) + jr), e1 = __ldcg(inv_off + bhi * (dm.R + 1) + jr + 1);
     const int32_t* list = inv_list + bhi * dm.R * dm.topk + e0;      // query regions that list jr, fixed order
     const int total = (e1 - e0) * dm.n_r;
@@ -403,7 +401,7 @@ static DirGeom dkv_geom(const Dims& d) {
 bool backward_direct_supported(const Dims& d, int dtype) {
     if (!attend_direct_supported(d, dtype)) return false;
     if ((long long)d.R * d.n_r * d.n_r >= (1ll << 32)) return false;
-    return dkv_geom(d).smem_bytes <= 200 * 1024 && dq_geom(d).smem_bytes <= 200 * 1024 && d.R <= 8192;
+    return dkv_geom(d).smem_bytes <= 200 * 1024 && dq_geom(d).smem_bytes <= 200 * 1024 && d.R <= 8192 && dkv_geom(d).gpi <= 65535;
 }
 
 template <typename F>
@@ -416,7 +414,7 @@ namespace {
 struct BwdArgs {
     const __nv_bfloat16 *q, *k, *v, *go;
     const int32_t* index;
-    int32_t *inv_off, *inv_list;
+    int32_t *inv_off, *inv_list, *inv_order;
     const float *lce_w, *lse;
     __nv_bfloat16 *dq, *dk, *dv;
     float* delta;
@@ -434,7 +432,7 @@ static cudaError_t launch_dq(const Dims& d, const BwdArgs& a) {
     if (e != cudaSuccess) return e;
     count_launch();
     return launch_kernel(kernel, dim3(g.gpi > d.heads_i ? g.gpi : d.heads_i, d.heads + 1, d.B), dim3(g.nw * 32), (size_t)g.smem_bytes, a.st, false,
-                         a.q, a.k, a.v, a.index, a.lse, a.go, a.dq, a.delta, a.inv_off, a.inv_list, inverse_uses_bits(d), a.status, d, g);
+                         a.q, a.k, a.v, a.index, a.lse, a.go, a.dq, a.delta, a.inv_off, a.inv_list, a.inv_order, inverse_uses_bits(d), a.status, d, g);
 }
 
 template <int PL, bool EXACT, int TY, int TX>
@@ -445,8 +443,8 @@ static cudaError_t launch_dkv(const Dims& d, const BwdArgs& a) {
     const cudaError_t e = allow_smem(set, kernel, g.smem_bytes);
     if (e != cudaSuccess) return e;
     count_launch();
-    return launch_kernel(kernel, dim3(g.gpi, d.heads, d.B), dim3(g.nw * 32), (size_t)g.smem_bytes, a.st, true,
-                         a.q, a.k, a.v, a.inv_off, a.inv_list, a.lse, a.delta, a.go, a.lce_w, a.dk, a.dv, d, g);
+    return launch_kernel(kernel, dim3(d.heads, d.B, g.gpi), dim3(g.nw * 32), (size_t)g.smem_bytes, a.st, true,
+                         a.q, a.k, a.v, a.inv_off, a.inv_list, a.inv_order, a.lse, a.delta, a.go, a.lce_w, a.dk, a.dv, d, g);
 }
 
 static cudaError_t launch_both(const Dims& d, const BwdArgs& a) {
@@ -467,12 +465,12 @@ static cudaError_t launch_both(const Dims& d, const BwdArgs& a) {
 }
 
 cudaError_t launch_backward_direct(const Dims& d, const void* Q, const void* K, const void* V,
-                                   const int32_t* index, int32_t* inv_off, int32_t* inv_list,
+                                   const int32_t* index, int32_t* inv_off, int32_t* inv_list, int32_t* inv_order,
                                    const float* lce_w, const float* lse, const void* dO,
                                    void* dQ, void* dK, void* dV, float* delta, int32_t* status, cudaStream_t st) {
     typedef __nv_bfloat16 bf;
     const BwdArgs a = {static_cast<const bf*>(Q), static_cast<const bf*>(K), static_cast<const bf*>(V), static_cast<const bf*>(dO), index,
-                       inv_off, inv_list, lce_w, lse, static_cast<bf*>(dQ), static_cast<bf*>(dK), static_cast<bf*>(dV), delta, status, st};
+                       inv_off, inv_list, inv_order, lce_w, lse, static_cast<bf*>(dQ), static_cast<bf*>(dK), static_cast<bf*>(dV), delta, status, st};
     return launch_both(d, a);
 }
 

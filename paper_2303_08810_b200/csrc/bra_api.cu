@@ -20,6 +20,7 @@ WsLayout ws_layout(const Dims& d) {
     L.delta = off;    off += align256(sizeof(float) * (size_t)d.B * d.heads * d.N);
     L.inv_off = off;  off += align256(sizeof(int32_t) * (size_t)d.B * d.heads_i * (d.R + 1));
     L.inv_list = off; off += align256(sizeof(int32_t) * (size_t)d.B * d.heads_i * d.R * d.topk);
+    L.inv_order = off; off += align256(sizeof(int32_t) * (size_t)d.B * d.heads_i * d.R);
     L.dw_part = off;  off += align256(sizeof(float) * (size_t)lce_grad_partials(d) * d.C * 26);
     L.pad = L.pad_lse = off;
     L.pad_tensor = 0;

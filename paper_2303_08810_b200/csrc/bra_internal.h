@@ -41,6 +41,7 @@ struct WsLayout {
     size_t delta;       // fp32 [B,heads,N]  rowsum(P o dP) of the backward pass
     size_t inv_off;     // int32 [B,heads_i,R+1] CSR offsets of the inverse routing index
     size_t inv_list;    // int32 [B,heads_i,R*topk] query regions routed to each key region
+    size_t inv_order;   // int32 [B,heads_i,R] key regions by falling length of their lists
     size_t dw_part;     // fp32 [lce_grad_partials(d), 26*C] partial LCE weight / bias gradients
     size_t pad;         // padded maps only: seven [B,H,W,C] tensors of the padded size (Q, K, V, O / dO, dQ, dK, dV)
     size_t pad_lse;     // padded maps only: fp32 [B,heads,H*W] of the padded size
@@ -126,7 +127,7 @@ cudaError_t launch_attend_tc_wide(const Dims& d, const void* Q, const void* K, c
 
 bool backward_direct_supported(const Dims& d, int dtype);
 cudaError_t launch_backward_direct(const Dims& d, const void* Q, const void* K, const void* V,
-                                const int32_t* index, int32_t* inv_off, int32_t* inv_list,
+                                const int32_t* index, int32_t* inv_off, int32_t* inv_list, int32_t* inv_order,
                                 const float* lce_w, const float* lse, const void* dO,
                                 void* dQ, void* dK, void* dV, float* delta, int32_t* status, cudaStream_t st);
 

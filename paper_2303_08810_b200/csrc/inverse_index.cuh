@@ -1,5 +1,7 @@
 // Inverse routing index of one (image, routing head): for each key region the query regions whose rows list it, in
-// entry order (query region, then slot) - the fixed order of the dK / dV sums - as CSR.
+// entry order (query region, then slot) - the fixed order of the dK / dV sums - as CSR; and the key regions by falling
+// length of their lists.  The dK / dV kernels start the longest first: where a map has a few kinds of content, the queries
+// of a kind all pick the same few regions (2 x 100 x 167 tokens, S = 16: 264 us in map order, 172 us with evenly spread lists).
 #pragma once
 
 #include "bra_internal.h"
@@ -11,7 +13,7 @@ constexpr int INVERSE_BITS_MAX = 40 * 1024;     // bytes of the bit matrix up to
 inline int inverse_words(const Dims& d) { return (d.R + 31) / 32; }
 inline bool inverse_uses_bits(const Dims& d) { return (size_t)d.R * inverse_words(d) * 4 <= INVERSE_BITS_MAX; }
 inline size_t inverse_smem(const Dims& d) {
-    return sizeof(int32_t) * ((size_t)d.R + 2 + (inverse_uses_bits(d) ? (size_t)d.R * inverse_words(d) : 0));
+    return sizeof(int32_t) * (2 * (size_t)d.R + 2 + (inverse_uses_bits(d) ? (size_t)d.R * inverse_words(d) : 0));
 }
 
 // One CTA.  A row of the index seldom names a region twice, so what has to be inverted is a bit matrix (key region x
@@ -21,7 +23,7 @@ inline size_t inverse_smem(const Dims& d) {
 // or a matrix that does not fit sends the CTA to the comparisons: warp w takes key regions w, w + nwarps, ..., sweeps
 // the entries 32 at a time and finds its region's hits with a ballot.  Entries outside [0, R) are in no list.
 __device__ __forceinline__ void inverse_index_job(const int32_t* __restrict__ index, int32_t* __restrict__ inv_off,
-                                                  int32_t* __restrict__ inv_list, int bh, int32_t* sm, bool use_bits, const Dims& dm) {
+                                                  int32_t* __restrict__ inv_list, int32_t* __restrict__ order, int bh, int32_t* sm, bool use_bits, const Dims& dm) {
     const int tid = threadIdx.x, nthreads = blockDim.x;
     const int lane = tid & 31, warp = tid >> 5, nwarps = nthreads >> 5;
     const int entries = dm.R * dm.topk, words = (dm.R + 31) >> 5;
@@ -29,7 +31,8 @@ __device__ __forceinline__ void inverse_index_job(const int32_t* __restrict__ in
     int32_t* off = inv_off + (size_t)bh * (dm.R + 1);
     int32_t* list = inv_list + (size_t)bh * entries;
     int32_t* count = sm;                                    // [R + 1]
-    uint32_t* bits = reinterpret_cast<uint32_t*>(sm + dm.R + 2);
+    int32_t* length = sm + dm.R + 2;                        // [R]
+    uint32_t* bits = reinterpret_cast<uint32_t*>(sm + 2 * dm.R + 2);
     int* repeated = sm + dm.R + 1;
     bool by_bits = use_bits;
     if (use_bits) {
@@ -70,13 +73,19 @@ __device__ __forceinline__ void inverse_index_job(const int32_t* __restrict__ in
                 const int o = __shfl_up_sync(0xffffffffu, incl, s);
                 if (lane >= s) incl += o;
             }
-            if (j < dm.R) count[j] = run + incl - n;
+            if (j < dm.R) { count[j] = run + incl - n; length[j] = n; }
             run += __shfl_sync(0xffffffffu, incl, 31);
         }
         if (lane == 0) count[dm.R] = run;
     }
     __syncthreads();
     for (int j = tid; j <= dm.R; j += nthreads) off[j] = count[j];
+    for (int j = tid; j < dm.R; j += nthreads) {            // longest list first, ties to the lower region
+        const int n = length[j];
+        int rank = 0;
+        for (int o = 0; o < dm.R; ++o) rank += length[o] > n || (length[o] == n && o < j);
+        order[(size_t)bh * dm.R + rank] = j;
+    }
     if (by_bits) {
         for (int j = tid; j < dm.R; j += nthreads) {
             int32_t* out = list + count[j];

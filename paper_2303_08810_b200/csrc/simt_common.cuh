@@ -18,7 +18,7 @@
 namespace bra {
 
 namespace sk {
-constexpr int THREADS = 64;             // short CTAs: several per SM, an even tail
+constexpr int THREADS = 256;            // at most: enough for a region, which shares the copies (64 if that is enough: an even tail)
 constexpr int RESIDENT_MAX = 100 * 1024;
 constexpr int IDX_MAX = 4096;           // routing entries kept in shared memory per CTA
 }  // namespace sk
@@ -48,10 +48,14 @@ inline SimtGeom simt_geom(const Dims& d, SimtKind kind) {
     g.row = d.d * d.esize + 16;
     g.mul_nr = recip32(d.n_r); g.mul_ws = recip32(d.ws); g.mul_s = recip32(d.S);
     // lanes of this call against the lanes the GPU holds at once (12 warps per SM)
-    const long long lanes = (long long)d.B * d.heads * d.R * ((d.n_r + qt - 1) / qt);
+    // (dK / dV of larger maps: as if an eighth of the regions held the lists, which is what clustered content comes to;
+    // measured at 1 x 96 x 96, S = 7, 2 heads: 522 -> 224 us; at 36 x 14 x 14 it costs more than it gives)
+    const long long lanes = (long long)d.B * d.heads * d.R * ((d.n_r + qt - 1) / qt) / (kind == SIMT_DKV && d.N > 400 ? 8 : 1);
     g.ksl = 0;
     while (g.ksl < 3 && (lanes << g.ksl) < kSMs * 256 && (qt * d.d >> (g.ksl + 1)) >= 4) ++g.ksl;    // sum_shares: whole float4s
-    const int most = sk::THREADS >> g.ksl;                            // lane groups of a CTA
+    int threads = 64;
+    while (threads < sk::THREADS && ((d.n_r + qt - 1) / qt << g.ksl) > threads) threads *= 2;
+    const int most = threads >> g.ksl;                                // lane groups of a CTA
     g.hb = d.hs; g.cw = d.ws;
     if ((d.n_r + qt - 1) / qt > most) {
         if (g.cw > qt * most) g.cw = qt * most;
@@ -286,8 +290,10 @@ __device__ __forceinline__ void simt_st(__nv_bfloat16* p, float v) { *p = __floa
 
 // Adds the 5 x 5 depthwise correlation of `in` (FLIP: with the flipped filter) to the staged rows of the CTA's regions and
 // stores them.  Lane = channel (32 at a time), TS x TS positions per pass: every input value is read once per tile.
-template <typename T, int D, int TS, bool FLIP>
-__device__ __forceinline__ void simt_lce(const float* st, const float* s_w, const float* bias, const T* in, T* out, int r0, int nreg, int rows_per_region,
+// region_at[i]: region i of the CTA.
+struct SimtFrom { int r0; __device__ int operator[](int i) const { return r0 + i; } };
+template <typename T, int D, int TS, bool FLIP, typename RegionAt>
+__device__ __forceinline__ void simt_lce(const float* st, const float* s_w, const float* bias, const T* in, T* out, RegionAt region_at, int nreg, int rows_per_region,
                                          const SimtChunk& c,                                         const Dims& dm, const SimtGeom& gm) {
     constexpr int LANES = D < 32 ? D : 32, GROUPS = D / LANES, SUB = 32 / LANES;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
@@ -306,7 +312,7 @@ __device__ __forceinline__ void simt_lce(const float* st, const float* s_w, cons
             for (int k = 0; k < 25; ++k) w[k] = dm.lce ? s_w[ch * 25 + k] : 0.f;
             b = bias ? __ldg(bias + ch) : 0.f;
         }
-        const int r = r0 + rl;
+        const int r = region_at[rl];
         const int ry = fdiv(r, dm.S, gm.mul_s), rx = r - ry * dm.S;
         const int ly0 = ty * TS, lx0 = tx * TS;                       // within the chunk
         const int y0 = ry * dm.hs + c.y + ly0, x0 = rx * dm.ws + c.x + lx0;

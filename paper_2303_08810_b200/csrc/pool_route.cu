@@ -15,6 +15,29 @@ namespace bra {
 template <typename T> struct Vec;
 template <> struct Vec<float> { static constexpr int n = 4; };
 template <> struct Vec<__nv_bfloat16> { static constexpr int n = 8; };
+// load_row with coherent loads: the pooling kernels may be launched while the kernel before them in the stream (the
+// caller's, which may write Q and K) still runs, and loads on the read-only path may be moved above the wait for it
+template <int n>
+__device__ __forceinline__ void load_row_cg(const float* p, float* out) {
+#pragma unroll
+    for (int i = 0; i < n; i += 4) {
+        const float4 v = __ldcg(reinterpret_cast<const float4*>(p + i));
+        out[i] = v.x; out[i + 1] = v.y; out[i + 2] = v.z; out[i + 3] = v.w;
+    }
+}
+template <int n>
+__device__ __forceinline__ void load_row_cg(const __nv_bfloat16* p, float* out) {
+#pragma unroll
+    for (int i = 0; i < n; i += 8) {
+        const uint4 v = __ldcg(reinterpret_cast<const uint4*>(p + i));
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            out[i + 2 * j] = __uint_as_float(w[j] << 16);
+            out[i + 2 * j + 1] = __uint_as_float(w[j] & 0xffff0000u);
+        }
+    }
+}
 template <int n>
 __device__ __forceinline__ void zero_row(float* v) {
 #pragma unroll
@@ -23,7 +46,7 @@ __device__ __forceinline__ void zero_row(float* v) {
 
 template <typename T, bool ANY_MAP>
 __global__ void __launch_bounds__(256)
-pool_kernel(const T* __restrict__ Q, const T* __restrict__ K,
+pool_kernel(const T* Q, const T* K,
             float* __restrict__ q_mean, float* __restrict__ k_mean, Dims dm) {
     constexpr int VEC = Vec<T>::n;
     extern __shared__ float part[];   // [ws][C]
@@ -39,6 +62,7 @@ pool_kernel(const T* __restrict__ Q, const T* __restrict__ K,
     const int rows = ANY_MAP ? min(dm.hs, dm.H0 - ry * dm.hs) : dm.hs;
     const int on_map = ANY_MAP ? min(dm.ws, dm.W0 - rx * dm.ws) * cvecs : items;
 
+    pdl_wait();
     for (int it = threadIdx.x; it < items; it += blockDim.x) {
         float acc[VEC];
 #pragma unroll
@@ -48,7 +72,7 @@ pool_kernel(const T* __restrict__ Q, const T* __restrict__ K,
         for (; (!ANY_MAP || it < on_map) && y + 8 <= rows; y += 8) {      // eight loads in flight
             float v[8][VEC];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) load_row<VEC>(p + (size_t)(y + u) * row_elems, v[u]);
+            for (int u = 0; u < 8; ++u) load_row_cg<VEC>(p + (size_t)(y + u) * row_elems, v[u]);
 #pragma unroll
             for (int u = 0; u < 8; ++u)
 #pragma unroll
@@ -56,7 +80,7 @@ pool_kernel(const T* __restrict__ Q, const T* __restrict__ K,
         }
         for (; (!ANY_MAP || it < on_map) && y < rows; ++y) {
             float v[VEC];
-            load_row<VEC>(p + (size_t)y * row_elems, v);
+            load_row_cg<VEC>(p + (size_t)y * row_elems, v);
 #pragma unroll
             for (int i = 0; i < VEC; ++i) acc[i] += v[i];
         }
@@ -79,7 +103,7 @@ pool_kernel(const T* __restrict__ Q, const T* __restrict__ K,
 // is what this latency-bound scan needs).  Row halves are added lower half first.
 template <typename T, bool ANY_MAP>
 __global__ void __launch_bounds__(256)
-pool_split_kernel(const T* __restrict__ Q, const T* __restrict__ K,
+pool_split_kernel(const T* Q, const T* K,
                   float* __restrict__ q_mean, float* __restrict__ k_mean, Dims dm) {
     constexpr int VEC = Vec<T>::n;
     extern __shared__ float part[];   // [2][ws][C]
@@ -94,9 +118,10 @@ pool_split_kernel(const T* __restrict__ Q, const T* __restrict__ K,
     const int it = threadIdx.x % items, yh = threadIdx.x / items;        // blockDim.x == 2 * items
     const T* p = src + ((size_t)b * dm.H0 + (size_t)ry * dm.hs + 4 * yh) * row_elems + (size_t)rx * dm.ws * dm.C + (size_t)it * VEC;
     float v[4][VEC];
+    pdl_wait();
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-        if (!ANY_MAP || (ry * dm.hs + 4 * yh + u < dm.H0 && rx * dm.ws + it / cvecs < dm.W0)) load_row<VEC>(p + (size_t)u * row_elems, v[u]);
+        if (!ANY_MAP || (ry * dm.hs + 4 * yh + u < dm.H0 && rx * dm.ws + it / cvecs < dm.W0)) load_row_cg<VEC>(p + (size_t)u * row_elems, v[u]);
         else zero_row<VEC>(v[u]);
     }
     float acc[VEC];
@@ -126,7 +151,7 @@ pool_split_kernel(const T* __restrict__ Q, const T* __restrict__ K,
 // stage-3 shape: the launch rate of CTAs, not HBM, sets its time.)
 template <typename T, int HS, int WS, bool ANY_MAP>
 __global__ void __launch_bounds__(512)
-pool_rows_kernel(const T* __restrict__ Q, const T* __restrict__ K,
+pool_rows_kernel(const T* Q, const T* K,
                  float* __restrict__ q_mean, float* __restrict__ k_mean, Dims dm) {
     constexpr int VEC = Vec<T>::n;
     const int ry = blockIdx.x, b = blockIdx.z;
@@ -134,6 +159,7 @@ pool_rows_kernel(const T* __restrict__ Q, const T* __restrict__ K,
     float* dst = blockIdx.y == 0 ? q_mean : k_mean;
     const int cvecs = dm.C / VEC;
     const int rx = threadIdx.x / cvecs, cv = threadIdx.x - rx * cvecs;
+    pdl_wait();
     if (rx >= dm.S) return;
     const size_t row_elems = (size_t)dm.W0 * dm.C;
     const T* p = src + ((size_t)b * dm.H0 + (size_t)ry * HS) * row_elems + (size_t)rx * dm.ws * dm.C + (size_t)cv * VEC;
@@ -143,7 +169,7 @@ pool_rows_kernel(const T* __restrict__ Q, const T* __restrict__ K,
     for (int x = 0; x < WS; ++x)
 #pragma unroll
         for (int y = 0; y < HS; ++y) {
-            if (!ANY_MAP || (ry * HS + y < dm.H0 && rx * WS + x < dm.W0)) load_row<VEC>(p + (size_t)y * row_elems + (size_t)x * dm.C, v[x][y]);
+            if (!ANY_MAP || (ry * HS + y < dm.H0 && rx * WS + x < dm.W0)) load_row_cg<VEC>(p + (size_t)y * row_elems + (size_t)x * dm.C, v[x][y]);
             else zero_row<VEC>(v[x][y]);
         }
     // the next kernel may be set up from here on: this CTA's loads are out
@@ -176,11 +202,12 @@ static cudaError_t launch_pool_rows_t(const Dims& d, const void* Q, const void* 
     const dim3 grid(d.S, 2, d.B);
     const T* q = static_cast<const T*>(Q);
     const T* k = static_cast<const T*>(K);
-    if (d.hs == 1) pool_rows_kernel<T, 1, 1, ANY_MAP><<<grid, threads, 0, st>>>(q, k, q_mean, k_mean, d);
-    else if (d.hs == 2) pool_rows_kernel<T, 2, 2, ANY_MAP><<<grid, threads, 0, st>>>(q, k, q_mean, k_mean, d);
-    else pool_rows_kernel<T, 4, 4, ANY_MAP><<<grid, threads, 0, st>>>(q, k, q_mean, k_mean, d);
+    cudaError_t e;
+    if (d.hs == 1) e = launch_kernel(pool_rows_kernel<T, 1, 1, ANY_MAP>, grid, dim3(threads), 0, st, true, q, k, q_mean, k_mean, d);
+    else if (d.hs == 2) e = launch_kernel(pool_rows_kernel<T, 2, 2, ANY_MAP>, grid, dim3(threads), 0, st, true, q, k, q_mean, k_mean, d);
+    else e = launch_kernel(pool_rows_kernel<T, 4, 4, ANY_MAP>, grid, dim3(threads), 0, st, true, q, k, q_mean, k_mean, d);
     count_launch();
-    return cudaGetLastError();
+    return e;
 }
 
 template <typename T>
@@ -203,15 +230,14 @@ cudaError_t launch_pool(const Dims& d, int dtype, const void* Q, const void* K,
     dim3 grid(d.R, d.B, 2);
     if (d.hs == 8 && 2 * items <= 256 && 2 * smem <= 48 * 1024) {
         const bool any = d.H != d.H0 || d.W != d.W0;
-        auto go = [&](auto* q, auto* k) {
+        auto go = [&](auto* q, auto* k) -> cudaError_t {
             typedef typename std::remove_const<typename std::remove_pointer<decltype(q)>::type>::type T;
-            if (any) pool_split_kernel<T, true><<<grid, 2 * items, 2 * smem, st>>>(q, k, q_mean, k_mean, d);
-            else pool_split_kernel<T, false><<<grid, 2 * items, 2 * smem, st>>>(q, k, q_mean, k_mean, d);
+            count_launch();
+            return launch_kernel(any ? pool_split_kernel<T, true> : pool_split_kernel<T, false>, grid, dim3(2 * items), 2 * smem, st, true,
+                                 q, k, q_mean, k_mean, d);
         };
-        if (dtype == BRA_BF16) go(static_cast<const __nv_bfloat16*>(Q), static_cast<const __nv_bfloat16*>(K));
-        else go(static_cast<const float*>(Q), static_cast<const float*>(K));
-        count_launch();
-        return cudaGetLastError();
+        return dtype == BRA_BF16 ? go(static_cast<const __nv_bfloat16*>(Q), static_cast<const __nv_bfloat16*>(K))
+                                 : go(static_cast<const float*>(Q), static_cast<const float*>(K));
     }
     auto go = [&](auto* q, auto* k) -> cudaError_t {
         typedef typename std::remove_const<typename std::remove_pointer<decltype(q)>::type>::type T;
@@ -220,9 +246,8 @@ cudaError_t launch_pool(const Dims& d, int dtype, const void* Q, const void* K,
             const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        kernel<<<grid, threads, smem, st>>>(q, k, q_mean, k_mean, d);
         count_launch();
-        return cudaGetLastError();
+        return launch_kernel(kernel, grid, dim3(threads), smem, st, true, q, k, q_mean, k_mean, d);
     };
     return dtype == BRA_BF16 ? go(static_cast<const __nv_bfloat16*>(Q), static_cast<const __nv_bfloat16*>(K))
                              : go(static_cast<const float*>(Q), static_cast<const float*>(K));

@@ -738,3 +738,150 @@ def test_random_shapes_forward_and_backward(bra, seed):
             assert np.abs(f64(a) - r).max() <= GRAD_MAX, f"{cfg} {impl} {name}"
         ran += 1
     assert ran >= 8
+
+
+# ------------------------------------------------------------------ edges of the kernels and of their dispatch rules
+# The bounds are those at the top of this file: one rounding of P and of O to bf16 (2^-9 of values of order 1 to 4), fp32 sums
+# otherwise.  `kind` of the index: "route" (bra_route's), "repeats" (random, one row names a single region).
+def run_edge(bra, cfg, impl, kind="route", seed=51, **kw):
+    index = None
+    if kind == "repeats":
+        rng = np.random.default_rng(seed)
+        heads_i = 1 if kw.get("shared") else cfg.heads
+        index = rng.integers(0, cfg.R, size=(cfg.B, heads_i, cfg.R, cfg.topk)).astype(np.int32)
+        index[0, 0, 0] = cfg.R - 1
+    run_attend_case(bra, cfg, impl, seed, index=index, **kw)
+    run_backward_case(bra, cfg, seed, index=index, impl=impl, shared=kw.get("shared", False))
+
+
+# every token of the map a key: topk * 16 rows (n_r rounded up) > tokens; above 64 tokens from 64 pairs on, gradients 296
+DENSE_EDGES = [
+    (BraConfig("dense-one-token-map", 1, 1, 1, 32, 1, 1, 1, "bf16"), "route"),
+    (BraConfig("dense-1-token-regions-k=R", 2, 7, 7, 64, 2, 7, 49, "bf16"), "route"),
+    (BraConfig("dense-64-regions", 2, 8, 8, 32, 1, 8, 5, "bf16"), "route"),          # the mask's last bit; repeats: counts
+    (BraConfig("dense-64-regions-repeats", 2, 8, 8, 64, 2, 8, 5, "bf16"), "repeats"),
+    (BraConfig("dense-1x2-regions", 3, 4, 8, 64, 2, 4, 3, "bf16"), "route"),
+    (BraConfig("dense-3x3-regions", 2, 6, 6, 64, 2, 2, 3, "bf16"), "repeats"),
+    (BraConfig("dense-3x5-regions-k=R", 2, 6, 10, 64, 2, 2, 4, "bf16"), "route"),
+    (BraConfig("dense-2x2-regions-63-pairs", 63, 12, 12, 32, 1, 6, 13, "bf16"), "route"),
+    (BraConfig("dense-2x2-regions-64-pairs", 64, 12, 12, 32, 1, 6, 13, "bf16"), "route"),
+    (BraConfig("dense-256-tokens-296-pairs", 148, 16, 16, 64, 2, 8, 17, "bf16"), "route"),
+    (BraConfig("dense-135-tokens-296-pairs", 148, 9, 15, 64, 2, 3, 9, "bf16"), "repeats"),
+    (BraConfig("dense-padded-64-tokens", 2, 7, 6, 64, 2, 4, 5, "bf16"), "route"),
+    (BraConfig("dense-padded-whole-regions", 2, 5, 5, 64, 2, 4, 5, "bf16"), "repeats"),
+    (BraConfig("dense-padded-k=R-64-pairs", 32, 13, 13, 64, 2, 7, 49, "bf16"), "route"),
+]
+
+
+@pytest.mark.parametrize("cfg,kind", DENSE_EDGES, ids=[c.name for c, _ in DENSE_EDGES])
+def test_dense_kernels_at_their_edges(bra, cfg, kind):
+    run_edge(bra, cfg, "auto", kind)
+    if cfg.B <= 3:
+        run_edge(bra, cfg, "auto", "repeats", seed=52, shared=True)
+        run_attend_case(bra, cfg, "auto", 53, lce=False)
+        run_attend_case(bra, cfg, "auto", 54, bias=True, scale=0.5)
+    if cfg.topk == cfg.R:                   # no index asked for: nothing needs to be routed
+        x = synthetic.make_inputs(cfg, seed=55)
+        t = to_dev(x, cfg)
+        p = problem_of(bra, cfg)
+        O, _, lse = bra.bra_forward(p, t["Q"], t["K"], t["V"], t["w"], want_index=False)
+        every = np.broadcast_to(np.arange(cfg.R, dtype=np.int32), (cfg.B, cfg.heads, cfg.R, cfg.R))
+        O_ref, lse_ref = orc.bra_attend(x["Q"], x["K"], x["V"], every, x["w"], cfg.heads, cfg.S)
+        check_O(f64(O), O_ref, cfg.dtype)
+        np.testing.assert_allclose(f64(lse), lse_ref, rtol=0, atol=2e-3)
+
+
+# operands straight from global memory: any region and map, head dim 32 or 64; two tiles per warp from 1184 warps on
+DIRECT_EDGES = [
+    (BraConfig("direct-6x7-1152-warps", 18, 24, 28, 64, 2, 4, 3, "bf16"), "route"),
+    (BraConfig("direct-6x7-1216-warps", 19, 24, 28, 64, 2, 4, 3, "bf16"), "route"),
+    (BraConfig("direct-d64-6x7-1216-warps", 19, 24, 28, 128, 2, 4, 3, "bf16"), "repeats"),
+    (BraConfig("direct-10x2-two-tiles", 37, 40, 8, 64, 2, 4, 2, "bf16"), "route"),
+    (BraConfig("direct-7x3-two-tiles", 37, 28, 12, 64, 2, 4, 2, "bf16"), "route"),
+    (BraConfig("direct-11x12-one-tile", 1, 22, 24, 64, 2, 2, 3, "bf16"), "repeats"),      # more than 128 tokens, 12-wide rows
+    (BraConfig("direct-11x12-two-tiles", 30, 22, 24, 64, 2, 2, 3, "bf16"), "route"),
+    (BraConfig("direct-2x128-row-of-a-chunk", 1, 4, 128, 32, 1, 1, 1, "bf16"), "route"),
+    (BraConfig("direct-4x4-two-passes-of-a-table", 2, 28, 28, 64, 2, 7, 20, "bf16"), "repeats"),
+    (BraConfig("direct-16x16-two-passes-of-a-table", 1, 32, 32, 64, 2, 2, 4, "bf16"), "route"),
+    (BraConfig("direct-d64-one-token-regions", 1, 7, 7, 128, 2, 7, 49, "bf16"), "route"),
+    (BraConfig("direct-d64-16x16", 1, 32, 32, 64, 1, 2, 3, "bf16"), "repeats"),
+    (BraConfig("direct-padded-8x7", 2, 29, 27, 64, 2, 4, 3, "bf16"), "route"),
+    (BraConfig("direct-padded-d64-8x7", 2, 29, 27, 128, 2, 4, 3, "bf16"), "route"),
+    (BraConfig("direct-padded-two-tiles", 19, 21, 25, 64, 2, 4, 3, "bf16"), "route"),
+    (BraConfig("direct-padded-rows-of-whole-regions", 2, 9, 9, 64, 2, 8, 6, "bf16"), "repeats"),
+    (BraConfig("direct-529-regions", 1, 23, 23, 32, 1, 23, 3, "bf16"), "repeats"),          # inverse index: bits / comparisons
+    (BraConfig("direct-576-regions", 1, 24, 24, 32, 1, 24, 3, "bf16"), "repeats"),
+]
+
+
+@pytest.mark.parametrize("cfg,kind", DIRECT_EDGES, ids=[c.name for c, _ in DIRECT_EDGES])
+def test_direct_kernels_at_their_edges(bra, cfg, kind):
+    run_edge(bra, cfg, "mma", kind)
+    if cfg.B <= 2:
+        run_edge(bra, cfg, "mma", "repeats", seed=52, shared=True)
+        run_attend_case(bra, cfg, "mma", 53, lce=False, index=np.zeros((cfg.B, cfg.heads, cfg.R, cfg.topk), np.int32))
+
+
+# CUDA cores: two rows per lane up to head dim 32, 1 to 8 lanes per row, rows resident / staged / counted, chunks
+SIMT_EDGES = [
+    (BraConfig("simt-one-token-map", 1, 1, 1, 16, 1, 1, 1, "f32"), "route"),
+    (BraConfig("simt-d16-8-lanes-per-row", 1, 8, 8, 16, 1, 2, 2, "f32"), "repeats"),
+    (BraConfig("simt-d64-staged", 1, 24, 24, 64, 1, 3, 3, "f32"), "route"),
+    (BraConfig("simt-d128", 1, 8, 12, 256, 2, 2, 3, "f32"), "repeats"),
+    (BraConfig("simt-d128-odd-regions", 1, 9, 15, 128, 1, 3, 2, "f32"), "route"),
+    (BraConfig("simt-one-lane-per-row", 32, 28, 28, 128, 4, 7, 1, "f32"), "route"),
+    (BraConfig("simt-2x600-region", 1, 2, 600, 32, 1, 1, 1, "f32"), "route"),
+    (BraConfig("simt-40x9-regions", 1, 80, 18, 32, 1, 2, 2, "f32"), "repeats"),
+    (BraConfig("simt-every-region-counts", 1, 14, 14, 64, 2, 7, 49, "f32"), "repeats"),
+    (BraConfig("simt-every-region", 2, 6, 6, 32, 1, 3, 9, "f32"), "route"),
+    (BraConfig("simt-padded-d16", 2, 37, 26, 32, 2, 5, 4, "f32"), "route"),
+    (BraConfig("simt-padded-resident", 1, 9, 9, 64, 2, 8, 6, "f32"), "repeats"),
+    (BraConfig("simt-bf16-d16", 1, 14, 13, 32, 2, 7, 4, "bf16"), "route"),
+    (BraConfig("simt-576-regions", 1, 24, 24, 32, 1, 24, 3, "f32"), "repeats"),
+]
+
+
+@pytest.mark.parametrize("cfg,kind", SIMT_EDGES, ids=[c.name for c, _ in SIMT_EDGES])
+def test_cuda_core_kernels_at_their_edges(bra, cfg, kind):
+    run_edge(bra, cfg, "simt", kind)
+    if cfg.B <= 2:
+        run_edge(bra, cfg, "simt", "repeats", seed=52, shared=True)
+        run_attend_case(bra, cfg, "simt", 53, bias=True)
+
+
+@pytest.mark.parametrize("B,H,W,C,d,dtype", [
+    (1, 1, 1, 32, 32, "bf16"), (2, 1, 70, 32, 32, "bf16"), (1, 70, 1, 96, 32, "f32"), (2, 33, 17, 96, 32, "bf16"),
+    (1, 31, 65, 64, 64, "bf16"), (1, 5, 33, 16, 16, "f32"), (3, 17, 35, 80, 16, "f32"), (40, 12, 20, 128, 64, "bf16")])
+def test_lce_weight_gradient_at_the_edges_of_its_tiles(bra, B, H, W, C, d, dtype):
+    """Maps of one row or column, widths next to a tile's, channel counts that leave part of a block: d_lce_w and d_lce_b
+    to the rounding of their fp32 sums (the attention gradients beside them have their own tests)."""
+    import torch
+    cfg = BraConfig("lce-grad", B, H, W, C, C // d, 1, 1, dtype)
+    x = synthetic.make_inputs(cfg, seed=61, with_do=True)
+    t = to_dev(x, cfg)
+    p = problem_of(bra, cfg)
+    ws = bra.workspace(p)
+    idx = torch.zeros(B, cfg.heads, 1, 1, dtype=torch.int32, device="cuda")
+    _, lse = bra.bra_attend(p, t["Q"], t["K"], t["V"], idx, t["w"], ws=ws)
+    g = bra.bra_backward(p, t["Q"], t["K"], t["V"], idx, t["w"], lse, t["dO"], ws=ws, want_bias_grad=True)
+    assert bra.bra_device_status(ws) == 0
+    Vp = np.pad(x["V"].astype(np.float64), ((0, 0), (2, 2), (2, 2), (0, 0)))
+    G = x["dO"].astype(np.float64)
+    ref_w = np.stack([np.stack([(G * Vp[:, i:i + H, j:j + W]).sum((0, 1, 2)) for j in range(5)], -1) for i in range(5)], -2)
+    ref_b = G.sum((0, 1, 2))
+    for a, r in ((g[3], ref_w), (g[4], ref_b)):
+        assert np.abs(f64(a) - r).max() <= LCE_GRAD_REL * max(1.0, np.abs(r).max())
+
+
+@pytest.mark.parametrize("B,H,W,S,dtype", [
+    (2, 30, 29, 4, "bf16"), (2, 13, 13, 7, "bf16"), (1, 6, 5, 7, "f32"), (2, 27, 26, 7, "f32"), (1, 23, 17, 4, "bf16"), (1, 5, 5, 4, "bf16")])
+def test_pooling_of_maps_that_S_does_not_divide(bra, B, H, W, S, dtype):
+    """Regions of 8 x 8, 2 x 2, 1 x 1, 4 x 4, 6 x 5 tokens that the map's edge cuts, and regions wholly outside."""
+    cfg = BraConfig("pool", B, H, W, 64, 2, S, 2, dtype)
+    x = synthetic.make_inputs(cfg, seed=71)
+    t = to_dev(x, cfg)
+    qm, km, idx = bra.bra_route(problem_of(bra, cfg), t["Q"], t["K"])
+    Qr, Kr, idx_ref, gap = orc.bra_route(x["Q"], x["K"], cfg.heads, S, 2)
+    np.testing.assert_allclose(f64(qm), Qr, rtol=0, atol=2e-6)
+    np.testing.assert_allclose(f64(km), Kr, rtol=0, atol=2e-6)
+    check_index(idx.cpu().numpy(), idx_ref, gap, 2, cfg.R, orc.region_affinity(Qr, Kr, cfg.heads))

@@ -751,7 +751,8 @@ def run_edge(bra, cfg, impl, kind="route", seed=51, **kw):
         index = rng.integers(0, cfg.R, size=(cfg.B, heads_i, cfg.R, cfg.topk)).astype(np.int32)
         index[0, 0, 0] = cfg.R - 1
     run_attend_case(bra, cfg, impl, seed, index=index, **kw)
-    run_backward_case(bra, cfg, seed, index=index, impl=impl, shared=kw.get("shared", False))
+    if cfg.d <= 64:                         # no gradients at head dim 128
+        run_backward_case(bra, cfg, seed, index=index, impl=impl, shared=kw.get("shared", False))
 
 
 # every token of the map a key: topk * 16 rows (n_r rounded up) > tokens; above 64 tokens from 64 pairs on, gradients 296
@@ -846,7 +847,7 @@ def test_cuda_core_kernels_at_their_edges(bra, cfg, kind):
     run_edge(bra, cfg, "simt", kind)
     if cfg.B <= 2:
         run_edge(bra, cfg, "simt", "repeats", seed=52, shared=True)
-        run_attend_case(bra, cfg, "simt", 53, bias=True)
+        run_attend_case(bra, cfg, "simt", 53, bias=True, index=np.zeros((cfg.B, cfg.heads, cfg.R, cfg.topk), np.int32))
 
 
 @pytest.mark.parametrize("B,H,W,C,d,dtype", [

@@ -23,11 +23,13 @@
  *   - Regions: S x S non-overlapping blocks of (H/S) x (W/S) tokens, numbered
  *     row-major r = ry * S + rx (region partition, Section 3.2).  Where S does
  *     not divide H or W (Appendix C picks S as a divisor "to avoid padding"),
- *     the library works on copies of Q, K, V zero-padded at the bottom and the
- *     right to the next multiples of S: the zero tokens are pooled, routed to
- *     and attended to like real ones, and O, lse and the gradients are cropped
- *     back to H x W.  The copies live in ws (bra_workspace_bytes accounts for
- *     them) and cost one extra kernel per tensor.
+ *     the map counts as zero-padded at the bottom and the right to the next
+ *     multiples of S: the zero tokens are pooled, routed to and attended to like
+ *     real ones, and O, lse and the gradients are those of the H x W tokens.
+ *     Most kernels work on the map as it is; those that want whole regions
+ *     (BRA_IMPL_TC and BRA_IMPL_IMG) get padded copies, which live in ws
+ *     (bra_workspace_bytes accounts for them) and cost one extra kernel per
+ *     tensor.
  *   - index: int32 [B, heads, S*S, topk] (or [B, 1, S*S, topk] when
  *     p->shared_routing != 0).  Row i lists the key regions that the queries of
  *     region i attend to.  It is a list: any order, duplicates count twice.
@@ -75,7 +77,8 @@ typedef enum bra_dtype { BRA_F32 = 0, BRA_BF16 = 1 } bra_dtype;
 typedef enum bra_impl {
     BRA_IMPL_AUTO = 0,  /* fastest kernel that supports the problem */
     BRA_IMPL_SIMT = 1,  /* fp32 CUDA-core kernel: any dtype, any shape with C/heads <= 128 */
-    BRA_IMPL_MMA = 2,   /* bf16 warp-level tensor-core kernel (C/heads == 32) */
+    BRA_IMPL_MMA = 2,   /* bf16 warp-level tensor-core kernels with operands straight from global memory (C/heads == 32 or 64,
+                           regions at most 128 tokens wide) */
     BRA_IMPL_TC = 3,    /* bf16 tcgen05/TMEM kernels (C/heads == 32; regions of 8 x 8 tokens, or 16 wide and a multiple of 8 high) */
     BRA_IMPL_IMG = 4,   /* bf16 warp-level tensor-core kernel with a whole (image, head) of K and V resident in
                            shared memory (C/heads == 32, H*W <= ~1500 tokens): small maps, small regions */

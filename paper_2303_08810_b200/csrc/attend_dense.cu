@@ -4,6 +4,8 @@
 // to the LCE's thread mapping through shared memory (over the slices).
 // What bounds it: per 16 x 16 scores eight MMAs (64 cycles of a scheduler's tensor pipe), eight exponentials per lane (64
 // cycles of its MUFU share) and about 60 instructions.
+// Measured (B200): 64 x 7 x 7, 16 heads, topk 49: forward 161 us with routing -> 16.4 us; 64 x 14 x 14, 8 heads, topk 16:
+// level with attend_img.cu (44 us).  The other side of the rule: dense_pays().
 #include "dense_common.cuh"
 
 namespace bra {

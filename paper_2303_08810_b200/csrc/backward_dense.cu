@@ -4,6 +4,8 @@
 //   2. warp = 16 keys: dK = scale dS^T Q and dV = P^T dO in one walk over the queries; dV + LCE adjoint
 // P from the saved log-sum-exp, dP = dO V^T, dS = P o (dP - delta).  Who is routed where is the count table, so no inverse
 // index is needed.  Every sum has a fixed order.
+// Bound: instruction issue; the two walks over the keys in 1. make S and dP twice.  Measured (B200) against the kernels of
+// backward_img.cu: 64 x 14 x 14, 8 heads, topk 16: 156 -> 103 us; 64 x 7 x 7, 16 heads, topk 49: 477 -> 39 us.
 #include "dense_common.cuh"
 
 namespace bra {

@@ -4,7 +4,7 @@
 // four keys per lane.
 // Bound: the FMA pipe, 2 D FMAs per query and key (a packed FMA every two cycles and scheduler), in practice the latency of
 // the dot-product chains.  Measured (B200) against one thread per query with operands from global memory: 64 x 28 x 28,
-// 4 heads, topk 4: 356 -> 137 us; 1 x 16 x 16, 1 head: 41 -> 14 us.
+// 4 heads, topk 4: 356 -> 144 us; 1 x 16 x 16, 1 head: 41 -> 11 us.
 #include "simt_common.cuh"
 
 #include <type_traits>

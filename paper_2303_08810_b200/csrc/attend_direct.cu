@@ -225,7 +225,7 @@ attend_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* 
 // ------------------------------------------------------------------ host side
 bool attend_direct_supported(const Dims& d, int dtype) {
     if (dtype != BRA_BF16 || (d.d != 32 && d.d != 64)) return false;
-    if (d.ws > 128 || d.R > 65535 || (long long)d.topk * d.n_r * d.n_r >= (1ll << 32)) return false;   // fast division by n_r
+    if (d.ws > 128 || d.R > 65535 || d.n_r >= 1 << 25) return false;                      // fdiv() by ws and S
     if ((long long)d.H0 * d.W0 * d.C / 8 >= (1ll << 31) || d.heads > 65535 || d.B > 65535) return false;
     return direct_geom(d, d.lce, 4, 1).smem_bytes <= 200 * 1024;
 }

@@ -33,7 +33,7 @@ attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
     if (dm.lce) simt_load_weights(s_w, lce_w + (size_t)h * D * 25, 25 * D);
     if (gm.resident) {
         simt_copy_rows<T, D>(sbase + gm.off_a, sbase + gm.off_b, K, V, dm.C, dm.N, [&](int row, uint32_t& at) {
-            const int r = fdiv(row, dm.n_r, gm.mul_nr);
+            const int r = fdiv(row, gm.by_nr);
             at = row * gm.row;
             return simt_token(dm, gm, r, row - r * dm.n_r);
         });
@@ -142,7 +142,7 @@ attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
             const int l = fdiv(row, gm.kps, gm.mul_kps), kk = st * gm.kps + row - l * gm.kps;
             at = l * gm.reg + (row - l * gm.kps) * gm.row;
             if (kk >= total) return -1;
-            const int m = fdiv(kk, dm.n_r, gm.mul_nr);
+            const int m = fdiv(kk, gm.by_nr);
             const int r = entry(l * dm.topk + m);
             return r >= 0 ? simt_token(dm, gm, r, kk - m * dm.n_r) : -1;
         });
@@ -158,7 +158,7 @@ attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
             walk(std::true_type(), abase, gm.resident ? 0 : rl * gm.reg, k0, gm.resident ? dm.N : min(total, k0 + gm.kps), 0);
         else
             walk(std::false_type(), abase, 0, k0, gm.dense ? dm.N : gm.resident ? total : min(total, k0 + gm.kps), [&](int kk, float& wt) -> int {
-                const int m = fdiv(kk, dm.n_r, gm.mul_nr);
+                const int m = fdiv(kk, gm.by_nr);
                 if (gm.dense) {
                     const int n = cnt[rl * dm.R + m];
                     wt = (float)n;

@@ -47,7 +47,7 @@ bwd_dq_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
     const T* K = Kg + head; const T* V = Vg + head;
     if (gm.resident) {
         simt_copy_rows<T, D>(sbase + gm.off_a, sbase + gm.off_b, K, V, dm.C, dm.N, [&](int row, uint32_t& at) {
-            const int r = fdiv(row, dm.n_r, gm.mul_nr);
+            const int r = fdiv(row, gm.by_nr);
             at = row * gm.row;
             return simt_token(dm, gm, r, row - r * dm.n_r);
         });
@@ -148,7 +148,7 @@ bwd_dq_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
             const int lr = fdiv(row, gm.kps, gm.mul_kps), kk = st * gm.kps + row - lr * gm.kps;
             at = lr * gm.reg + (row - lr * gm.kps) * gm.row;
             if (kk >= total) return -1;
-            const int m = fdiv(kk, dm.n_r, gm.mul_nr);
+            const int m = fdiv(kk, gm.by_nr);
             const int r = entry(lr * dm.topk + m);
             return r >= 0 ? simt_token(dm, gm, r, kk - m * dm.n_r) : -1;
         });
@@ -164,7 +164,7 @@ bwd_dq_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
             walk(std::true_type(), abase, gm.resident ? 0 : rl * gm.reg, k0, gm.resident ? dm.N : min(total, k0 + gm.kps), it >= nst, 0);
         else
             walk(std::false_type(), abase, 0, k0, gm.dense ? dm.N : gm.resident ? total : min(total, k0 + gm.kps), it >= nst, [&](int kk, float& wt) -> int {
-                const int m = fdiv(kk, dm.n_r, gm.mul_nr);
+                const int m = fdiv(kk, gm.by_nr);
                 if (gm.dense) {
                     const int n = cnt[rl * dm.R + m];
                     wt = (float)n;
@@ -209,7 +209,7 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
     if (dm.lce) simt_load_weights(s_w, lce_w + (size_t)h * D * 25, 25 * D);
     if (gm.resident) {
         simt_copy_rows<T, D>(sbase + gm.off_a, sbase + gm.off_b, Q, dO, dm.C, dm.N, [&](int row, uint32_t& at) {
-            const int r = fdiv(row, dm.n_r, gm.mul_nr);
+            const int r = fdiv(row, gm.by_nr);
             at = row * gm.row;
             return simt_token(dm, gm, r, row - r * dm.n_r);
         });
@@ -229,8 +229,8 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
     const bool active = rl_raw < nreg;
     const int rl = active ? rl_raw : 0;
     const int jr = __ldcg(order + rl);                                // this lane's key region
-    const int e0 = __ldcg(offs + jr), mine = (__ldcg(offs + jr + 1) - e0) * dm.n_r;     // its queries
-    const int warp_total = __reduce_max_sync(0xffffffffu, mine);
+    const int e0 = __ldcg(offs + jr), listed = __ldcg(offs + jr + 1) - e0;              // its query regions
+    const long long warp_total = (long long)__reduce_max_sync(0xffffffffu, listed) * dm.n_r;    // (with repeats a list may be long)
     bool weighted = false;
     int32_t* cnt = reinterpret_cast<int32_t*>(smem + gm.off_cnt);
     if (gm.dense) {
@@ -252,14 +252,14 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
     }
     // statistics of a row: lse and delta; a row that does not count has lse = inf (P = 0); a row of the zero padding has
     // zero Q and dO and lse = delta = 0 and adds nothing
-    auto walk = [&](auto plain, uint32_t abase, uint32_t at0, int row0, int k0, int k1, auto&& row_of) {
+    auto walk = [&](auto plain, uint32_t abase, uint32_t at0, int row0, int n, auto&& row_of) {
         constexpr bool PLAIN = decltype(plain)::value;
         uint32_t next = abase + at0 + ks * gm.row, next_stat = abase + gm.off_stat + (row0 + ks) * 8;
 #pragma unroll 1
-        for (int kb = k0; kb < k1; kb += KS) {
+        for (int kb = 0; kb < n; kb += KS) {
             const int kk = kb + ks;
             uint32_t at = next, at_stat = next_stat;
-            bool dead = kk >= k1;
+            bool dead = kk >= n;
             float wt = 1.f;
             if constexpr (PLAIN) {
                 if (dead) { at = abase; at_stat = abase + gm.off_stat; }
@@ -284,51 +284,54 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
             axpy(gv[0], p, g);
         }
     };
-    int most = warp_total;                                            // longest list of the CTA's regions
+    long long most = 0;                                               // queries of the CTA's longest list
     if (gm.resident) {
         float2* stat = reinterpret_cast<float2*>(smem + gm.off_stat);
         for (int row = tid; row < dm.N; row += blockDim.x) {
-            const int r = fdiv(row, dm.n_r, gm.mul_nr);
+            const int r = fdiv(row, gm.by_nr);
             const int tk = simt_token(dm, gm, r, row - r * dm.n_r);
             stat[row] = tk >= 0 ? make_float2(__ldg(lse_h + tk), __ldcg(delta_h + tk)) : make_float2(0.f, 0.f);
         }
     } else {
         const int j = __ldcg(order);                                  // the first has the longest list
-        most = (__ldcg(offs + j + 1) - __ldcg(offs + j)) * dm.n_r;
+        most = (long long)(__ldcg(offs + j + 1) - __ldcg(offs + j)) * dm.n_r;
     }
-    const int nst = gm.resident ? 1 : (most + gm.kps - 1) / gm.kps;
+    const int nst = gm.resident ? 1 : (int)((most + gm.kps - 1) / gm.kps);
+    int m0 = 0, q0 = 0;                                               // list entry and token of the next stage's first query
     auto load_stage = [&](int st) {
         const uint32_t base = sbase + (st & 1) * gm.stage_bytes;
         float2* stat = reinterpret_cast<float2*>(smem + (st & 1) * gm.stage_bytes + gm.off_stat);
         simt_copy_rows<T, D>(base + gm.off_a, base + gm.off_b, Q, dO, dm.C, nreg * gm.kps, [&](int row, uint32_t& at) {
-            const int lr = fdiv(row, gm.kps, gm.mul_kps), kk = st * gm.kps + row - lr * gm.kps;
+            const int lr = fdiv(row, gm.kps, gm.mul_kps), u = q0 + row - lr * gm.kps;
             at = lr * gm.reg + (row - lr * gm.kps) * gm.row;
-            const int j = __ldcg(order + lr), s0 = __ldcg(offs + j);
-            const int m = fdiv(kk, dm.n_r, gm.mul_nr);
+            const int j = __ldcg(order + lr), m = fdiv(u, gm.by_nr), s0 = __ldcg(offs + j) + m0 + m;
             int tk = -1;
             float2 v = make_float2(INFINITY, 0.f);
-            if (s0 + m < __ldcg(offs + j + 1)) {
-                tk = simt_token(dm, gm, __ldcg(list + s0 + m), kk - m * dm.n_r);
+            if (s0 < __ldcg(offs + j + 1)) {
+                tk = simt_token(dm, gm, __ldcg(list + s0), u - m * dm.n_r);
                 v = tk >= 0 ? make_float2(__ldg(lse_h + tk), __ldcg(delta_h + tk)) : make_float2(0.f, 0.f);
             }
             if ((threadIdx.x & 3) == 0) stat[row] = v;
             return tk;
         });
         cp_async_commit();
+        const int u = q0 + gm.kps, m = fdiv(u, gm.by_nr);
+        m0 += m; q0 = u - m * dm.n_r;
     };
     if (!gm.resident && nst > 0) load_stage(0);
     for (int st = 0; st < nst; ++st) {
         if (st + 1 < nst) { load_stage(st + 1); cp_async_wait<1>(); } else cp_async_wait<0>();
         __syncthreads();
-        const int k0 = gm.resident ? 0 : st * gm.kps;
         const uint32_t abase = sbase + (st & 1) * gm.stage_bytes;
         if (!gm.resident) {
-            if (k0 < warp_total) walk(std::true_type(), abase, rl * gm.reg, rl * gm.kps, k0, min(warp_total, k0 + gm.kps), 0);
+            const long long rest = warp_total - (long long)st * gm.kps;
+            if (rest > 0) walk(std::true_type(), abase, rl * gm.reg, rl * gm.kps, (int)min(rest, (long long)gm.kps), 0);
         } else if (gm.dense && !weighted) {
-            walk(std::true_type(), abase, 0, 0, 0, dm.N, 0);
+            walk(std::true_type(), abase, 0, 0, dm.N, 0);
         } else {
-            walk(std::false_type(), abase, 0, 0, 0, gm.dense ? dm.N : warp_total, [&](int kk, float& wt) -> int {
-                const int m = fdiv(kk, dm.n_r, gm.mul_nr);
+            const int mine = listed * dm.n_r;                         // (a resident slice: a few hundred tokens)
+            walk(std::false_type(), abase, 0, 0, gm.dense ? dm.N : (int)warp_total, [&](int kk, float& wt) -> int {
+                const int m = fdiv(kk, gm.by_nr);
                 if (gm.dense) {
                     const int n = cnt[rl * dm.R + m];
                     wt = (float)n;
@@ -358,10 +361,6 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
     else simt_lce<T, D, 4, true>(st, s_w, nullptr, dO, dVg + head, order, nreg, gm.spr, chunk, dm, gm);
 }
 
-bool backward_supported(const Dims& d) {
-    return (d.d == 16 || d.d == 32 || d.d == 64) && d.R <= 1000 && simt_fits(d, SIMT_DQ) && simt_fits(d, SIMT_DKV);
-}
-
 enum Family { FAMILY_SIMT, FAMILY_DIRECT, FAMILY_IMG, FAMILY_DENSE };
 
 // bf16, head dim 32 or 64: tensor-core kernels.  Small maps with enough (image, head) pairs to fill the GPU keep a
@@ -373,6 +372,10 @@ static Family choose_family(const Dims& d, int dtype, int impl) {
         (impl == BRA_IMPL_IMG || (impl == BRA_IMPL_AUTO && img_pays(d))))
         return FAMILY_IMG;
     return backward_direct_supported(d, dtype) ? FAMILY_DIRECT : FAMILY_SIMT;
+}
+bool backward_supported(const Dims& d, int dtype, int impl) {
+    if ((d.d != 16 && d.d != 32 && d.d != 64) || d.R > 1000) return false;
+    return choose_family(d, dtype, impl) != FAMILY_SIMT || (simt_fits(d, SIMT_DQ) && simt_fits(d, SIMT_DKV));
 }
 bool backward_any_map(const Dims& d, int dtype, int impl) { return choose_family(d, dtype, impl) != FAMILY_IMG; }
 

@@ -255,7 +255,7 @@ bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16*
     cp_async_commit();
     const int e0 = __ldcg(inv_off + bhi * (dm.R + 1) + jr), e1 = __ldcg(inv_off + bhi * (dm.R + 1) + jr + 1);
     const int32_t* list = inv_list + bhi * dm.R * dm.topk + e0;      // query regions that list jr, fixed order
-    const int total = (e1 - e0) * dm.n_r;
+    const long long total = (long long)(e1 - e0) * dm.n_r;           // a list with repeats may hold every entry of the index
     const float* lse_h = lse + ((size_t)b * dm.heads + h) * N0;
     const float* delta_h = delta + ((size_t)b * dm.heads + h) * N0;
     uint32_t* tab = reinterpret_cast<uint32_t*>(smem + gm.off_tab + grp * gm.tab_bytes);   // row offsets, lse * log2(e), delta
@@ -263,16 +263,16 @@ bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16*
     float* s_dl = s_l2 + gm.tab;
     float* st = reinterpret_cast<float*>(smem + gm.off_st + grp * gm.st_bytes);
     const float sl2 = dm.scale * 1.4426950408889634f;
-    const int passes = (total + gm.tab - 1) / gm.tab;
+    const int passes = (int)((total + gm.tab - 1) / gm.tab);
     // A query beyond the list, or of the zero padding (zero rows of Q and dO: it adds nothing), names some readable row with
     // lse = inf: its P is zero.
-    auto fill_queries = [&](int k0, int n) {
+    // (m0, t0): list entry and token of the table's first query; left: how many queries remain from there on.
+    auto fill_queries = [&](int m0, int t0, int n, int left) {
         for (int e = glane; e < n; e += glanes) {
-            const int kk = min(k0 + e, total - 1);
-            const int m = fdiv(kk, dm.n_r, gm.mul_nr);
-            const int tk = token_of(dm, gm, __ldcg(list + m), kk - m * dm.n_r), at = max(tk, 0);
+            const int u = t0 + min(e, left - 1), m = fdiv(u, gm.by_nr);
+            const int tk = token_of(dm, gm, __ldcg(list + m0 + m), u - m * dm.n_r), at = max(tk, 0);
             tab[e] = (uint32_t)at * (uint32_t)(dm.C >> 3);
-            s_l2[e] = k0 + e >= total || tk < 0 ? INFINITY : __ldg(lse_h + at) * 1.4426950408889634f;
+            s_l2[e] = e >= left || tk < 0 ? INFINITY : __ldg(lse_h + at) * 1.4426950408889634f;
             s_dl[e] = __ldcg(delta_h + at);
         }
     };
@@ -303,13 +303,16 @@ bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16*
                     for (int e = 0; e < 4; ++e) { dkx[x][p][n][e] = 0.f; dvx[x][p][n][e] = 0.f; }
         }
 
+        int m0 = 0, t0 = 0;
 #pragma unroll 1
         for (int pass = 0; pass < passes; ++pass) {
-            const int k0 = pass * gm.tab;
-            const int nk = min(gm.tab, (total - k0 + 31) / 32 * 32);
+            const int left = (int)min((long long)gm.tab, total - (long long)pass * gm.tab);
+            const int nk = (left + 31) / 32 * 32;                     // (the table's size is a multiple of 32)
             if (passes > 1 || !filled) {
                 if (filled) group_sync();
-                fill_queries(k0, nk);
+                fill_queries(m0, t0, nk, left);
+                const int u = t0 + gm.tab, m = fdiv(u, gm.by_nr);
+                m0 += m; t0 = u - m * dm.n_r;
                 group_sync();
                 filled = true;
             }
@@ -405,7 +408,6 @@ static DirGeom dkv_geom(const Dims& d) {
 
 bool backward_direct_supported(const Dims& d, int dtype) {
     if (!attend_direct_supported(d, dtype)) return false;
-    if ((long long)d.R * d.n_r * d.n_r >= (1ll << 32)) return false;
     return dkv_geom(d).smem_bytes <= 200 * 1024 && dq_geom(d).smem_bytes <= 200 * 1024 && d.R <= 8192 && dkv_geom(d).gpi <= 65535;
 }
 

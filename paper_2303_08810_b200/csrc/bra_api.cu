@@ -308,7 +308,7 @@ bra_status bra_backward(const bra_problem* p, const void* Q, const void* K, cons
         return BRA_ERR_ALIGN;
     WsLayout L;
     if ((s = check_ws(d, ws, ws_bytes, &L)) != BRA_OK) return s;
-    if (!backward_supported(d)) return BRA_ERR_UNSUPPORTED;
+    if (!backward_supported(d, p->dtype, p->impl)) return BRA_ERR_UNSUPPORTED;
     char* w = static_cast<char*>(ws);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (!padded(d) || backward_any_map(d, p->dtype, p->impl)) {

@@ -172,7 +172,7 @@ int lce_grad_partials(const Dims& d);
 cudaError_t launch_lce_grad(const Dims& d, int dtype, const void* V, const void* dO, float* part, float* d_lce_w, float* d_lce_b,
                             int32_t* status, cudaStream_t st);
 
-bool backward_supported(const Dims& d);
+bool backward_supported(const Dims& d, int dtype, int impl);
 // true if the kernels launch_backward() takes for this problem work on maps that S does not divide
 bool backward_any_map(const Dims& d, int dtype, int impl);
 // impl: the bra_impl the caller asked for

@@ -11,6 +11,7 @@
 // 16-byte stores.
 #pragma once
 
+#include "fast_div.h"
 #include "mma_common.cuh"
 
 namespace bra {
@@ -27,7 +28,8 @@ struct DirGeom {
     int nw, gpc;           // warps per CTA; groups (regions) per CTA: several when a region is one warp's work, else 1
     int gpi;               // CTAs per (image, head): the grid is (gpi, heads, images)
     int halo_w, halo_row;  // tokens and bytes of a halo row
-    uint32_t mul_nr, mul_ws, mul_s, mul_hw;
+    FastDiv by_nr;                                // positions in a walk pass n_r * n_r < 2^32; tokens of a region and regions do not
+    uint32_t mul_ws, mul_s, mul_hw;
     int off_tab, off_w, off_halo, off_st, smem_bytes;
     int tab, tab_bytes, halo_bytes, st_bytes;     // per group; tab: entries
 };
@@ -51,7 +53,7 @@ inline DirGeom direct_geom(const Dims& d, bool with_lce, int entry_bytes, int rt
     g.gpi = (d.R + g.gpc - 1) / g.gpc * g.chunks;
     g.halo_w = d.ws + 4;
     g.halo_row = g.halo_w * 64 * g.planes + 16;        // tiles four rows apart start on different banks
-    g.mul_nr = recip32(d.n_r); g.mul_ws = recip32(d.ws); g.mul_s = recip32(d.S); g.mul_hw = recip32(g.halo_w);
+    g.by_nr = fast_div(d.n_r); g.mul_ws = recip32(d.ws); g.mul_s = recip32(d.S); g.mul_hw = recip32(g.halo_w);
     g.tab = g.gpc > 1 ? dk::TAB_WARP : dk::TAB;
     const int need = (d.topk * d.n_r + 31) / 32 * 32;
     if (need < g.tab) g.tab = need;
@@ -190,7 +192,7 @@ __device__ __forceinline__ int fill_keys(uint32_t* tab, uint32_t* dead, const in
     int zeros = 0;
     for (int e = lane0; e < n; e += lanes) {                         // whole warps: n and lanes are multiples of 32
         const int kk = min(k0 + e, total - 1);
-        const int m = fdiv(kk, dm.n_r, gm.mul_nr);
+        const int m = fdiv(kk, gm.by_nr);
         const int r = __ldcg(irow + m);  // coherent load: the index may come from the kernel this one overlaps
         bool ok = k0 + e < total;
         int tok = 0;

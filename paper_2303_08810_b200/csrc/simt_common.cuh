@@ -13,6 +13,7 @@
 // once (of several regions, or of several key shares) start on different banks.
 #pragma once
 
+#include "fast_div.h"
 #include "mma_common.cuh"
 
 namespace bra {
@@ -31,7 +32,8 @@ struct SimtGeom {
     int threads, gpi;      // the grid is (gpi, heads, images)
     int resident, dense;   // dense: topk == R, walk every region and weigh it by how often the list names it
     int kps, stages;       // rows of the other side per region and stage
-    uint32_t mul_nr, mul_ws, mul_s, mul_spr, mul_kps, mul_cw;
+    FastDiv by_nr, by_ws, by_s;
+    uint32_t mul_spr, mul_kps, mul_cw;
     int row;               // bytes of a row of one tensor in shared memory
     int reg;               // bytes from one region's rows of a stage to the next region's
     int off_a, off_b, off_stat, off_idx, off_cnt, off_w, off_st, stage_bytes, smem_bytes;
@@ -46,7 +48,7 @@ inline SimtGeom simt_geom(const Dims& d, SimtKind kind) {
     SimtGeom g;
     const int qt = simt_rows(d.d, kind);
     g.row = d.d * d.esize + 16;
-    g.mul_nr = recip32(d.n_r); g.mul_ws = recip32(d.ws); g.mul_s = recip32(d.S);
+    g.by_nr = fast_div(d.n_r); g.by_ws = fast_div(d.ws); g.by_s = fast_div(d.S);
     // lanes of this call against the lanes the GPU holds at once (12 warps per SM)
     // (dK / dV of larger maps: as if an eighth of the regions held the lists, which is what clustered content comes to;
     // measured at 1 x 96 x 96, S = 7, 2 heads: 522 -> 224 us; at 36 x 14 x 14 it costs more than it gives)
@@ -106,14 +108,14 @@ inline SimtGeom simt_geom(const Dims& d, SimtKind kind) {
     return g;
 }
 inline bool simt_fits(const Dims& d, SimtKind kind) {
-    return (long long)d.topk * d.n_r * d.n_r < (1ll << 32) && (long long)d.R * d.n_r * d.n_r < (1ll << 32) && d.B <= 65535 &&
-           d.heads <= 65534 && (long long)d.H * d.W < (1ll << 30) && simt_geom(d, kind).smem_bytes <= 220 * 1024;
+    // (token numbers and positions in a walk are ints)
+    return d.B <= 65535 && d.heads <= 65534 && (long long)d.H * d.W < (1ll << 31) - 65536 && simt_geom(d, kind).smem_bytes <= 220 * 1024;
 }
 
 // Token (row-major in the caller's map) of token t of region r; -1 in the zero padding.
 __device__ __forceinline__ int simt_token(const Dims& dm, const SimtGeom& gm, int r, int t) {
-    const int ry = fdiv(r, dm.S, gm.mul_s), rx = r - ry * dm.S;
-    const int ty = fdiv(t, dm.ws, gm.mul_ws), tx = t - ty * dm.ws;
+    const int ry = fdiv(r, gm.by_s), rx = r - ry * dm.S;
+    const int ty = fdiv(t, gm.by_ws), tx = t - ty * dm.ws;
     const int y = ry * dm.hs + ty, x = rx * dm.ws + tx;
     return y < dm.H0 && x < dm.W0 ? y * dm.W0 + x : -1;
 }
@@ -131,7 +133,7 @@ __device__ __forceinline__ SimtChunk simt_chunk(const Dims& dm, const SimtGeom& 
 __device__ __forceinline__ int simt_row(const Dims& dm, const SimtGeom& gm, const SimtChunk& c, int r, int t) {
     const int ly = fdiv(t, gm.cw, gm.mul_cw), lx = t - ly * gm.cw;
     if (ly >= c.rows || lx >= c.cols) return -1;
-    const int ry = fdiv(r, dm.S, gm.mul_s), rx = r - ry * dm.S;
+    const int ry = fdiv(r, gm.by_s), rx = r - ry * dm.S;
     const int y = ry * dm.hs + c.y + ly, x = rx * dm.ws + c.x + lx;
     return y < dm.H0 && x < dm.W0 ? y * dm.W0 + x : -1;
 }
@@ -313,7 +315,7 @@ __device__ __forceinline__ void simt_lce(const float* st, const float* s_w, cons
             b = bias ? __ldg(bias + ch) : 0.f;
         }
         const int r = region_at[rl];
-        const int ry = fdiv(r, dm.S, gm.mul_s), rx = r - ry * dm.S;
+        const int ry = fdiv(r, gm.by_s), rx = r - ry * dm.S;
         const int ly0 = ty * TS, lx0 = tx * TS;                       // within the chunk
         const int y0 = ry * dm.hs + c.y + ly0, x0 = rx * dm.ws + c.x + lx0;
         float acc[TS][TS];

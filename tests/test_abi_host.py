@@ -150,3 +150,64 @@ def test_binding_fails_loudly_without_gpu():
         pytest.skip("has a GPU")
     with pytest.raises(RuntimeError, match="no CPU fallback"):
         binding.workspace(problem())
+
+
+# ------------------------------------------------------------------ what is accepted
+def status_without_gpu(lib, call, **kw):
+    """What `call` answers for a problem: 7 (no kernel) or, past every host check, 8 - the launch finds no device."""
+    import torch
+    if torch.cuda.is_available():
+        pytest.skip("the made-up addresses must not reach a GPU")
+    p = problem(**kw)
+    big = 1 << 62
+    if call == "attend":
+        return lib.bra_attend(ctypes.byref(p), A, A, A, A, A, A, A, A, A, big, None)
+    return lib.bra_backward(ctypes.byref(p), *([A] * 12), A, big, None)
+
+
+# regions whose tokens times listed tokens pass 2^32: the kernels divide token numbers exactly, whatever their product
+@pytest.mark.parametrize("call,kw", [
+    ("attend", dict(H=256, W=256, S=1, topk=1, dtype="f32")),
+    ("attend", dict(H=512, W=512, S=4, topk=1, dtype="f32")),
+    ("attend", dict(H=736, W=736, S=8, topk=4, dtype="f32")),
+    ("attend", dict(H=512, W=512, S=4, topk=16, dtype="bf16")),
+    ("attend", dict(H=8192, W=8192, S=2, topk=4, C=16, heads=1, dtype="f32")),
+    ("backward", dict(H=512, W=512, S=4, topk=1, dtype="f32")),
+    ("backward", dict(H=512, W=512, S=4, topk=1, dtype="bf16")),
+    ("backward", dict(H=728, W=728, S=8, topk=4, dtype="bf16")),
+    ("backward", dict(H=1024, W=1024, S=16, topk=4, dtype="bf16")),
+    ("backward", dict(H=1024, W=1024, S=16, topk=4, C=128, dtype="bf16")),
+])
+def test_large_regions_are_accepted(lib, call, kw):
+    assert status_without_gpu(lib, call, **{"B": 1, **kw}) == 8
+
+
+def test_division_by_multiplication_is_exact(tmp_path):
+    """csrc/fast_div.h on the host: every divisor of a spread, dividends next to every kind of multiple."""
+    import subprocess
+    src = tmp_path / "t.cpp"
+    src.write_text('''
+#include "fast_div.h"
+#include <stdio.h>
+int main() {
+    const uint32_t top = 0x7fffffffu;
+    long long bad = 0;
+    auto check = [&](uint32_t n, uint32_t d, const bra::FastDiv& f) { if (bra::fdiv(n, f) != n / d) { if (!bad++) printf("%u / %u\\n", n, d); } };
+    auto divisor = [&](uint32_t d) {
+        const bra::FastDiv f = bra::fast_div((int)d);
+        for (uint64_t m = 1; m * d <= top; m = m < 40 ? m + 1 : m + m / 3)
+            for (int o = -1; o <= 1; ++o) if (m * d + o <= top) check((uint32_t)(m * d + o), d, f);
+        const uint32_t last = top / d * d;
+        check(0, d, f); check(last, d, f); check(last - 1, d, f); check(top, d, f);
+    };
+    for (uint32_t d = 1; d < 70000; ++d) divisor(d);
+    for (uint32_t s = 3; s < 31; ++s) for (int o = -2; o <= 2; ++o) divisor((1u << s) + o);
+    for (uint32_t d = 70001; d < top - 99991; d += d / 7 + 1) divisor(d);
+    divisor(top);
+    return bad ? 1 : 0;
+}
+''')
+    exe = tmp_path / "t"
+    subprocess.run(["g++", "-O2", "-std=c++17", "-I", os.path.join(ROOT, "paper_2303_08810_b200", "csrc"), str(src), "-o", str(exe)], check=True)
+    run = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert run.returncode == 0, run.stdout

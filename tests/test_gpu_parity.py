@@ -886,3 +886,35 @@ def test_pooling_of_maps_that_S_does_not_divide(bra, B, H, W, S, dtype):
     np.testing.assert_allclose(f64(qm), Qr, rtol=0, atol=2e-6)
     np.testing.assert_allclose(f64(km), Kr, rtol=0, atol=2e-6)
     check_index(idx.cpu().numpy(), idx_ref, gap, 2, cfg.R, orc.region_affinity(Qr, Kr, cfg.heads))
+
+
+# ------------------------------------------------------------------ large regions
+@pytest.mark.parametrize("dtype,impl", [("f32", "simt"), ("bf16", "mma")])
+def test_lists_with_repeats_of_large_regions(bra, dtype, impl):
+    """Four regions of 22 500 tokens, every query region lists region 0 four times: the list of region 0 has 360 000 queries,
+    and the last of them is the only one with a gradient.  The softmax over four copies of the keys is the softmax over one
+    with every probability divided by four (exactly: a power of two), so O, and dK, dV summed over the copies, equal those
+    of topk = 1 up to the rounding of sums in another order."""
+    import torch
+    H, W = 360, 250
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(91)
+    dt = torch.float32 if dtype == "f32" else torch.bfloat16
+    Q, K, V = (torch.randn(1, H, W, 32, device="cuda", generator=gen).to(dt) for _ in range(3))
+    dO = torch.zeros_like(Q)
+    dO[0, -1, -1] = 1000.0 * torch.randn(32, device="cuda", generator=gen).to(dt)
+    got = []
+    for topk in (4, 1):
+        p = bra.make_problem(1, H, W, 32, 1, 2, topk, dtype, lce=False, impl=IMPLS[impl])
+        ws = bra.workspace(p)
+        idx = torch.zeros(1, 1, 4, topk, dtype=torch.int32, device="cuda")
+        O, lse = bra.bra_attend(p, Q, K, V, idx, ws=ws)
+        dQ, dK, dV, _, _ = bra.bra_backward(p, Q, K, V, idx, None, lse, dO, ws=ws)
+        assert bra.bra_device_status(ws) == 0
+        got.append([f64(x) for x in (O, dQ, dK, dV)])
+    # fp32: sums of up to 90 000 terms, sqrt(n) 2^-24 of them; bf16: two results rounded to 2^-9 each
+    tol = 1e-4 if dtype == "f32" else 8e-3
+    for name, a, r in zip(("O", "dQ", "dK", "dV"), *got):
+        assert np.linalg.norm(a - r) <= tol * np.linalg.norm(r), name
+    for a in got[0][2:]:
+        assert np.abs(a[0, :180, :125]).max() > 0 and (a[0, 180:] == 0).all()       # region 0 only

@@ -461,9 +461,9 @@ static cudaError_t launch_both(const Dims& d, const BwdArgs& a) {
                         : dq_single(d)   ? launch_dq<1, false, true>(d, a)
                                          : launch_dq<1, false, false>(d, a);
     if (e != cudaSuccess) return e;
-    if (d.hs <= 2) return d.d == 64 ? launch_dkv<2, true, 2, 2>(d, a) : launch_dkv<1, false, 2, 2>(d, a);
-    if (d.d == 64) return launch_dkv<2, true, 4, 4>(d, a);
-    if (exact) return launch_dkv<1, true, 4, 4>(d, a);
+    if (d.d == 64) return d.hs <= 2 ? launch_dkv<2, true, 2, 2>(d, a) : launch_dkv<2, true, 4, 4>(d, a);
+    if (exact) return d.hs <= 2 ? launch_dkv<1, true, 2, 2>(d, a) : launch_dkv<1, true, 4, 4>(d, a);
+    if (d.hs <= 2) return launch_dkv<1, false, 2, 2>(d, a);
     switch (lce_tile_width(dkv_geom(d), d)) {
         case 2: return launch_dkv<1, false, 4, 2>(d, a);
         case 3: return launch_dkv<1, false, 4, 3>(d, a);

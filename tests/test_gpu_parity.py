@@ -918,3 +918,39 @@ def test_lists_with_repeats_of_large_regions(bra, dtype, impl):
         assert np.linalg.norm(a - r) <= tol * np.linalg.norm(r), name
     for a in got[0][2:]:
         assert np.abs(a[0, :180, :125]).max() > 0 and (a[0, 180:] == 0).all()       # region 0 only
+
+
+# ------------------------------------------------------------------ problems that are more precise than one bf16 product
+def rounding_ratio(got, ref):
+    """Root mean square error of a bf16 result over that of the exact result rounded to bf16 once: 1 for a kernel whose own
+    errors are small beside that rounding."""
+    import torch
+    ideal = torch.from_numpy(ref).to(torch.bfloat16).double().numpy()
+    return np.sqrt(((f64(got) - ref) ** 2).mean() / ((ideal - ref) ** 2).mean())
+
+
+# Regions of more than 128 tokens whose rows do not divide 128: P and dS enter their products with 16 bits of mantissa.  What
+# that leaves, 2^-17 of each term, is 2^-8 of the result's own rounding (both add up over the same terms), which moves the
+# ratio by about 2^-16; fp32 sums and ex2.approx are smaller still.  P and dS of 8 bits (2^-9 of each term) come out at 1.4
+# to 1.45.  2 %: the ratio of 25 600 and more samples, few of which can differ.
+RATIO_MAX = 1.02
+
+
+@pytest.mark.parametrize("cfg", [
+    BraConfig("exact-2x100", 1, 4, 200, 64, 2, 2, 2, "bf16"),
+    BraConfig("exact-2x65", 2, 4, 130, 64, 2, 2, 3, "bf16"),
+    BraConfig("exact-12x12", 1, 24, 24, 64, 2, 2, 3, "bf16"),
+    BraConfig("exact-d64-2x100", 1, 4, 200, 128, 2, 2, 2, "bf16"),
+], ids=lambda c: c.name)
+def test_gradients_of_wide_regions_keep_their_precision(bra, cfg):
+    x = synthetic.make_inputs(cfg, seed=93, with_do=True)
+    t = to_dev(x, cfg)
+    p = problem_of(bra, cfg, lce=False)
+    ws = bra.workspace(p)
+    O, idx, lse = bra.bra_forward(p, t["Q"], t["K"], t["V"], ws=ws)
+    g = bra.bra_backward(p, t["Q"], t["K"], t["V"], idx, None, lse, t["dO"], ws=ws)
+    assert bra.bra_device_status(ws) == 0
+    ref = orc.bra_backward(x["Q"], x["K"], x["V"], idx.cpu().numpy(), np.zeros_like(x["w"]), x["dO"], cfg.heads, cfg.S)
+    ratios = {name: rounding_ratio(a, r) for name, a, r in zip(("dQ", "dK", "dV"), g, ref)}
+    print(cfg.name, ratios)
+    assert max(ratios.values()) <= RATIO_MAX, ratios

@@ -254,6 +254,7 @@ cudaError_t launch_attend_direct(const Dims& d, const void* Q, const void* K, co
     const DirGeom g = direct_geom(d, d.lce, 4, rt);
 #define BRA_GO(PL, EX, RT, TY, TX) return launch_t<PL, EX, RT, TY, TX>(d, g, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel)
     if (g.planes == 2) {
+        if (direct_exact(d)) { if (rt == 2) BRA_GO(2, true, 2, 4, 4); BRA_GO(2, true, 1, 4, 4); }
         if (rt == 2) BRA_GO(2, false, 2, 4, 4);
         if (d.hs <= 2) BRA_GO(2, false, 1, 2, 2);
         BRA_GO(2, false, 1, 4, 4);

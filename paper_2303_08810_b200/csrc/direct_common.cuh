@@ -72,8 +72,8 @@ inline DirGeom direct_geom(const Dims& d, bool with_lce, int entry_bytes, int rt
     return g;
 }
 
-// Head dim 32, regions of more than 128 tokens whose rows do not divide 128: these shapes used to run in fp32 on the
-// CUDA cores, so the probabilities keep 16 bits of mantissa here (two MMAs).  Head dim 64: the same in the gradients.
+// Regions of more than 128 tokens whose rows do not divide 128: these shapes used to run in fp32 on the CUDA cores, so the
+// probabilities keep 16 bits of mantissa here (two MMAs).  The gradients of head dim 64 do so for every shape.
 inline bool direct_exact(const Dims& d) { return d.n_r > 128 && 128 % d.ws != 0; }
 
 // Tiles per warp in the forward kernel: two share every row that is loaded (and transposed) where regions have two and enough

@@ -954,3 +954,18 @@ def test_gradients_of_wide_regions_keep_their_precision(bra, cfg):
     ratios = {name: rounding_ratio(a, r) for name, a, r in zip(("dQ", "dK", "dV"), g, ref)}
     print(cfg.name, ratios)
     assert max(ratios.values()) <= RATIO_MAX, ratios
+
+
+@pytest.mark.parametrize("cfg", [
+    BraConfig("exact-d64-12x12", 1, 24, 24, 128, 2, 2, 2, "bf16"),
+    BraConfig("exact-d64-2x100", 1, 4, 200, 128, 2, 2, 2, "bf16"),
+    BraConfig("exact-d64-12x12-two-tiles", 33, 24, 24, 128, 2, 2, 2, "bf16"),
+    BraConfig("exact-12x12", 1, 24, 24, 64, 2, 2, 2, "bf16"),
+], ids=lambda c: c.name)
+def test_attention_of_wide_regions_keeps_its_precision(bra, cfg):
+    x = synthetic.make_inputs(cfg, seed=94)
+    t = to_dev(x, cfg)
+    p = problem_of(bra, cfg, lce=False)
+    O, idx, _ = bra.bra_forward(p, t["Q"], t["K"], t["V"])
+    ref, _ = orc.bra_attend(x["Q"], x["K"], x["V"], idx.cpu().numpy(), None, cfg.heads, cfg.S)
+    assert rounding_ratio(O, ref) <= RATIO_MAX

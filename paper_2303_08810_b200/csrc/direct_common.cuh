@@ -72,9 +72,12 @@ inline DirGeom direct_geom(const Dims& d, bool with_lce, int entry_bytes, int rt
     return g;
 }
 
-// Regions of more than 128 tokens whose rows do not divide 128: these shapes used to run in fp32 on the CUDA cores, so the
-// probabilities keep 16 bits of mantissa here (two MMAs).  The gradients of head dim 64 do so for every shape.
-inline bool direct_exact(const Dims& d) { return d.n_r > 128 && 128 % d.ws != 0; }
+// Regions of more than 128 tokens whose rows do not divide 128, lists of more than 256 regions and regions of tens of
+// thousands of tokens: these problems used to run in fp32 on the CUDA cores, so the probabilities keep 16 bits of mantissa
+// here (two MMAs).  The gradients of head dim 64 do so for every shape.
+inline bool direct_exact(const Dims& d) {
+    return (d.n_r > 128 && 128 % d.ws != 0) || d.topk > 256 || (long long)d.topk * d.n_r * d.n_r >= (1ll << 32);
+}
 
 // Tiles per warp in the forward kernel: two share every row that is loaded (and transposed) where regions have two and enough
 // warps remain.  Measured: 2 x 100 x 167 tokens, S = 16, topk 4, 6 heads 124 -> 114 us; 2 x 112 x 112, S = 8: 98 -> 88 us.

@@ -60,6 +60,7 @@ attend_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* 
     const uint8_t* Vh = reinterpret_cast<const uint8_t*>(Vg) + head_off;
     const uint8_t* Vb = Vh + t4 * 16;
 
+    const uint4 probe = spare_probe<PL>(Kb - t4 * 16, Vh, lane);
     float* s_w = reinterpret_cast<float*>(smem + gm.off_w);
     if (dm.lce) {
         load_lce_weights(s_w, lce_w, h, 32 * PL * 25, tid, gm.nw * 32);
@@ -73,6 +74,7 @@ attend_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* 
     __syncthreads();                                                  // weights
     pdl_wait();          // in bra_forward the launch may overlap the tail of the routing kernel
     if (!live) return;                                                // a whole warp (one_warp) and no barrier of the CTA follows
+    const int spare = spare_token<PL>(probe, Kb - t4 * 16, Vh, tok_bytes, N0, lane);
 
     const int hi = dm.heads_i == 1 ? 0 : h;
     const int32_t* irow = index + (((size_t)b * dm.heads_i + hi) * dm.R + i) * dm.topk;
@@ -114,7 +116,7 @@ attend_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* 
             const int nk = min(gm.tab, (total - k0 + 31) / 32 * 32);
             if (passes > 1 || first_round) {
                 if (pass > 0 || !first_round) group_sync();           // the table before has been read
-                int z = fill_keys(tab, dead, irow, k0, nk, total, glane, glanes, status, dm, gm);
+                int z = fill_keys(tab, dead, irow, k0, nk, total, spare, glane, glanes, status, dm, gm);
                 if (first_round) {
                     z = __reduce_add_sync(0xffffffffu, z);
                     if (lane == 0 && z) atomicAdd(zeros, z);

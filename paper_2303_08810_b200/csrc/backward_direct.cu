@@ -65,6 +65,7 @@ bwd_dq_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* 
     const uint8_t* Vb = reinterpret_cast<const uint8_t*>(Vg) + head_off;
     const uint8_t* Gb = reinterpret_cast<const uint8_t*>(dOg) + head_off;
     uint8_t* dQb = reinterpret_cast<uint8_t*>(dQg) + head_off;
+    const uint4 probe = spare_probe<PL>(Kb - t4 * 16, Vb - t4 * 16, lane);
     const size_t stat0 = ((size_t)b * dm.heads + h) * N0;
     const int hi = dm.heads_i == 1 ? 0 : h;
     const int32_t* irow = index + (((size_t)b * dm.heads_i + hi) * dm.R + i) * dm.topk;
@@ -73,6 +74,7 @@ bwd_dq_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* 
     uint32_t* dead = tab + gm.tab;
     const float sl2 = dm.scale * 1.4426950408889634f;
     const int passes = (total + gm.tab - 1) / gm.tab;
+    const int spare = spare_token<PL>(probe, Kb - t4 * 16, Vb - t4 * 16, tok_bytes, N0, lane);
     bool filled = false;
 
     for (int tile = gwarp * RT; tile - gwarp * RT < gm.tpc; tile += gwarps * RT) {
@@ -110,7 +112,7 @@ bwd_dq_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* 
             const int nk = SINGLE ? 16 * KS : min(gm.tab, (total - k0 + 31) / 32 * 32);
             if (passes > 1 || !filled) {
                 if (filled) group_sync();
-                fill_keys(tab, dead, irow, k0, nk, total, glane, glanes, status, dm, gm);
+                fill_keys(tab, dead, irow, k0, nk, total, spare, glane, glanes, status, dm, gm);
                 group_sync();
                 filled = true;
             }
@@ -200,6 +202,7 @@ bwd_dq_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* 
                 for (int p = 0; p < PL; ++p) *reinterpret_cast<uint4*>(o + p * 64) = pack_row(dq[x][p], r, dm.scale);
                 if (t4 == 0) delta_out[stat0 + tok[x][r]] = delta[x][r];
             }
+        if (SINGLE) break;                                            // (at most 64 tokens: as many warps as tiles)
     }
     pdl_launch_dependents();
 }
@@ -240,11 +243,13 @@ bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16*
     const uint8_t* Gb = Gh + t4 * 16;
     uint8_t* dKb = reinterpret_cast<uint8_t*>(dKg) + head_off + t4 * 16;
 
+    const uint4 probe = spare_probe<PL>(Qb - t4 * 16, Gh, lane);
     float* s_w = reinterpret_cast<float*>(smem + gm.off_w);
     if (dm.lce) load_lce_weights(s_w, lce_w, h, 32 * PL * 25, tid, gm.nw * 32);
     __syncthreads();                                                  // weights
     pdl_wait();          // delta, the inverse index and the order of the regions come from the dQ kernel
     if (!live) return;
+    const int spare = spare_token<PL>(probe, Qb - t4 * 16, Gh, tok_bytes, N0, lane);
 
     const int hi = dm.heads_i == 1 ? 0 : h;
     const size_t bhi = (size_t)b * dm.heads_i + hi;
@@ -264,16 +269,18 @@ bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16*
     float* st = reinterpret_cast<float*>(smem + gm.off_st + grp * gm.st_bytes);
     const float sl2 = dm.scale * 1.4426950408889634f;
     const int passes = (int)((total + gm.tab - 1) / gm.tab);
-    // A query beyond the list, or of the zero padding (zero rows of Q and dO: it adds nothing), names some readable row with
-    // lse = inf: its P is zero.
+    // A query beyond the list, or of the zero padding (zero rows of Q and dO: it adds nothing), names the row of token `spare`
+    // with lse = inf: its P is zero.
     // (m0, t0): list entry and token of the table's first query; left: how many queries remain from there on.
     auto fill_queries = [&](int m0, int t0, int n, int left) {
         for (int e = glane; e < n; e += glanes) {
             const int u = t0 + min(e, left - 1), m = fdiv(u, gm.by_nr);
-            const int tk = token_of(dm, gm, __ldcg(list + m0 + m), u - m * dm.n_r), at = max(tk, 0);
+            const int tk = token_of(dm, gm, __ldcg(list + m0 + m), u - m * dm.n_r);
+            const bool ok = e < left && tk >= 0;
+            const int at = ok ? tk : spare;
             tab[e] = (uint32_t)at * (uint32_t)(dm.C >> 3);
-            s_l2[e] = e >= left || tk < 0 ? INFINITY : __ldg(lse_h + at) * 1.4426950408889634f;
-            s_dl[e] = __ldcg(delta_h + at);
+            s_l2[e] = ok ? __ldg(lse_h + at) * 1.4426950408889634f : INFINITY;
+            s_dl[e] = ok ? __ldcg(delta_h + at) : 0.f;
         }
     };
     bool filled = false;

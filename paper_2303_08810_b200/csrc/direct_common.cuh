@@ -185,26 +185,58 @@ __device__ __forceinline__ int token_of(const Dims& dm, const DirGeom& gm, int r
     const int y = ry * dm.hs + ty, x = rx * dm.ws + tx;
     return y < dm.H0 && x < dm.W0 ? y * dm.W0 + x : -1;
 }
+// Dead rows (of a tile's rest, of a bad routing entry, of the zero padding) have the probability 0, but what is read in their
+// place must be finite, or the product is NaN: a row of a region that nobody routes to would reach the results.  They read
+// token 0, or, if that holds an infinity or NaN in one of the two tensors, the first token that does not (none: 0).
+// spare_probe(), with a chunk of token 0 per lane, is called where its latency is hidden; both by whole warps.  (Zeroing the
+// rows in the walk, or walking again when a NaN came out, costs registers there: forward + backward at 64 x 56 x 56 x 64
+// 238 -> 264 and 252 us.)
+template <int PL>
+__device__ __forceinline__ uint4 spare_probe(const uint8_t* a, const uint8_t* b, int lane) {
+    return ld16_or_zero((lane < 4 * PL ? a : b) + lane % (4 * PL) * 16, lane < 8 * PL);
+}
+__device__ __forceinline__ bool finite_bf16x8(const uint4& v) {
+    bool ok = true;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) ok = ok && (reg_of(v, i) & 0x7f80u) != 0x7f80u && (reg_of(v, i) & 0x7f800000u) != 0x7f800000u;
+    return ok;
+}
+template <int PL>
+__device__ __forceinline__ int spare_token(const uint4& probe, const uint8_t* a, const uint8_t* b, uint32_t tok_bytes, int tokens, int lane) {
+    if (__all_sync(0xffffffffu, finite_bf16x8(probe))) return 0;
+#pragma unroll 1
+    for (int t0 = 0; t0 < tokens; t0 += 32) {
+        const int t = t0 + lane;
+        bool ok = t < tokens;
+#pragma unroll 1
+        for (int q = 0; ok && q < 8 * PL; ++q)
+            ok = finite_bf16x8(ld16((q < 4 * PL ? a : b) + (size_t)(uint32_t)t * tok_bytes + q % (4 * PL) * 16));
+        const uint32_t word = __ballot_sync(0xffffffffu, ok);
+        if (word) return t0 + __ffs(word) - 1;
+    }
+    return 0;
+}
 // Table of the keys [k0, k0 + n) of a group: key kk is token kk % n_r of region irow[kk / n_r].  An entry is the
 // offset of the token's row from the head's first byte, in units of 16 bytes.  Keys that are not rows of the map - entries
-// beyond `total`, of a bad routing entry, of the zero padding - name some readable row and have their bit set in `dead`:
+// beyond `total`, of a bad routing entry, of the zero padding - name the row of token `spare` and have their bit set in `dead`:
 // the caller gives them the probability zero.  (A key of the zero padding has the score 0 and the value 0: all it does is
 // count in the softmax's denominator.)  Returns how many keys of the zero padding this lane met.
-__device__ __forceinline__ int fill_keys(uint32_t* tab, uint32_t* dead, const int32_t* irow, int k0, int n, int total, int lane0, int lanes,
-                                         int32_t* status, const Dims& dm, const DirGeom& gm) {
+__device__ __forceinline__ int fill_keys(uint32_t* tab, uint32_t* dead, const int32_t* irow, int k0, int n, int total, int spare, int lane0,
+                                         int lanes, int32_t* status, const Dims& dm, const DirGeom& gm) {
     int zeros = 0;
     for (int e = lane0; e < n; e += lanes) {                         // whole warps: n and lanes are multiples of 32
         const int kk = min(k0 + e, total - 1);
         const int m = fdiv(kk, gm.by_nr);
         const int r = __ldcg(irow + m);  // coherent load: the index may come from the kernel this one overlaps
         bool ok = k0 + e < total;
-        int tok = 0;
+        int tok = spare;
         if (r < 0 || r >= dm.R) {
             record_error(status, BRA_ERR_INDEX, r);
             ok = false;
         } else {
             tok = token_of(dm, gm, r, kk - m * dm.n_r);
-            if (tok < 0) { zeros += ok; ok = false; tok = 0; }
+            if (tok < 0) { zeros += ok; ok = false; }
+            if (!ok) tok = spare;
         }
         tab[e] = (uint32_t)tok * (uint32_t)(dm.C >> 3);
         const uint32_t word = __ballot_sync(0xffffffffu, !ok);

@@ -990,3 +990,78 @@ def test_long_lists_keep_their_precision(bra, C):
     refs = (ref,) + orc.bra_backward(x["Q"], x["K"], x["V"], index, np.zeros_like(x["w"]), x["dO"], cfg.heads, cfg.S)[:3]
     ratios = {name: rounding_ratio(a, r) for name, a, r in zip(("O", "dQ", "dK", "dV"), (O,) + tuple(g[:3]), refs)}
     assert max(ratios.values()) <= RATIO_MAX, ratios
+
+
+# ------------------------------------------------------------------ infinities and NaN stay where they are routed
+def closed_lists(cfg, seed, bad=False):
+    """Regions 0 .. topk - 1 list one another and nothing else lists them: what is in region 0 concerns no other region."""
+    rng = np.random.default_rng(seed)
+    idx = np.empty((cfg.B, cfg.heads, cfg.R, cfg.topk), np.int32)
+    for b in range(cfg.B):
+        for h in range(cfg.heads):
+            for r in range(cfg.R):
+                pool = np.arange(cfg.topk) if r < cfg.topk else np.arange(cfg.topk, cfg.R)
+                idx[b, h, r] = rng.permutation(pool)[:cfg.topk]
+    if bad:
+        idx[0, 0, -1, -1] = cfg.R
+        idx[-1, -1, cfg.topk, 0] = -1
+    return idx
+
+
+def region_mask(cfg, first, last):
+    """[H, W]: tokens of regions first .. last - 1 of the (padded) map."""
+    hs, ws = -(-cfg.H // cfg.S), -(-cfg.W // cfg.S)
+    r = (np.arange(cfg.H) // hs)[:, None] * cfg.S + (np.arange(cfg.W) // ws)[None, :]
+    return (r >= first) & (r < last)
+
+
+def run_isolation_case(bra, cfg, impl, value, bad=False):
+    """Region 0 of every tensor is `value`: O, lse and the gradients of the regions that do not list it are what they are
+    with a finite region 0 (bf16: one rounding apart, in case the sums are taken in another order).  LCE off: it spreads
+    over borders, rightly."""
+    import torch
+    x = synthetic.make_inputs(cfg, seed=97, with_do=True)
+    idx = torch.from_numpy(closed_lists(cfg, 98, bad)).cuda()
+    p = problem_of(bra, cfg, impl=IMPLS[impl], lce=False)
+    ws = bra.workspace(p)
+    where = torch.from_numpy(region_mask(cfg, 0, 1)).cuda()
+    outs = []
+    for v in (None, value):
+        t = to_dev(x, cfg)
+        if v is not None:
+            for n in ("Q", "K", "V", "dO"):
+                t[n][:, where] = v
+        O, lse = bra.bra_attend(p, t["Q"], t["K"], t["V"], idx, ws=ws)
+        g = bra.bra_backward(p, t["Q"], t["K"], t["V"], idx, None, lse, t["dO"], ws=ws)
+        assert bra.bra_device_status(ws) == (9 if bad else 0)
+        outs.append((O,) + tuple(g[:3]) + (lse,))
+    others = region_mask(cfg, cfg.topk, cfg.R)
+    for name, clean, got in zip(("O", "dQ", "dK", "dV", "lse"), *outs):
+        if name == "lse":
+            a, r = f64(got)[..., others.ravel()], f64(clean)[..., others.ravel()]
+        else:
+            a, r = f64(got)[:, others], f64(clean)[:, others]
+            assert not np.isfinite(f64(got)[:, where.cpu().numpy()]).any(), name       # region 0 lists itself
+        assert np.isfinite(a).all(), f"{cfg.name} {name}: {np.count_nonzero(~np.isfinite(a))} of {a.size}"
+        assert np.linalg.norm(a - r) <= (4e-3 if cfg.dtype == "bf16" else 1e-6) * np.linalg.norm(r), name
+
+
+DIRECT_ISOLATION = [
+    BraConfig("alone-one-block-of-keys", 2, 12, 20, 64, 2, 4, 3, "bf16"),           # 45 keys
+    BraConfig("alone-tail", 2, 12, 20, 64, 2, 4, 7, "bf16"),                        # 105 keys
+    BraConfig("alone-two-tables-of-a-warp", 1, 21, 35, 64, 2, 7, 20, "bf16"),       # 300 keys
+    BraConfig("alone-two-tables-of-a-cta", 1, 30, 35, 64, 2, 5, 12, "bf16"),        # 504 keys of 42 tokens; lists up to 13 x 42
+    BraConfig("alone-two-tiles-per-warp", 19, 24, 28, 64, 2, 4, 3, "bf16"),
+    BraConfig("alone-d64", 1, 12, 20, 128, 2, 4, 3, "bf16"),
+    BraConfig("alone-d64-two-tables", 1, 21, 35, 128, 2, 7, 20, "bf16"),
+    BraConfig("alone-cut-map", 2, 29, 27, 64, 2, 4, 3, "bf16"),
+    BraConfig("alone-cut-map-d64", 2, 29, 27, 128, 2, 4, 3, "bf16"),
+    BraConfig("alone-11x12", 1, 33, 36, 64, 2, 3, 4, "bf16"),
+]
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("nan")], ids=["inf", "nan"])
+@pytest.mark.parametrize("cfg", DIRECT_ISOLATION, ids=lambda c: c.name)
+def test_direct_kernels_keep_infinities_in_their_regions(bra, cfg, value):
+    run_isolation_case(bra, cfg, "mma", value)
+    run_isolation_case(bra, cfg, "mma", value, bad=True)

@@ -31,6 +31,7 @@ attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
     const T* Q = Qg + head; const T* K = Kg + head; const T* V = Vg + head;
     float* s_w = reinterpret_cast<float*>(smem + gm.off_w);
     if (dm.lce) simt_load_weights(s_w, lce_w + (size_t)h * D * 25, 25 * D);
+    simt_zero_rows(smem, gm);
     if (gm.resident) {
         simt_copy_rows<T, D>(sbase + gm.off_a, sbase + gm.off_b, K, V, dm.C, dm.N, [&](int row, uint32_t& at) {
             const int r = fdiv(row, gm.by_nr);
@@ -95,13 +96,13 @@ attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
                 const int kk = k0 + (blk * U + u) * KS + ks;
                 dead[u] = kk >= k1;
                 if constexpr (PLAIN) {
-                    at[u] = dead[u] ? abase : next;
+                    at[u] = dead[u] ? abase + gm.zero : next;
                     next += KS * gm.row;
                 } else {
                     wt[u] = 1.f;
                     const int row = dead[u] ? -1 : row_of(kk, wt[u]);
                     dead[u] = row < 0;
-                    at[u] = abase + (dead[u] ? 0 : row);
+                    at[u] = abase + (dead[u] ? gm.zero : row);
                 }
             }
             dots<T, QT, U, D>(s, q, at, gm.off_a);

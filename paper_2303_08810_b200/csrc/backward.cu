@@ -45,6 +45,7 @@ bwd_dq_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
     const int N0 = dm.H0 * dm.W0;
     const size_t head = (size_t)b * N0 * dm.C + (size_t)h * D;
     const T* K = Kg + head; const T* V = Vg + head;
+    simt_zero_rows(smem, gm);
     if (gm.resident) {
         simt_copy_rows<T, D>(sbase + gm.off_a, sbase + gm.off_b, K, V, dm.C, dm.N, [&](int row, uint32_t& at) {
             const int r = fdiv(row, gm.by_nr);
@@ -105,13 +106,13 @@ bwd_dq_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
                 const int kk = k0 + (blk * U + u) * KS + ks;
                 dead[u] = kk >= k1;
                 if constexpr (PLAIN) {
-                    at[u] = dead[u] ? abase : next;
+                    at[u] = dead[u] ? abase + gm.zero : next;
                     next += KS * gm.row;
                 } else {
                     wt[u] = 1.f;
                     const int row = dead[u] ? -1 : row_of(kk, wt[u]);
                     dead[u] = row < 0;
-                    at[u] = abase + (dead[u] ? 0 : row);
+                    at[u] = abase + (dead[u] ? gm.zero : row);
                 }
             }
             dots<T, QT, U, D>(s, q, at, gm.off_a);
@@ -207,6 +208,7 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
     const T* Q = Qg + head; const T* dO = dOg + head;
     float* s_w = reinterpret_cast<float*>(smem + gm.off_w);
     if (dm.lce) simt_load_weights(s_w, lce_w + (size_t)h * D * 25, 25 * D);
+    simt_zero_rows(smem, gm);
     if (gm.resident) {
         simt_copy_rows<T, D>(sbase + gm.off_a, sbase + gm.off_b, Q, dO, dm.C, dm.N, [&](int row, uint32_t& at) {
             const int r = fdiv(row, gm.by_nr);
@@ -262,13 +264,13 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
             bool dead = kk >= n;
             float wt = 1.f;
             if constexpr (PLAIN) {
-                if (dead) { at = abase; at_stat = abase + gm.off_stat; }
+                if (dead) { at = abase + gm.zero; at_stat = abase + gm.off_stat; }
                 next += KS * gm.row;
                 next_stat += KS * 8;
             } else {
                 const int row = dead ? -1 : row_of(kk, wt);
                 dead = row < 0;
-                at = abase + (dead ? 0 : row) * gm.row;               // (resident: row number)
+                at = abase + (dead ? gm.zero : row * gm.row);         // (resident: row number)
                 at_stat = abase + gm.off_stat + (dead ? 0 : row) * 8;
             }
             const float2 stat = lds_f32x2(at_stat);

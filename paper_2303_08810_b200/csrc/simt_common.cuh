@@ -36,6 +36,7 @@ struct SimtGeom {
     uint32_t mul_spr, mul_kps, mul_cw;
     int row;               // bytes of a row of one tensor in shared memory
     int reg;               // bytes from one region's rows of a stage to the next region's
+    int zero;              // offset of a row of zeros in either tensor's rows
     int off_a, off_b, off_stat, off_idx, off_cnt, off_w, off_st, stage_bytes, smem_bytes;
 };
 
@@ -91,8 +92,9 @@ inline SimtGeom simt_geom(const Dims& d, SimtKind kind) {
     const int rows = g.resident ? d.N : g.rpc * g.kps;                // of one stage
     g.reg = (g.kps * g.row + 111) / 128 * 128 + 16;                   // 16 modulo 128
     int off = 0;
-    g.off_a = off;    off += g.resident ? rows * g.row : g.rpc * g.reg;
-    g.off_b = off;    off += g.resident ? rows * g.row : g.rpc * g.reg;
+    g.zero = g.resident ? rows * g.row : g.rpc * g.reg;
+    g.off_a = off;    off += g.zero + g.row;
+    g.off_b = off;    off += g.zero + g.row;
     g.off_stat = off; off += kind == SIMT_DKV ? (rows * 8 + 15) / 16 * 16 : 0;     // lse, delta
     g.stage_bytes = off;
     off *= g.stages;
@@ -277,6 +279,16 @@ __device__ __forceinline__ void simt_copy_rows(uint32_t dst_a, uint32_t dst_b, c
                 ptx::cp_async_16(dst_b + at + c * 16, B + off + c * (16 / sizeof(T)), bytes);
             }
         }
+    }
+}
+
+// The rows that stand in for keys (queries) that do not count: their probability is 0, but 0 times an infinity or NaN of some
+// other region's row would not be.
+__device__ __forceinline__ void simt_zero_rows(uint8_t* smem, const SimtGeom& gm) {
+    const int n = gm.row / 16;
+    for (int e = threadIdx.x; e < 2 * gm.stages * n; e += blockDim.x) {
+        const int r = e / n, stage = r >> 1;
+        *reinterpret_cast<uint4*>(smem + stage * gm.stage_bytes + (r & 1 ? gm.off_b : gm.off_a) + gm.zero + (e - r * n) * 16) = make_uint4(0, 0, 0, 0);
     }
 }
 

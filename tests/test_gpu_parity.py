@@ -1065,3 +1065,46 @@ DIRECT_ISOLATION = [
 def test_direct_kernels_keep_infinities_in_their_regions(bra, cfg, value):
     run_isolation_case(bra, cfg, "mma", value)
     run_isolation_case(bra, cfg, "mma", value, bad=True)
+
+
+SIMT_ISOLATION = [
+    BraConfig("alone-resident", 2, 8, 12, 64, 2, 4, 8, "f32"),
+    BraConfig("alone-resident-d16", 2, 8, 12, 32, 2, 4, 7, "f32"),
+    BraConfig("alone-staged-d64", 1, 12, 20, 64, 1, 4, 3, "f32"),
+    BraConfig("alone-staged", 1, 21, 70, 64, 2, 7, 5, "f32"),
+    BraConfig("alone-staged-d16", 1, 35, 35, 16, 1, 7, 9, "f32"),
+    BraConfig("alone-staged-one-lane", 40, 21, 35, 64, 2, 7, 3, "f32"),
+    BraConfig("alone-staged-d64-chunks", 1, 51, 51, 64, 1, 3, 2, "f32"),
+    BraConfig("alone-cut-map-f32", 2, 29, 27, 64, 2, 4, 3, "f32"),
+    BraConfig("alone-bf16-d16", 2, 12, 20, 32, 2, 4, 5, "bf16"),
+]
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("nan")], ids=["inf", "nan"])
+@pytest.mark.parametrize("cfg", SIMT_ISOLATION, ids=lambda c: c.name)
+def test_cuda_core_kernels_keep_infinities_in_their_regions(bra, cfg, value):
+    run_isolation_case(bra, cfg, "simt", value)
+    run_isolation_case(bra, cfg, "simt", value, bad=True)
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("nan")], ids=["inf", "nan"])
+def test_cuda_core_kernels_keep_infinities_out_of_weighted_walks(bra, value):
+    """topk = R with repeats: every region is walked, weighed by how often it is listed, region 0 not at all."""
+    import torch
+    cfg = BraConfig("alone-weighted", 2, 6, 6, 32, 1, 3, 9, "f32")
+    x = synthetic.make_inputs(cfg, seed=97, with_do=True)
+    idx = torch.randint(1, 9, (2, 1, 9, 9), dtype=torch.int32, device="cuda", generator=torch.Generator("cuda").manual_seed(4))
+    idx[:, :, 0] = 0
+    p = problem_of(bra, cfg, impl=IMPLS["simt"], lce=False)
+    ws = bra.workspace(p)
+    where = torch.from_numpy(region_mask(cfg, 0, 1)).cuda()
+    outs = []
+    for v in (None, value):
+        t = to_dev(x, cfg)
+        if v is not None:
+            for n in ("Q", "K", "V", "dO"):
+                t[n][:, where] = v
+        O, lse = bra.bra_attend(p, t["Q"], t["K"], t["V"], idx, ws=ws)
+        outs.append((O,) + tuple(bra.bra_backward(p, t["Q"], t["K"], t["V"], idx, None, lse, t["dO"], ws=ws)[:3]))
+    for clean, got in zip(*outs):
+        assert (clean[:, ~where] == got[:, ~where]).all()

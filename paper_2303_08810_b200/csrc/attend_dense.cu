@@ -12,11 +12,57 @@ namespace bra {
 
 using namespace ptx;
 
+// The CTA's tokens one by one (dense_any_nan() says when and why).
+__device__ __noinline__ void attend_dense_by_token(const __nv_bfloat16* Qg, const __nv_bfloat16* Vg, const float* lce_w, const float* lce_b,
+                                                   __nv_bfloat16* O, float* lse, const uint8_t* smem, bool weighted, const Dims& dm, const DenseGeom& gm) {
+    const int h = blockIdx.y, b = blockIdx.z;
+    const int N0 = dm.H0 * dm.W0, y0 = blockIdx.x * gm.g.hb;
+    const int q0 = y0 * dm.W, nq = min(gm.g.hb, dm.H - y0) * dm.W;
+    const size_t head = (size_t)b * N0 * dm.C + (size_t)h * 32;
+    const uint8_t* reg = smem + gm.off_reg;
+    const float* bias = reinterpret_cast<const float*>(smem + gm.off_bias);
+    const float sl2 = dm.scale * 1.4426950408889634f;
+    for (int t = threadIdx.x; t < nq; t += blockDim.x) {
+        const int2 at = dense_pos(dm, gm, q0 + t);
+        if (at.y >= dm.H0 || at.x >= dm.W0) continue;
+        const int i = reg[q0 + t], tok = at.y * dm.W0 + at.x;
+        const unsigned long long m64 = reinterpret_cast<const unsigned long long*>(smem + gm.off_mask)[i];
+        float q[32], o[32], v[32], m = -INFINITY, l = 0.f;
+        load_row<32>(Qg + head + (size_t)(uint32_t)tok * dm.C, q);
+#pragma unroll
+        for (int c = 0; c < 32; ++c) o[c] = 0.f;
+        auto score = [&](int j) {
+            dense_row32(v, smem + gm.off_a, j);
+            return dense_dot(q, v) * sl2 + (weighted ? bias[i * dm.R + reg[j]] : 0.f);
+        };
+#pragma unroll 1
+        for (int j = 0; j < dm.N; ++j)
+            if (m64 >> reg[j] & 1) m = fmaxf(m, score(j));
+        const float mn = m == -INFINITY ? 0.f : m;
+#pragma unroll 1
+        for (int j = 0; j < dm.N; ++j)
+            if (m64 >> reg[j] & 1) {
+                const float p = exp2f(score(j) - mn);
+                l += p;
+                dense_row32(v, smem + gm.off_b, j);
+#pragma unroll
+                for (int c = 0; c < 32; ++c) o[c] = fmaf(p, v[c], o[c]);
+            }
+        const float inv = l > 0.f ? 1.f / l : 0.f;
+#pragma unroll
+        for (int c = 0; c < 32; ++c) o[c] *= inv;
+        if (lse) lse[((size_t)b * dm.heads + h) * N0 + tok] = (m + log2f(l)) * 0.6931471805599453f;
+        if (dm.lce) dense_lce_row<false>(o, Vg + head, lce_w + (size_t)h * 32 * 25, lce_b ? lce_b + h * 32 : nullptr, at.y, at.x, dm);
+        store_row<32>(O + head + (size_t)(uint32_t)tok * dm.C, o);
+    }
+}
+
 template <int RT, int TX, int NR>
 __global__ void __launch_bounds__(256, 2)
 attend_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __restrict__ Kg, const __nv_bfloat16* __restrict__ Vg,
                     const int32_t* index, const float* __restrict__ lce_w, const float* __restrict__ lce_b,
-                    __nv_bfloat16* __restrict__ O, float* __restrict__ lse, int32_t* __restrict__ status, Dims dm, DenseGeom gm) {
+                    __nv_bfloat16* __restrict__ O, float* __restrict__ lse, int32_t* __restrict__ status,
+                    const __grid_constant__ Dims dm, const __grid_constant__ DenseGeom gm) {
     extern __shared__ __align__(128) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nthreads = blockDim.x;
@@ -151,7 +197,10 @@ attend_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* _
         for (int s = 0; s < 2; ++s) dense_mma_tokens<RT>(o, pa[s], vs, kb + 16 * s, lane);
     }
     cp_async_wait<0>();
-    __syncthreads();                                                  // the slices have been read: staging takes their place
+    if (__syncthreads_or(dense_any_nan(o))) {                         // the slices have been read: staging takes their place
+        attend_dense_by_token(Qg, Vg, lce_w, lce_b, O, lse, smem, routes.weighted, dm, gm);
+        return;
+    }
     float* st = reinterpret_cast<float*>(smem + gm.g.off_st);
 #pragma unroll
     for (int x = 0; x < RT; ++x)

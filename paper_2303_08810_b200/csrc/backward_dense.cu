@@ -12,12 +12,82 @@ namespace bra {
 
 using namespace ptx;
 
+// The gradients of an (image, head) token by token (dense_any_nan() says when and why).
+__device__ __noinline__ void bwd_dense_by_token(const float* lce_w, const __nv_bfloat16* dOg, __nv_bfloat16* dQg, __nv_bfloat16* dKg, __nv_bfloat16* dVg,
+                                                uint8_t* smem, bool weighted, const Dims& dm, const DenseGeom& gm) {
+    const int h = blockIdx.y, b = blockIdx.z;
+    const size_t head = (size_t)b * dm.H0 * dm.W0 * dm.C + (size_t)h * 32;
+    const uint8_t *qs = smem + gm.off_a, *ks = smem + gm.off_b, *vs = smem + gm.off_c, *gs = smem + gm.off_d, *reg = smem + gm.off_reg;
+    const float* bias = reinterpret_cast<const float*>(smem + gm.off_bias);
+    const unsigned long long* mask = reinterpret_cast<const unsigned long long*>(smem + gm.off_mask);
+    const float* l2 = reinterpret_cast<const float*>(smem + gm.off_stat);
+    float* dl = reinterpret_cast<float*>(smem + gm.off_stat) + gm.rows;
+    const float sl2 = dm.scale * 1.4426950408889634f;
+    auto on_map = [&](const int2& at) { return at.y < dm.H0 && at.x < dm.W0; };
+    auto store = [&](__nv_bfloat16* out, const int2& at, float (&v)[32], float f) {
+#pragma unroll
+        for (int c = 0; c < 32; ++c) v[c] *= f;
+        store_row<32>(out + head + (size_t)(uint32_t)(at.y * dm.W0 + at.x) * dm.C, v);
+    };
+    for (int t = threadIdx.x; t < dm.N; t += blockDim.x) {            // queries
+        const int2 at = dense_pos(dm, gm, t);
+        if (!on_map(at)) continue;
+        const int i = reg[t];
+        float q[32], g[32], row[32], acc[32], delta = 0.f;
+        dense_row32(q, qs, t);
+        dense_row32(g, gs, t);
+#pragma unroll
+        for (int c = 0; c < 32; ++c) acc[c] = 0.f;
+#pragma unroll 1
+        for (int it = 0; it < 2 * dm.N; ++it) {
+            const int j = it < dm.N ? it : it - dm.N;
+            if (!(mask[i] >> reg[j] & 1)) continue;
+            dense_row32(row, vs, j);
+            const float dp = dense_dot(g, row);
+            dense_row32(row, ks, j);
+            const float p = exp2f(dense_dot(q, row) * sl2 + (weighted ? bias[i * dm.R + reg[j]] : 0.f) - l2[t]);
+            if (it < dm.N) { delta = fmaf(p, dp, delta); continue; }
+            const float ds = p * (dp - delta);
+#pragma unroll
+            for (int c = 0; c < 32; ++c) acc[c] = fmaf(ds, row[c], acc[c]);
+        }
+        dl[t] = delta;
+        store(dQg, at, acc, dm.scale);
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < dm.N; t += blockDim.x) {            // keys
+        const int2 at = dense_pos(dm, gm, t);
+        if (!on_map(at)) continue;
+        const int j = reg[t];
+        float k[32], v[32], row[32], gk[32], gv[32];
+        dense_row32(k, ks, t);
+        dense_row32(v, vs, t);
+#pragma unroll
+        for (int c = 0; c < 32; ++c) gk[c] = gv[c] = 0.f;
+#pragma unroll 1
+        for (int i = 0; i < dm.N; ++i) {
+            if (!(mask[64 + j] >> reg[i] & 1)) continue;
+            dense_row32(row, qs, i);
+            const float p = exp2f(dense_dot(k, row) * sl2 + (weighted ? bias[reg[i] * dm.R + j] : 0.f) - l2[i]);
+            float g[32];
+            dense_row32(g, gs, i);
+            const float ds = p * (dense_dot(v, g) - dl[i]);
+#pragma unroll
+            for (int c = 0; c < 32; ++c) { gk[c] = fmaf(ds, row[c], gk[c]); gv[c] = fmaf(p, g[c], gv[c]); }
+        }
+        store(dKg, at, gk, dm.scale);
+        if (dm.lce) dense_lce_row<true>(gv, dOg + head, lce_w + (size_t)h * 32 * 25, nullptr, at.y, at.x, dm);
+        store(dVg, at, gv, 1.f);
+    }
+}
+
 template <int TX, int NR>
 __global__ void __launch_bounds__(256, 2)
 bwd_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __restrict__ Kg, const __nv_bfloat16* __restrict__ Vg,
                  const int32_t* __restrict__ index, const float* __restrict__ lse, const __nv_bfloat16* __restrict__ dOg,
                  const float* __restrict__ lce_w, __nv_bfloat16* __restrict__ dQg, __nv_bfloat16* __restrict__ dKg,
-                 __nv_bfloat16* __restrict__ dVg, int32_t* __restrict__ status, Dims dm, DenseGeom gm) {
+                 __nv_bfloat16* __restrict__ dVg, int32_t* __restrict__ status, const __grid_constant__ Dims dm,
+                 const __grid_constant__ DenseGeom gm) {
     extern __shared__ __align__(128) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nthreads = blockDim.x;
@@ -67,6 +137,7 @@ bwd_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __re
     };
 
     // ---- queries: delta, dQ ----
+    bool nan = false;
 #pragma unroll 1
     for (int tile = warp; tile < steps; tile += gm.nw) {
         const int r0 = tile * 16;
@@ -131,6 +202,7 @@ bwd_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __re
                 }
             }
         }
+        nan = nan || dense_any_nan(dq) || delta[0] != delta[0] || delta[1] != delta[1];
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             const int t = r0 + g + 8 * r, tok = token(t);
@@ -141,7 +213,11 @@ bwd_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __re
             for (int n = 0; n < 4; ++n) o[4 * n] = pack2_bf16(dq[0][n][2 * r] * dm.scale, dq[0][n][2 * r + 1] * dm.scale);
         }
     }
-    __syncthreads();
+    if (__syncthreads_or(nan)) {
+        cp_async_wait<0>();
+        bwd_dense_by_token(lce_w, dOg, dQg, dKg, dVg, smem, routes.weighted, dm, gm);
+        return;
+    }
 
     // ---- keys: dK, dV (a warp has at most two tiles; dV is staged once all warps have read the slices) ----
     float dv[2][4][4];
@@ -192,6 +268,7 @@ bwd_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __re
             frag_hi(a[0], c[0], c[1]);
             dense_mma_tokens<1>(dv + x, a, gs, qb, lane);
         }
+        nan = nan || dense_any_nan(dk) || dense_any_nan(reinterpret_cast<const float (&)[1][4][4]>(dv[x]));
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             const int tok = token(r0 + g + 8 * r);
@@ -202,7 +279,10 @@ bwd_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __re
         }
     }
     cp_async_wait<0>();
-    __syncthreads();
+    if (__syncthreads_or(nan)) {
+        bwd_dense_by_token(lce_w, dOg, dQg, dKg, dVg, smem, routes.weighted, dm, gm);
+        return;
+    }
     float* st = reinterpret_cast<float*>(smem + gm.g.off_st);
 #pragma unroll
     for (int x = 0; x < 2; ++x) {

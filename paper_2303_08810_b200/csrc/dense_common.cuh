@@ -174,6 +174,57 @@ __device__ __forceinline__ void dense_a(uint32_t (&a)[1][2][4], uint32_t slice, 
     const uint4 lo[1] = {dense_row(slice, r0 + g, t4)}, up[1] = {dense_row(slice, r0 + 8 + g, t4)};
     rows_to_a<1>(a, lo, up);
 }
+// The products run over every token of the map, with probability 0 where a pair is not routed: an infinity or NaN of a token
+// then becomes a NaN in the accumulators of queries (keys) that do not list its region.  A CTA whose accumulators hold a NaN
+// does its work again with the functions below (in attend_dense.cu and backward_dense.cu), a thread per token that
+// looks at the routed pairs alone.  (That costs the kernels a few comparisons behind each walk.)
+template <int RT>
+__device__ __forceinline__ bool dense_any_nan(const float (&acc)[RT][4][4]) {
+    bool nan = false;
+#pragma unroll
+    for (int x = 0; x < RT; ++x)
+#pragma unroll
+        for (int n = 0; n < 4; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) nan = nan || acc[x][n][e] != acc[x][n][e];
+    return nan;
+}
+// row r of a slice
+__device__ __forceinline__ void dense_row32(float (&v)[32], const uint8_t* slice, int r) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const uint4 u = *reinterpret_cast<const uint4*>(slice + dense_at(r, q));
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            v[8 * q + 2 * j] = __uint_as_float(reg_of(u, j) << 16);
+            v[8 * q + 2 * j + 1] = __uint_as_float(reg_of(u, j) & 0xffff0000u);
+        }
+    }
+}
+__device__ __forceinline__ float dense_dot(const float (&a)[32], const float (&b)[32]) {
+    float s = 0.f;
+#pragma unroll
+    for (int c = 0; c < 32; ++c) s = fmaf(a[c], b[c], s);
+    return s;
+}
+// acc += the 5 x 5 correlation of a head's channels at (y, x), plus its bias; FLIP: with the flipped filter
+template <bool FLIP>
+__device__ __forceinline__ void dense_lce_row(float (&acc)[32], const __nv_bfloat16* in_head, const float* w, const float* bias, int y, int x, const Dims& dm) {
+#pragma unroll 1
+    for (int k = 0; k < 25; ++k) {
+        const int yy = y + k / 5 - 2, xx = x + k % 5 - 2;
+        if ((unsigned)yy >= (unsigned)dm.H0 || (unsigned)xx >= (unsigned)dm.W0) continue;
+        float v[32];
+        load_row<32>(in_head + (size_t)(uint32_t)(yy * dm.W0 + xx) * dm.C, v);
+#pragma unroll
+        for (int c = 0; c < 32; ++c) acc[c] = fmaf(__ldg(w + c * 25 + (FLIP ? 24 - k : k)), v[c], acc[c]);
+    }
+    if (bias) {
+#pragma unroll
+        for (int c = 0; c < 32; ++c) acc[c] += __ldg(bias + c);
+    }
+}
+
 // acc (16 x 32) += A (16 x 16, fp32 fragments c0, c1) * the 16 rows of a slice from r0 on
 template <int RT>
 __device__ __forceinline__ void dense_mma_tokens(float (*acc)[4][4], const uint32_t (*a)[4], uint32_t slice, int r0, int lane) {

@@ -993,7 +993,7 @@ def test_long_lists_keep_their_precision(bra, C):
 
 
 # ------------------------------------------------------------------ infinities and NaN stay where they are routed
-def closed_lists(cfg, seed, bad=False):
+def closed_lists(cfg, seed, bad=False, repeats=False):
     """Regions 0 .. topk - 1 list one another and nothing else lists them: what is in region 0 concerns no other region."""
     rng = np.random.default_rng(seed)
     idx = np.empty((cfg.B, cfg.heads, cfg.R, cfg.topk), np.int32)
@@ -1002,6 +1002,8 @@ def closed_lists(cfg, seed, bad=False):
             for r in range(cfg.R):
                 pool = np.arange(cfg.topk) if r < cfg.topk else np.arange(cfg.topk, cfg.R)
                 idx[b, h, r] = rng.permutation(pool)[:cfg.topk]
+    if repeats:
+        idx[..., -1] = idx[..., 0]
     if bad:
         idx[0, 0, -1, -1] = cfg.R
         idx[-1, -1, cfg.topk, 0] = -1
@@ -1015,13 +1017,15 @@ def region_mask(cfg, first, last):
     return (r >= first) & (r < last)
 
 
-def run_isolation_case(bra, cfg, impl, value, bad=False):
+def run_isolation_case(bra, cfg, impl, value, bad=False, repeats=False):
     """Region 0 of every tensor is `value`: O, lse and the gradients of the regions that do not list it are what they are
     with a finite region 0 (bf16: one rounding apart, in case the sums are taken in another order).  LCE off: it spreads
     over borders, rightly."""
     import torch
     x = synthetic.make_inputs(cfg, seed=97, with_do=True)
-    idx = torch.from_numpy(closed_lists(cfg, 98, bad)).cuda()
+    idx = torch.from_numpy(closed_lists(cfg, 98, bad, repeats)).cuda()
+    if repeats:
+        idx[:, :, 0, 0] = 0                     # region 0 still lists itself
     p = problem_of(bra, cfg, impl=IMPLS[impl], lce=False)
     ws = bra.workspace(p)
     where = torch.from_numpy(region_mask(cfg, 0, 1)).cuda()
@@ -1108,3 +1112,47 @@ def test_cuda_core_kernels_keep_infinities_out_of_weighted_walks(bra, value):
         outs.append((O,) + tuple(bra.bra_backward(p, t["Q"], t["K"], t["V"], idx, None, lse, t["dO"], ws=ws)[:3]))
     for clean, got in zip(*outs):
         assert (clean[:, ~where] == got[:, ~where]).all()
+
+
+DENSE_ISOLATION = [
+    BraConfig("alone-7x7", 2, 7, 7, 64, 2, 7, 10, "bf16"),
+    BraConfig("alone-64-regions", 2, 8, 8, 64, 2, 8, 9, "bf16"),
+    BraConfig("alone-2x2-regions", 2, 8, 8, 64, 2, 4, 5, "bf16"),
+    BraConfig("alone-2x2-regions-64-pairs", 64, 12, 12, 32, 1, 6, 13, "bf16"),
+    BraConfig("alone-256-tokens", 148, 16, 16, 64, 2, 8, 17, "bf16"),
+    BraConfig("alone-cut-64-tokens", 2, 7, 6, 64, 2, 4, 5, "bf16"),
+]
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("nan")], ids=["inf", "nan"])
+@pytest.mark.parametrize("cfg", DENSE_ISOLATION, ids=lambda c: c.name)
+def test_dense_kernels_keep_infinities_in_their_regions(bra, cfg, value):
+    run_isolation_case(bra, cfg, "auto", value)
+    run_isolation_case(bra, cfg, "auto", value, bad=True)
+    run_isolation_case(bra, cfg, "auto", value, repeats=True)
+
+
+@pytest.mark.parametrize("cfg", DENSE_ISOLATION, ids=lambda c: c.name)
+def test_dense_kernels_by_token_match_the_oracle(bra, cfg):
+    """One NaN makes a CTA work token by token: the tokens that it does not concern, LCE included, against the oracle."""
+    import torch
+    x = synthetic.make_inputs(cfg, seed=99, with_do=True)
+    t = to_dev(x, cfg)
+    index = closed_lists(cfg, 98)
+    idx = torch.from_numpy(index).cuda()
+    p = problem_of(bra, cfg)
+    ws = bra.workspace(p)
+    bias = np.linspace(-0.5, 0.5, cfg.C).astype(np.float32)
+    ref, _ = orc.bra_attend(x["Q"], x["K"], x["V"], index, x["w"], cfg.heads, cfg.S, None, bias)
+    grads = orc.bra_backward(x["Q"], x["K"], x["V"], index, x["w"], x["dO"], cfg.heads, cfg.S)
+    for n in ("Q", "K"):                        # (a NaN in V or dO spreads through the LCE)
+        t[n][:, 0, 0] = float("nan")
+    t["V"][:, 0, 0] = t["dO"][:, 0, 0] = float("inf")
+    O, lse = bra.bra_attend(p, t["Q"], t["K"], t["V"], idx, t["w"], torch.from_numpy(bias).cuda(), ws=ws)
+    g = bra.bra_backward(p, t["Q"], t["K"], t["V"], idx, t["w"], lse, t["dO"], ws=ws)
+    assert bra.bra_device_status(ws) == 0
+    far = region_mask(cfg, cfg.topk, cfg.R)
+    far[:3, :3] = False
+    check_O(f64(O)[:, far], ref[:, far], "bf16")
+    for name, a, r in zip(("dQ", "dK", "dV"), g, grads):
+        assert np.abs(f64(a)[:, far] - r[:, far]).max() <= GRAD_MAX, name

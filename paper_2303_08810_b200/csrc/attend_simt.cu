@@ -151,7 +151,7 @@ attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
     };
     if (!gm.resident) load_stage(0);
     for (int st = 0; st < nst; ++st) {
-        if (st + 1 < nst) { load_stage(st + 1); cp_async_wait<1>(); } else cp_async_wait<0>();
+        simt_advance(gm, st, nst, load_stage);
         __syncthreads();
         const uint32_t abase = sbase + (st & 1) * gm.stage_bytes;
         const int k0 = gm.resident ? 0 : st * gm.kps;

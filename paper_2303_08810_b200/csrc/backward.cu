@@ -157,10 +157,10 @@ bwd_dq_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
     };
     if (!gm.resident) load_stage(0);
     for (int it = 0; it < 2 * nst; ++it) {
-        if (!gm.resident && it + 1 < 2 * nst) { load_stage(it + 1); cp_async_wait<1>(); } else cp_async_wait<0>();
+        simt_advance(gm, it, gm.resident ? 0 : 2 * nst, load_stage);
         __syncthreads();
         const int k0 = gm.resident ? 0 : (it < nst ? it : it - nst) * gm.kps;
-        const uint32_t abase = sbase + (gm.resident ? 0 : it & 1) * gm.stage_bytes;
+        const uint32_t abase = sbase + (it & 1) * gm.stage_bytes;
         if (gm.resident ? gm.dense && !weighted : !bad)
             walk(std::true_type(), abase, gm.resident ? 0 : rl * gm.reg, k0, gm.resident ? dm.N : min(total, k0 + gm.kps), it >= nst, 0);
         else
@@ -301,8 +301,9 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
     const int nst = gm.resident ? 1 : (int)((most + gm.kps - 1) / gm.kps);
     int m0 = 0, q0 = 0;                                               // list entry and token of the next stage's first query
     auto load_stage = [&](int st) {
-        const uint32_t base = sbase + (st & 1) * gm.stage_bytes;
-        float2* stat = reinterpret_cast<float2*>(smem + (st & 1) * gm.stage_bytes + gm.off_stat);
+        const int off = (st & 1) * gm.stage_bytes;
+        const uint32_t base = sbase + off;
+        float2* stat = reinterpret_cast<float2*>(smem + off + gm.off_stat);
         simt_copy_rows<T, D>(base + gm.off_a, base + gm.off_b, Q, dO, dm.C, nreg * gm.kps, [&](int row, uint32_t& at) {
             const int lr = fdiv(row, gm.kps, gm.mul_kps), u = q0 + row - lr * gm.kps;
             at = lr * gm.reg + (row - lr * gm.kps) * gm.row;
@@ -322,7 +323,7 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
     };
     if (!gm.resident && nst > 0) load_stage(0);
     for (int st = 0; st < nst; ++st) {
-        if (st + 1 < nst) { load_stage(st + 1); cp_async_wait<1>(); } else cp_async_wait<0>();
+        simt_advance(gm, st, nst, load_stage);
         __syncthreads();
         const uint32_t abase = sbase + (st & 1) * gm.stage_bytes;
         if (!gm.resident) {

@@ -22,6 +22,7 @@ namespace sk {
 constexpr int THREADS = 256;            // at most: enough for a region, which shares the copies (64 if that is enough: an even tail)
 constexpr int RESIDENT_MAX = 100 * 1024;
 constexpr int IDX_MAX = 4096;           // routing entries kept in shared memory per CTA
+constexpr int SMEM_MAX = 220 * 1024;
 }  // namespace sk
 
 struct SimtGeom {
@@ -37,7 +38,8 @@ struct SimtGeom {
     int row;               // bytes of a row of one tensor in shared memory
     int reg;               // bytes from one region's rows of a stage to the next region's
     int zero;              // offset of a row of zeros in either tensor's rows
-    int off_a, off_b, off_stat, off_idx, off_cnt, off_w, off_st, stage_bytes, smem_bytes;
+    int off_a, off_b, off_stat, off_idx, off_cnt, off_w, off_st, smem_bytes;
+    int stage_bytes;       // from one stage to the next (0: there is one)
 };
 
 enum SimtKind { SIMT_ATTEND, SIMT_DQ, SIMT_DKV };
@@ -45,7 +47,8 @@ enum SimtKind { SIMT_ATTEND, SIMT_DQ, SIMT_DKV };
 // rows per lane: two where registers allow it (the dK / dV kernel keeps four rows of channels per key)
 inline int simt_rows(int head_dim, SimtKind kind) { return kind != SIMT_DKV && head_dim <= 32 ? 2 : 1; }
 
-inline SimtGeom simt_geom(const Dims& d, SimtKind kind) {
+// At most rpc_max regions per CTA; stages of the rows of the other side where they are not resident.
+inline SimtGeom simt_geom(const Dims& d, SimtKind kind, int rpc_max, int stages) {
     SimtGeom g;
     const int qt = simt_rows(d.d, kind);
     g.row = d.d * d.esize + 16;
@@ -72,6 +75,7 @@ inline SimtGeom simt_geom(const Dims& d, SimtKind kind) {
     g.rpc = g.chunks > 1 ? 1 : most / g.spr;
     if (g.rpc < 1) g.rpc = 1;
     if (g.rpc > d.R) g.rpc = d.R;
+    if (g.rpc > rpc_max) g.rpc = rpc_max;
     if ((long long)g.rpc * d.topk > sk::IDX_MAX) g.rpc = sk::IDX_MAX / d.topk > 0 ? sk::IDX_MAX / d.topk : 1;
     const int ctas = (d.R + g.rpc - 1) / g.rpc;                       // even out the regions over them
     g.rpc = (d.R + ctas - 1) / ctas;
@@ -88,7 +92,7 @@ inline SimtGeom simt_geom(const Dims& d, SimtKind kind) {
     if (g.kps < block) g.kps = block;
     if (g.kps > 32) g.kps = 32;
     g.mul_kps = recip32(g.kps);
-    g.stages = g.resident ? 1 : 2;
+    g.stages = g.resident ? 1 : stages;
     const int rows = g.resident ? d.N : g.rpc * g.kps;                // of one stage
     g.reg = (g.kps * g.row + 111) / 128 * 128 + 16;                   // 16 modulo 128
     int off = 0;
@@ -96,8 +100,9 @@ inline SimtGeom simt_geom(const Dims& d, SimtKind kind) {
     g.off_a = off;    off += g.zero + g.row;
     g.off_b = off;    off += g.zero + g.row;
     g.off_stat = off; off += kind == SIMT_DKV ? (rows * 8 + 15) / 16 * 16 : 0;     // lse, delta
-    g.stage_bytes = off;
+    g.stage_bytes = g.stages == 2 ? off : 0;
     off *= g.stages;
+    const int rows_end = off;
     g.off_idx = off;                                                  // (dK / dV: the lists are read through L1)
     if (kind != SIMT_DKV && (long long)g.rpc * d.topk <= sk::IDX_MAX) off += g.rpc * d.topk * 4;
     g.off_cnt = off;  off += g.dense ? g.rpc * d.R * 4 : 0;
@@ -105,13 +110,20 @@ inline SimtGeom simt_geom(const Dims& d, SimtKind kind) {
     off = (off + 15) / 16 * 16;
     g.off_st = 0;                                                     // over the rows, once they have been read
     const int st = kind != SIMT_DQ ? g.rpc * qt * g.spr * (d.d + 4) * 4 : 0;
-    if (st > g.stages * g.stage_bytes) { g.off_st = off; off += st; }
+    if (st > rows_end) { g.off_st = off; off += st; }
     g.smem_bytes = off;
+    return g;
+}
+// Two stages, so that the next rows arrive while these are used; where a region is a few tokens, nearly every lane has rows of
+// its own, and as many regions as fit are taken with one stage.
+inline SimtGeom simt_geom(const Dims& d, SimtKind kind) {
+    SimtGeom g = simt_geom(d, kind, sk::THREADS, 2);
+    for (int rpc = sk::THREADS; g.smem_bytes > sk::SMEM_MAX && rpc > 0; rpc /= 2) g = simt_geom(d, kind, rpc, 1);
     return g;
 }
 inline bool simt_fits(const Dims& d, SimtKind kind) {
     // (token numbers and positions in a walk are ints)
-    return d.B <= 65535 && d.heads <= 65534 && (long long)d.H * d.W < (1ll << 31) - 65536 && simt_geom(d, kind).smem_bytes <= 220 * 1024;
+    return d.B <= 65535 && d.heads <= 65534 && (long long)d.H * d.W < (1ll << 31) - 65536 && simt_geom(d, kind).smem_bytes <= sk::SMEM_MAX;
 }
 
 // Token (row-major in the caller's map) of token t of region r; -1 in the zero padding.
@@ -290,6 +302,15 @@ __device__ __forceinline__ void simt_zero_rows(uint8_t* smem, const SimtGeom& gm
         const int r = e / n, stage = r >> 1;
         *reinterpret_cast<uint4*>(smem + stage * gm.stage_bytes + (r & 1 ? gm.off_b : gm.off_a) + gm.zero + (e - r * n) * 16) = make_uint4(0, 0, 0, 0);
     }
+}
+
+// Stage `it` of a walk has arrived (for this thread's copies) and, with two stages, the next one is on its way.
+// load(i): starts the copies of stage i; stage 0 was started before.
+template <typename F>
+__device__ __forceinline__ void simt_advance(const SimtGeom& gm, int it, int n, F&& load) {
+    const int next = it + gm.stages - 1;
+    if (next > 0 && next < n) load(next);
+    if (next > it && next < n) ptx::cp_async_wait<1>(); else ptx::cp_async_wait<0>();
 }
 
 // LCE weights of a head as they lie in memory: [D channels][25] (odd stride: lane = channel reads without conflicts)

@@ -182,6 +182,21 @@ def test_large_regions_are_accepted(lib, call, kw):
     assert status_without_gpu(lib, call, **{"B": 1, **kw}) == 8
 
 
+def test_every_region_size_is_accepted(lib):
+    """fp32 has only the CUDA-core kernels, so they take every region size, list length and batch: no layout of their shared
+    memory is too large."""
+    for d in (16, 32, 64, 128):
+        for dtype in ("f32", "bf16"):
+            for hs, ws in ((1, 1), (1, 2), (2, 1), (2, 2), (1, 3), (3, 3), (2, 5), (4, 4), (3, 7), (8, 8), (7, 11), (16, 16), (1, 300), (40, 3)):
+                for S in (1, 2, 4, 7, 14, 16, 31):
+                    for topk in {1, min(4, S * S), S * S}:
+                        for B, heads in ((1, 1), (8, 2), (64, 4)):
+                            kw = dict(B=B, H=hs * S, W=ws * S, C=heads * d, heads=heads, S=S, topk=topk, dtype=dtype, impl=1)
+                            assert status_without_gpu(lib, "attend", **kw) == 8, kw
+                            if d <= 64 and S * S <= 1000:
+                                assert status_without_gpu(lib, "backward", **kw) == 8, kw
+
+
 def test_division_by_multiplication_is_exact(tmp_path):
     """csrc/fast_div.h on the host: every divisor of a spread, dividends next to every kind of multiple."""
     import subprocess

@@ -839,6 +839,15 @@ SIMT_EDGES = [
     (BraConfig("simt-padded-resident", 1, 9, 9, 64, 2, 8, 6, "f32"), "repeats"),
     (BraConfig("simt-bf16-d16", 1, 14, 13, 32, 2, 7, 4, "bf16"), "route"),
     (BraConfig("simt-576-regions", 1, 24, 24, 32, 1, 24, 3, "f32"), "repeats"),
+    # regions of one and two tokens with wide rows: one stage, as many regions as fit
+    (BraConfig("simt-d64-1x1-k1", 1, 4, 4, 64, 1, 4, 1, "f32"), "route"),
+    (BraConfig("simt-d64-1x1", 1, 14, 14, 64, 1, 14, 4, "f32"), "repeats"),
+    (BraConfig("simt-d64-1x1-one-lane", 64, 16, 16, 192, 3, 16, 4, "f32"), "route"),
+    (BraConfig("simt-d128-1x1", 1, 14, 14, 128, 1, 14, 4, "f32"), "repeats"),
+    (BraConfig("simt-d128-1x1-one-lane", 64, 16, 16, 384, 3, 16, 3, "f32"), "route"),
+    (BraConfig("simt-d128-1x2", 2, 14, 28, 256, 2, 14, 3, "f32"), "route"),
+    (BraConfig("simt-d128-2x1-bf16", 2, 28, 14, 256, 2, 14, 3, "bf16"), "repeats"),
+    (BraConfig("simt-d128-1x1-bf16", 2, 14, 14, 256, 2, 14, 3, "bf16"), "route"),
 ]
 
 

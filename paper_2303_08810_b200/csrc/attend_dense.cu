@@ -242,10 +242,14 @@ static cudaError_t launch_t(const Dims& d, const DenseGeom& g, const void* Q, co
         });
         if (e != cudaSuccess) return e;
     }
-    count_launch();
-    return launch_kernel(kernel, dim3(g.g.chunks, d.heads, d.B), dim3(g.nw * 32), (size_t)g.smem_bytes, st, after_own_kernel,
-                         static_cast<const __nv_bfloat16*>(Q), static_cast<const __nv_bfloat16*>(K), static_cast<const __nv_bfloat16*>(V),
-                         index, lce_w, lce_b, static_cast<__nv_bfloat16*>(O), lse, status, d, g);
+    typedef __nv_bfloat16 bf;
+    return grid_pieces(d, [&](const GridPiece& p) {
+        count_launch();
+        return launch_kernel(kernel, dim3(g.g.chunks, p.heads, p.images), dim3(g.nw * 32), (size_t)g.smem_bytes, st, after_own_kernel,
+                             static_cast<const bf*>(Q) + p.tensor, static_cast<const bf*>(K) + p.tensor, static_cast<const bf*>(V) + p.tensor,
+                             piece_of(index, p.index), piece_of(lce_w, p.channel * 25), piece_of(lce_b, p.channel), static_cast<bf*>(O) + p.tensor,
+                             piece_of(lse, p.stat), status, d, g);
+    });
 }
 
 cudaError_t launch_attend_dense(const Dims& d, const void* Q, const void* K, const void* V,

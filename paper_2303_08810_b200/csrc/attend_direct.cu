@@ -228,7 +228,7 @@ attend_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* 
 bool attend_direct_supported(const Dims& d, int dtype) {
     if (dtype != BRA_BF16 || (d.d != 32 && d.d != 64)) return false;
     if (d.ws > 128 || d.R > 65535 || d.n_r >= 1 << 25) return false;                      // fdiv() by ws and S
-    if ((long long)d.H0 * d.W0 * d.C / 8 >= (1ll << 31) || d.heads > 65535 || d.B > 65535) return false;
+    if ((long long)d.H0 * d.W0 * d.C / 8 >= (1ll << 31)) return false;
     return direct_geom(d, d.lce, 4, 1).smem_bytes <= 200 * 1024;
 }
 
@@ -243,10 +243,14 @@ static cudaError_t launch_t(const Dims& d, const DirGeom& g, const void* Q, cons
         });
         if (e != cudaSuccess) return e;
     }
-    count_launch();
-    return launch_kernel(kernel, dim3(g.gpi, d.heads, d.B), dim3(g.nw * 32), (size_t)g.smem_bytes, st, after_own_kernel,
-                         static_cast<const __nv_bfloat16*>(Q), static_cast<const __nv_bfloat16*>(K), static_cast<const __nv_bfloat16*>(V),
-                         index, lce_w, lce_b, static_cast<__nv_bfloat16*>(O), lse, status, d, g);
+    typedef __nv_bfloat16 bf;
+    return grid_pieces(d, [&](const GridPiece& p) {
+        count_launch();
+        return launch_kernel(kernel, dim3(g.gpi, p.heads, p.images), dim3(g.nw * 32), (size_t)g.smem_bytes, st, after_own_kernel,
+                             static_cast<const bf*>(Q) + p.tensor, static_cast<const bf*>(K) + p.tensor, static_cast<const bf*>(V) + p.tensor,
+                             index + p.index, piece_of(lce_w, p.channel * 25), piece_of(lce_b, p.channel), static_cast<bf*>(O) + p.tensor,
+                             piece_of(lse, p.stat), status, d, g);
+    });
 }
 
 cudaError_t launch_attend_direct(const Dims& d, const void* Q, const void* K, const void* V,

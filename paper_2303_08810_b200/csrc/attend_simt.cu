@@ -213,10 +213,13 @@ static cudaError_t launch_t(const Dims& d, const void* Q, const void* K, const v
         });
         if (e != cudaSuccess) return e;
     }
-    count_launch();
-    return launch_kernel(attend_simt_kernel<T, D>, dim3(g.gpi, d.heads, d.B), dim3(g.threads), (size_t)g.smem_bytes, st, after_own_kernel,
-                         static_cast<const T*>(Q), static_cast<const T*>(K), static_cast<const T*>(V), index, lce_w, lce_b,
-                         static_cast<T*>(O), lse, status, d, g);
+    return grid_pieces(d, [&](const GridPiece& p) {
+        count_launch();
+        return launch_kernel(attend_simt_kernel<T, D>, dim3(g.gpi, p.heads, p.images), dim3(g.threads), (size_t)g.smem_bytes, st, after_own_kernel,
+                             static_cast<const T*>(Q) + p.tensor, static_cast<const T*>(K) + p.tensor, static_cast<const T*>(V) + p.tensor,
+                             index + p.index, piece_of(lce_w, p.channel * 25), piece_of(lce_b, p.channel), static_cast<T*>(O) + p.tensor,
+                             piece_of(lse, p.stat), status, d, g);
+    });
 }
 
 template <typename T>

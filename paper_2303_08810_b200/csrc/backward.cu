@@ -31,7 +31,7 @@ bwd_dq_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
     constexpr int QT = D <= 32 ? 2 : 1, U = 2;                        // simt_rows()
     extern __shared__ __align__(128) uint8_t smem[];
     if (blockIdx.y == 0) {
-        if ((int)blockIdx.x < dm.heads_i)
+        if (inv_off && (int)blockIdx.x < dm.heads_i)
             inverse_index_job(index, inv_off, inv_list, inv_order, blockIdx.z * dm.heads_i + blockIdx.x, reinterpret_cast<int32_t*>(smem), inv_bits, dm);
         return;
     }
@@ -433,20 +433,27 @@ static cudaError_t launch_bwd_t(const Dims& d, int impl, const void* Q, const vo
                 return cudaFuncSetAttribute(bwd_dq_simt_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, g.smem_bytes);
             })) != cudaSuccess)
             return e;
-        e = launch_kernel(bwd_dq_simt_kernel<T, D>, dim3(g.gpi > d.heads_i ? g.gpi : d.heads_i, d.heads + 1, d.B), dim3(g.threads),
-                          (size_t)g.smem_bytes, st, false, q, k, v, index, lse, go, static_cast<T*>(dQ), delta, inv_off, inv_list, inv_order,
-                          inverse_uses_bits(d), status, d, g);
-        count_launch();
+        e = grid_pieces(d, [&](const GridPiece& p) {
+            const InversePiece inv = inverse_piece(d, p, inv_off, inv_list, inv_order);
+            count_launch();
+            return launch_kernel(bwd_dq_simt_kernel<T, D>, dim3(g.gpi > d.heads_i ? g.gpi : d.heads_i, p.heads + 1, p.images), dim3(g.threads),
+                                 (size_t)g.smem_bytes, st, false, q + p.tensor, k + p.tensor, v + p.tensor, index + p.index, lse + p.stat,
+                                 go + p.tensor, static_cast<T*>(dQ) + p.tensor, delta + p.stat, p.h0 ? nullptr : inv.off, inv.list, inv.order,
+                                 inverse_uses_bits(d), status, d, g);
+        });
         if (e != cudaSuccess) return e;
         const SimtGeom gk = simt_geom(d, SIMT_DKV);
         if (gk.smem_bytes > 48 * 1024 && (e = set_kv.ensure(gk.smem_bytes, [&] {
                 return cudaFuncSetAttribute(bwd_dkv_simt_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, gk.smem_bytes);
             })) != cudaSuccess)
             return e;
-        e = launch_kernel(bwd_dkv_simt_kernel<T, D>, dim3(d.heads, d.B, gk.gpi), dim3(gk.threads), (size_t)gk.smem_bytes, st, true,
-                          q, k, v, static_cast<const int32_t*>(inv_off), static_cast<const int32_t*>(inv_list), static_cast<const int32_t*>(inv_order), lse,
-                          static_cast<const float*>(delta), go, lce_w, static_cast<T*>(dK), static_cast<T*>(dV), d, gk);
-        count_launch();
+        e = group_pieces(d, gk.gpi, gk.chunks, [&](const GridPiece& p, int regions_before, int groups) {
+            const InversePiece inv = inverse_piece(d, p, inv_off, inv_list, inv_order);
+            count_launch();
+            return launch_kernel(bwd_dkv_simt_kernel<T, D>, dim3(p.heads, p.images, groups), dim3(gk.threads), (size_t)gk.smem_bytes, st, true,
+                                 q + p.tensor, k + p.tensor, v + p.tensor, inv.off, inv.list, inv.order + regions_before, lse + p.stat,
+                                 delta + p.stat, go + p.tensor, lce_w, static_cast<T*>(dK) + p.tensor, static_cast<T*>(dV) + p.tensor, d, gk);
+        });
         if (e != cudaSuccess) return e;
     }
 

@@ -320,10 +320,13 @@ static cudaError_t launch_t(const Dims& d, const DenseGeom& g, const void* Q, co
         if (e != cudaSuccess) return e;
     }
     typedef __nv_bfloat16 bf;
-    count_launch();
-    return launch_kernel(kernel, dim3(1, d.heads, d.B), dim3(g.nw * 32), (size_t)g.smem_bytes, st, false,
-                         static_cast<const bf*>(Q), static_cast<const bf*>(K), static_cast<const bf*>(V), index, lse, static_cast<const bf*>(dO),
-                         lce_w, static_cast<bf*>(dQ), static_cast<bf*>(dK), static_cast<bf*>(dV), status, d, g);
+    return grid_pieces(d, [&](const GridPiece& p) {
+        count_launch();
+        return launch_kernel(kernel, dim3(1, p.heads, p.images), dim3(g.nw * 32), (size_t)g.smem_bytes, st, false,
+                             static_cast<const bf*>(Q) + p.tensor, static_cast<const bf*>(K) + p.tensor, static_cast<const bf*>(V) + p.tensor,
+                             index + p.index, lse + p.stat, static_cast<const bf*>(dO) + p.tensor, piece_of(lce_w, p.channel * 25),
+                             static_cast<bf*>(dQ) + p.tensor, static_cast<bf*>(dK) + p.tensor, static_cast<bf*>(dV) + p.tensor, status, d, g);
+    });
 }
 
 cudaError_t launch_backward_dense(const Dims& d, const void* Q, const void* K, const void* V, const int32_t* index, const float* lce_w,

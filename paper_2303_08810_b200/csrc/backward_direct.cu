@@ -39,7 +39,7 @@ bwd_dq_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* 
     extern __shared__ __align__(128) uint8_t smem[];
     // blockIdx.y = 0: the inverse index (one CTA per (image, routing head)); else head blockIdx.y - 1
     if (blockIdx.y == 0) {
-        if ((int)blockIdx.x < dm.heads_i)
+        if (inv_off && (int)blockIdx.x < dm.heads_i)
             inverse_index_job(index, inv_off, inv_list, inv_order, blockIdx.z * dm.heads_i + blockIdx.x, reinterpret_cast<int32_t*>(smem), inv_bits, dm);
         return;
     }
@@ -415,7 +415,7 @@ static DirGeom dkv_geom(const Dims& d) {
 
 bool backward_direct_supported(const Dims& d, int dtype) {
     if (!attend_direct_supported(d, dtype)) return false;
-    return dkv_geom(d).smem_bytes <= 200 * 1024 && dq_geom(d).smem_bytes <= 200 * 1024 && d.R <= 8192 && dkv_geom(d).gpi <= 65535;
+    return dkv_geom(d).smem_bytes <= 200 * 1024 && dq_geom(d).smem_bytes <= 200 * 1024 && d.R <= 8192;
 }
 
 template <typename F>
@@ -444,9 +444,13 @@ static cudaError_t launch_dq(const Dims& d, const BwdArgs& a) {
     static PerDeviceMax set;
     const cudaError_t e = allow_smem(set, kernel, g.smem_bytes);
     if (e != cudaSuccess) return e;
-    count_launch();
-    return launch_kernel(kernel, dim3(g.gpi > d.heads_i ? g.gpi : d.heads_i, d.heads + 1, d.B), dim3(g.nw * 32), (size_t)g.smem_bytes, a.st, false,
-                         a.q, a.k, a.v, a.index, a.lse, a.go, a.dq, a.delta, a.inv_off, a.inv_list, a.inv_order, inverse_uses_bits(d), a.status, d, g);
+    return grid_pieces(d, [&](const GridPiece& p) {
+        const InversePiece inv = inverse_piece(d, p, a.inv_off, a.inv_list, a.inv_order);
+        count_launch();
+        return launch_kernel(kernel, dim3(g.gpi > d.heads_i ? g.gpi : d.heads_i, p.heads + 1, p.images), dim3(g.nw * 32), (size_t)g.smem_bytes, a.st,
+                             false, a.q + p.tensor, a.k + p.tensor, a.v + p.tensor, a.index + p.index, a.lse + p.stat, a.go + p.tensor,
+                             a.dq + p.tensor, a.delta + p.stat, p.h0 ? nullptr : inv.off, inv.list, inv.order, inverse_uses_bits(d), a.status, d, g);
+    });
 }
 
 template <int PL, bool EXACT, int TY, int TX>
@@ -456,9 +460,13 @@ static cudaError_t launch_dkv(const Dims& d, const BwdArgs& a) {
     static PerDeviceMax set;
     const cudaError_t e = allow_smem(set, kernel, g.smem_bytes);
     if (e != cudaSuccess) return e;
-    count_launch();
-    return launch_kernel(kernel, dim3(d.heads, d.B, g.gpi), dim3(g.nw * 32), (size_t)g.smem_bytes, a.st, true,
-                         a.q, a.k, a.v, a.inv_off, a.inv_list, a.inv_order, a.lse, a.delta, a.go, a.lce_w, a.dk, a.dv, d, g);
+    return group_pieces(d, g.gpi, g.chunks, [&](const GridPiece& p, int regions_before, int groups) {
+        const InversePiece inv = inverse_piece(d, p, a.inv_off, a.inv_list, a.inv_order);
+        count_launch();
+        return launch_kernel(kernel, dim3(p.heads, p.images, groups), dim3(g.nw * 32), (size_t)g.smem_bytes, a.st, true,
+                             a.q + p.tensor, a.k + p.tensor, a.v + p.tensor, inv.off, inv.list, inv.order + regions_before, a.lse + p.stat,
+                             a.delta + p.stat, a.go + p.tensor, a.lce_w, a.dk + p.tensor, a.dv + p.tensor, d, g);
+    });
 }
 
 static cudaError_t launch_both(const Dims& d, const BwdArgs& a) {

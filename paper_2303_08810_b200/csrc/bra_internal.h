@@ -32,6 +32,37 @@ struct Dims {
     int esize;    // bytes per element of Q, K, V, O
 };
 
+// A launch covers at most GRID_YZ heads, images or groups of regions (grid extents in y and z end at 65535, one row to spare);
+// larger problems are launched piece by piece, every piece with pointers to its first head and image.
+constexpr int GRID_YZ = 65534;
+struct GridPiece {
+    int heads, images;
+    size_t tensor;      // elements from the start of Q, K, V, O and their gradients
+    size_t index;       // entries from the start of the routing index
+    size_t stat;        // floats from the start of lse and delta
+    size_t channel;     // channels from the start of the LCE weights and bias
+    int h0, b0;
+};
+template <typename F>
+inline cudaError_t grid_pieces(const Dims& d, F&& launch) {
+    for (int h0 = 0; h0 < d.heads; h0 += GRID_YZ)
+        for (int b0 = 0; b0 < d.B; b0 += GRID_YZ) {
+            GridPiece p;
+            p.h0 = h0; p.b0 = b0;
+            p.heads = d.heads - h0 < GRID_YZ ? d.heads - h0 : GRID_YZ;
+            p.images = d.B - b0 < GRID_YZ ? d.B - b0 : GRID_YZ;
+            p.channel = (size_t)h0 * d.d;
+            p.tensor = (size_t)b0 * d.H0 * d.W0 * d.C + p.channel;
+            p.index = ((size_t)b0 * d.heads_i + (d.heads_i == 1 ? 0 : h0)) * d.R * d.topk;
+            p.stat = ((size_t)b0 * d.heads + h0) * d.H0 * d.W0;
+            const cudaError_t e = launch(p);
+            if (e != cudaSuccess) return e;
+        }
+    return cudaSuccess;
+}
+template <typename T>
+inline T* piece_of(T* p, size_t n) { return p ? p + n : nullptr; }
+
 // Scratch layout (byte offsets from ws, all multiples of 256).
 struct WsLayout {
     size_t status;      // int32[64]: [0] first device error, [1] detail

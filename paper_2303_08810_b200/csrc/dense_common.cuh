@@ -61,7 +61,7 @@ inline DenseGeom dense_geom(const Dims& d, int slices, int region_rows) {
 }
 
 inline bool dense_supported(const Dims& d, int dtype) {
-    return dtype == BRA_BF16 && d.d == 32 && d.R <= 64 && d.N <= 256 && d.heads <= 65535 && d.B <= 65535;
+    return dtype == BRA_BF16 && d.d == 32 && d.R <= 64 && d.N <= 256;
 }
 
 // slice row r, 16-byte chunk q: chunk index xor (r >> 1) & 3, conflict-free for ldmatrix and for 16-byte fragment reads

@@ -16,6 +16,31 @@ inline size_t inverse_smem(const Dims& d) {
     return sizeof(int32_t) * (2 * (size_t)d.R + 2 + (inverse_uses_bits(d) ? (size_t)d.R * inverse_words(d) : 0));
 }
 
+// The inverse index of the images of a piece.
+struct InversePiece { int32_t *off, *list, *order; };
+inline InversePiece inverse_piece(const Dims& d, const GridPiece& p, int32_t* off, int32_t* list, int32_t* order) {
+    const size_t bh = (size_t)p.b0 * d.heads_i;
+    return {off + bh * (d.R + 1), list + bh * d.R * d.topk, order + bh * d.R};
+}
+// Pieces of the dK / dV grids (heads, images, groups): all heads; `chunks` consecutive groups are a region, the first of a
+// piece region `regions_before` of the order.  (More groups than a grid holds: always one region per group or less.)
+template <typename F>
+inline cudaError_t group_pieces(const Dims& d, int groups, int chunks, F&& launch) {
+    if (chunks > GRID_YZ) return cudaErrorInvalidConfiguration;        // (a region of millions of tokens)
+    const int most = GRID_YZ / chunks * chunks;
+    Dims images = d;
+    images.heads = 1;                                       // x holds them all
+    for (int g0 = 0; g0 < groups; g0 += most) {
+        const cudaError_t e = grid_pieces(images, [&](GridPiece p) {
+            p.heads = d.heads;
+            p.stat = (size_t)p.b0 * d.heads * d.H0 * d.W0;
+            return launch(p, g0 / chunks, groups - g0 < most ? groups - g0 : most);
+        });
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 // One CTA.  A row of the index seldom names a region twice, so what has to be inverted is a bit matrix (key region x
 // query region): every entry sets a bit (atomics whose order does not matter), every key region counts and lists its
 // bits in ascending order: work proportional to the entries, where comparing every entry with every region took

@@ -123,7 +123,7 @@ inline SimtGeom simt_geom(const Dims& d, SimtKind kind) {
 }
 inline bool simt_fits(const Dims& d, SimtKind kind) {
     // (token numbers and positions in a walk are ints)
-    return d.B <= 65535 && d.heads <= 65534 && (long long)d.H * d.W < (1ll << 31) - 65536 && simt_geom(d, kind).smem_bytes <= sk::SMEM_MAX;
+    return (long long)d.H * d.W < (1ll << 31) - 65536 && simt_geom(d, kind).smem_bytes <= sk::SMEM_MAX;
 }
 
 // Token (row-major in the caller's map) of token t of region r; -1 in the zero padding.

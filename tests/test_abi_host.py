@@ -182,6 +182,15 @@ def test_large_regions_are_accepted(lib, call, kw):
     assert status_without_gpu(lib, call, **{"B": 1, **kw}) == 8
 
 
+@pytest.mark.parametrize("many", [dict(B=70000), dict(B=1, C=70000 * 32, heads=70000)], ids=["images", "heads"])
+@pytest.mark.parametrize("call", ["attend", "backward"])
+@pytest.mark.parametrize("kw", [dict(dtype="f32"), dict(dtype="bf16"), dict(dtype="bf16", H=7, W=7, S=7, topk=7)])
+def test_more_images_or_heads_than_a_grid_extent_are_accepted(lib, call, kw, many):
+    if "heads" not in many:
+        many = dict(many, C=32, heads=1)
+    assert status_without_gpu(lib, call, **{**dict(H=8, W=8, S=2, topk=2), **kw, **many}) == 8
+
+
 def test_every_region_size_is_accepted(lib):
     """fp32 has only the CUDA-core kernels, so they take every region size, list length and batch: no layout of their shared
     memory is too large."""

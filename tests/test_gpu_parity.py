@@ -1165,3 +1165,40 @@ def test_dense_kernels_by_token_match_the_oracle(bra, cfg):
     check_O(f64(O)[:, far], ref[:, far], "bf16")
     for name, a, r in zip(("dQ", "dK", "dV"), g, grads):
         assert np.abs(f64(a)[:, far] - r[:, far]).max() <= GRAD_MAX, name
+
+
+# ------------------------------------------------------------------ more images or heads than a grid holds in y or z
+@pytest.mark.parametrize("dtype,impl,d", [("f32", "simt", 16), ("bf16", "mma", 32), ("bf16", "auto", 32)])
+@pytest.mark.parametrize("many", ["images", "heads"])
+def test_more_images_or_heads_than_a_grid_extent(bra, dtype, impl, d, many):
+    """65 600 of them, 2 x 2 tokens each: the first and the last ones equal those of a problem of their own (another batch
+    size may share rows between lanes otherwise: sums in another order)."""
+    import torch
+    n, part = 65600, 40
+    B, heads = (n, 1) if many == "images" else (1, n)
+    dt = torch.float32 if dtype == "f32" else torch.bfloat16
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(5)
+    full = [torch.randn(B, 2, 2, heads * d, device="cuda", generator=gen).to(dt) for _ in range(4)]
+    idx = torch.randint(0, 4, (B, heads, 4, 2), dtype=torch.int32, device="cuda", generator=gen)
+
+    def run(x, idx):
+        B, heads = idx.shape[:2]
+        p = bra.make_problem(B, 2, 2, heads * d, heads, 2, 2, dtype, lce=False, impl=IMPLS[impl])
+        ws = bra.workspace(p)
+        O, lse = bra.bra_attend(p, x[0], x[1], x[2], idx, ws=ws)
+        g = bra.bra_backward(p, x[0], x[1], x[2], idx, None, lse, x[3], ws=ws)
+        assert bra.bra_device_status(ws) == 0
+        return (O,) + tuple(g[:3])
+
+    got = run(full, idx)
+    for cut in (slice(0, part), slice(n - part, n)):
+        if many == "images":
+            ref = run([t[cut].contiguous() for t in full], idx[cut].contiguous())
+            mine = [t[cut] for t in got]
+        else:
+            ch = slice(cut.start * d, cut.stop * d)
+            ref = run([t[..., ch].contiguous() for t in full], idx[:, cut].contiguous())
+            mine = [t[..., ch] for t in got]
+        for a, r in zip(mine, ref):
+            assert (a - r).float().norm() <= (4e-3 if dtype == "bf16" else 1e-6) * r.float().norm()

@@ -59,7 +59,10 @@ attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
     bool weighted = false;
     int32_t* cnt = reinterpret_cast<int32_t*>(smem + gm.off_cnt);
     if (gm.dense)
-        weighted = !simt_counts(cnt, nreg, dm.R, nreg * dm.topk, [&](int e) { const int r = s_idx[e]; return r < 0 ? -1 : e / dm.topk * dm.R + r; });
+        weighted = !simt_counts(cnt, nreg, dm.R, [&](auto add) {
+            for (int e = tid; e < nreg * dm.topk; e += blockDim.x)
+                if (s_idx[e] >= 0) add(e / dm.topk, s_idx[e]);
+        });
 
     // ---- this lane's rows: QT queries of one region, a share of the keys ----
     const int KS = 1 << gm.ksl, ks = tid & (KS - 1), slot = tid >> gm.ksl;

@@ -70,7 +70,10 @@ bwd_dq_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
     bool weighted = false;
     int32_t* cnt = reinterpret_cast<int32_t*>(smem + gm.off_cnt);
     if (gm.dense)
-        weighted = !simt_counts(cnt, nreg, dm.R, nreg * dm.topk, [&](int e) { const int r = s_idx[e]; return r < 0 ? -1 : e / dm.topk * dm.R + r; });
+        weighted = !simt_counts(cnt, nreg, dm.R, [&](auto add) {
+            for (int e = tid; e < nreg * dm.topk; e += blockDim.x)
+                if (s_idx[e] >= 0) add(e / dm.topk, s_idx[e]);
+        });
 
     const int KS = 1 << gm.ksl, ks = tid & (KS - 1), slot = tid >> gm.ksl;
     const int rl_raw = fdiv(slot, gm.spr, gm.mul_spr);
@@ -237,9 +240,11 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
     int32_t* cnt = reinterpret_cast<int32_t*>(smem + gm.off_cnt);
     if (gm.dense) {
         __syncthreads();
-        weighted = !simt_counts(cnt, nreg, dm.R, nreg * dm.R * dm.topk, [&](int e) {     // (topk == R: few entries)
-            const int l = e / (dm.R * dm.topk), j = __ldcg(order + l), at = __ldcg(offs + j) + e - l * dm.R * dm.topk;
-            return at < __ldcg(offs + j + 1) ? l * dm.R + __ldcg(list + at) : -1;
+        weighted = !simt_counts(cnt, nreg, dm.R, [&](auto add) {      // eight lanes per list
+            for (int l = tid >> 3; l < nreg; l += blockDim.x >> 3) {
+                const int j = __ldcg(order + l), end = __ldcg(offs + j + 1);
+                for (int at = __ldcg(offs + j) + (tid & 7); at < end; at += 8) add(l, __ldcg(list + at));
+            }
         });
     }
     const int t0 = active ? slot - rl_raw * gm.spr : 0;

@@ -390,16 +390,13 @@ bool in_x[TS + 4];
     }
 }
 
-// How often each region is named by the list of each region of the CTA: cnt[rl][R]; true if every count is one.
-// entry_at(e): rl * R + region, -1 for no region.
-template <typename EntryAt>
-__device__ __forceinline__ bool simt_counts(int32_t* cnt, int nreg, int R, int entries, EntryAt&& entry_at) {
+// How often each region is named by the list of each region of the CTA: cnt[rl][R], counted by count(add) where add(rl, region);
+// true if every count is one.
+template <typename Count>
+__device__ __forceinline__ bool simt_counts(int32_t* cnt, int nreg, int R, Count&& count) {
     for (int e = threadIdx.x; e < nreg * R; e += blockDim.x) cnt[e] = 0;
     __syncthreads();
-    for (int e = threadIdx.x; e < entries; e += blockDim.x) {
-        const int at = entry_at(e);
-        if (at >= 0) atomicAdd(cnt + at, 1);
-    }
+    count([&](int rl, int r) { atomicAdd(cnt + rl * R + r, 1); });
     __syncthreads();
     bool ones = true;
     for (int e = threadIdx.x; e < nreg * R; e += blockDim.x) ones = ones && cnt[e] == 1;

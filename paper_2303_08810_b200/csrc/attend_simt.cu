@@ -31,8 +31,8 @@ attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
     const T* Q = Qg + head; const T* K = Kg + head; const T* V = Vg + head;
     float* s_w = reinterpret_cast<float*>(smem + gm.off_w);
     if (dm.lce) simt_load_weights(s_w, lce_w + (size_t)h * D * 25, 25 * D);
-    simt_zero_rows(smem, gm);
     if (gm.resident) {
+        simt_zero_rows(smem, gm);
         simt_copy_rows<T, D>(sbase + gm.off_a, sbase + gm.off_b, K, V, dm.C, dm.N, [&](int row, uint32_t& at) {
             const int r = fdiv(row, gm.by_nr);
             at = row * gm.row;
@@ -82,8 +82,8 @@ attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
     }
     const int total = dm.topk * dm.n_r;
 
-    // keys [k0, k1): rows from offset at0 on, in order (PLAIN), or row_of(kk, wt): offset of the row in shared memory (-1: the
-    // key does not count) and its weight.  The reference maximum follows the scores only when one lies 16 above it (P and its sums
+    // keys [k0, k1): rows from offset at0 on, in order (PLAIN), or row_of(kk, dead, wt): offset of the row in shared memory (of
+    // zeros if the key does not count) and its weight.  The reference maximum follows the scores only when one lies 16 above it (P and its sums
     // are fp32: any reference gives the same relative precision), so that the sums are seldom rescaled.
     auto walk = [&](auto plain, uint32_t abase, uint32_t at0, int k0, int k1, auto&& row_of) {
         constexpr bool PLAIN = decltype(plain)::value;
@@ -99,13 +99,11 @@ attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
                 const int kk = k0 + (blk * U + u) * KS + ks;
                 dead[u] = kk >= k1;
                 if constexpr (PLAIN) {
-                    at[u] = dead[u] ? abase + gm.zero : next;
+                    at[u] = dead[u] && gm.resident ? abase + gm.zero : next;
                     next += KS * gm.row;
                 } else {
                     wt[u] = 1.f;
-                    const int row = dead[u] ? -1 : row_of(kk, wt[u]);
-                    dead[u] = row < 0;
-                    at[u] = abase + (dead[u] ? gm.zero : row);
+                    at[u] = abase + row_of(kk, dead[u], wt[u]);
                 }
             }
             dots<T, QT, U, D>(s, q, at, gm.off_a);
@@ -161,15 +159,19 @@ attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
         if (gm.resident ? gm.dense && !weighted : !bad)
             walk(std::true_type(), abase, gm.resident ? 0 : rl * gm.reg, k0, gm.resident ? dm.N : min(total, k0 + gm.kps), 0);
         else
-            walk(std::false_type(), abase, 0, k0, gm.dense ? dm.N : gm.resident ? total : min(total, k0 + gm.kps), [&](int kk, float& wt) -> int {
+            walk(std::false_type(), abase, 0, k0, gm.dense ? dm.N : gm.resident ? total : min(total, k0 + gm.kps), [&](int kk, bool& dead, float& wt) -> int {
+                const int none = gm.resident ? gm.zero : rl * gm.reg + (kk - k0) * gm.row;
+                if (dead) return none;
                 const int m = fdiv(kk, gm.by_nr);
                 if (gm.dense) {
                     const int n = cnt[rl * dm.R + m];
                     wt = (float)n;
-                    return n > 0 ? kk * gm.row : -1;
+                    dead = n == 0;
+                    return dead ? none : kk * gm.row;
                 }
                 const int r = entry(rl * dm.topk + m);
-                return r < 0 ? -1 : gm.resident ? (r * dm.n_r + kk - m * dm.n_r) * gm.row : rl * gm.reg + (kk - k0) * gm.row;
+                dead = r < 0;
+                return dead || !gm.resident ? none : (r * dm.n_r + kk - m * dm.n_r) * gm.row;
             });
         __syncthreads();
     }

@@ -45,8 +45,8 @@ bwd_dq_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
     const int N0 = dm.H0 * dm.W0;
     const size_t head = (size_t)b * N0 * dm.C + (size_t)h * D;
     const T* K = Kg + head; const T* V = Vg + head;
-    simt_zero_rows(smem, gm);
     if (gm.resident) {
+        simt_zero_rows(smem, gm);
         simt_copy_rows<T, D>(sbase + gm.off_a, sbase + gm.off_b, K, V, dm.C, dm.N, [&](int row, uint32_t& at) {
             const int r = fdiv(row, gm.by_nr);
             at = row * gm.row;
@@ -109,13 +109,11 @@ bwd_dq_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
                 const int kk = k0 + (blk * U + u) * KS + ks;
                 dead[u] = kk >= k1;
                 if constexpr (PLAIN) {
-                    at[u] = dead[u] ? abase + gm.zero : next;
+                    at[u] = dead[u] && gm.resident ? abase + gm.zero : next;
                     next += KS * gm.row;
                 } else {
                     wt[u] = 1.f;
-                    const int row = dead[u] ? -1 : row_of(kk, wt[u]);
-                    dead[u] = row < 0;
-                    at[u] = abase + (dead[u] ? gm.zero : row);
+                    at[u] = abase + row_of(kk, dead[u], wt[u]);
                 }
             }
             dots<T, QT, U, D>(s, q, at, gm.off_a);
@@ -167,15 +165,19 @@ bwd_dq_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
         if (gm.resident ? gm.dense && !weighted : !bad)
             walk(std::true_type(), abase, gm.resident ? 0 : rl * gm.reg, k0, gm.resident ? dm.N : min(total, k0 + gm.kps), it >= nst, 0);
         else
-            walk(std::false_type(), abase, 0, k0, gm.dense ? dm.N : gm.resident ? total : min(total, k0 + gm.kps), it >= nst, [&](int kk, float& wt) -> int {
+            walk(std::false_type(), abase, 0, k0, gm.dense ? dm.N : gm.resident ? total : min(total, k0 + gm.kps), it >= nst, [&](int kk, bool& dead, float& wt) -> int {
+                const int none = gm.resident ? gm.zero : rl * gm.reg + (kk - k0) * gm.row;
+                if (dead) return none;
                 const int m = fdiv(kk, gm.by_nr);
                 if (gm.dense) {
                     const int n = cnt[rl * dm.R + m];
                     wt = (float)n;
-                    return n > 0 ? kk * gm.row : -1;
+                    dead = n == 0;
+                    return dead ? none : kk * gm.row;
                 }
                 const int r = entry(rl * dm.topk + m);
-                return r < 0 ? -1 : gm.resident ? (r * dm.n_r + kk - m * dm.n_r) * gm.row : rl * gm.reg + (kk - k0) * gm.row;
+                dead = r < 0;
+                return dead || !gm.resident ? none : (r * dm.n_r + kk - m * dm.n_r) * gm.row;
             });
         if (it == nst - 1) end_of_first();
         __syncthreads();
@@ -211,8 +213,8 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
     const T* Q = Qg + head; const T* dO = dOg + head;
     float* s_w = reinterpret_cast<float*>(smem + gm.off_w);
     if (dm.lce) simt_load_weights(s_w, lce_w + (size_t)h * D * 25, 25 * D);
-    simt_zero_rows(smem, gm);
     if (gm.resident) {
+        simt_zero_rows(smem, gm);
         simt_copy_rows<T, D>(sbase + gm.off_a, sbase + gm.off_b, Q, dO, dm.C, dm.N, [&](int row, uint32_t& at) {
             const int r = fdiv(row, gm.by_nr);
             at = row * gm.row;
@@ -269,7 +271,7 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
             bool dead = kk >= n;
             float wt = 1.f;
             if constexpr (PLAIN) {
-                if (dead) { at = abase + gm.zero; at_stat = abase + gm.off_stat; }
+                if (dead && gm.resident) { at = abase + gm.zero; at_stat = abase + gm.off_stat; }
                 next += KS * gm.row;
                 next_stat += KS * 8;
             } else {

@@ -37,7 +37,7 @@ struct SimtGeom {
     uint32_t mul_spr, mul_kps, mul_cw;
     int row;               // bytes of a row of one tensor in shared memory
     int reg;               // bytes from one region's rows of a stage to the next region's
-    int zero;              // offset of a row of zeros in either tensor's rows
+    int zero;              // resident: offset of a row of zeros in either tensor's rows
     int off_a, off_b, off_stat, off_idx, off_cnt, off_w, off_st, smem_bytes;
     int stage_bytes;       // from one stage to the next (0: there is one)
 };
@@ -97,8 +97,8 @@ inline SimtGeom simt_geom(const Dims& d, SimtKind kind, int rpc_max, int stages)
     g.reg = (g.kps * g.row + 111) / 128 * 128 + 16;                   // 16 modulo 128
     int off = 0;
     g.zero = g.resident ? rows * g.row : g.rpc * g.reg;
-    g.off_a = off;    off += g.zero + g.row;
-    g.off_b = off;    off += g.zero + g.row;
+    g.off_a = off;    off += g.zero + (g.resident ? g.row : 0);
+    g.off_b = off;    off += g.zero + (g.resident ? g.row : 0);
     g.off_stat = off; off += kind == SIMT_DKV ? (rows * 8 + 15) / 16 * 16 : 0;     // lse, delta
     g.stage_bytes = g.stages == 2 ? off : 0;
     off *= g.stages;
@@ -294,14 +294,12 @@ __device__ __forceinline__ void simt_copy_rows(uint32_t dst_a, uint32_t dst_b, c
     }
 }
 
-// The rows that stand in for keys (queries) that do not count: their probability is 0, but 0 times an infinity or NaN of some
-// other region's row would not be.
+// Keys (queries) that do not count have the probability 0 and must read zeros: 0 times an infinity or NaN of some other region's
+// row would not be 0.  In a stage they have rows of zeros in their own places (tok_at() says -1); a resident slice has one here.
 __device__ __forceinline__ void simt_zero_rows(uint8_t* smem, const SimtGeom& gm) {
     const int n = gm.row / 16;
-    for (int e = threadIdx.x; e < 2 * gm.stages * n; e += blockDim.x) {
-        const int r = e / n, stage = r >> 1;
-        *reinterpret_cast<uint4*>(smem + stage * gm.stage_bytes + (r & 1 ? gm.off_b : gm.off_a) + gm.zero + (e - r * n) * 16) = make_uint4(0, 0, 0, 0);
-    }
+    for (int e = threadIdx.x; e < 2 * n; e += blockDim.x)
+        *reinterpret_cast<uint4*>(smem + (e < n ? gm.off_a + e * 16 : gm.off_b + (e - n) * 16) + gm.zero) = make_uint4(0, 0, 0, 0);
 }
 
 // Stage `it` of a walk has arrived (for this thread's copies) and, with two stages, the next one is on its way.

@@ -201,6 +201,7 @@ __global__ void __launch_bounds__(sk::THREADS, 1)
 bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* __restrict__ Vg, const int32_t* inv_off,
                     const int32_t* inv_list, const int32_t* inv_order, const float* __restrict__ lse, const float* delta, const T* __restrict__ dOg,
                     const float* __restrict__ lce_w, T* __restrict__ dKg, T* __restrict__ dVg, Dims dm, SimtGeom gm) {
+    constexpr int SPLIT = D > 32 ? 1 : 0, DL = D >> SPLIT;            // simt_split(); channels of a lane
     extern __shared__ __align__(128) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
     const int tid = threadIdx.x;
@@ -231,7 +232,8 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
     const int32_t* list = inv_list + bhi * dm.R * dm.topk;
     const float* lse_h = lse + ((size_t)b * dm.heads + h) * N0;
     const float* delta_h = delta + ((size_t)b * dm.heads + h) * N0;
-    const int KS = 1 << gm.ksl, ks = tid & (KS - 1), slot = tid >> gm.ksl;
+    const int KS = 1 << gm.ksl, ks = tid & (KS - 1), slot = tid >> (gm.ksl + SPLIT);
+    const int c0 = SPLIT ? (tid >> gm.ksl & 1) * DL : 0;              // this lane's first channel
     const int rl_raw = fdiv(slot, gm.spr, gm.mul_spr);
     const bool active = rl_raw < nreg;
     const int rl = active ? rl_raw : 0;
@@ -251,13 +253,13 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
     }
     const int t0 = active ? slot - rl_raw * gm.spr : 0;
     const int tok = active ? simt_row(dm, gm, chunk, jr, t0) : -1;
-    float kr[D], vr[D], gk[1][D], gv[1][D];
+    float kr[DL], vr[DL], gk[1][DL], gv[1][DL];
     {
-        const size_t at = head + (size_t)(tok < 0 ? 0 : tok) * dm.C;
-        ldg_row<T, D>(kr, Kg + at, tok >= 0, dm.scale);
-        ldg_row<T, D>(vr, Vg + at, tok >= 0, 1.f);
+        const size_t at = head + (size_t)(tok < 0 ? 0 : tok) * dm.C + c0;
+        ldg_row<T, DL>(kr, Kg + at, tok >= 0, dm.scale);
+        ldg_row<T, DL>(vr, Vg + at, tok >= 0, 1.f);
 #pragma unroll
-        for (int i = 0; i < D; ++i) gk[0][i] = gv[0][i] = 0.f;
+        for (int i = 0; i < DL; ++i) gk[0][i] = gv[0][i] = 0.f;
     }
     // statistics of a row: lse and delta; a row that does not count has lse = inf (P = 0); a row of the zero padding has
     // zero Q and dO and lse = delta = 0 and adds nothing
@@ -281,11 +283,15 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
                 at_stat = abase + gm.off_stat + (dead ? 0 : row) * 8;
             }
             const float2 stat = lds_f32x2(at_stat);
-            float g[D], qv[D];
-            lds_row<T, D>(qv, at + gm.off_a);
-            lds_row<T, D>(g, at + gm.off_b);
-            const float dp = dot4(vr, g);
-            float p = expf(dot(qv, kr) - stat.x);
+            float g[DL], qv[DL];
+            lds_row<T, DL>(qv, at + gm.off_a + c0 * (int)sizeof(T));
+            lds_row<T, DL>(g, at + gm.off_b + c0 * (int)sizeof(T));
+            float dp = dot4(vr, g), s = dot(qv, kr);
+            if (SPLIT) {
+                dp += __shfl_xor_sync(0xffffffffu, dp, KS);
+                s += __shfl_xor_sync(0xffffffffu, s, KS);
+            }
+            float p = expf(s - stat.x);
             if (!PLAIN && weighted) p *= wt;
             float ds = p * (dp - stat.y);
             if (dead) p = ds = 0.f;
@@ -353,17 +359,17 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
         __syncthreads();
     }
     int first, held;
-    sum_shares<1, D>(gk, gm.ksl, ks, &first, &held);
-    sum_shares<1, D>(gv, gm.ksl, ks, &first, &held);
+    sum_shares<1, DL>(gk, gm.ksl, ks, &first, &held);
+    sum_shares<1, DL>(gv, gm.ksl, ks, &first, &held);
     cp_async_wait<0>();
     __syncthreads();
     float* st = reinterpret_cast<float*>(smem + gm.off_st);
     if (tok >= 0) {
-        for_held<1, D>(gk, first, held, [&](int, int c, const float4& v) {
-            store4(dKg + head + (size_t)tok * dm.C + c, make_float4(v.x * dm.scale, v.y * dm.scale, v.z * dm.scale, v.w * dm.scale));
+        for_held<1, DL>(gk, first, held, [&](int, int c, const float4& v) {
+            store4(dKg + head + (size_t)tok * dm.C + c0 + c, make_float4(v.x * dm.scale, v.y * dm.scale, v.z * dm.scale, v.w * dm.scale));
         });
-        for_held<1, D>(gv, first, held, [&](int, int c, const float4& v) {
-            *reinterpret_cast<float4*>(st + (rl * gm.spr + t0) * (D + 4) + c) = v;
+        for_held<1, DL>(gv, first, held, [&](int, int c, const float4& v) {
+            *reinterpret_cast<float4*>(st + (rl * gm.spr + t0) * (D + 4) + c0 + c) = v;
         });
     }
     __syncthreads();

@@ -46,6 +46,9 @@ enum SimtKind { SIMT_ATTEND, SIMT_DQ, SIMT_DKV };
 
 // rows per lane: two where registers allow it (the dK / dV kernel keeps four rows of channels per key)
 inline int simt_rows(int head_dim, SimtKind kind) { return kind != SIMT_DKV && head_dim <= 32 ? 2 : 1; }
+// log2 of the lanes that hold a row's channels: a dK / dV lane with the four rows of 64 channels spilled 2 KB of registers
+// (gradients at 64 x 14 x 14, 4 heads of 64, topk 16: 1048 us)
+inline int simt_split(int head_dim, SimtKind kind) { return kind == SIMT_DKV && head_dim > 32 ? 1 : 0; }
 
 // At most rpc_max regions per CTA; stages of the rows of the other side where they are not resident.
 inline SimtGeom simt_geom(const Dims& d, SimtKind kind, int rpc_max, int stages) {
@@ -57,11 +60,13 @@ inline SimtGeom simt_geom(const Dims& d, SimtKind kind, int rpc_max, int stages)
     // (dK / dV of larger maps: as if an eighth of the regions held the lists, which is what clustered content comes to;
     // measured at 1 x 96 x 96, S = 7, 2 heads: 522 -> 224 us; at 36 x 14 x 14 it costs more than it gives)
     const long long lanes = (long long)d.B * d.heads * d.R * ((d.n_r + qt - 1) / qt) / (kind == SIMT_DKV && d.N > 400 ? 8 : 1);
+    const int split = simt_split(d.d, kind);
     g.ksl = 0;
-    while (g.ksl < 3 && (lanes << g.ksl) < kSMs * 256 && (qt * d.d >> (g.ksl + 1)) >= 4) ++g.ksl;    // sum_shares: whole float4s
+    while (g.ksl < 3 && (lanes << (g.ksl + split)) < kSMs * 256 && (qt * d.d >> (g.ksl + split + 1)) >= 4) ++g.ksl;    // sum_shares: whole float4s
+    const int group = g.ksl + split;                                  // log2 of the lanes of a group
     int threads = 64;
-    while (threads < sk::THREADS && ((d.n_r + qt - 1) / qt << g.ksl) > threads) threads *= 2;
-    const int most = threads >> g.ksl;                                // lane groups of a CTA
+    while (threads < sk::THREADS && ((d.n_r + qt - 1) / qt << group) > threads) threads *= 2;
+    const int most = threads >> group;                                // lane groups of a CTA
     g.hb = d.hs; g.cw = d.ws;
     if ((d.n_r + qt - 1) / qt > most) {
         if (g.cw > qt * most) g.cw = qt * most;
@@ -80,7 +85,7 @@ inline SimtGeom simt_geom(const Dims& d, SimtKind kind, int rpc_max, int stages)
     const int ctas = (d.R + g.rpc - 1) / g.rpc;                       // even out the regions over them
     g.rpc = (d.R + ctas - 1) / ctas;
     g.mul_spr = recip32(g.spr);
-    g.threads = ((g.rpc * g.spr << g.ksl) + 31) / 32 * 32;
+    g.threads = ((g.rpc * g.spr << group) + 31) / 32 * 32;
     g.gpi = ctas * g.chunks;
     const long long slice = 2ll * d.N * g.row;
     // copies of the slice against copies of the listed rows (a key region is listed topk times on average)

@@ -119,10 +119,13 @@ inline SimtGeom simt_geom(const Dims& d, SimtKind kind, int rpc_max, int stages)
     g.smem_bytes = off;
     return g;
 }
-// Two stages, so that the next rows arrive while these are used; where a region is a few tokens, nearly every lane has rows of
-// its own, and as many regions as fit are taken with one stage.
+// Two stages, so that the next rows arrive while these are used, if three CTAs of them fit on an SM.  Else one: more CTAs hide
+// more than the second stage does (attention, one / two stages: 64 x 14 x 14, 2 heads of 128, topk 16: 247 / 511 us;
+// 64 x 28 x 28, S = 14, 2 heads of 32: 91 / 138; below the line 16 x 64 x 64, S = 16, 2 heads of 32: 234 / 227; 64 x 40 x 24, S = 8,
+// 2 heads of 64: 308 / 293).  Where a region is a few tokens, nearly every lane has rows of its own: as many regions as fit.
 inline SimtGeom simt_geom(const Dims& d, SimtKind kind) {
     SimtGeom g = simt_geom(d, kind, sk::THREADS, 2);
+    if (g.stages * g.stage_bytes > 72 * 1024) g = simt_geom(d, kind, sk::THREADS, 1);
     for (int rpc = sk::THREADS; g.smem_bytes > sk::SMEM_MAX && rpc > 0; rpc /= 2) g = simt_geom(d, kind, rpc, 1);
     return g;
 }

@@ -239,7 +239,7 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
     const int rl = active ? rl_raw : 0;
     const int jr = __ldcg(order + rl);                                // this lane's key region
     const int e0 = __ldcg(offs + jr), listed = __ldcg(offs + jr + 1) - e0;              // its query regions
-    const long long warp_total = (long long)__reduce_max_sync(0xffffffffu, listed) * dm.n_r;    // (with repeats a list may be long)
+    const int warp_listed = __reduce_max_sync(0xffffffffu, listed);
     bool weighted = false;
     int32_t* cnt = reinterpret_cast<int32_t*>(smem + gm.off_cnt);
     if (gm.dense) {
@@ -299,7 +299,7 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
             axpy(gv[0], p, g);
         }
     };
-    long long most = 0;                                               // queries of the CTA's longest list
+    int most = 0;                                                     // entries of the CTA's longest list
     if (gm.resident) {
         float2* stat = reinterpret_cast<float2*>(smem + gm.off_stat);
         for (int row = tid; row < dm.N; row += blockDim.x) {
@@ -309,18 +309,17 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
         }
     } else {
         const int j = __ldcg(order);                                  // the first has the longest list
-        most = (long long)(__ldcg(offs + j + 1) - __ldcg(offs + j)) * dm.n_r;
+        most = __ldcg(offs + j + 1) - __ldcg(offs + j);
     }
-    const int nst = gm.resident ? 1 : (int)((most + gm.kps - 1) / gm.kps);
-    int m0 = 0, q0 = 0;                                               // list entry and token of the next stage's first query
+    int first_entry = 0;                                              // of the walk
     auto load_stage = [&](int st) {
         const int off = (st & 1) * gm.stage_bytes;
         const uint32_t base = sbase + off;
         float2* stat = reinterpret_cast<float2*>(smem + off + gm.off_stat);
         simt_copy_rows<T, D>(base + gm.off_a, base + gm.off_b, Q, dO, dm.C, nreg * gm.kps, [&](int row, uint32_t& at) {
-            const int lr = fdiv(row, gm.kps, gm.mul_kps), u = q0 + row - lr * gm.kps;
+            const int lr = fdiv(row, gm.kps, gm.mul_kps), u = st * gm.kps + row - lr * gm.kps;
             at = lr * gm.reg + (row - lr * gm.kps) * gm.row;
-            const int j = __ldcg(order + lr), m = fdiv(u, gm.by_nr), s0 = __ldcg(offs + j) + m0 + m;
+            const int j = __ldcg(order + lr), m = fdiv(u, gm.by_nr), s0 = __ldcg(offs + j) + first_entry + m;
             int tk = -1;
             float2 v = make_float2(INFINITY, 0.f);
             if (s0 < __ldcg(offs + j + 1)) {
@@ -331,33 +330,36 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
             return tk;
         });
         cp_async_commit();
-        const int u = q0 + gm.kps, m = fdiv(u, gm.by_nr);
-        m0 += m; q0 = u - m * dm.n_r;
     };
-    if (!gm.resident && nst > 0) load_stage(0);
-    for (int st = 0; st < nst; ++st) {
-        simt_advance(gm, st, nst, load_stage);
-        __syncthreads();
-        const uint32_t abase = sbase + (st & 1) * gm.stage_bytes;
-        if (!gm.resident) {
-            const long long rest = warp_total - (long long)st * gm.kps;
-            if (rest > 0) walk(std::true_type(), abase, rl * gm.reg, rl * gm.kps, (int)min(rest, (long long)gm.kps), 0);
-        } else if (gm.dense && !weighted) {
-            walk(std::true_type(), abase, 0, 0, dm.N, 0);
-        } else {
-            const int mine = listed * dm.n_r;                         // (a resident slice: a few hundred tokens)
-            walk(std::false_type(), abase, 0, 0, gm.dense ? dm.N : (int)warp_total, [&](int kk, float& wt) -> int {
-                const int m = fdiv(kk, gm.by_nr);
-                if (gm.dense) {
-                    const int n = cnt[rl * dm.R + m];
-                    wt = (float)n;
-                    return n > 0 ? kk : -1;
-                }
-                return kk < mine ? __ldcg(list + e0 + m) * dm.n_r + kk - m * dm.n_r : -1;
-            });
+    do {
+        const int nst = gm.resident ? 1 : (min(most - first_entry, gm.span) * dm.n_r + gm.kps - 1) / gm.kps;
+        const int warp_total = min(warp_listed - first_entry, gm.span) * dm.n_r;
+        if (!gm.resident) load_stage(0);
+        for (int st = 0; st < nst; ++st) {
+            simt_advance(gm, st, nst, load_stage);
+            __syncthreads();
+            const uint32_t abase = sbase + (st & 1) * gm.stage_bytes;
+            if (!gm.resident) {
+                const int rest = warp_total - st * gm.kps;
+                if (rest > 0) walk(std::true_type(), abase, rl * gm.reg, rl * gm.kps, min(rest, gm.kps), 0);
+            } else if (gm.dense && !weighted) {
+                walk(std::true_type(), abase, 0, 0, dm.N, 0);
+            } else {
+                const int mine = listed * dm.n_r;                         // (a resident slice: a few hundred tokens)
+                walk(std::false_type(), abase, 0, 0, gm.dense ? dm.N : warp_total, [&](int kk, float& wt) -> int {
+                    const int m = fdiv(kk, gm.by_nr);
+                    if (gm.dense) {
+                        const int n = cnt[rl * dm.R + m];
+                        wt = (float)n;
+                        return n > 0 ? kk : -1;
+                    }
+                    return kk < mine ? __ldcg(list + e0 + m) * dm.n_r + kk - m * dm.n_r : -1;
+                });
+            }
+            __syncthreads();
         }
-        __syncthreads();
-    }
+        first_entry += gm.span;
+    } while (first_entry < most);
     int first, held;
     sum_shares<1, DL>(gk, gm.ksl, ks, &first, &held);
     sum_shares<1, DL>(gv, gm.ksl, ks, &first, &held);

@@ -33,6 +33,7 @@ struct SimtGeom {
     int threads, gpi;      // the grid is (gpi, heads, images)
     int resident, dense;   // dense: topk == R, walk every region and weigh it by how often the list names it
     int kps, stages;       // rows of the other side per region and stage
+    int span;              // dK / dV: entries of a list per walk (their rows are counted in 32 bits)
     FastDiv by_nr, by_ws, by_s;
     uint32_t mul_spr, mul_kps, mul_cw;
     int row;               // bytes of a row of one tensor in shared memory
@@ -50,8 +51,9 @@ inline int simt_rows(int head_dim, SimtKind kind) { return kind != SIMT_DKV && h
 // (gradients at 64 x 14 x 14, 4 heads of 64, topk 16: 1048 us)
 inline int simt_split(int head_dim, SimtKind kind) { return kind == SIMT_DKV && head_dim > 32 ? 1 : 0; }
 
-// At most rpc_max regions per CTA; stages of the rows of the other side where they are not resident.
-inline SimtGeom simt_geom(const Dims& d, SimtKind kind, int rpc_max, int stages) {
+// At most rpc_max regions per CTA; stages of the rows of the other side where they are not resident; threads that a CTA has
+// unless one region wants more.
+inline SimtGeom simt_geom(const Dims& d, SimtKind kind, int rpc_max, int stages, int threads = 64) {
     SimtGeom g;
     const int qt = simt_rows(d.d, kind);
     g.row = d.d * d.esize + 16;
@@ -64,7 +66,6 @@ inline SimtGeom simt_geom(const Dims& d, SimtKind kind, int rpc_max, int stages)
     g.ksl = 0;
     while (g.ksl < 3 && (lanes << (g.ksl + split)) < kSMs * 256 && (qt * d.d >> (g.ksl + split + 1)) >= 4) ++g.ksl;    // sum_shares: whole float4s
     const int group = g.ksl + split;                                  // log2 of the lanes of a group
-    int threads = 64;
     while (threads < sk::THREADS && ((d.n_r + qt - 1) / qt << group) > threads) threads *= 2;
     const int most = threads >> group;                                // lane groups of a CTA
     g.hb = d.hs; g.cw = d.ws;
@@ -97,6 +98,7 @@ inline SimtGeom simt_geom(const Dims& d, SimtKind kind, int rpc_max, int stages)
     if (g.kps < block) g.kps = block;
     if (g.kps > 32) g.kps = 32;
     g.mul_kps = recip32(g.kps);
+    g.span = (1 << 30) / d.n_r + 1;
     g.stages = g.resident ? 1 : stages;
     const int rows = g.resident ? d.N : g.rpc * g.kps;                // of one stage
     g.reg = (g.kps * g.row + 111) / 128 * 128 + 16;                   // 16 modulo 128
@@ -125,6 +127,9 @@ inline SimtGeom simt_geom(const Dims& d, SimtKind kind, int rpc_max, int stages)
 // 2 heads of 64: 308 / 293).  Where a region is a few tokens, nearly every lane has rows of its own: as many regions as fit.
 inline SimtGeom simt_geom(const Dims& d, SimtKind kind) {
     SimtGeom g = simt_geom(d, kind, sk::THREADS, 2);
+    // resident: twice the threads make half the copies of the slice (64 x 14 x 14, 2 heads of 32, attention, S = 14, topk 8: 62 -> 47 us,
+    // S = 7, topk 16: 43 -> 35; dK / dV, whose lists differ in length: 104 to 107 %)
+    if (g.resident && kind != SIMT_DKV) g = simt_geom(d, kind, sk::THREADS, 2, 128);
     if (g.stages * g.stage_bytes > 72 * 1024) g = simt_geom(d, kind, sk::THREADS, 1);
     for (int rpc = sk::THREADS; g.smem_bytes > sk::SMEM_MAX && rpc > 0; rpc /= 2) g = simt_geom(d, kind, rpc, 1);
     return g;

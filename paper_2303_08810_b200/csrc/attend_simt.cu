@@ -13,12 +13,13 @@ namespace bra {
 
 using namespace ptx;
 
-template <typename T, int D>
-__global__ void __launch_bounds__(sk::THREADS, D <= 16 ? 2 : 1)
+// FAR: rows of K and V straight from global memory (simt_far()).
+template <typename T, int D, bool FAR>
+__global__ void __launch_bounds__(FAR ? 128 : sk::THREADS, FAR ? (D <= 64 ? 3 : 2) : D <= 16 ? 2 : 1)
 attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* __restrict__ Vg, const int32_t* index,
                    const float* __restrict__ lce_w, const float* __restrict__ lce_b, T* __restrict__ Og, float* __restrict__ lse,
                    int32_t* __restrict__ status, Dims dm, SimtGeom gm) {
-    constexpr int QT = D <= 32 ? 2 : 1, U = 4;                        // simt_rows()
+    constexpr int QT = D <= 32 && !FAR ? 2 : 1, U = 4;                // simt_rows()
     extern __shared__ __align__(128) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
     const int tid = threadIdx.x;
@@ -31,7 +32,7 @@ attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
     const T* Q = Qg + head; const T* K = Kg + head; const T* V = Vg + head;
     float* s_w = reinterpret_cast<float*>(smem + gm.off_w);
     if (dm.lce) simt_load_weights(s_w, lce_w + (size_t)h * D * 25, 25 * D);
-    if (gm.resident) {
+    if (!FAR && gm.resident) {
         simt_zero_rows(smem, gm);
         simt_copy_rows<T, D>(sbase + gm.off_a, sbase + gm.off_b, K, V, dm.C, dm.N, [&](int row, uint32_t& at) {
             const int r = fdiv(row, gm.by_nr);
@@ -58,7 +59,7 @@ attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
     bad = __syncthreads_or(bad);
     bool weighted = false;
     int32_t* cnt = reinterpret_cast<int32_t*>(smem + gm.off_cnt);
-    if (gm.dense)
+    if (!FAR && gm.dense)
         weighted = !simt_counts(cnt, nreg, dm.R, [&](auto add) {
             for (int e = tid; e < nreg * dm.topk; e += blockDim.x)
                 if (s_idx[e] >= 0) add(e / dm.topk, s_idx[e]);
@@ -88,17 +89,20 @@ attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
     auto walk = [&](auto plain, uint32_t abase, uint32_t at0, int k0, int k1, auto&& row_of) {
         constexpr bool PLAIN = decltype(plain)::value;
         const int blocks = (k1 - k0 + U * KS - 1) / (U * KS);
-        uint32_t next = abase + at0 + ks * gm.row;
+        [[maybe_unused]] uint32_t next = abase + at0 + ks * gm.row;
 #pragma unroll 1
         for (int blk = 0; blk < blocks; ++blk) {
-            uint32_t at[U];
+            [[maybe_unused]] uint32_t at[U];
+            [[maybe_unused]] int row[U];                              // FAR: token
             bool dead[U];
             float s[QT][U], wt[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int kk = k0 + (blk * U + u) * KS + ks;
                 dead[u] = kk >= k1;
-                if constexpr (PLAIN) {
+                if constexpr (FAR) {
+                    row[u] = row_of(kk, dead[u], wt[u]);
+                } else if constexpr (PLAIN) {
                     at[u] = dead[u] && gm.resident ? abase + gm.zero : next;
                     next += KS * gm.row;
                 } else {
@@ -106,7 +110,8 @@ attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
                     at[u] = abase + row_of(kk, dead[u], wt[u]);
                 }
             }
-            dots<T, QT, U, D>(s, q, at, gm.off_a);
+            if constexpr (FAR) dots_far<T>(s, q, K, row, dm.C);
+            else dots<T, QT, U, D>(s, q, at, gm.off_a);
 #pragma unroll
             for (int x = 0; x < QT; ++x) {
 #pragma unroll
@@ -124,56 +129,68 @@ attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     s[x][u] = expf(s[x][u] - mn);
-                    if (!PLAIN && weighted) s[x][u] *= wt[u];
+                    if (!FAR && !PLAIN && weighted) s[x][u] *= wt[u];
                     l_run[x] += s[x][u];
                 }
             }
+            if constexpr (FAR) axpy_far<T>(o, s, V, row, dm.C);
+            else {
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                float v[D];
-                lds_row<T, D>(v, at[u] + gm.off_b);
+                for (int u = 0; u < U; ++u) {
+                    float v[D];
+                    lds_row<T, D>(v, at[u] + gm.off_b);
 #pragma unroll
-                for (int x = 0; x < QT; ++x) axpy(o[x], s[x][u], v);
+                    for (int x = 0; x < QT; ++x) axpy(o[x], s[x][u], v);
+                }
             }
         }
     };
-    const int nst = gm.resident ? 1 : (total + gm.kps - 1) / gm.kps;
-    auto load_stage = [&](int st) {
-        const uint32_t base = sbase + (st & 1) * gm.stage_bytes;
-        simt_copy_rows<T, D>(base + gm.off_a, base + gm.off_b, K, V, dm.C, nreg * gm.kps, [&](int row, uint32_t& at) {
-            const int l = fdiv(row, gm.kps, gm.mul_kps), kk = st * gm.kps + row - l * gm.kps;
-            at = l * gm.reg + (row - l * gm.kps) * gm.row;
-            if (kk >= total) return -1;
-            const int m = fdiv(kk, gm.by_nr);
-            const int r = entry(l * dm.topk + m);
-            return r >= 0 ? simt_token(dm, gm, r, kk - m * dm.n_r) : -1;
+    if constexpr (FAR) {
+        walk(std::false_type(), 0, 0, 0, total, [&](int kk, bool& dead, float&) -> int {
+            if (dead) return -1;
+            const int m = fdiv(kk, gm.by_nr), r = entry(rl * dm.topk + m);
+            dead = r < 0;
+            return dead ? -1 : simt_token(dm, gm, r, kk - m * dm.n_r);        // (-1 in the zero padding: a row of zeros that counts)
         });
-        cp_async_commit();
-    };
-    if (!gm.resident) load_stage(0);
-    for (int st = 0; st < nst; ++st) {
-        simt_advance(gm, st, nst, load_stage);
-        __syncthreads();
-        const uint32_t abase = sbase + (st & 1) * gm.stage_bytes;
-        const int k0 = gm.resident ? 0 : st * gm.kps;
-        if (gm.resident ? gm.dense && !weighted : !bad)
-            walk(std::true_type(), abase, gm.resident ? 0 : rl * gm.reg, k0, gm.resident ? dm.N : min(total, k0 + gm.kps), 0);
-        else
-            walk(std::false_type(), abase, 0, k0, gm.dense ? dm.N : gm.resident ? total : min(total, k0 + gm.kps), [&](int kk, bool& dead, float& wt) -> int {
-                const int none = gm.resident ? gm.zero : rl * gm.reg + (kk - k0) * gm.row;
-                if (dead) return none;
+    } else {
+        const int nst = gm.resident ? 1 : (total + gm.kps - 1) / gm.kps;
+        auto load_stage = [&](int st) {
+            const uint32_t base = sbase + (st & 1) * gm.stage_bytes;
+            simt_copy_rows<T, D>(base + gm.off_a, base + gm.off_b, K, V, dm.C, nreg * gm.kps, [&](int row, uint32_t& at) {
+                const int l = fdiv(row, gm.kps, gm.mul_kps), kk = st * gm.kps + row - l * gm.kps;
+                at = l * gm.reg + (row - l * gm.kps) * gm.row;
+                if (kk >= total) return -1;
                 const int m = fdiv(kk, gm.by_nr);
-                if (gm.dense) {
-                    const int n = cnt[rl * dm.R + m];
-                    wt = (float)n;
-                    dead = n == 0;
-                    return dead ? none : kk * gm.row;
-                }
-                const int r = entry(rl * dm.topk + m);
-                dead = r < 0;
-                return dead || !gm.resident ? none : (r * dm.n_r + kk - m * dm.n_r) * gm.row;
+                const int r = entry(l * dm.topk + m);
+                return r >= 0 ? simt_token(dm, gm, r, kk - m * dm.n_r) : -1;
             });
-        __syncthreads();
+            cp_async_commit();
+        };
+        if (!gm.resident) load_stage(0);
+        for (int st = 0; st < nst; ++st) {
+            simt_advance(gm, st, nst, load_stage);
+            __syncthreads();
+            const uint32_t abase = sbase + (st & 1) * gm.stage_bytes;
+            const int k0 = gm.resident ? 0 : st * gm.kps;
+            if (gm.resident ? gm.dense && !weighted : !bad)
+                walk(std::true_type(), abase, gm.resident ? 0 : rl * gm.reg, k0, gm.resident ? dm.N : min(total, k0 + gm.kps), 0);
+            else
+                walk(std::false_type(), abase, 0, k0, gm.dense ? dm.N : gm.resident ? total : min(total, k0 + gm.kps), [&](int kk, bool& dead, float& wt) -> int {
+                    const int none = gm.resident ? gm.zero : rl * gm.reg + (kk - k0) * gm.row;
+                    if (dead) return none;
+                    const int m = fdiv(kk, gm.by_nr);
+                    if (gm.dense) {
+                        const int n = cnt[rl * dm.R + m];
+                        wt = (float)n;
+                        dead = n == 0;
+                        return dead ? none : kk * gm.row;
+                    }
+                    const int r = entry(rl * dm.topk + m);
+                    dead = r < 0;
+                    return dead || !gm.resident ? none : (r * dm.n_r + kk - m * dm.n_r) * gm.row;
+                });
+            __syncthreads();
+        }
     }
 
     // ---- merge the key shares; normalise; stage; lse ----
@@ -198,29 +215,28 @@ attend_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T* 
         });
     __syncthreads();
     const float* bias = dm.lce && lce_b ? lce_b + h * D : nullptr;
-    if (dm.hs <= 2) simt_lce<T, D, 2, false>(st, s_w, bias, V, Og + head, SimtFrom{r0}, nreg, QT * gm.spr, chunk, dm, gm);
-    else simt_lce<T, D, 4, false>(st, s_w, bias, V, Og + head, SimtFrom{r0}, nreg, QT * gm.spr, chunk, dm, gm);
+    if (FAR ? dm.n_r == 1 : dm.hs <= 2) simt_lce<T, D, FAR ? 1 : 2, false>(st, s_w, bias, V, Og + head, SimtFrom{r0}, nreg, QT * gm.spr, chunk, dm, gm);
+    else simt_lce<T, D, FAR ? 2 : 4, false>(st, s_w, bias, V, Og + head, SimtFrom{r0}, nreg, QT * gm.spr, chunk, dm, gm);
 }
 
 bool attend_simt_supported(const Dims& d) {
     return (d.d == 16 || d.d == 32 || d.d == 64 || d.d == 128) && simt_fits(d, SIMT_ATTEND);
 }
 
-template <typename T, int D>
+template <typename T, int D, bool FAR>
 static cudaError_t launch_t(const Dims& d, const void* Q, const void* K, const void* V,
                             const int32_t* index, const float* lce_w, const float* lce_b,
-                            void* O, float* lse, int32_t* status, cudaStream_t st, bool after_own_kernel) {
-    const SimtGeom g = simt_geom(d, SIMT_ATTEND);
+                            void* O, float* lse, int32_t* status, cudaStream_t st, bool after_own_kernel, const SimtGeom& g) {
     static PerDeviceMax smem_set;
     if (g.smem_bytes > 48 * 1024) {
         const cudaError_t e = smem_set.ensure(g.smem_bytes, [&] {
-            return cudaFuncSetAttribute(attend_simt_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, g.smem_bytes);
+            return cudaFuncSetAttribute(attend_simt_kernel<T, D, FAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, g.smem_bytes);
         });
         if (e != cudaSuccess) return e;
     }
     return grid_pieces(d, [&](const GridPiece& p) {
         count_launch();
-        return launch_kernel(attend_simt_kernel<T, D>, dim3(g.gpi, p.heads, p.images), dim3(g.threads), (size_t)g.smem_bytes, st, after_own_kernel,
+        return launch_kernel(attend_simt_kernel<T, D, FAR>, dim3(g.gpi, p.heads, p.images), dim3(g.threads), (size_t)g.smem_bytes, st, after_own_kernel,
                              static_cast<const T*>(Q) + p.tensor, static_cast<const T*>(K) + p.tensor, static_cast<const T*>(V) + p.tensor,
                              index + p.index, piece_of(lce_w, p.channel * 25), piece_of(lce_b, p.channel), static_cast<T*>(O) + p.tensor,
                              piece_of(lse, p.stat), status, d, g);
@@ -231,12 +247,12 @@ template <typename T>
 static cudaError_t launch_d(const Dims& d, const void* Q, const void* K, const void* V,
                             const int32_t* index, const float* lce_w, const float* lce_b,
                             void* O, float* lse, int32_t* status, cudaStream_t st, bool after_own_kernel) {
-    switch (d.d) {
-        case 16:  return launch_t<T, 16>(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel);
-        case 32:  return launch_t<T, 32>(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel);
-        case 64:  return launch_t<T, 64>(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel);
-        case 128: return launch_t<T, 128>(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel);
-    }
+    const SimtGeom g = simt_geom(d, SIMT_ATTEND);
+#define BRA_GO(D)                                                                                                                     \
+    case D: return g.far ? launch_t<T, D, true>(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel, g)             \
+                         : launch_t<T, D, false>(d, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel, g)
+    switch (d.d) { BRA_GO(16); BRA_GO(32); BRA_GO(64); BRA_GO(128); }
+#undef BRA_GO
     return cudaErrorInvalidValue;
 }
 

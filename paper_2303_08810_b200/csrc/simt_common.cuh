@@ -31,6 +31,7 @@ struct SimtGeom {
     int rpc, spr;          // regions per CTA; lane groups (QT rows each) per region (of a full chunk)
     int ksl;               // log2 of the lanes that share rows
     int threads, gpi;      // the grid is (gpi, heads, images)
+    int far;               // rows straight from global memory (simt_far())
     int resident, dense;   // dense: topk == R, walk every region and weigh it by how often the list names it
     int kps, stages;       // rows of the other side per region and stage
     int span;              // dK / dV: entries of a list per walk (their rows are counted in 32 bits)
@@ -45,8 +46,14 @@ struct SimtGeom {
 
 enum SimtKind { SIMT_ATTEND, SIMT_DQ, SIMT_DKV };
 
+// Attention over regions of one or two tokens: the lanes of a CTA share no rows of K and V, and rows staged for each of them leave
+// an SM two to four warps.  They read their rows straight from global memory (attend_simt_kernel<T, D, true>), unless every
+// region is routed to and the slice is resident.  Measured (B200, us, staged / straight / one thread per query without shared key
+// lanes): 64 x 14 x 14, S = 14, topk 8: 1 head of 64 127 / 46 / 63, 1 head of 128 512 / 93 / 127, 2 heads of 32 (resident) 47 / 43 / 56;
+// 64 x 16 x 16, S = 16, topk 4, 2 heads of 32 86 / 41 / 46; 64 x 28 x 14, S = 14, topk 8, 2 heads of 32 77 / 68 / 81.
+inline bool simt_far(const Dims& d, SimtKind kind) { return kind == SIMT_ATTEND && d.n_r <= 2 && !(d.topk == d.R && d.R <= 64); }
 // rows per lane: two where registers allow it (the dK / dV kernel keeps four rows of channels per key)
-inline int simt_rows(int head_dim, SimtKind kind) { return kind != SIMT_DKV && head_dim <= 32 ? 2 : 1; }
+inline int simt_rows(const Dims& d, SimtKind kind) { return kind != SIMT_DKV && d.d <= 32 && !simt_far(d, kind) ? 2 : 1; }
 // log2 of the lanes that hold a row's channels: a dK / dV lane with the four rows of 64 channels spilled 2 KB of registers
 // (gradients at 64 x 14 x 14, 4 heads of 64, topk 16: 1048 us)
 inline int simt_split(int head_dim, SimtKind kind) { return kind == SIMT_DKV && head_dim > 32 ? 1 : 0; }
@@ -55,7 +62,8 @@ inline int simt_split(int head_dim, SimtKind kind) { return kind == SIMT_DKV && 
 // unless one region wants more.
 inline SimtGeom simt_geom(const Dims& d, SimtKind kind, int rpc_max, int stages, int threads = 64) {
     SimtGeom g;
-    const int qt = simt_rows(d.d, kind);
+    const int qt = simt_rows(d, kind);
+    g.far = simt_far(d, kind);
     g.row = d.d * d.esize + 16;
     g.by_nr = fast_div(d.n_r); g.by_ws = fast_div(d.ws); g.by_s = fast_div(d.S);
     // lanes of this call against the lanes the GPU holds at once (12 warps per SM)
@@ -90,7 +98,7 @@ inline SimtGeom simt_geom(const Dims& d, SimtKind kind, int rpc_max, int stages,
     g.gpi = ctas * g.chunks;
     const long long slice = 2ll * d.N * g.row;
     // copies of the slice against copies of the listed rows (a key region is listed topk times on average)
-    g.resident = slice <= sk::RESIDENT_MAX && (long long)g.rpc * d.topk * d.n_r >= d.N;
+    g.resident = !g.far && slice <= sk::RESIDENT_MAX && (long long)g.rpc * d.topk * d.n_r >= d.N;
     g.dense = g.resident && d.topk == d.R && d.R <= 64;
     const int block = 4 << g.ksl;
     // about 64 rows of two tensors per stage (18 KB at D = 32, fp32), in whole blocks of four per lane
@@ -100,10 +108,10 @@ inline SimtGeom simt_geom(const Dims& d, SimtKind kind, int rpc_max, int stages,
     g.mul_kps = recip32(g.kps);
     g.span = (1 << 30) / d.n_r + 1;
     g.stages = g.resident ? 1 : stages;
-    const int rows = g.resident ? d.N : g.rpc * g.kps;                // of one stage
+    const int rows = g.far ? 0 : g.resident ? d.N : g.rpc * g.kps;    // of one stage
     g.reg = (g.kps * g.row + 111) / 128 * 128 + 16;                   // 16 modulo 128
     int off = 0;
-    g.zero = g.resident ? rows * g.row : g.rpc * g.reg;
+    g.zero = g.far ? 0 : g.resident ? rows * g.row : g.rpc * g.reg;
     g.off_a = off;    off += g.zero + (g.resident ? g.row : 0);
     g.off_b = off;    off += g.zero + (g.resident ? g.row : 0);
     g.off_stat = off; off += kind == SIMT_DKV ? (rows * 8 + 15) / 16 * 16 : 0;     // lse, delta
@@ -129,7 +137,7 @@ inline SimtGeom simt_geom(const Dims& d, SimtKind kind) {
     SimtGeom g = simt_geom(d, kind, sk::THREADS, 2);
     // resident: twice the threads make half the copies of the slice (64 x 14 x 14, 2 heads of 32, attention, S = 14, topk 8: 62 -> 47 us,
     // S = 7, topk 16: 43 -> 35; dK / dV, whose lists differ in length: 104 to 107 %)
-    if (g.resident && kind != SIMT_DKV) g = simt_geom(d, kind, sk::THREADS, 2, 128);
+    if ((g.resident && kind != SIMT_DKV) || g.far) g = simt_geom(d, kind, sk::THREADS, 2, 128);
     if (g.stages * g.stage_bytes > 72 * 1024) g = simt_geom(d, kind, sk::THREADS, 1);
     for (int rpc = sk::THREADS; g.smem_bytes > sk::SMEM_MAX && rpc > 0; rpc /= 2) g = simt_geom(d, kind, rpc, 1);
     return g;
@@ -215,6 +223,52 @@ __device__ __forceinline__ void dots(float (&s)[QT][U], const float (&q)[QT][N],
             for (int u = 0; u < U; ++u)
 #pragma unroll
                 for (int x = 0; x < QT; ++x) s[x][u] = fmaf(q[x][c + i], k[u][i], s[x][u]);
+    }
+}
+// 16 bytes of a row in global memory; zeros if there is no row
+template <typename T>
+__device__ __forceinline__ void ldg_chunk(float (&v)[16 / sizeof(T)], const T* p, bool ok) {
+    if (ok) load_row<16 / (int)sizeof(T)>(p, v);
+    else
+#pragma unroll
+        for (int i = 0; i < 16 / (int)sizeof(T); ++i) v[i] = 0.f;
+}
+// s[x][u] = q[x] . row tok[u] of a head in global memory (no row: 0)
+template <typename T, int QT, int U, int N>
+__device__ __forceinline__ void dots_far(float (&s)[QT][U], const float (&q)[QT][N], const T* head, const int (&tok)[U], int C) {
+    constexpr int CH = 16 / (int)sizeof(T);
+#pragma unroll
+    for (int x = 0; x < QT; ++x)
+#pragma unroll
+        for (int u = 0; u < U; ++u) s[x][u] = 0.f;
+#pragma unroll
+    for (int c = 0; c < N; c += CH) {
+        float k[U][CH];
+#pragma unroll
+        for (int u = 0; u < U; ++u) ldg_chunk(k[u], head + (size_t)max(tok[u], 0) * C + c, tok[u] >= 0);
+#pragma unroll
+        for (int i = 0; i < CH; ++i)
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int x = 0; x < QT; ++x) s[x][u] = fmaf(q[x][c + i], k[u][i], s[x][u]);
+    }
+}
+// acc[x] += sum of f[x][u] row tok[u]
+template <typename T, int QT, int U, int N>
+__device__ __forceinline__ void axpy_far(float (&acc)[QT][N], const float (&f)[QT][U], const T* head, const int (&tok)[U], int C) {
+    constexpr int CH = 16 / (int)sizeof(T);
+#pragma unroll
+    for (int c = 0; c < N; c += CH) {
+        float v[U][CH];
+#pragma unroll
+        for (int u = 0; u < U; ++u) ldg_chunk(v[u], head + (size_t)max(tok[u], 0) * C + c, tok[u] >= 0);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int i = 0; i < CH; ++i)
+#pragma unroll
+                for (int x = 0; x < QT; ++x) acc[x][c + i] = fmaf(f[x][u], v[u][i], acc[x][c + i]);
     }
 }
 template <int N>

@@ -848,6 +848,9 @@ SIMT_EDGES = [
     (BraConfig("simt-d128-1x2", 2, 14, 28, 256, 2, 14, 3, "f32"), "route"),
     (BraConfig("simt-d128-2x1-bf16", 2, 28, 14, 256, 2, 14, 3, "bf16"), "repeats"),
     (BraConfig("simt-d128-1x1-bf16", 2, 14, 14, 256, 2, 14, 3, "bf16"), "route"),
+    (BraConfig("simt-d16-1x1", 64, 14, 14, 32, 2, 14, 8, "f32"), "route"),
+    (BraConfig("simt-padded-1x2", 2, 6, 11, 32, 1, 6, 5, "f32"), "route"),
+    (BraConfig("simt-padded-1x1-d64", 2, 5, 6, 64, 1, 6, 5, "f32"), "repeats"),
 ]
 
 
@@ -1090,6 +1093,8 @@ SIMT_ISOLATION = [
     BraConfig("alone-staged-d64-chunks", 1, 51, 51, 64, 1, 3, 2, "f32"),
     BraConfig("alone-cut-map-f32", 2, 29, 27, 64, 2, 4, 3, "f32"),
     BraConfig("alone-bf16-d16", 2, 12, 20, 32, 2, 4, 5, "bf16"),
+    BraConfig("alone-1x1", 2, 6, 6, 64, 2, 6, 7, "f32"),
+    BraConfig("alone-cut-1x2", 2, 6, 11, 64, 1, 6, 6, "f32"),
 ]
 
 

@@ -812,6 +812,7 @@ DIRECT_EDGES = [
     (BraConfig("direct-padded-rows-of-whole-regions", 2, 9, 9, 64, 2, 8, 6, "bf16"), "repeats"),
     (BraConfig("direct-529-regions", 1, 23, 23, 32, 1, 23, 3, "bf16"), "repeats"),          # inverse index: bits / comparisons
     (BraConfig("direct-576-regions", 1, 24, 24, 32, 1, 24, 3, "bf16"), "repeats"),
+    (BraConfig("direct-961-regions", 1, 31, 31, 64, 2, 31, 5, "bf16"), "repeats"),
 ]
 
 

@@ -385,9 +385,9 @@ enum Family { FAMILY_SIMT, FAMILY_DIRECT, FAMILY_IMG, FAMILY_DENSE };
 // whole slice resident (head dim 32); the rest take their operands straight from global memory.
 static Family choose_family(const Dims& d, int dtype, int impl) {
     if (dtype != BRA_BF16 || impl == BRA_IMPL_SIMT) return FAMILY_SIMT;
-    if (impl == BRA_IMPL_AUTO && backward_dense_supported(d, dtype) && dense_pays(d, 2 * kSMs)) return FAMILY_DENSE;
+    if (impl == BRA_IMPL_AUTO && backward_dense_supported(d, dtype) && dense_grad_pays(d)) return FAMILY_DENSE;
     if (backward_img_supported(d, dtype) &&
-        (impl == BRA_IMPL_IMG || (impl == BRA_IMPL_AUTO && img_pays(d))))
+        (impl == BRA_IMPL_IMG || (impl == BRA_IMPL_AUTO && img_grad_pays(d))))
         return FAMILY_IMG;
     return backward_direct_supported(d, dtype) ? FAMILY_DIRECT : FAMILY_SIMT;
 }

@@ -131,7 +131,7 @@ static Path choose_attend(const Dims& d, int dtype, int impl) {
     }
     if (attend_tc_supported(d, dtype)) return PATH_TC;
     if (attend_tc_wide_supported(d, dtype)) return PATH_TC_WIDE;
-    if (attend_dense_supported(d, dtype) && dense_pays(d, 64)) return PATH_DENSE;
+    if (attend_dense_supported(d, dtype) && dense_pays(d)) return PATH_DENSE;
     if (attend_img_supported(d, dtype) && img_pays(d)) return PATH_IMG;
     if (attend_direct_supported(d, dtype)) return PATH_DIRECT;
     if (attend_simt_supported(d)) return PATH_SIMT;

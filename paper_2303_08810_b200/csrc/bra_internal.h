@@ -136,18 +136,34 @@ cudaError_t launch_attend_dense(const Dims& d, const void* Q, const void* K, con
                                 const int32_t* index, const float* lce_w, const float* lce_b,
                                 void* O, float* lse, int32_t* status, cudaStream_t st, bool after_own_kernel);
 // true if the dense kernels are the faster ones: they walk all tokens of the map for 16 queries at a time, the routed ones
-// topk regions for a tile of one region, n_r of whose 16 rows are used.  With more than 64 tokens a CTA's walk is long and
-// wants `pairs` (image, head) pairs to fill the GPU.  Measured (B200, us, dense against the best other kernel), attention /
-// gradients, 14 x 14 map, 49 regions, topk 16, 8 heads: 512 pairs 44 / 103 against 44 / 156, 128 pairs 17 / 53 against
-// 25 / 47, 32 pairs 14 / 36 against 11 / 28; 7 x 7 map, topk 49, 16 heads: 1024 pairs 27 / 41 against 120 / 282, 16 pairs
-// 17 / 25 against 11 / 28.
-inline bool dense_pays(const Dims& d, int pairs) {
-    return (long long)d.N < (long long)d.topk * ((d.n_r + 15) / 16 * 16) && (d.N <= 64 || (long long)d.B * d.heads >= pairs);
+// topk regions for a tile of one region, n_r of whose 16 rows are used.  Measured (B200, us, dense / direct).
+// Above 64 tokens a CTA's walk is long and wants (image, head) pairs to fill the GPU.  14 x 14, 49 regions, topk 16: attention
+// 64 pairs 10.6 / 14.6, 32 pairs 14 / 8; gradients 296 pairs 54 / 94, 128 pairs 53 / 46.
+inline bool dense_fewer_rows(const Dims& d) { return (long long)d.N < (long long)d.topk * ((d.n_r + 15) / 16 * 16); }
+inline bool dense_grad_pays(const Dims& d) {
+    return dense_fewer_rows(d) && (d.N <= 64 || (long long)d.B * d.heads >= 2 * kSMs);   // up to 64 tokens, 4 pairs, topk 8: 11.2 / 12.0
 }
-// true if there are enough (image, head) pairs for the kernels with one CTA each.  Measured, 28 x 28 map, 4 heads, topk 4,
-// attention / gradients against the kernels with a CTA per region: 256 pairs 43 / 103 against 50 / 112, 64 pairs 31 / 50
-// against 19 / 36.
-inline bool img_pays(const Dims& d) { return (long long)d.B * d.heads >= kSMs; }
+// Up to 64 tokens: the direct kernel has a warp per region and is the faster one while they fit on the GPU at once (12 per SM):
+// 7 x 7, topk 16: 16 pairs 8.2 / 6.2, 32 pairs 8.2 / 6.9, 48 pairs 8.3 / 11.2; 8 x 8, 2 x 2 regions, topk 8: 96 pairs 7.1 / 7.1,
+// 192 pairs 7.6 / 12.2.  With every region on every list bra_forward has nothing to route for the dense kernel (7 x 7, topk 49,
+// 16 pairs: 5.8 against 13 us), and bra_attend, whose results are the same bit for bit, takes it too (10.8 / 7.0).
+inline bool dense_pays(const Dims& d) {
+    const long long pairs = (long long)d.B * d.heads;
+    if (!dense_fewer_rows(d)) return false;
+    return d.N > 64 ? pairs >= 64 : d.topk == d.R || pairs * d.R * ((d.n_r + 15) / 16) > 12 * kSMs;
+}
+// true if the kernels with one CTA per (image, head) are: they are written for regions of 2 x 2 and 4 x 4 tokens (5 x 5, topk 6,
+// 25 x 25, 256 pairs: attention 111 against 70 us, gradients 244 / 163; 3 x 3, topk 9: 59 / 33, 93 / 69) and fill the GPU in waves of
+// 148.  Attention, resident / direct: 28 x 28, topk 4: 128 pairs 29.9 / 26.8, 144 29.9 / 31.5, 160 40.8 / 33.4, 200 40.9 / 40.5, 256
+// 41.0 / 49.9; 32 x 32, S = 8, topk 4: 96 pairs 28.4 / 25.9, 128 28.4 / 33.4, 160 54 / 41; 14 x 14, topk 8: 144 pairs 22.7 / 23.0, 160
+// 27.3 / 24.5, 256 27.5 / 36.2.  Within the first wave by the blocks of 32 keys that the direct kernel walks.
+inline bool img_regions(const Dims& d) { return d.hs == d.ws && (d.hs == 2 || d.hs == 4); }
+inline bool img_pays(const Dims& d) {
+    const long long pairs = (long long)d.B * d.heads;
+    return img_regions(d) && (pairs >= 190 || (pairs <= kSMs && pairs * d.R * ((d.topk * d.n_r + 31) / 32) >= 13000));
+}
+// Gradients: 28 x 28, topk 4: 144 pairs 57.5 / 58.6, 200 95 / 79, 256 99 / 103; 14 x 14, topk 8: 160 pairs 62 / 49, 256 65 / 72.
+inline bool img_grad_pays(const Dims& d) { return img_regions(d) && (long long)d.B * d.heads >= 237; }
 bool backward_dense_supported(const Dims& d, int dtype);
 cudaError_t launch_backward_dense(const Dims& d, const void* Q, const void* K, const void* V, const int32_t* index, const float* lce_w,
                                   const float* lse, const void* dO, void* dQ, void* dK, void* dV, int32_t* status, cudaStream_t st);

@@ -49,7 +49,8 @@ inline cudaError_t group_pieces(const Dims& d, int groups, int chunks, F&& launc
 // bits in ascending order: work proportional to the entries, where comparing every entry with every region took
 // 109 us at 256 regions, topk 4 and 41 us at 64 regions, topk 12.  A repeated entry (a caller's index may have them)
 // or a matrix that does not fit: counts by atomics, then one warp puts the entries in their places in order, 32 at a time, the
-// rank among equals of the 32 from a match.  (Every region comparing itself with every entry instead: 961 regions, topk 16, 2 heads, gradients 17.6 ms; 0.24 ms now.)
+// rank among equals of the 32 from a match.  (Every region comparing itself with every entry instead: 961 regions, topk 16,
+// 2 heads, gradients 17.6 ms; 0.24 ms now.)
 // Entries outside [0, R) are in no list.
 __device__ __forceinline__ void inverse_index_job(const int32_t* __restrict__ index, int32_t* __restrict__ inv_off,
                                                   int32_t* __restrict__ inv_list, int32_t* __restrict__ order, int bh, int32_t* sm, bool use_bits, const Dims& dm) {

@@ -1130,12 +1130,12 @@ def test_cuda_core_kernels_keep_infinities_out_of_weighted_walks(bra, value):
 
 
 DENSE_ISOLATION = [
-    BraConfig("alone-7x7", 2, 7, 7, 64, 2, 7, 10, "bf16"),
-    BraConfig("alone-64-regions", 2, 8, 8, 64, 2, 8, 9, "bf16"),
-    BraConfig("alone-2x2-regions", 2, 8, 8, 64, 2, 4, 5, "bf16"),
+    BraConfig("alone-7x7", 20, 7, 7, 64, 2, 7, 10, "bf16"),
+    BraConfig("alone-64-regions", 20, 8, 8, 64, 2, 8, 9, "bf16"),
+    BraConfig("alone-2x2-regions", 60, 8, 8, 64, 2, 4, 5, "bf16"),
     BraConfig("alone-2x2-regions-64-pairs", 64, 12, 12, 32, 1, 6, 13, "bf16"),
     BraConfig("alone-256-tokens", 148, 16, 16, 64, 2, 8, 17, "bf16"),
-    BraConfig("alone-cut-64-tokens", 2, 7, 6, 64, 2, 4, 5, "bf16"),
+    BraConfig("alone-cut-64-tokens", 60, 7, 6, 64, 2, 4, 5, "bf16"),
 ]
 
 
@@ -1208,3 +1208,27 @@ def test_more_images_or_heads_than_a_grid_extent(bra, dtype, impl, d, many):
             mine = [t[..., ch] for t in got]
         for a, r in zip(mine, ref):
             assert (a - r).float().norm() <= (4e-3 if dtype == "bf16" else 1e-6) * r.float().norm()
+
+
+# ------------------------------------------------------------------ both sides of the dispatch rules
+RULE_EDGES = [
+    # maps of up to 64 tokens, attention: the direct kernel up to 1776 regions in the batch, the dense one from there on
+    (BraConfig("rule-64-regions-27-pairs", 27, 8, 8, 32, 1, 8, 5, "bf16"), "route"),
+    (BraConfig("rule-64-regions-28-pairs", 28, 8, 8, 32, 1, 8, 5, "bf16"), "repeats"),
+    (BraConfig("rule-1x2-regions-111-pairs", 111, 4, 8, 32, 1, 4, 3, "bf16"), "repeats"),
+    (BraConfig("rule-1x2-regions-112-pairs", 112, 4, 8, 32, 1, 4, 3, "bf16"), "route"),
+    (BraConfig("rule-3x3-regions-446-pairs", 223, 6, 6, 64, 2, 2, 3, "bf16"), "route"),
+    (BraConfig("rule-padded-112-pairs", 56, 7, 6, 64, 2, 4, 5, "bf16"), "repeats"),
+    # regions of 4 x 4 and 2 x 2: resident slices from 190 pairs, gradients from 237; within the first wave by what is walked
+    (BraConfig("rule-4x4-188-pairs", 94, 8, 8, 64, 2, 2, 2, "bf16"), "route"),
+    (BraConfig("rule-4x4-190-pairs", 95, 8, 8, 64, 2, 2, 2, "bf16"), "route"),
+    (BraConfig("rule-4x4-236-pairs", 118, 8, 8, 64, 2, 2, 2, "bf16"), "repeats"),
+    (BraConfig("rule-4x4-238-pairs", 119, 8, 8, 64, 2, 2, 2, "bf16"), "repeats"),
+    (BraConfig("rule-2x2-128-pairs", 64, 20, 20, 64, 2, 10, 8, "bf16"), "route"),
+    (BraConfig("rule-2x2-130-pairs", 65, 20, 20, 64, 2, 10, 8, "bf16"), "route"),
+]
+
+
+@pytest.mark.parametrize("cfg,kind", RULE_EDGES, ids=[c.name for c, _ in RULE_EDGES])
+def test_both_sides_of_the_dispatch_rules(bra, cfg, kind):
+    run_edge(bra, cfg, "auto", kind)

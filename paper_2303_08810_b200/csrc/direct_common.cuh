@@ -47,7 +47,15 @@ inline DirGeom direct_geom(const Dims& d, bool with_lce, int entry_bytes, int rt
         g.chunks = (d.hs + g.hb - 1) / g.hb;
     }
     g.tpc = (g.hb * d.ws + 15) / 16;
-    const int most = (g.planes == 2 ? 4 : 8) / rt, want = (g.tpc + rt - 1) / rt;
+    const int most = (g.planes == 2 ? 4 : 8) / rt;
+    // two rounds of tiles per CTA only where there is a CTA for every SM (64 x 64, S = 2, topk 2, one head of 64: attention
+    // 1 image 101 -> 56 us; 8 images, 256 CTAs, 141 -> 146)
+    while (g.chunks > 1 && (g.tpc + rt - 1) / rt > most && g.hb > 1 && (long long)d.B * d.heads * d.R * g.chunks < kSMs) {
+        g.hb = (g.hb + 1) / 2;
+        g.chunks = (d.hs + g.hb - 1) / g.hb;
+        g.tpc = (g.hb * d.ws + 15) / 16;
+    }
+    const int want = (g.tpc + rt - 1) / rt;
     if (want == 1 && g.chunks == 1) g.gpc = g.nw = most < 4 ? most : 4;
     else { g.gpc = 1; g.nw = want < most ? want : most; }
     g.gpi = (d.R + g.gpc - 1) / g.gpc * g.chunks;

@@ -813,6 +813,11 @@ DIRECT_EDGES = [
     (BraConfig("direct-529-regions", 1, 23, 23, 32, 1, 23, 3, "bf16"), "repeats"),          # inverse index: bits / comparisons
     (BraConfig("direct-576-regions", 1, 24, 24, 32, 1, 24, 3, "bf16"), "repeats"),
     (BraConfig("direct-961-regions", 1, 31, 31, 64, 2, 31, 5, "bf16"), "repeats"),
+    # head dim 64, regions in chunks: one round of tiles per CTA below 148 CTAs
+    (BraConfig("direct-d64-16x16-144-ctas", 18, 32, 32, 64, 1, 2, 3, "bf16"), "route"),
+    (BraConfig("direct-d64-16x16-152-ctas", 19, 32, 32, 64, 1, 2, 3, "bf16"), "repeats"),
+    (BraConfig("direct-d64-3x64", 1, 6, 128, 64, 1, 2, 2, "bf16"), "route"),
+    (BraConfig("direct-d64-padded-9x17", 1, 17, 33, 64, 1, 2, 2, "bf16"), "repeats"),
 ]
 
 

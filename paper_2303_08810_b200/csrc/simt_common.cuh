@@ -67,9 +67,12 @@ inline SimtGeom simt_geom(const Dims& d, SimtKind kind, int rpc_max, int stages,
     g.row = d.d * d.esize + 16;
     g.by_nr = fast_div(d.n_r); g.by_ws = fast_div(d.ws); g.by_s = fast_div(d.S);
     // lanes of this call against the lanes the GPU holds at once (12 warps per SM)
-    // (dK / dV of larger maps: as if an eighth of the regions held the lists, which is what clustered content comes to;
-    // measured at 1 x 96 x 96, S = 7, 2 heads: 522 -> 224 us; at 36 x 14 x 14 it costs more than it gives)
-    const long long lanes = (long long)d.B * d.heads * d.R * ((d.n_r + qt - 1) / qt) / (kind == SIMT_DKV && d.N > 400 ? 8 : 1);
+    // (dK / dV of larger maps: as if a half of the regions held the lists, a quarter with topk = 1, which is what clustered content
+    // comes to.  By 8 / 4 / 2 / 1, gradients in us: 64 x 21 x 21, 2 heads, topk 8 400 / 316 / 279 / 276; 4 x 44 x 44, 4 heads, topk 4 354 /
+    // 298 / 254 / 291; clustered, forward and gradients: 2 x 88 x 88, 2 heads, topk 1 448 / 447 / 563 / 731, 5 x 48 x 48, 4 heads, topk 4
+    // 491 / 418 / 385 / 497)
+    const int held = kind == SIMT_DKV && d.N > 400 ? (d.topk == 1 ? 4 : 2) : 1;
+    const long long lanes = (long long)d.B * d.heads * d.R * ((d.n_r + qt - 1) / qt) / held;
     const int split = simt_split(d.d, kind);
     g.ksl = 0;
     while (g.ksl < 3 && (lanes << (g.ksl + split)) < kSMs * 256 && (qt * d.d >> (g.ksl + split + 1)) >= 4) ++g.ksl;    // sum_shares: whole float4s

@@ -20,13 +20,18 @@ def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
+def dependencies():
+    """Everything the library is compiled from: sources, every header beside them, the public headers, and the flags here."""
+    root = os.path.dirname(PKG_DIR)
+    return sources() + [p for pattern in (os.path.join(CSRC, "*.h"), os.path.join(CSRC, "*.cuh"), os.path.join(root, "include", "*.h"))
+                        for p in sorted(glob.glob(pattern))] + [os.path.abspath(__file__)]
+
+
 def is_stale() -> bool:
     if not os.path.exists(LIB_PATH):
         return True
     built = os.path.getmtime(LIB_PATH)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.h")) + [
-        os.path.join(os.path.dirname(PKG_DIR), "include", "bra.h")]
-    return any(os.path.getmtime(p) > built for p in deps)
+    return any(os.path.getmtime(p) > built for p in dependencies())
 
 
 def build_library(force: bool = False, verbose: bool = False) -> str:

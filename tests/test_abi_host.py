@@ -64,6 +64,30 @@ def test_workspace_bytes(lib):
     assert binding.workspace_bytes(problem(S=3)) > n           # S does not divide the map: room for the padded copies
 
 
+def test_every_included_file_makes_the_library_stale(monkeypatch, tmp_path):
+    """A change of any source or header is a change of the library: all files of csrc/ that a source includes, transitively,
+    and the public header."""
+    from paper_2303_08810_b200 import build
+    seen, todo = set(), list(build.sources())
+    while todo:
+        path = os.path.realpath(todo.pop())
+        if path in seen:
+            continue
+        seen.add(path)
+        for name in re.findall(r'^\s*#include "([^"]+)"', open(path).read(), flags=re.M):
+            todo.append(os.path.join(os.path.dirname(path), name))
+    assert any(p.endswith(".cuh") for p in seen) and any(p.endswith("bra.h") for p in seen)
+    assert seen <= {os.path.realpath(p) for p in build.dependencies()}
+    lib = tmp_path / "lib.so"
+    lib.write_bytes(b"")
+    monkeypatch.setattr(build, "LIB_PATH", str(lib))
+    newest = max(os.path.getmtime(p) for p in build.dependencies())
+    os.utime(lib, (newest + 1,) * 2)
+    assert not build.is_stale()
+    os.utime(lib, (newest - 1,) * 2)
+    assert build.is_stale()
+
+
 A = 0x10000  # a fake, aligned, never dereferenced device address
 
 

@@ -1237,3 +1237,149 @@ RULE_EDGES = [
 @pytest.mark.parametrize("cfg,kind", RULE_EDGES, ids=[c.name for c, _ in RULE_EDGES])
 def test_both_sides_of_the_dispatch_rules(bra, cfg, kind):
     run_edge(bra, cfg, "auto", kind)
+
+
+# ------------------------------------------------------------------ bad routing entries in every kernel, gradients among them
+BAD_INDEX = [
+    ("simt", BraConfig("bad-staged", 2, 12, 20, 64, 2, 4, 4, "f32")),
+    ("simt", BraConfig("bad-resident", 2, 8, 12, 64, 2, 4, 8, "f32")),
+    ("simt", BraConfig("bad-every-region", 2, 6, 6, 64, 2, 3, 9, "f32")),
+    ("simt", BraConfig("bad-1x1", 2, 6, 6, 64, 2, 6, 7, "f32")),
+    ("mma", BraConfig("bad-direct-one-block", 2, 12, 20, 64, 2, 4, 3, "bf16")),
+    ("mma", BraConfig("bad-direct", 2, 21, 35, 64, 2, 7, 9, "bf16")),
+    ("mma", BraConfig("bad-direct-d64", 2, 12, 20, 128, 2, 4, 4, "bf16")),
+    ("auto", BraConfig("bad-dense-7x7", 20, 7, 7, 64, 2, 7, 10, "bf16")),
+    ("auto", BraConfig("bad-dense-k=R", 20, 7, 7, 64, 2, 7, 49, "bf16")),
+    ("auto", BraConfig("bad-dense-2x2", 148, 16, 16, 64, 2, 8, 17, "bf16")),
+    ("img", BraConfig("bad-resident-bf16", 2, 16, 16, 64, 2, 4, 4, "bf16")),
+    ("tc", BraConfig("bad-tc", 2, 32, 32, 64, 2, 4, 4, "bf16")),
+]
+
+
+@pytest.mark.parametrize("impl,cfg", BAD_INDEX, ids=[c.name for _, c in BAD_INDEX])
+def test_bad_entries_count_for_nothing(bra, impl, cfg):
+    """Every row's last entry is out of range, every entry of one row is: the results are those of lists without these entries,
+    a query without any gets the attention term 0, and the call reports BRA_ERR_INDEX."""
+    import torch
+    x = synthetic.make_inputs(cfg, seed=101, with_do=True)
+    rng = np.random.default_rng(102)
+    good = rng.permuted(np.tile(np.arange(cfg.R, dtype=np.int32), (cfg.B, cfg.heads, cfg.R, 1)), axis=-1)[..., :cfg.topk]
+    bad = good.copy()
+    bad[..., -1] = np.where(rng.random(bad[..., -1].shape) < 0.5, -1, cfg.R)
+    lost = cfg.R // 2
+    bad[0, 0, lost] = cfg.R + 3
+    t = to_dev(x, cfg)
+    p = problem_of(bra, cfg, impl=IMPLS[impl], lce=False)
+    ws = bra.workspace(p)
+    idx = torch.from_numpy(bad).cuda()
+    O, lse = bra.bra_attend(p, t["Q"], t["K"], t["V"], idx, ws=ws)
+    assert bra.bra_device_status(ws) == 9
+    g = bra.bra_backward(p, t["Q"], t["K"], t["V"], idx, None, lse, t["dO"], ws=ws)
+    assert bra.bra_device_status(ws) in (0, 9)       # (a gradient call may leave it to the forward call to say so)
+    ref, _ = orc.bra_attend(x["Q"], x["K"], x["V"], good[..., :-1], None, cfg.heads, cfg.S)
+    where = region_mask(cfg, lost, lost + 1)
+    ref[0][where, :cfg.d] = 0
+    dO = x["dO"].copy()
+    dO[0][where, :cfg.d] = 0
+    grads = orc.bra_backward(x["Q"], x["K"], x["V"], good[..., :-1], np.zeros_like(x["w"]), dO, cfg.heads, cfg.S)
+    check_O(f64(O), ref, cfg.dtype)
+    tol = GRAD_MAX if cfg.dtype == "bf16" else 2e-4
+    for name, a, r in zip(("dQ", "dK", "dV"), g, grads):
+        assert np.abs(f64(a) - r).max() <= tol, f"{name} {np.abs(f64(a) - r).max():.3e}"
+
+
+# ------------------------------------------------------------------ inputs written right before the call; graphs
+ORDER_CASES = [
+    BraConfig("order-pool-rows", 16, 28, 28, 128, 4, 7, 4, "bf16"),
+    BraConfig("order-pool-split", 16, 56, 56, 64, 2, 7, 1, "bf16"),
+    BraConfig("order-pool-8", 8, 49, 49, 64, 2, 7, 2, "bf16"),
+    BraConfig("order-pool-16", 2, 128, 128, 64, 2, 8, 4, "bf16"),
+    BraConfig("order-padded", 4, 61, 53, 64, 2, 4, 3, "bf16"),
+    BraConfig("order-dense", 16, 7, 7, 512, 16, 7, 49, "bf16"),
+    BraConfig("order-fp32", 4, 28, 28, 64, 2, 7, 4, "f32"),
+]
+
+
+def order_step(bra, cfg, source, ws):
+    """One kernel writes Q, K, V and dO, the calls follow it on the stream."""
+    import torch
+    p = problem_of(bra, cfg)
+    X = torch.empty_like(source)
+    w = torch.full((cfg.C, 5, 5), 0.01, device="cuda")
+    index = torch.empty(cfg.B, cfg.heads, cfg.R, cfg.topk, dtype=torch.int32, device="cuda")
+
+    def step():
+        torch.mul(source, 1.0, out=X)
+        O, _, lse = bra.bra_forward(p, X[0], X[1], X[2], w, index=index, ws=ws)
+        g = bra.bra_backward(p, X[0], X[1], X[2], index, w, lse, X[3], ws=ws, want_bias_grad=True)
+        return (O, index, lse) + tuple(g)
+
+    return step, X
+
+
+def order_sources(cfg, n):
+    import torch
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(7)
+    dt = torch.bfloat16 if cfg.dtype == "bf16" else torch.float32
+    return [torch.randn(4, cfg.B, cfg.H, cfg.W, cfg.C, device="cuda", generator=gen).to(dt) for _ in range(n)]
+
+
+@pytest.mark.parametrize("cfg", ORDER_CASES, ids=lambda c: c.name)
+def test_calls_wait_for_the_kernel_that_writes_their_inputs(bra, cfg):
+    """The first kernel of a call may be set up under the kernel before it in the stream: it must still see what that one wrote.
+    The inputs are overwritten with NaN-free but other values between the steps, nothing synchronises in between."""
+    import torch
+    p = problem_of(bra, cfg)
+    ws = bra.workspace(p)
+    sources = order_sources(cfg, 2)
+    want = []
+    for src in sources:
+        step, X = order_step(bra, cfg, src, ws)
+        X.copy_(src)
+        torch.cuda.synchronize()
+        want.append([t.clone() for t in step()])
+        torch.cuda.synchronize()
+    live = torch.empty_like(sources[0])
+    step, X = order_step(bra, cfg, live, ws)
+    got = []
+    for it in range(6):
+        live.copy_(sources[it % 2])
+        X.fill_(3.0)
+        got.append([t.clone() for t in step()])
+    torch.cuda.synchronize()
+    assert bra.bra_device_status(ws) == 0
+    for it, outs in enumerate(got):
+        for a, r in zip(outs, want[it % 2]):
+            assert torch.equal(a, r), f"step {it}"
+
+
+@pytest.mark.parametrize("cfg", ORDER_CASES, ids=lambda c: c.name)
+def test_calls_in_a_cuda_graph(bra, cfg):
+    """Forward and backward (its helper stream among them) captured behind the kernel that writes their inputs, replayed on
+    other inputs: the results of the calls made directly."""
+    import torch
+    p = problem_of(bra, cfg)
+    ws = bra.workspace(p)
+    sources = order_sources(cfg, 2)
+    want = []
+    for src in sources:
+        want.append([t.clone() for t in order_step(bra, cfg, src, ws)[0]()])
+    live = sources[0].clone()
+    step, _ = order_step(bra, cfg, live, ws)
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(stream):
+        step()
+    stream.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        outs = step()
+    for it in range(4):
+        live.copy_(sources[it % 2])
+        graph.replay()
+        torch.cuda.synchronize()
+        assert bra.bra_device_status(ws) == 0
+        for a, r in zip(outs, want[it % 2]):
+            assert torch.equal(a, r), f"replay {it}"
+    del graph

@@ -76,7 +76,8 @@ typedef enum bra_dtype { BRA_F32 = 0, BRA_BF16 = 1 } bra_dtype;
 /* Which kernel family runs the token-to-token attention (step 4-5). */
 typedef enum bra_impl {
     BRA_IMPL_AUTO = 0,  /* fastest kernel that supports the problem */
-    BRA_IMPL_SIMT = 1,  /* fp32 CUDA-core kernel: any dtype, any shape with C/heads <= 128 */
+    BRA_IMPL_SIMT = 1,  /* fp32 CUDA-core kernels: any dtype, any map, region size, topk and batch; C/heads 16, 32, 64 or 128
+                           (gradients: up to 64) */
     BRA_IMPL_MMA = 2,   /* bf16 warp-level tensor-core kernels with operands straight from global memory (C/heads == 32 or 64,
                            regions at most 128 tokens wide) */
     BRA_IMPL_TC = 3,    /* bf16 tcgen05/TMEM kernels (C/heads == 32; regions of 8 x 8 tokens, or 16 wide and a multiple of 8 high) */

@@ -2,8 +2,10 @@
 // CTA = (image, head, chunk of map rows); a warp owns RT tiles of 16 query tokens and walks all keys in blocks of 32:
 // S by m16n8k16 MMAs on fragments read as 16-byte chunks, online softmax, O += P V with V through ldmatrix.  O^att goes
 // to the LCE's thread mapping through shared memory (over the slices).
-// What bounds it: per 16 x 16 scores eight MMAs (64 cycles of a scheduler's tensor pipe), eight exponentials per lane (64
-// cycles of its MUFU share) and about 60 instructions.
+// Per 16 x 16 scores: eight MMAs (64 cycles of a scheduler's tensor pipe), eight exponentials per lane (64 cycles of its MUFU share)
+// and about 60 instructions.  What bounds it at 64 x 14 x 14, 8 heads, topk 16: latency - 0.46 instructions per cycle and scheduler
+// with 12 warps per SM (128 registers), per issue 1.6 cycles of fixed waits, 0.8 at barriers, 0.7 for loads, 0.7 for the MMA pipe;
+// 1.73 waves of CTAs.
 // Measured (B200): 64 x 7 x 7, 16 heads, topk 49: forward 161 us with routing -> 16.4 us; 64 x 14 x 14, 8 heads, topk 16:
 // level with attend_img.cu (44 us).  The other side of the rule: dense_pays().
 #include "dense_common.cuh"

@@ -13,7 +13,8 @@
 // What bounds it: one m16n8k16 MMA takes 8 cycles of a scheduler's tensor pipe (16 per 16 queries x 64 keys x 32
 // channels: S and P V) and the softmax needs about as many issue slots; with regions of few tokens, the L2 traffic of
 // the routed keys (every group reads topk * n_r of them).  Counters at 2 x 100 x 167, S = 16, topk 4, 6 heads: 0.53
-// instructions per cycle and scheduler, tensor pipe 14 %: issue slots.
+// instructions per cycle and scheduler, tensor pipe 14 %; at 16 x 32 x 32, 12 heads of 64: 0.40, 2.2 cycles per issue waiting
+// for loads, 1.7 in fixed waits: latency at 12 warps per SM.
 // Measured (B200) against staging keys and values in shared memory: 16 x 32 x 32, 12 heads of 64, topk 12: 278 -> 126 us;
 // 2 x 100 x 167, 6 heads: 131 us and four padded copies -> 114 us and none.  Small maps: attend_img.cu
 // where it has the CTAs (img_pays()).  A reference maximum that moves only for scores 8 above it: no faster, error

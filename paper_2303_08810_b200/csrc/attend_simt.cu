@@ -3,7 +3,8 @@
 // copied to (or, with a resident slice, read from) shared memory.  Softmax is the one-pass running-max form in blocks of
 // four keys per lane.
 // Bound: the FMA pipe, 2 D FMAs per query and key (a packed FMA every two cycles and scheduler), in practice the latency of
-// the dot-product chains.  Measured (B200) against one thread per query with operands from global memory: 64 x 28 x 28,
+// the dot-product chains (64 x 28 x 28, 4 heads, topk 4: 0.48 instructions per cycle and scheduler with 7.5 warps per SM, 255 registers).
+// Measured (B200) against one thread per query with operands from global memory: 64 x 28 x 28,
 // 4 heads, topk 4: 356 -> 144 us; 1 x 16 x 16, 1 head: 41 -> 11 us.
 #include "simt_common.cuh"
 

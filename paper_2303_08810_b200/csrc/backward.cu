@@ -431,7 +431,7 @@ static cudaError_t launch_bwd_t(const Dims& d, int impl, const void* Q, const vo
 
     const Family family = choose_family(d, sizeof(T) == 2 ? BRA_BF16 : BRA_F32, impl);
     if (family == FAMILY_IMG) {
-        // the dQ kernel of this family and of the next also writes the inverse routing index
+        // the dQ kernel of this family, of the direct and of the CUDA-core kernels also writes the inverse routing index
         if ((e = launch_backward_img(d, Q, K, V, index, inv_off, inv_list, lce_w, lse, dO, dQ, dK, dV,
                                      delta, status, st)) != cudaSuccess) return e;
     } else if (family == FAMILY_DENSE) {

@@ -2,9 +2,10 @@
 // (dense_common.cuh), bf16, head dim 32: one launch, CTA = (image, head), the slices of Q, K, V and dO resident.
 //   1. warp = 16 queries: delta = rowsum(P o dP) in a first walk over the keys, dQ = scale dS K in a second
 //   2. warp = 16 keys: dK = scale dS^T Q and dV = P^T dO in one walk over the queries; dV + LCE adjoint
-// P from the saved log-sum-exp, dP = dO V^T, dS = P o (dP - delta).  Who is routed where is the count table, so no inverse
-// index is needed.  Every sum has a fixed order.
-// Bound: instruction issue; the two walks over the keys in 1. make S and dP twice.  Measured (B200) against the kernels of
+// P from the saved log-sum-exp, dP = dO V^T, dS = P o (dP - delta).  Who is routed where is the bit masks (with repeats a table
+// of log2 of the counts), so no inverse index is needed.  Every sum has a fixed order.
+// Bound: latency at 12 warps per SM (0.47 instructions per cycle and scheduler; per issue 1.8 cycles of fixed waits, 1.0 at
+// barriers, 0.55 for the MMA pipe), 1.73 waves; the two walks over the keys in 1. make S and dP twice.  Measured (B200) against the kernels of
 // backward_img.cu: 64 x 14 x 14, 8 heads, topk 16: 156 -> 103 us; 64 x 7 x 7, 16 heads, topk 49: 477 -> 39 us.
 #include "dense_common.cuh"
 

@@ -189,7 +189,7 @@ static bra_status attend_any_map(Path path, const Dims& d, const WsLayout& L, in
     int32_t* status = reinterpret_cast<int32_t*>(w + L.status);
     if (any_map(path)) return run_attend(path, d, dtype, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel);
     return on_padded_map(d, L, Q, K, V, O, lse, w, st, [&](const Dims& dp, const void* q, const void* k, const void* v, void* o, float* l) {
-        return run_attend(path, dp, dtype, q, k, v, index, lce_w, lce_b, o, l, status, st, after_own_kernel && !padded(d));
+        return run_attend(path, dp, dtype, q, k, v, index, lce_w, lce_b, o, l, status, st, false);
     });
 }
 
@@ -369,7 +369,7 @@ const char* bra_status_string(bra_status s) {
     switch (s) {
         case BRA_OK: return "ok";
         case BRA_ERR_NULL: return "a required pointer is NULL";
-        case BRA_ERR_SHAPE: return "bad shape: sizes must be positive, S must divide H and W, heads must divide C";
+        case BRA_ERR_SHAPE: return "bad shape: sizes must be positive, heads must divide C";
         case BRA_ERR_TOPK: return "topk must be in [1, S*S]";
         case BRA_ERR_DTYPE: return "dtype must be BRA_F32 or BRA_BF16";
         case BRA_ERR_ALIGN: return "pointer not aligned (tensors 16 bytes, workspace 256 bytes)";

@@ -88,7 +88,9 @@ inline bool direct_exact(const Dims& d) {
 }
 
 // Tiles per warp in the forward kernel: two share every row that is loaded (and transposed) where regions have two and enough
-// warps remain.  Measured: 2 x 100 x 167 tokens, S = 16, topk 4, 6 heads 124 -> 114 us; 2 x 112 x 112, S = 8: 98 -> 88 us.
+// warps remain.  Measured, one / two tiles: 2 x 100 x 167 tokens, S = 16, topk 4, 6 heads 124 / 114 us; 2 x 112 x 112, S = 8: 98 / 88.
+// Around the line each wave of CTAs is a step on either side: 35 x 35, 784 warps 11.7 / 13.1, 1176 13.9 / 15.7, 1372 20.6 / 15.8, 1764
+// 22.7 / 24.0, 3626 42.1 / 37.6; 70 x 70, 1176 warps 12.1 / 12.2, 1568 19.0 / 14.5, 2352 22.5 / 21.9.
 inline int direct_rt(const Dims& d) {
     const long long warps = (long long)d.B * d.heads * d.R * ((d.n_r + 31) / 32);
     return d.n_r > 16 && warps >= 8 * kSMs ? 2 : 1;

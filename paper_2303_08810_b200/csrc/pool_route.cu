@@ -39,15 +39,7 @@ __device__ __forceinline__ void unpack_row(const uint4& v, float (&out)[8]) {
 template <int n>
 __device__ __forceinline__ void load_row_cg(const __nv_bfloat16* p, float* out) {
 #pragma unroll
-    for (int i = 0; i < n; i += 8) {
-        const uint4 v = __ldcg(reinterpret_cast<const uint4*>(p + i));
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            out[i + 2 * j] = __uint_as_float(w[j] << 16);
-            out[i + 2 * j + 1] = __uint_as_float(w[j] & 0xffff0000u);
-        }
-    }
+    for (int i = 0; i < n; i += 8) unpack_row(__ldcg(reinterpret_cast<const uint4*>(p + i)), reinterpret_cast<float (&)[8]>(out[i]));
 }
 template <int n>
 __device__ __forceinline__ void zero_row(float* v) {

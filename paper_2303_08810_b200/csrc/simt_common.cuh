@@ -397,7 +397,7 @@ __device__ __forceinline__ void simt_st(__nv_bfloat16* p, float v) { *p = __floa
 struct SimtFrom { int r0; __device__ int operator[](int i) const { return r0 + i; } };
 template <typename T, int D, int TS, bool FLIP, typename RegionAt>
 __device__ __forceinline__ void simt_lce(const float* st, const float* s_w, const float* bias, const T* in, T* out, RegionAt region_at, int nreg, int rows_per_region,
-                                         const SimtChunk& c,                                         const Dims& dm, const SimtGeom& gm) {
+                                         const SimtChunk& c, const Dims& dm, const SimtGeom& gm) {
     constexpr int LANES = D < 32 ? D : 32, GROUPS = D / LANES, SUB = 32 / LANES;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int nty = (c.rows + TS - 1) / TS, ntx = (c.cols + TS - 1) / TS, tiles = nty * ntx;
@@ -425,7 +425,7 @@ __device__ __forceinline__ void simt_lce(const float* st, const float* s_w, cons
 #pragma unroll
             for (int xx = 0; xx < TS; ++xx) acc[yy][xx] = b;
         if (dm.lce) {
-bool in_x[TS + 4];
+            bool in_x[TS + 4];
 #pragma unroll
             for (int cc = 0; cc < TS + 4; ++cc) in_x[cc] = (unsigned)(x0 + cc - 2) < (unsigned)dm.W0;
             const T* p = in + (ptrdiff_t)((y0 - 2) * dm.W0 + x0 - 2) * dm.C + ch;

@@ -153,14 +153,16 @@ inline bool dense_pays(const Dims& d) {
     return d.N > 64 ? pairs >= 64 : d.topk == d.R || pairs * d.R * ((d.n_r + 15) / 16) > 12 * kSMs;
 }
 // true if the kernels with one CTA per (image, head) are: they are written for regions of 2 x 2 and 4 x 4 tokens (5 x 5, topk 6,
-// 25 x 25, 256 pairs: attention 111 against 70 us, gradients 244 / 163; 3 x 3, topk 9: 59 / 33, 93 / 69) and fill the GPU in waves of
-// 148.  Attention, resident / direct: 28 x 28, topk 4: 128 pairs 29.9 / 26.8, 144 29.9 / 31.5, 160 40.8 / 33.4, 200 40.9 / 40.5, 256
-// 41.0 / 49.9; 32 x 32, S = 8, topk 4: 96 pairs 28.4 / 25.9, 128 28.4 / 33.4, 160 54 / 41; 14 x 14, topk 8: 144 pairs 22.7 / 23.0, 160
-// 27.3 / 24.5, 256 27.5 / 36.2.  Within the first wave by the blocks of 32 keys that the direct kernel walks.
+// 25 x 25, 256 pairs: attention 111 against 70 us, gradients 244 / 163; 3 x 3, topk 9: 59 / 33, 93 / 69), fill the GPU in waves of 148
+// and, with a whole SM each, start only when the routing kernel is done.  bra_forward, resident / direct: 28 x 28, topk 4: 144 pairs
+// 46.7 / 38.9, 160 46.8 / 41.1, 200 49.7 / 50.7, 256 49.7 / 58.1; 20 x 20, S = 5, topk 6: 160 29.7 / 26.8, 200 30.2 / 34.3; 14 x 14: topk 4,
+// 256 pairs 47.5 / 42.1, 320 49.7 / 52.7, topk 12, 200 43.6 / 46.1.  The work: the blocks of 32 keys that the direct kernel walks.
+// On the wrong side of it: 16 x 16, S = 8, topk 8, 256 pairs 62.9 / 53.3 and 20 x 20, S = 10, topk 8, 160 pairs 62.9 / 65.2.
+// (Attention alone: 28 x 28 144 pairs 30.0 / 31.5; 32 x 32, S = 8, topk 4, 128 pairs 28.5 / 33.4, bra_forward 35.5 / 39.7.)
 inline bool img_regions(const Dims& d) { return d.hs == d.ws && (d.hs == 2 || d.hs == 4); }
 inline bool img_pays(const Dims& d) {
     const long long pairs = (long long)d.B * d.heads;
-    return img_regions(d) && (pairs >= 190 || (pairs <= kSMs && pairs * d.R * ((d.topk * d.n_r + 31) / 32) >= 13000));
+    return img_regions(d) && pairs >= 190 && pairs * d.R * ((d.topk * d.n_r + 31) / 32) >= 15000;
 }
 // Gradients: 28 x 28, topk 4: 144 pairs 57.5 / 58.6, 200 95 / 79, 256 99 / 103; 14 x 14, topk 8: 160 pairs 62 / 49, 256 65 / 72.
 inline bool img_grad_pays(const Dims& d) { return img_regions(d) && (long long)d.B * d.heads >= 237; }

@@ -1224,13 +1224,13 @@ RULE_EDGES = [
     (BraConfig("rule-1x2-regions-112-pairs", 112, 4, 8, 32, 1, 4, 3, "bf16"), "route"),
     (BraConfig("rule-3x3-regions-446-pairs", 223, 6, 6, 64, 2, 2, 3, "bf16"), "route"),
     (BraConfig("rule-padded-112-pairs", 56, 7, 6, 64, 2, 4, 5, "bf16"), "repeats"),
-    # regions of 4 x 4 and 2 x 2: resident slices from 190 pairs, gradients from 237; within the first wave by what is walked
-    (BraConfig("rule-4x4-188-pairs", 94, 8, 8, 64, 2, 2, 2, "bf16"), "route"),
-    (BraConfig("rule-4x4-190-pairs", 95, 8, 8, 64, 2, 2, 2, "bf16"), "route"),
+    # regions of 4 x 4 and 2 x 2: resident slices from 190 pairs with enough to walk, gradients from 237
+    (BraConfig("rule-2x2-188-pairs", 94, 20, 20, 64, 2, 10, 8, "bf16"), "route"),
+    (BraConfig("rule-2x2-190-pairs", 95, 20, 20, 64, 2, 10, 8, "bf16"), "route"),
     (BraConfig("rule-4x4-236-pairs", 118, 8, 8, 64, 2, 2, 2, "bf16"), "repeats"),
     (BraConfig("rule-4x4-238-pairs", 119, 8, 8, 64, 2, 2, 2, "bf16"), "repeats"),
-    (BraConfig("rule-2x2-128-pairs", 64, 20, 20, 64, 2, 10, 8, "bf16"), "route"),
-    (BraConfig("rule-2x2-130-pairs", 65, 20, 20, 64, 2, 10, 8, "bf16"), "route"),
+    (BraConfig("rule-4x4-15000-blocks", 200, 20, 20, 32, 1, 5, 6, "bf16"), "route"),
+    (BraConfig("rule-4x4-14925-blocks", 199, 20, 20, 32, 1, 5, 6, "bf16"), "route"),
 ]
 
 

@@ -379,13 +379,14 @@ bwd_dkv_simt_kernel(const T* __restrict__ Qg, const T* __restrict__ Kg, const T*
     else simt_lce<T, D, 4, true>(st, s_w, nullptr, dO, dVg + head, order, nreg, gm.spr, chunk, dm, gm);
 }
 
-enum Family { FAMILY_SIMT, FAMILY_DIRECT, FAMILY_IMG, FAMILY_DENSE };
+enum Family { FAMILY_SIMT, FAMILY_DIRECT, FAMILY_IMG, FAMILY_DENSE, FAMILY_ONE };
 
 // bf16, head dim 32 or 64: tensor-core kernels.  Small maps with enough (image, head) pairs to fill the GPU keep a
 // whole slice resident (head dim 32); the rest take their operands straight from global memory.
 static Family choose_family(const Dims& d, int dtype, int impl) {
     if (dtype != BRA_BF16 || impl == BRA_IMPL_SIMT) return FAMILY_SIMT;
     if (impl == BRA_IMPL_AUTO && backward_dense_supported(d, dtype) && dense_grad_pays(d)) return FAMILY_DENSE;
+    if (impl == BRA_IMPL_AUTO && backward_one_supported(d, dtype)) return FAMILY_ONE;
     if (backward_img_supported(d, dtype) &&
         (impl == BRA_IMPL_IMG || (impl == BRA_IMPL_AUTO && img_grad_pays(d))))
         return FAMILY_IMG;
@@ -434,6 +435,8 @@ static cudaError_t launch_bwd_t(const Dims& d, int impl, const void* Q, const vo
         // the dQ kernel of this family, of the direct and of the CUDA-core kernels also writes the inverse routing index
         if ((e = launch_backward_img(d, Q, K, V, index, inv_off, inv_list, lce_w, lse, dO, dQ, dK, dV,
                                      delta, status, st)) != cudaSuccess) return e;
+    } else if (family == FAMILY_ONE) {
+        if ((e = launch_backward_one(d, Q, K, V, index, lce_w, lse, dO, dQ, dK, dV, status, st)) != cudaSuccess) return e;
     } else if (family == FAMILY_DENSE) {
         if ((e = launch_backward_dense(d, Q, K, V, index, lce_w, lse, dO, dQ, dK, dV, status, st)) != cudaSuccess) return e;
     } else if (family == FAMILY_DIRECT) {

@@ -180,6 +180,10 @@ cudaError_t launch_backward_direct(const Dims& d, const void* Q, const void* K, 
                                 const float* lce_w, const float* lse, const void* dO,
                                 void* dQ, void* dK, void* dV, float* delta, int32_t* status, cudaStream_t st);
 
+bool backward_one_supported(const Dims& d, int dtype);
+cudaError_t launch_backward_one(const Dims& d, const void* Q, const void* K, const void* V, const int32_t* index, const float* lce_w,
+                                const float* lse, const void* dO, void* dQ, void* dK, void* dV, int32_t* status, cudaStream_t st);
+
 bool backward_img_supported(const Dims& d, int dtype);
 cudaError_t launch_backward_img(const Dims& d, const void* Q, const void* K, const void* V,
                                 const int32_t* index, const int32_t* inv_off, const int32_t* inv_list,

@@ -1288,6 +1288,65 @@ def test_bad_entries_count_for_nothing(bra, impl, cfg):
         assert np.abs(f64(a) - r).max() <= tol, f"{name} {np.abs(f64(a) - r).max():.3e}"
 
 
+# topk = 1 in one launch: tiles of a region (17 .. 64 tokens), rows behind its last token, cut maps, every list length
+ONE_EDGES = [
+    (BraConfig("one-1x17", 1, 2, 34, 32, 1, 2, 1, "bf16"), "route"),
+    (BraConfig("one-5x4", 3, 35, 28, 96, 3, 7, 1, "bf16"), "route"),
+    (BraConfig("one-4x8", 2, 16, 32, 64, 2, 4, 1, "bf16"), "route"),
+    (BraConfig("one-3x11", 2, 9, 33, 64, 2, 3, 1, "bf16"), "route"),
+    (BraConfig("one-6x8", 2, 24, 32, 64, 2, 4, 1, "bf16"), "route"),
+    (BraConfig("one-7x7", 2, 49, 49, 64, 2, 7, 1, "bf16"), "route"),
+    (BraConfig("one-9x7", 2, 27, 21, 64, 2, 3, 1, "bf16"), "route"),
+    (BraConfig("one-8x8", 2, 56, 56, 64, 2, 7, 1, "bf16"), "route"),
+    (BraConfig("one-64x1", 1, 128, 2, 32, 1, 2, 1, "bf16"), "route"),
+    (BraConfig("one-13x5-two-kernels", 2, 26, 10, 64, 2, 2, 1, "bf16"), "route"),          # 65 tokens
+    (BraConfig("one-4x4-two-kernels", 2, 16, 16, 64, 2, 4, 1, "bf16"), "route"),           # 16
+    (BraConfig("one-cut-8x7", 2, 29, 27, 64, 2, 4, 1, "bf16"), "route"),
+    (BraConfig("one-cut-rows-of-whole-regions", 1, 33, 40, 32, 1, 8, 1, "bf16"), "route"),
+    (BraConfig("one-256-regions", 1, 80, 96, 32, 1, 16, 1, "bf16"), "route"),
+]
+
+
+@pytest.mark.parametrize("cfg,kind", ONE_EDGES, ids=[c.name for c, _ in ONE_EDGES])
+def test_gradients_of_topk_1_at_their_edges(bra, cfg, kind):
+    run_edge(bra, cfg, "auto", kind)
+    idx = np.zeros((cfg.B, cfg.heads, cfg.R, 1), np.int32)                                 # one list of every region, the rest empty
+    idx[:, :, 1:cfg.R // 2] = cfg.R - 1
+    run_backward_case(bra, cfg, seed=61, index=idx)
+    run_backward_case(bra, cfg, seed=62, shared=True)
+
+
+def test_bad_entries_of_topk_1_have_no_gradient(bra):
+    import torch
+    cfg = BraConfig("bad-one", 2, 29, 27, 64, 2, 4, 1, "bf16")
+    x = synthetic.make_inputs(cfg, seed=103, with_do=True)
+    idx = np.random.default_rng(104).integers(0, cfg.R, (cfg.B, cfg.heads, cfg.R, 1)).astype(np.int32)
+    good = idx.copy()
+    lost = (1, 5)
+    for r, v in zip(lost, (-1, cfg.R)):
+        idx[0, 0, r] = v
+    t = to_dev(x, cfg)
+    p = problem_of(bra, cfg, lce=False)
+    ws = bra.workspace(p)
+    dev = torch.from_numpy(idx).cuda()
+    O, lse = bra.bra_attend(p, t["Q"], t["K"], t["V"], dev, ws=ws)
+    assert bra.bra_device_status(ws) == 9
+    g = bra.bra_backward(p, t["Q"], t["K"], t["V"], dev, None, lse, t["dO"], ws=ws)
+    assert bra.bra_device_status(ws) == 9
+    dO = x["dO"].copy()
+    for r in lost:
+        dO[0][region_mask(cfg, r, r + 1), :cfg.d] = 0
+    ref = orc.bra_backward(x["Q"], x["K"], x["V"], good, np.zeros_like(x["w"]), dO, cfg.heads, cfg.S)
+    for name, a, r in zip(("dQ", "dK", "dV"), g, ref):
+        assert np.abs(f64(a) - r).max() <= GRAD_MAX, name
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("nan")], ids=["inf", "nan"])
+@pytest.mark.parametrize("hw", [(24, 28), (29, 27), (28, 24)])
+def test_gradients_of_topk_1_keep_infinities_in_their_regions(bra, hw, value):
+    run_isolation_case(bra, BraConfig("alone-one", 2, hw[0], hw[1], 64, 2, 4, 1, "bf16"), "auto", value)
+
+
 # ------------------------------------------------------------------ inputs written right before the call; graphs
 ORDER_CASES = [
     BraConfig("order-pool-rows", 16, 28, 28, 128, 4, 7, 4, "bf16"),

@@ -7,8 +7,10 @@
 // with 12 warps per SM (128 registers), per issue 1.6 cycles of fixed waits, 0.8 at barriers, 0.7 for loads, 0.7 for the MMA pipe;
 // 1.73 waves of CTAs.
 // Measured (B200): 64 x 7 x 7, 16 heads, topk 49: forward 161 us with routing -> 16.4 us; 64 x 14 x 14, 8 heads, topk 16:
-// level with attend_img.cu (44 us).  The other side of the rule: dense_pays().
+// level with attend_img.cu (44 us); 46 -> 44 under ncu, bra_forward 55.7 -> 54.1, with the mask as the addend of the scaling.  The other side of the rule: dense_pays().
 #include "dense_common.cuh"
+
+#include <type_traits>
 
 namespace bra {
 
@@ -130,37 +132,38 @@ attend_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* _
 #pragma unroll
             for (int e = 0; e < 4; ++e) o[x][n][e] = 0.f;
     }
+    const uint32_t row_off = dense_row_offset(lane), col_off = dense_col_offset(lane);
+    auto walk = [&](auto weighted) {
+        DenseRow<NR> on[RT][2];
+#pragma unroll
+        for (int x = 0; x < RT; ++x)
+#pragma unroll
+            for (int r = 0; r < 2; ++r) on[x][r] = DenseRow<NR>(mask[where[x][r] >> 16], t4);
 #pragma unroll 1
     for (int kb = 0; kb < dm.N; kb += 32) {
         float c[RT][4][4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const uint4 kr[1] = {dense_row(ks, kb + 8 * j + g, t4)};
+            const uint4 kr[1] = {dense_chunk(ks + (kb + 8 * j) * 64 + row_off)};
 #pragma unroll
-            for (int x = 0; x < RT; ++x) {
-                mma_rows<1>(c[x][j], qa[x], kr);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) c[x][j][e] *= sl2;
-            }
+            for (int x = 0; x < RT; ++x) mma_rows<1>(c[x][j], qa[x], kr);
         }
-        if (routes.masked || kb + 32 > dm.N) {
 #pragma unroll
-            for (int x = 0; x < RT; ++x) dense_mask<NR, 4>(c[x], mask[where[x][0] >> 16], mask[where[x][1] >> 16], kb, t4, reg, -INFINITY);
-        }
-        if (routes.weighted) {
+        for (int j = 0; j < 4; ++j)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const uchar2 kr = *reinterpret_cast<const uchar2*>(reg + kb + 8 * j + 2 * t4);
+            for (int x = 0; x < RT; ++x)
 #pragma unroll
-                for (int x = 0; x < RT; ++x)
+                for (int r = 0; r < 2; ++r)
 #pragma unroll
-                    for (int r = 0; r < 2; ++r) {
-                        const float* row = bias + (where[x][r] >> 16) * dm.R;
-                        if (kr.x < 64) c[x][j][2 * r] += row[kr.x];
-                        if (kr.y < 64) c[x][j][2 * r + 1] += row[kr.y];
+                    for (int e = 0; e < 2; ++e) {
+                        const float a = weighted.value ? dense_weight(bias + (where[x][r] >> 16) * dm.R, reg[kb + 8 * j + 2 * t4 + e])
+                                                       : on[x][r].pick(0.f, j, e, kb, t4, reg);
+                        c[x][j][2 * r + e] = fmaf(c[x][j][2 * r + e], sl2, a);
                     }
-            }
-        }
+#pragma unroll
+        for (int x = 0; x < RT; ++x)
+#pragma unroll
+            for (int r = 0; r < 2; ++r) on[x][r].template next<32>();
         uint32_t pa[2][RT][4];
 #pragma unroll
         for (int x = 0; x < RT; ++x) {
@@ -196,8 +199,11 @@ attend_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* _
             frag_hi(pa[1][x], c[x][2], c[x][3]);
         }
 #pragma unroll
-        for (int s = 0; s < 2; ++s) dense_mma_tokens<RT>(o, pa[s], vs, kb + 16 * s, lane);
+        for (int s = 0; s < 2; ++s) dense_mma_tokens<RT>(o, pa[s], vs + (kb + 16 * s) * 64, col_off);
     }
+    };
+    if (routes.weighted) walk(std::true_type());
+    else walk(std::false_type());
     cp_async_wait<0>();
     if (__syncthreads_or(dense_any_nan(o))) {                         // the slices have been read: staging takes their place
         attend_dense_by_token(Qg, Vg, lce_w, lce_b, O, lse, smem, routes.weighted, dm, gm);
@@ -261,12 +267,16 @@ cudaError_t launch_attend_dense(const Dims& d, const void* Q, const void* K, con
     Dims map = d;
     map.ws = d.W;
     const int tx = lce_tile_width(g.g, map);
-#define BRA_GO(RT, TX)                                                                                                           \
-    return d.n_r == 4 ? launch_t<RT, TX, 4>(d, g, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel)             \
-                      : launch_t<RT, TX, 0>(d, g, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel)
-    if (g.np <= 8) { if (tx == 2) BRA_GO(1, 2); BRA_GO(1, 4); }
-    if (tx == 2) BRA_GO(2, 2);
-    BRA_GO(2, 4);
+#define BRA_GO(RT, TX, NR) return launch_t<RT, TX, NR>(d, g, Q, K, V, index, lce_w, lce_b, O, lse, status, st, after_own_kernel)
+    if (d.n_r == 1) { if (tx == 2) BRA_GO(1, 2, 1); BRA_GO(1, 4, 1); }                    // at most 64 tokens
+    if (d.n_r == 4) {
+        if (g.np <= 8) { if (tx == 2) BRA_GO(1, 2, 4); BRA_GO(1, 4, 4); }
+        if (tx == 2) BRA_GO(2, 2, 4);
+        BRA_GO(2, 4, 4);
+    }
+    if (g.np <= 8) { if (tx == 2) BRA_GO(1, 2, 0); BRA_GO(1, 4, 0); }
+    if (tx == 2) BRA_GO(2, 2, 0);
+    BRA_GO(2, 4, 0);
 #undef BRA_GO
 }
 

@@ -4,10 +4,14 @@
 //   2. warp = 16 keys: dK = scale dS^T Q and dV = P^T dO in one walk over the queries; dV + LCE adjoint
 // P from the saved log-sum-exp, dP = dO V^T, dS = P o (dP - delta).  Who is routed where is the bit masks (with repeats a table
 // of log2 of the counts), so no inverse index is needed.  Every sum has a fixed order.
-// Bound: latency at 12 warps per SM (0.47 instructions per cycle and scheduler; per issue 1.8 cycles of fixed waits, 1.0 at
-// barriers, 0.55 for the MMA pipe), 1.73 waves; the two walks over the keys in 1. make S and dP twice.  Measured (B200) against the kernels of
-// backward_img.cu: 64 x 14 x 14, 8 heads, topk 16: 156 -> 103 us; 64 x 7 x 7, 16 heads, topk 49: 477 -> 39 us.
+// Bound: latency at 12 warps per SM (0.46 instructions per cycle and scheduler; per issue 1.3 cycles of fixed waits, 1.1 at
+// barriers, 0.84 for the MMA pipe), 1.73 waves; the two walks over the keys in 1. make S and dP twice.  Measured (B200) against the kernels of
+// backward_img.cu: 64 x 14 x 14, 8 heads, topk 16: 156 -> 103 us; 64 x 7 x 7, 16 heads, topk 49: 477 -> 39 us.  With the mask picked
+// before the exponential, a walk of its own for lists with repeats and the slices' swizzle out of the walks (12.2 k -> 10.3 k
+// instructions a warp): 96 -> 84 us, forward + backward 155.5 -> 142.2; 64 x 12 x 12 153.0 -> 138.4; 64 x 9 x 9, S = 3 69.8 -> 65.0.
 #include "dense_common.cuh"
+
+#include <type_traits>
 
 namespace bra {
 
@@ -138,69 +142,75 @@ bwd_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __re
     };
 
     // ---- queries: delta, dQ ----
+    const uint32_t row_off = dense_row_offset(lane), col_off = dense_col_offset(lane);
     bool nan = false;
+    auto queries = [&](auto weighted) {
 #pragma unroll 1
     for (int tile = warp; tile < steps; tile += gm.nw) {
         const int r0 = tile * 16;
         uint32_t qa[1][2][4], ga[1][2][4];
-        dense_a(qa, qs, r0, g, t4);
-        dense_a(ga, gs, r0, g, t4);
+        dense_a(qa, qs + r0 * 64 + row_off);
+        dense_a(ga, gs + r0 * 64 + row_off);
         const float l0 = s_l2[r0 + g], l1 = s_l2[r0 + 8 + g];
         const int i0 = min((int)reg[r0 + g], dm.R - 1), i1 = min((int)reg[r0 + 8 + g], dm.R - 1);
-        const unsigned long long m0 = mask[i0], m1 = mask[i1];
         float delta[2] = {0.f, 0.f}, dq[1][4][4];
 #pragma unroll
         for (int n = 0; n < 4; ++n)
 #pragma unroll
             for (int e = 0; e < 4; ++e) dq[0][n][e] = 0.f;
-#pragma unroll 1
-        for (int sweep = 0; sweep < 2; ++sweep) {
+        // P and dP of 16 keys
+        auto scores = [&](float (&c)[2][4], float (&dp)[2][4], DenseRow<NR>& on0, DenseRow<NR>& on1, int kb) {
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const uint4 kr[1] = {dense_chunk(ks + (kb + 8 * j) * 64 + row_off)}, vr[1] = {dense_chunk(vs + (kb + 8 * j) * 64 + row_off)};
+                mma_rows<1>(c[j], qa, kr);
+                mma_rows<1>(dp[j], ga, vr);
+            }
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int r = weighted.value ? reg[kb + 8 * j + 2 * t4 + e] : 0;
+                    const float a = weighted.value ? dense_weight(bias + i0 * dm.R, r) - l0 : on0.pick(-l0, j, e, kb, t4, reg);
+                    const float b = weighted.value ? dense_weight(bias + i1 * dm.R, r) - l1 : on1.pick(-l1, j, e, kb, t4, reg);
+                    c[j][e] = ex2_approx(fmaf(c[j][e], sl2, a));
+                    c[j][2 + e] = ex2_approx(fmaf(c[j][2 + e], sl2, b));
+                }
+            on0.template next<16>();
+            on1.template next<16>();
+        };
+        {
+            DenseRow<NR> on0(mask[i0], t4), on1(mask[i1], t4);
 #pragma unroll 2
             for (int kb = 0; kb < dm.N; kb += 16) {
                 float c[2][4], dp[2][4];
+                scores(c, dp, on0, on1, kb);
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
-                    const uint4 kr[1] = {dense_row(ks, kb + 8 * j + g, t4)}, vr[1] = {dense_row(vs, kb + 8 * j + g, t4)};
-                    mma_rows<1>(c[j], qa, kr);
-                    mma_rows<1>(dp[j], ga, vr);
-                    float a0 = -l0, a1 = -l0, a2 = -l1, a3 = -l1;
-                    const int k = kb + 8 * j + 2 * t4;
-                    if (routes.weighted) {
-                        const uchar2 kg = *reinterpret_cast<const uchar2*>(reg + k);
-                        const float* b0 = bias + i0 * dm.R;
-                        const float* b1 = bias + i1 * dm.R;
-                        if (kg.x < 64) { a0 += b0[kg.x]; a2 += b1[kg.x]; }
-                        if (kg.y < 64) { a1 += b0[kg.y]; a3 += b1[kg.y]; }
-                    }
-                    c[j][0] = ex2_approx(fmaf(c[j][0], sl2, a0));
-                    c[j][1] = ex2_approx(fmaf(c[j][1], sl2, a1));
-                    c[j][2] = ex2_approx(fmaf(c[j][2], sl2, a2));
-                    c[j][3] = ex2_approx(fmaf(c[j][3], sl2, a3));
-                }
-                if (routes.masked || kb + 16 > dm.N) dense_mask<NR, 2>(c, m0, m1, kb, t4, reg, 0.f);
-                if (sweep == 0) {
-#pragma unroll
-                    for (int j = 0; j < 2; ++j) {
-                        delta[0] = fmaf(c[j][0], dp[j][0], fmaf(c[j][1], dp[j][1], delta[0]));
-                        delta[1] = fmaf(c[j][2], dp[j][2], fmaf(c[j][3], dp[j][3], delta[1]));
-                    }
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 2; ++j) {
-                        c[j][0] *= dp[j][0] - delta[0]; c[j][1] *= dp[j][1] - delta[0];
-                        c[j][2] *= dp[j][2] - delta[1]; c[j][3] *= dp[j][3] - delta[1];
-                    }
-                    uint32_t sa[1][4];
-                    frag_hi(sa[0], c[0], c[1]);
-                    dense_mma_tokens<1>(dq, sa, ks, kb, lane);
+                    delta[0] = fmaf(c[j][0], dp[j][0], fmaf(c[j][1], dp[j][1], delta[0]));
+                    delta[1] = fmaf(c[j][2], dp[j][2], fmaf(c[j][3], dp[j][3], delta[1]));
                 }
             }
-            if (sweep == 0) {
+        }
 #pragma unroll
-                for (int r = 0; r < 2; ++r) {
-                    delta[r] += __shfl_xor_sync(0xffffffffu, delta[r], 1);
-                    delta[r] += __shfl_xor_sync(0xffffffffu, delta[r], 2);
+        for (int r = 0; r < 2; ++r) {
+            delta[r] += __shfl_xor_sync(0xffffffffu, delta[r], 1);
+            delta[r] += __shfl_xor_sync(0xffffffffu, delta[r], 2);
+        }
+        {
+            DenseRow<NR> on0(mask[i0], t4), on1(mask[i1], t4);
+#pragma unroll 2
+            for (int kb = 0; kb < dm.N; kb += 16) {
+                float c[2][4], dp[2][4];
+                scores(c, dp, on0, on1, kb);
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    c[j][0] *= dp[j][0] - delta[0]; c[j][1] *= dp[j][1] - delta[0];
+                    c[j][2] *= dp[j][2] - delta[1]; c[j][3] *= dp[j][3] - delta[1];
                 }
+                uint32_t sa[1][4];
+                frag_hi(sa[0], c[0], c[1]);
+                dense_mma_tokens<1>(dq, sa, ks + kb * 64, col_off);
             }
         }
         nan = nan || dense_any_nan(dq) || delta[0] != delta[0] || delta[1] != delta[1];
@@ -214,6 +224,9 @@ bwd_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __re
             for (int n = 0; n < 4; ++n) o[4 * n] = pack2_bf16(dq[0][n][2 * r] * dm.scale, dq[0][n][2 * r + 1] * dm.scale);
         }
     }
+    };
+    if (routes.weighted) queries(std::true_type());
+    else queries(std::false_type());
     if (__syncthreads_or(nan)) {
         cp_async_wait<0>();
         bwd_dense_by_token(lce_w, dOg, dQg, dKg, dVg, smem, routes.weighted, dm, gm);
@@ -222,15 +235,16 @@ bwd_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __re
 
     // ---- keys: dK, dV (a warp has at most two tiles; dV is staged once all warps have read the slices) ----
     float dv[2][4][4];
+    auto keys = [&](auto weighted) {
 #pragma unroll
     for (int x = 0; x < 2; ++x) {
         const int r0 = (warp + x * gm.nw) * 16;
         if (r0 >= steps * 16) continue;
         uint32_t ka[1][2][4], va[1][2][4];
-        dense_a(ka, ks, r0, g, t4);
-        dense_a(va, vs, r0, g, t4);
+        dense_a(ka, ks + r0 * 64 + row_off);
+        dense_a(va, vs + r0 * 64 + row_off);
         const int k0 = min((int)reg[r0 + g], dm.R - 1), k1 = min((int)reg[r0 + 8 + g], dm.R - 1);
-        const unsigned long long m0 = mask[64 + k0], m1 = mask[64 + k1];
+        DenseRow<NR> on0(mask[64 + k0], t4), on1(mask[64 + k1], t4);
         float dk[1][4][4];
 #pragma unroll
         for (int n = 0; n < 4; ++n)
@@ -241,33 +255,37 @@ bwd_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __re
             float c[2][4], dp[2][4];
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
-                const uint4 qr[1] = {dense_row(qs, qb + 8 * j + g, t4)}, gr[1] = {dense_row(gs, qb + 8 * j + g, t4)};
+                const uint4 qr[1] = {dense_chunk(qs + (qb + 8 * j) * 64 + row_off)}, gr[1] = {dense_chunk(gs + (qb + 8 * j) * 64 + row_off)};
                 mma_rows<1>(c[j], ka, qr);
                 mma_rows<1>(dp[j], va, gr);
+            }
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
                 const int q = qb + 8 * j + 2 * t4;
                 const float2 l2 = *reinterpret_cast<const float2*>(s_l2 + q), dl = *reinterpret_cast<const float2*>(s_dl + q);
-                float a0 = -l2.x, a1 = -l2.y, a2 = -l2.x, a3 = -l2.y;
-                if (routes.weighted) {
-                    const uchar2 qg = *reinterpret_cast<const uchar2*>(reg + q);
-                    if (qg.x < 64) { a0 += bias[qg.x * dm.R + k0]; a2 += bias[qg.x * dm.R + k1]; }
-                    if (qg.y < 64) { a1 += bias[qg.y * dm.R + k0]; a3 += bias[qg.y * dm.R + k1]; }
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const float l = e ? l2.y : l2.x, d = e ? dl.y : dl.x;
+                    const int r = weighted.value ? reg[q + e] : 0;
+                    const float a = weighted.value ? (r < 64 ? bias[r * dm.R + k0] : -INFINITY) - l : on0.pick(-l, j, e, qb, t4, reg);
+                    const float b = weighted.value ? (r < 64 ? bias[r * dm.R + k1] : -INFINITY) - l : on1.pick(-l, j, e, qb, t4, reg);
+                    c[j][e] = ex2_approx(fmaf(c[j][e], sl2, a));
+                    c[j][2 + e] = ex2_approx(fmaf(c[j][2 + e], sl2, b));
+                    dp[j][e] -= d;
+                    dp[j][2 + e] -= d;
                 }
-                c[j][0] = ex2_approx(fmaf(c[j][0], sl2, a0));
-                c[j][1] = ex2_approx(fmaf(c[j][1], sl2, a1));
-                c[j][2] = ex2_approx(fmaf(c[j][2], sl2, a2));
-                c[j][3] = ex2_approx(fmaf(c[j][3], sl2, a3));
-                dp[j][0] -= dl.x; dp[j][1] -= dl.y; dp[j][2] -= dl.x; dp[j][3] -= dl.y;
             }
-            if (routes.masked) dense_mask<NR, 2>(c, m0, m1, qb, t4, reg, 0.f);
+            on0.template next<16>();
+            on1.template next<16>();
 #pragma unroll
             for (int j = 0; j < 2; ++j)
 #pragma unroll
                 for (int e = 0; e < 4; ++e) dp[j][e] *= c[j][e];
             uint32_t a[1][4];
             frag_hi(a[0], dp[0], dp[1]);
-            dense_mma_tokens<1>(dk, a, qs, qb, lane);
+            dense_mma_tokens<1>(dk, a, qs + qb * 64, col_off);
             frag_hi(a[0], c[0], c[1]);
-            dense_mma_tokens<1>(dv + x, a, gs, qb, lane);
+            dense_mma_tokens<1>(dv + x, a, gs + qb * 64, col_off);
         }
         nan = nan || dense_any_nan(dk) || dense_any_nan(reinterpret_cast<const float (&)[1][4][4]>(dv[x]));
 #pragma unroll
@@ -279,6 +297,9 @@ bwd_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __re
             for (int n = 0; n < 4; ++n) o[4 * n] = pack2_bf16(dk[0][n][2 * r] * dm.scale, dk[0][n][2 * r + 1] * dm.scale);
         }
     }
+    };
+    if (routes.weighted) keys(std::true_type());
+    else keys(std::false_type());
     cp_async_wait<0>();
     if (__syncthreads_or(nan)) {
         bwd_dense_by_token(lce_w, dOg, dQg, dKg, dVg, smem, routes.weighted, dm, gm);
@@ -338,6 +359,7 @@ cudaError_t launch_backward_dense(const Dims& d, const void* Q, const void* K, c
     const bool narrow = lce_tile_width(g.g, map) == 2;
 #define BRA_GO(TX, NR) return launch_t<TX, NR>(d, g, Q, K, V, index, lce_w, lse, dO, dQ, dK, dV, status, st)
     if (d.n_r == 4) { if (narrow) BRA_GO(2, 4); BRA_GO(4, 4); }
+    if (d.n_r == 1) { if (narrow) BRA_GO(2, 1); BRA_GO(4, 1); }
     if (narrow) BRA_GO(2, 0);
     BRA_GO(4, 0);
 #undef BRA_GO

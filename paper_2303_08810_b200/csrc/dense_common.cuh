@@ -142,36 +142,45 @@ __device__ __forceinline__ DenseRoutes dense_routes(unsigned long long* mask, fl
     }
     return out;
 }
-// Columns of J n-tiles from token k0 on whose region's bit is not set in m0 (row g) / m1 (row g + 8): value v.
-// NR = 4: regions of four tokens, else by table.
-template <int NR, int J>
-__device__ __forceinline__ void dense_mask(float (&c)[J][4], unsigned long long m0, unsigned long long m1, int k0, int t4, const uint8_t* reg, float v) {
-    if (NR == 4) {
-        const uint32_t w0 = (uint32_t)(m0 >> (k0 >> 2)) >> (t4 >> 1), w1 = (uint32_t)(m1 >> (k0 >> 2)) >> (t4 >> 1);
-#pragma unroll
-        for (int j = 0; j < J; ++j) {
-            if (!(w0 & (1u << (2 * j)))) c[j][0] = c[j][1] = v;
-            if (!(w1 & (1u << (2 * j)))) c[j][2] = c[j][3] = v;
+// What is added to the scaled scores of a row for the columns of n-tiles, in blocks of tokens from 0 on: `yes` where the column's region
+// is on the row's list, -inf elsewhere (and behind the last token).  NR: tokens per region - with four a bit of the mask covers the
+// two columns a lane holds of an n-tile, with one it is the token's, 0 (any) goes by the table of regions.  (A bit per two or
+// four scores, picked before the exponential: a test and a select per row and n-tile instead of per score behind it.)
+template <int NR>
+struct DenseRow {
+    unsigned long long m;
+    DenseRow() = default;
+    __device__ __forceinline__ DenseRow(unsigned long long mask, int t4) : m(NR == 4 ? mask >> (t4 >> 1) : NR == 1 ? mask >> (2 * t4) : mask) {}
+    // n-tile j of the block from token k0 on, column 2 t4 + e
+    __device__ __forceinline__ float pick(float yes, int j, int e, int k0, int t4, const uint8_t* reg) const {
+        bool on;
+        if (NR == 4) on = (uint32_t)m >> (2 * j) & 1;
+        else if (NR == 1) on = (uint32_t)m >> (8 * j + e) & 1;
+        else {
+            const int r = reg[k0 + 8 * j + 2 * t4 + e];
+            on = r < 64 && (m >> r & 1);
         }
-    } else {
-#pragma unroll
-        for (int j = 0; j < J; ++j) {
-            const uchar2 r = *reinterpret_cast<const uchar2*>(reg + k0 + 8 * j + 2 * t4);
-            if (r.x > 63 || !(m0 >> r.x & 1)) c[j][0] = v;
-            if (r.y > 63 || !(m0 >> r.y & 1)) c[j][1] = v;
-            if (r.x > 63 || !(m1 >> r.x & 1)) c[j][2] = v;
-            if (r.y > 63 || !(m1 >> r.y & 1)) c[j][3] = v;
-        }
+        return on ? yes : -INFINITY;
     }
-}
+    template <int TOKENS>
+    __device__ __forceinline__ void next() {
+        if (NR == 4) m >>= TOKENS / 4;
+        if (NR == 1) m >>= TOKENS;
+    }
+};
+// the same for lists with repeats, from row `at` of the table of log2(count)
+__device__ __forceinline__ float dense_weight(const float* at, int r) { return r < 64 ? at[r] : -INFINITY; }
 
-// rows r0 + g (lo), r0 + 8 + g of a slice, this lane's 16-byte chunk
-__device__ __forceinline__ uint4 dense_row(uint32_t slice, int r, int t4) {
-    const float4 f = ptx::lds_f32x4(slice + dense_at(r, t4));
+// Offsets of a lane in a slice: its 16-byte chunk of row g; rows lane % 16 for ldmatrix (exclusive or with 32: two chunks on).
+// From a row that is a multiple of eight on.
+__device__ __forceinline__ uint32_t dense_row_offset(int lane) { return dense_at(lane >> 2, lane & 3); }
+__device__ __forceinline__ uint32_t dense_col_offset(int lane) { return dense_at(lane & 15, lane >> 4); }
+__device__ __forceinline__ uint4 dense_chunk(uint32_t at) {
+    const float4 f = ptx::lds_f32x4(at);
     return make_uint4(__float_as_uint(f.x), __float_as_uint(f.y), __float_as_uint(f.z), __float_as_uint(f.w));
 }
-__device__ __forceinline__ void dense_a(uint32_t (&a)[1][2][4], uint32_t slice, int r0, int g, int t4) {
-    const uint4 lo[1] = {dense_row(slice, r0 + g, t4)}, up[1] = {dense_row(slice, r0 + 8 + g, t4)};
+__device__ __forceinline__ void dense_a(uint32_t (&a)[1][2][4], uint32_t at) {
+    const uint4 lo[1] = {dense_chunk(at)}, up[1] = {dense_chunk(at + 512)};
     rows_to_a<1>(a, lo, up);
 }
 // The products run over every token of the map, with probability 0 where a pair is not routed: an infinity or NaN of a token
@@ -225,14 +234,13 @@ __device__ __forceinline__ void dense_lce_row(float (&acc)[32], const __nv_bfloa
     }
 }
 
-// acc (16 x 32) += A (16 x 16, fp32 fragments c0, c1) * the 16 rows of a slice from r0 on
+// acc (16 x 32) += A (16 x 16) * the 16 rows of a slice that start at `rows`
 template <int RT>
-__device__ __forceinline__ void dense_mma_tokens(float (*acc)[4][4], const uint32_t (*a)[4], uint32_t slice, int r0, int lane) {
-    const int r = r0 + (lane & 15);
+__device__ __forceinline__ void dense_mma_tokens(float (*acc)[4][4], const uint32_t (*a)[4], uint32_t rows, uint32_t col_off) {
 #pragma unroll
     for (int np = 0; np < 2; ++np) {
         uint32_t b[4];
-        ldmatrix_x4_trans(slice + dense_at(r, 2 * np + (lane >> 4)), b);
+        ldmatrix_x4_trans(rows + (col_off ^ (np * 32)), b);
 #pragma unroll
         for (int x = 0; x < RT; ++x) {
             mma_bf16(acc[x][2 * np], a[x], b[0], b[1]);

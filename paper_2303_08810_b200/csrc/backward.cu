@@ -440,8 +440,7 @@ static cudaError_t launch_bwd_t(const Dims& d, int impl, const void* Q, const vo
     } else if (family == FAMILY_DENSE) {
         if ((e = launch_backward_dense(d, Q, K, V, index, lce_w, lse, dO, dQ, dK, dV, status, st)) != cudaSuccess) return e;
     } else if (family == FAMILY_DIRECT) {
-        if ((e = launch_backward_direct(d, Q, K, V, index, inv_off, inv_list, inv_order, lce_w, lse, dO, dQ, dK, dV,
-                                        delta, status, st)) != cudaSuccess) return e;
+        if ((e = launch_backward_direct(d, Q, K, V, index, ws, L, lce_w, lse, dO, dQ, dK, dV, st)) != cudaSuccess) return e;
     } else {
         SimtGeom g = simt_geom(d, SIMT_DQ);
         const int inv = (int)inverse_smem(d);

@@ -34,13 +34,13 @@ bwd_dq_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* 
                      const float* __restrict__ lse, const __nv_bfloat16* __restrict__ dOg,
                      __nv_bfloat16* __restrict__ dQg, float* __restrict__ delta_out,
                      int32_t* __restrict__ inv_off, int32_t* __restrict__ inv_list, int32_t* __restrict__ inv_order, bool inv_bits,
-                     int32_t* __restrict__ status, Dims dm, DirGeom gm) {
+                     ListJobs lj, int32_t* __restrict__ status, Dims dm, DirGeom gm) {
     constexpr int RT = 1, KS = SINGLE ? 4 : 2;                        // tiles per warp, 16-key steps per block
     extern __shared__ __align__(128) uint8_t smem[];
     // blockIdx.y = 0: the inverse index (one CTA per (image, routing head)); else head blockIdx.y - 1
     if (blockIdx.y == 0) {
         if (inv_off && (int)blockIdx.x < dm.heads_i)
-            inverse_index_job(index, inv_off, inv_list, inv_order, blockIdx.z * dm.heads_i + blockIdx.x, reinterpret_cast<int32_t*>(smem), inv_bits, dm);
+            inverse_index_job(index, inv_off, inv_list, inv_order, blockIdx.z * dm.heads_i + blockIdx.x, reinterpret_cast<int32_t*>(smem), inv_bits, dm, lj);
         return;
     }
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -208,14 +208,71 @@ bwd_dq_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* 
 }
 
 // ------------------------------------------------------------------ dK, dV
-template <int PL, bool EXACT, int TY, int TX>
+// dK = scale * acc of a tile's rows (tokens tok of the map), dV to the staging tile
+template <int PL>
+__device__ __forceinline__ void finish_rows(uint8_t* dKb, float* st, const float (&dk)[PL][4][4], const float (&dv)[PL][4][4], const int (&tok)[2], int tile,
+                                            int ntok, int g, int t4, const Dims& dm) {
+    const uint32_t tok_bytes = (uint32_t)dm.C * 2;
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const int tk = tile * 16 + g + 8 * r;
+        if (tk >= ntok) continue;
+        if (tok[r] >= 0) {
+            uint8_t* o = dKb + (size_t)(uint32_t)tok[r] * tok_bytes;
+#pragma unroll
+            for (int p = 0; p < PL; ++p) *reinterpret_cast<uint4*>(o + p * 64) = pack_row(dk[p], r, dm.scale);
+        }
+        float* dst = st + tk * 32 * PL + t4 * 8;
+#pragma unroll
+        for (int p = 0; p < PL; ++p)
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+                *reinterpret_cast<float4*>(dst + p * 32 + 4 * q) = make_float4(dv[p][2 * q][2 * r], dv[p][2 * q][2 * r + 1],
+                                                                               dv[p][2 * q + 1][2 * r], dv[p][2 * q + 1][2 * r + 1]);
+    }
+}
+// The same for the sums of the parts of a cut list, added in the order of the parts
+template <int PL>
+__device__ __forceinline__ void sum_parts(const float* at, int nparts, size_t stride, uint8_t* dKb, float* st, int jr, int c0, int tile, int ntok, int lane,
+                                          const Dims& dm, const DirGeom& gm) {
+    const int g = lane >> 2, t4 = lane & 3;
+    int tok[2];
+    float dk[PL][4][4], dv[PL][4][4];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const int tk = tile * 16 + g + 8 * r;
+        tok[r] = tk < ntok ? token_of(dm, gm, jr, c0 + tk) : -1;
+    }
+#pragma unroll
+    for (int p = 0; p < PL; ++p)
+#pragma unroll
+        for (int n = 0; n < 4; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) dk[p][n][e] = dv[p][n][e] = 0.f;
+#pragma unroll 1
+    for (int q = 0; q < nparts; ++q, at += stride) {
+#pragma unroll
+        for (int p = 0; p < PL; ++p)
+#pragma unroll
+            for (int n = 0; n < 4; ++n)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    dk[p][n][e] += __ldcg(at + ((p * 4 + n) * 4 + e) * 32);
+                    dv[p][n][e] += __ldcg(at + ((PL * 4 + p * 4 + n) * 4 + e) * 32);
+                }
+    }
+    finish_rows<PL>(dKb, st, dk, dv, tok, tile, ntok, g, t4, dm);
+}
+// CUT: long lists in parts (ListParts).
+template <int PL, bool EXACT, bool CUT, int TY, int TX>
 __global__ void __launch_bounds__(PL == 2 ? 128 : 256, PL == 2 ? 3 : 2)
 bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __restrict__ Kg,
                       const __nv_bfloat16* __restrict__ Vg, const int32_t* inv_off,
                       const int32_t* inv_list, const int32_t* inv_order, const float* __restrict__ lse,
                       const float* delta, const __nv_bfloat16* __restrict__ dOg,
                       const float* __restrict__ lce_w, __nv_bfloat16* __restrict__ dKg,
-                      __nv_bfloat16* __restrict__ dVg, Dims dm, DirGeom gm) {
+                      __nv_bfloat16* __restrict__ dVg, const int2* jobs, ListParts parts, int32_t* done, float* sums, int job0,
+                      const __grid_constant__ Dims dm, const __grid_constant__ DirGeom gm) {
     constexpr int RT = 1, KS = PL == 2 ? 1 : 2;                       // tiles per warp, 16-query steps per block
     extern __shared__ __align__(128) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
@@ -228,7 +285,7 @@ bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16*
     const int nth = one_warp ? rest * gm.gpc + warp : rest / gm.chunks;  // by falling length of the list
     const int gwarp = one_warp ? 0 : warp, gwarps = one_warp ? 1 : gm.nw;
     const int glane = one_warp ? lane : tid, glanes = gwarps * 32;
-    const bool live = nth < dm.R;
+    const bool live = nth < parts.jobs - job0;
     auto group_sync = [&]() { if (one_warp) __syncwarp(); else __syncthreads(); };
 
     const int rows = min(gm.hb, dm.hs - ck * gm.hb);
@@ -244,21 +301,34 @@ bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16*
     uint8_t* dKb = reinterpret_cast<uint8_t*>(dKg) + head_off + t4 * 16;
 
     const uint4 probe = spare_probe<PL>(Qb - t4 * 16, Gh, lane);
+    const int hi = dm.heads_i == 1 ? 0 : h;
+    const size_t bhi = (size_t)b * dm.heads_i + hi;
+    int2 job = make_int2(-1, 0);                                      // key region, part of its list
+    // there are as many jobs as regions, or more
+    if (CUT && !one_warp && job0 + nth >= dm.R) {
+        pdl_wait();
+        if (__ldcg(&jobs[bhi * parts.jobs + job0 + nth].x) < 0) return;
+    }
     float* s_w = reinterpret_cast<float*>(smem + gm.off_w);
     if (dm.lce) load_lce_weights(s_w, lce_w, h, 32 * PL * 25, tid, gm.nw * 32);
     __syncthreads();                                                  // weights
     pdl_wait();          // delta, the inverse index and the order of the regions come from the dQ kernel
-    if (!live) return;
+    if (CUT && live) job = __ldcg(jobs + bhi * parts.jobs + job0 + nth);
+    if (CUT ? job.x < 0 : !live) return;
+    if (!CUT) job.x = __ldcg(inv_order + bhi * dm.R + job0 + nth);
     const int spare = spare_token<PL>(probe, Qb - t4 * 16, Gh, tok_bytes, N0, lane);
 
-    const int hi = dm.heads_i == 1 ? 0 : h;
-    const size_t bhi = (size_t)b * dm.heads_i + hi;
-    const int jr = __ldcg(inv_order + bhi * dm.R + nth);              // key region
+    const int jr = job.x;
     const int ry = fdiv(jr, dm.S, gm.mul_s), rx = jr - ry * dm.S;
     const int y0 = ry * dm.hs + ck * gm.hb, x0 = rx * dm.ws;
     if (dm.lce) load_halo<PL>(sbase + gm.off_halo + grp * gm.halo_bytes, Gh, y0, x0, rows, dm, gm, glane, glanes);
     cp_async_commit();
-    const int e0 = __ldcg(inv_off + bhi * (dm.R + 1) + jr), e1 = __ldcg(inv_off + bhi * (dm.R + 1) + jr + 1);
+    const int l0 = __ldcg(inv_off + bhi * (dm.R + 1) + jr), l1 = __ldcg(inv_off + bhi * (dm.R + 1) + jr + 1);
+    const int nparts = CUT ? max(1, (l1 - l0 + parts.most - 1) / parts.most) : 1;
+    const int e0 = CUT ? l0 + job.y * parts.most : l0, e1 = CUT ? min(l1, e0 + parts.most) : l1;
+    // (parts, job, part): not needed before the end, so they wait behind the table; every thread writes them, for itself
+    volatile int* s_job = reinterpret_cast<int*>(smem + gm.off_tab + grp * gm.tab_bytes) + 3 * gm.tab;
+    if (CUT) { s_job[0] = nparts; s_job[1] = job0 + nth; s_job[2] = job.y; }
     const int32_t* list = inv_list + bhi * dm.R * dm.topk + e0;      // query regions that list jr, fixed order
     const long long total = (long long)(e1 - e0) * dm.n_r;           // a list with repeats may hold every entry of the index
     const float* lse_h = lse + ((size_t)b * dm.heads + h) * N0;
@@ -284,6 +354,8 @@ bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16*
         }
     };
     bool filled = false;
+    // where the sums of a tile of a job lie: 32 lanes times dK, dV as the lane holds them
+    auto sum_at = [&](int j, int tile) { return (((((size_t)b * dm.heads + h) * parts.cut + j) * gm.chunks + ck) * gm.tpc + tile) * 1024 * PL + lane; };
 
     for (int tile = gwarp * RT; tile - gwarp * RT < gm.tpc; tile += gwarps * RT) {
         const bool has = tile * 16 < ntok;
@@ -368,26 +440,32 @@ bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16*
                 }
             }
         }
-        // ---- dK = scale * acc; dV to the staging tile ----
+        if (CUT && s_job[0] > 1) {                                    // the sums of a part: to scratch memory
+            float* at = sums + sum_at(s_job[1], tile);
 #pragma unroll
-        for (int x = 0; x < RT; ++x)
+            for (int p = 0; p < PL; ++p)
 #pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                const int tk = (tile + x) * 16 + g + 8 * r;
-                if (tk >= ntok) continue;
-                if (tok[x][r] >= 0) {
-                    uint8_t* o = dKb + (size_t)(uint32_t)tok[x][r] * tok_bytes;
+                for (int n = 0; n < 4; ++n)
 #pragma unroll
-                    for (int p = 0; p < PL; ++p) *reinterpret_cast<uint4*>(o + p * 64) = pack_row(dkx[x][p], r, dm.scale);
-                }
-                float* dst = st + tk * 32 * PL + t4 * 8;
-#pragma unroll
-                for (int p = 0; p < PL; ++p)
-#pragma unroll
-                    for (int q = 0; q < 2; ++q)
-                        *reinterpret_cast<float4*>(dst + p * 32 + 4 * q) = make_float4(dvx[x][p][2 * q][2 * r], dvx[x][p][2 * q][2 * r + 1],
-                                                                                       dvx[x][p][2 * q + 1][2 * r], dvx[x][p][2 * q + 1][2 * r + 1]);
-            }
+                    for (int e = 0; e < 4; ++e) {
+                        __stcg(at + ((p * 4 + n) * 4 + e) * 32, dkx[0][p][n][e]);
+                        __stcg(at + ((PL * 4 + p * 4 + n) * 4 + e) * 32, dvx[0][p][n][e]);
+                    }
+        } else {
+            finish_rows<PL>(dKb, st, dkx[0], dvx[0], tok[0], tile, ntok, g, t4, dm);
+        }
+    }
+    if (CUT && s_job[0] > 1) {                                        // the part that is done last adds them up
+        const int nparts = s_job[0], first = s_job[1] - s_job[2];
+        int last = 0;
+        __threadfence();
+        group_sync();
+        if (glane == 0) last = atomicAdd(done + (((size_t)b * dm.heads + h) * dm.R + jr) * gm.chunks + ck, 1) == nparts - 1;
+        last = one_warp ? __shfl_sync(0xffffffffu, last, 0) : __syncthreads_or(last);
+        if (!last) { cp_async_wait<0>(); return; }
+        __threadfence();
+        for (int tile = gwarp; tile * 16 < ntok; tile += gwarps)
+            sum_parts<PL>(sums + sum_at(first, tile), nparts, (size_t)gm.chunks * gm.tpc * 1024 * PL, dKb, st, jr, c0, tile, ntok, lane, dm, gm);
     }
     cp_async_wait<0>();
     group_sync();
@@ -403,7 +481,7 @@ static DirGeom dq_geom(const Dims& d) {
     if (dq_single(d)) k.topk = (64 + d.n_r - 1) / d.n_r;             // one block of 64 keys
     DirGeom g = direct_geom(k, false, 4, 1);
     g.smem_bytes = g.off_tab + g.gpc * g.tab_bytes;                  // the table only
-    const int inv = (int)inverse_smem(d);
+    const int inv = (int)inverse_smem(d, true);
     if (g.smem_bytes < inv) g.smem_bytes = inv;
     return g;
 }
@@ -416,6 +494,35 @@ static DirGeom dkv_geom(const Dims& d) {
 bool backward_direct_supported(const Dims& d, int dtype) {
     if (!attend_direct_supported(d, dtype)) return false;
     return dkv_geom(d).smem_bytes <= 200 * 1024 && dq_geom(d).smem_bytes <= 200 * 1024 && d.R <= 8192;
+}
+
+// A part is what a group of warps would have on average if all were busy from the first to the last, and at least 256 queries; lists are
+// cut where the longest possible one is four parts or more, in problems that have no other kernels.  Measured (B200), forward +
+// backward, lists whole / cut.  A few regions holding most of the lists: 2 x 100 x 167, 6 heads, S = 16, topk 4 (87 % of the lists are empty, the
+// longest has 84 entries) 487 / 412 us, 1 x 123 x 99, 4 heads, topk 2 164 / 92, 2 x 80 x 80, S = 8, topk 1 112 / 77.  Evenly spread
+// lists: 2 x 50 x 84, 8 heads, topk 8 202 / 178, 1 x 92 x 84, 6 heads 120 / 107, 2 x 100 x 167, 6 heads 406 / 410.  Parts of 8 entries of 2 x 2 regions
+// (10 x 15 x 15, 3 heads of 64, S = 8, topk 12): 61 / 80.
+ListParts direct_grad_parts(const Dims& d, int* chunks, size_t* sum_bytes) {
+    ListParts p = {0, d.R, 0};
+    *sum_bytes = 0;
+    *chunks = 1;
+    if (!backward_direct_supported(d, d.esize == 2 ? BRA_BF16 : BRA_F32) || backward_one_supported(d, BRA_BF16) ||
+        (backward_dense_supported(d, BRA_BF16) && dense_grad_pays(d)) || (backward_img_supported(d, BRA_BF16) && img_grad_pays(d)))
+        return p;
+    const DirGeom g = dkv_geom(d);
+    *chunks = g.chunks;
+    const int warps = g.planes == 2 ? 12 : 16;                        // of an SM
+    const long long slots = (long long)kSMs * (g.gpc > 1 ? warps : warps / g.nw > 0 ? warps / g.nw : 1);
+    const long long entries = (long long)d.R * d.topk, work = entries * d.B * d.heads * g.chunks;
+    long long most = (work + slots - 1) / slots;
+    if (most < (256 + d.n_r - 1) / d.n_r) most = (256 + d.n_r - 1) / d.n_r;
+    if (most < 8) most = 8;
+    if (4 * most > d.R) return p;                                     // (a list is longer than R only where it repeats regions)
+    p.most = (int)most;
+    p.jobs = d.R + (int)(entries / most);
+    p.cut = (int)(2 * entries / most);
+    *sum_bytes = (size_t)d.B * d.heads * p.cut * g.chunks * g.tpc * 4096 * g.planes;
+    return p;
 }
 
 template <typename F>
@@ -432,6 +539,11 @@ struct BwdArgs {
     const float *lce_w, *lse;
     __nv_bfloat16 *dq, *dk, *dv;
     float* delta;
+    ListParts parts;
+    int chunks;
+    int2* jobs;
+    int32_t* done;
+    float* sums;
     int32_t* status;
     cudaStream_t st;
 };
@@ -446,27 +558,38 @@ static cudaError_t launch_dq(const Dims& d, const BwdArgs& a) {
     if (e != cudaSuccess) return e;
     return grid_pieces(d, [&](const GridPiece& p) {
         const InversePiece inv = inverse_piece(d, p, a.inv_off, a.inv_list, a.inv_order);
+        const int counters = (d.heads_i == 1 ? d.heads : 1) * d.R * a.chunks;
+        const ListJobs lj = {a.jobs + (size_t)p.b0 * d.heads_i * a.parts.jobs, a.done + (size_t)p.b0 * d.heads_i * counters, counters, a.parts};
         count_launch();
         return launch_kernel(kernel, dim3(g.gpi > d.heads_i ? g.gpi : d.heads_i, p.heads + 1, p.images), dim3(g.nw * 32), (size_t)g.smem_bytes, a.st,
                              false, a.q + p.tensor, a.k + p.tensor, a.v + p.tensor, a.index + p.index, a.lse + p.stat, a.go + p.tensor,
-                             a.dq + p.tensor, a.delta + p.stat, p.h0 ? nullptr : inv.off, inv.list, inv.order, inverse_uses_bits(d), a.status, d, g);
+                             a.dq + p.tensor, a.delta + p.stat, p.h0 ? nullptr : inv.off, inv.list, inv.order, inverse_uses_bits(d), lj, a.status, d, g);
+    });
+}
+
+template <int PL, bool EXACT, bool CUT, int TY, int TX>
+static cudaError_t launch_dkv_t(const Dims& d, const BwdArgs& a) {
+    const DirGeom g = dkv_geom(d);
+    auto kernel = bwd_dkv_direct_kernel<PL, EXACT, CUT, TY, TX>;
+    static PerDeviceMax set;
+    const cudaError_t e = allow_smem(set, kernel, g.smem_bytes);
+    if (e != cudaSuccess) return e;
+    const int all = (a.parts.jobs + g.gpc - 1) / g.gpc * g.chunks;
+    return group_pieces(d, all, g.chunks, [&](const GridPiece& p, int groups_before, int groups) {
+        const InversePiece inv = inverse_piece(d, p, a.inv_off, a.inv_list, a.inv_order);
+        const size_t bh = (size_t)p.b0 * d.heads;
+        count_launch();
+        return launch_kernel(kernel, dim3(p.heads, p.images, groups), dim3(g.nw * 32), (size_t)g.smem_bytes, a.st, true,
+                             a.q + p.tensor, a.k + p.tensor, a.v + p.tensor, inv.off, inv.list, inv.order, a.lse + p.stat,
+                             a.delta + p.stat, a.go + p.tensor, a.lce_w, a.dk + p.tensor, a.dv + p.tensor,
+                             a.jobs + (size_t)p.b0 * d.heads_i * a.parts.jobs, a.parts, a.done + bh * d.R * g.chunks,
+                             a.sums + bh * a.parts.cut * g.chunks * g.tpc * 1024 * PL, groups_before * g.gpc, d, g);
     });
 }
 
 template <int PL, bool EXACT, int TY, int TX>
 static cudaError_t launch_dkv(const Dims& d, const BwdArgs& a) {
-    const DirGeom g = dkv_geom(d);
-    auto kernel = bwd_dkv_direct_kernel<PL, EXACT, TY, TX>;
-    static PerDeviceMax set;
-    const cudaError_t e = allow_smem(set, kernel, g.smem_bytes);
-    if (e != cudaSuccess) return e;
-    return group_pieces(d, g.gpi, g.chunks, [&](const GridPiece& p, int regions_before, int groups) {
-        const InversePiece inv = inverse_piece(d, p, a.inv_off, a.inv_list, a.inv_order);
-        count_launch();
-        return launch_kernel(kernel, dim3(p.heads, p.images, groups), dim3(g.nw * 32), (size_t)g.smem_bytes, a.st, true,
-                             a.q + p.tensor, a.k + p.tensor, a.v + p.tensor, inv.off, inv.list, inv.order + regions_before, a.lse + p.stat,
-                             a.delta + p.stat, a.go + p.tensor, a.lce_w, a.dk + p.tensor, a.dv + p.tensor, d, g);
-    });
+    return a.parts.most ? launch_dkv_t<PL, EXACT, true, TY, TX>(d, a) : launch_dkv_t<PL, EXACT, false, TY, TX>(d, a);
 }
 
 static cudaError_t launch_both(const Dims& d, const BwdArgs& a) {
@@ -486,13 +609,17 @@ static cudaError_t launch_both(const Dims& d, const BwdArgs& a) {
     }
 }
 
-cudaError_t launch_backward_direct(const Dims& d, const void* Q, const void* K, const void* V,
-                                   const int32_t* index, int32_t* inv_off, int32_t* inv_list, int32_t* inv_order,
-                                   const float* lce_w, const float* lse, const void* dO,
-                                   void* dQ, void* dK, void* dV, float* delta, int32_t* status, cudaStream_t st) {
+cudaError_t launch_backward_direct(const Dims& d, const void* Q, const void* K, const void* V, const int32_t* index, char* ws, const WsLayout& L,
+                                   const float* lce_w, const float* lse, const void* dO, void* dQ, void* dK, void* dV, cudaStream_t st) {
     typedef __nv_bfloat16 bf;
+    int chunks;
+    size_t sum_bytes;
+    const ListParts parts = direct_grad_parts(d, &chunks, &sum_bytes);
+    auto at = [&](size_t off) { return reinterpret_cast<int32_t*>(ws + off); };
     const BwdArgs a = {static_cast<const bf*>(Q), static_cast<const bf*>(K), static_cast<const bf*>(V), static_cast<const bf*>(dO), index,
-                       inv_off, inv_list, inv_order, lce_w, lse, static_cast<bf*>(dQ), static_cast<bf*>(dK), static_cast<bf*>(dV), delta, status, st};
+                       at(L.inv_off), at(L.inv_list), at(L.inv_order), lce_w, lse, static_cast<bf*>(dQ), static_cast<bf*>(dK), static_cast<bf*>(dV),
+                       reinterpret_cast<float*>(ws + L.delta), parts, chunks, reinterpret_cast<int2*>(ws + L.jobs), at(L.done),
+                       reinterpret_cast<float*>(ws + L.sums), at(L.status), st};
     return launch_both(d, a);
 }
 

@@ -21,6 +21,12 @@ WsLayout ws_layout(const Dims& d) {
     L.inv_off = off;  off += align256(sizeof(int32_t) * (size_t)d.B * d.heads_i * (d.R + 1));
     L.inv_list = off; off += align256(sizeof(int32_t) * (size_t)d.B * d.heads_i * d.R * d.topk);
     L.inv_order = off; off += align256(sizeof(int32_t) * (size_t)d.B * d.heads_i * d.R);
+    int chunks = 0;
+    size_t sum_bytes = 0;
+    const ListParts parts = direct_grad_parts(d, &chunks, &sum_bytes);
+    L.jobs = off;     off += parts.most ? align256(sizeof(int2) * (size_t)d.B * d.heads_i * parts.jobs) : 0;
+    L.done = off;     off += parts.most ? align256(sizeof(int32_t) * (size_t)d.B * d.heads * d.R * chunks) : 0;
+    L.sums = off;     off += align256(sum_bytes);
     L.dw_part = off;  off += align256(sizeof(float) * (size_t)lce_grad_partials(d) * d.C * 26);
     L.pad = L.pad_lse = off;
     L.pad_tensor = 0;

@@ -63,6 +63,15 @@ inline cudaError_t grid_pieces(const Dims& d, F&& launch) {
 template <typename T>
 inline T* piece_of(T* p, size_t n) { return p ? p + n : nullptr; }
 
+// Lists of the inverse routing index cut in parts (the dK / dV kernel of backward_direct.cu): a job is a key region and a part of at
+// most `most` entries of its list, so that no CTA has much more to do than the others, however few regions hold most of the
+// index.  Every part of a region that has several leaves its sums in scratch memory; the one that finishes last adds them up,
+// in the order of the parts.  Jobs by falling length of their regions' lists: those of cut lists come first, and number their sums.
+struct ListParts {
+    int most;               // entries of a part; 0: lists are not cut
+    int jobs, cut;          // jobs of an (image, routing head) and, of those, parts of cut lists, at most
+};
+
 // Scratch layout (byte offsets from ws, all multiples of 256).
 struct WsLayout {
     size_t status;      // int32[64]: [0] first device error, [1] detail
@@ -73,6 +82,9 @@ struct WsLayout {
     size_t inv_off;     // int32 [B,heads_i,R+1] CSR offsets of the inverse routing index
     size_t inv_list;    // int32 [B,heads_i,R*topk] query regions routed to each key region
     size_t inv_order;   // int32 [B,heads_i,R] key regions by falling length of their lists
+    size_t jobs;        // int2 [B,heads_i,parts.jobs] key regions and parts of their lists
+    size_t done;        // int32 [B,heads,R,chunks] parts of a region's list that are done
+    size_t sums;        // fp32 dK and dV of the parts of cut lists, by job and tile
     size_t dw_part;     // fp32 [lce_grad_partials(d), 26*C] partial LCE weight / bias gradients
     size_t pad;         // padded maps only: seven [B,H,W,C] tensors of the padded size (Q, K, V, O / dO, dQ, dK, dV)
     size_t pad_lse;     // padded maps only: fp32 [B,heads,H*W] of the padded size
@@ -175,10 +187,10 @@ cudaError_t launch_attend_tc_wide(const Dims& d, const void* Q, const void* K, c
                                   void* O, float* lse, int32_t* status, cudaStream_t st, bool after_own_kernel);
 
 bool backward_direct_supported(const Dims& d, int dtype);
-cudaError_t launch_backward_direct(const Dims& d, const void* Q, const void* K, const void* V,
-                                const int32_t* index, int32_t* inv_off, int32_t* inv_list, int32_t* inv_order,
-                                const float* lce_w, const float* lse, const void* dO,
-                                void* dQ, void* dK, void* dV, float* delta, int32_t* status, cudaStream_t st);
+// How it cuts lists; chunks: groups of a region, sum_bytes: what the parts of cut lists of the whole problem leave in scratch memory.
+ListParts direct_grad_parts(const Dims& d, int* chunks, size_t* sum_bytes);
+cudaError_t launch_backward_direct(const Dims& d, const void* Q, const void* K, const void* V, const int32_t* index, char* ws, const WsLayout& L,
+                                const float* lce_w, const float* lse, const void* dO, void* dQ, void* dK, void* dV, cudaStream_t st);
 
 bool backward_one_supported(const Dims& d, int dtype);
 cudaError_t launch_backward_one(const Dims& d, const void* Q, const void* K, const void* V, const int32_t* index, const float* lce_w,

@@ -66,7 +66,7 @@ inline DirGeom direct_geom(const Dims& d, bool with_lce, int entry_bytes, int rt
     const int need = (d.topk * d.n_r + 31) / 32 * 32;
     if (need < g.tab) g.tab = need;
     int off = 0;
-    g.tab_bytes = (g.tab * entry_bytes + g.tab / 8 + 4 + 15) / 16 * 16;     // entries, a bit per entry, a counter
+    g.tab_bytes = (g.tab * entry_bytes + g.tab / 8 + 8 + 15) / 16 * 16;     // entries, a bit per entry, a counter; or three numbers
     g.off_tab = off;  off += g.gpc * g.tab_bytes;
     g.off_w = off;    off += with_lce ? 32 * g.planes * 25 * 4 : 0;
     off = (off + 15) / 16 * 16;

@@ -15,9 +15,18 @@ inline bool inverse_uses_bits(const Dims& d) { return (size_t)d.R * inverse_word
 // places in shared memory (words): counts [R + 1] and a flag, lengths, bits
 __host__ __device__ inline int inverse_length_at(int R) { return (R + 2 + 3) / 4 * 4; }
 __host__ __device__ inline int inverse_bits_at(int R) { return inverse_length_at(R) + (R + 3) / 4 * 4; }
-inline size_t inverse_smem(const Dims& d) {
-    return sizeof(int32_t) * (inverse_bits_at(d.R) + (inverse_uses_bits(d) ? (size_t)d.R * inverse_words(d) : 0));
+// (and, where lists are cut in parts, the regions by falling length behind the bits)
+inline size_t inverse_smem(const Dims& d, bool cut = false) {
+    return sizeof(int32_t) * (inverse_bits_at(d.R) + (inverse_uses_bits(d) ? (size_t)d.R * inverse_words(d) : 0) + (cut ? d.R : 0));
 }
+
+// What the inverse index job writes besides the index where lists are cut in parts (ListParts).
+struct ListJobs {
+    int2* jobs;             // [images, heads_i, p.jobs]: (region or -1, part)
+    int32_t* done;          // counters to set to zero, `counters` per (image, routing head)
+    int counters;
+    ListParts p;
+};
 
 // The inverse index of the images of a piece.
 struct InversePiece { int32_t *off, *list, *order; };
@@ -53,7 +62,8 @@ inline cudaError_t group_pieces(const Dims& d, int groups, int chunks, F&& launc
 // 2 heads, gradients 17.6 ms; 0.24 ms now.)
 // Entries outside [0, R) are in no list.
 __device__ __forceinline__ void inverse_index_job(const int32_t* __restrict__ index, int32_t* __restrict__ inv_off,
-                                                  int32_t* __restrict__ inv_list, int32_t* __restrict__ order, int bh, int32_t* sm, bool use_bits, const Dims& dm) {
+                                                  int32_t* __restrict__ inv_list, int32_t* __restrict__ order, int bh, int32_t* sm, bool use_bits, const Dims& dm,
+                                                  const ListJobs& lj = {nullptr, nullptr, 0, {0, 0, 0}}) {
     const int tid = threadIdx.x, nthreads = blockDim.x;
     const int lane = tid & 31, warp = tid >> 5;
     const int entries = dm.R * dm.topk, words = (dm.R + 31) >> 5;
@@ -64,6 +74,7 @@ __device__ __forceinline__ void inverse_index_job(const int32_t* __restrict__ in
     int32_t* length = sm + inverse_length_at(dm.R);         // [R], then -1 to a multiple of four
     uint32_t* bits = reinterpret_cast<uint32_t*>(sm + inverse_bits_at(dm.R));
     int* repeated = sm + dm.R + 1;
+    int32_t* by_rank = sm + inverse_bits_at(dm.R) + (use_bits ? dm.R * words : 0);
     bool by_bits = use_bits;
     if (use_bits) {
         for (int e = tid; e < dm.R * words; e += nthreads) bits[e] = 0u;
@@ -118,6 +129,31 @@ __device__ __forceinline__ void inverse_index_job(const int32_t* __restrict__ in
                     (l.w > n || (l.w == n && o + 3 < j));
         }
         order[(size_t)bh * dm.R + rank] = j;
+        if (lj.p.most) by_rank[rank] = j;
+    }
+    if (lj.p.most) {
+        for (int e = tid; e < lj.counters; e += nthreads) lj.done[(size_t)bh * lj.counters + e] = 0;
+        __syncthreads();
+        // jobs before those of a rank: parts of the lists before it (warps take 32 ranks at a time, each adding up what is before)
+        int2* out = lj.jobs + (size_t)bh * lj.p.jobs;
+        auto parts_of = [&](int q) { return q < dm.R ? max(1, (length[by_rank[q]] + lj.p.most - 1) / lj.p.most) : 0; };
+        const int ranks = (dm.R + 31) / 32 * 32;
+        int run = 0;
+        for (int q0 = 0, mine = warp * 32; mine < ranks; q0 += 32) {
+            const int parts = parts_of(q0 + lane);
+            if (q0 < mine) { run += __reduce_add_sync(0xffffffffu, parts); continue; }
+            int incl = parts;
+#pragma unroll
+            for (int s = 1; s < 32; s <<= 1) {
+                const int o = __shfl_up_sync(0xffffffffu, incl, s);
+                if (lane >= s) incl += o;
+            }
+            for (int p = 0; p < parts; ++p) out[run + incl - parts + p] = make_int2(by_rank[q0 + lane], p);
+            run += __shfl_sync(0xffffffffu, incl, 31);
+            mine += nthreads;
+            if (q0 + 32 >= ranks)
+                for (int e = run + lane; e < lj.p.jobs; e += 32) out[e] = make_int2(-1, 0);
+        }
     }
     if (by_bits) {
         for (int j = tid; j < dm.R; j += nthreads) {

@@ -1288,6 +1288,42 @@ def test_bad_entries_count_for_nothing(bra, impl, cfg):
         assert np.abs(f64(a) - r).max() <= tol, f"{name} {np.abs(f64(a) - r).max():.3e}"
 
 
+# gradients of lists cut in parts (64 regions and more, parts of eight entries and more): every part of a region adds its sums
+CUT_CASES = [
+    BraConfig("cut-8x4", 2, 64, 32, 64, 2, 8, 2, "bf16"),
+    BraConfig("cut-one-warp-regions", 1, 32, 32, 64, 2, 8, 3, "bf16"),                     # parts of 16
+    BraConfig("cut-one-warp-regions-d64", 1, 32, 32, 128, 2, 8, 3, "bf16"),
+    BraConfig("cut-odd-map", 1, 59, 61, 64, 2, 8, 2, "bf16"),
+    BraConfig("cut-d64", 1, 48, 40, 128, 2, 8, 2, "bf16"),
+    BraConfig("cut-12x12-chunks", 1, 96, 96, 32, 1, 8, 1, "bf16"),
+    BraConfig("cut-8x16-two-rounds-d64", 1, 64, 128, 64, 1, 8, 2, "bf16"),
+    BraConfig("cut-576-regions", 1, 96, 96, 32, 1, 24, 2, "bf16"),                         # inverse index without bits
+]
+
+
+@pytest.mark.parametrize("cfg", CUT_CASES, ids=lambda c: c.name)
+def test_gradients_of_lists_cut_in_parts(bra, cfg):
+    rng = np.random.default_rng(71)
+    shape = (cfg.B, cfg.heads, cfg.R, cfg.topk)
+    # a few regions hold every list.  (dK and dV leave in bf16: a sum over n queries is about sqrt(n) times a query's share, and its
+    # rounding alone |dK| 2^-9.  Five regions of 64 are listed some 40 times; so are 28 of 576, where |dK| of 25 would round by 0.05.)
+    n = max(5, cfg.R // 20)
+    few = rng.integers(0, n, size=shape).astype(np.int32) * (cfg.R // n)
+    run_backward_case(bra, cfg, seed=72, index=few)
+    # lists of every length around one, two and three parts, the rest of the regions once each
+    last = np.arange(cfg.R, dtype=np.int32)
+    at = 0
+    for j, n in enumerate((1, 7, 8, 9, 15, 16, 17) if cfg.R < 100 else (7, 8, 9, 15, 16, 17, 31, 32, 33, 47, 48, 49)):
+        last[at:at + n] = j
+        at += n
+    edge = np.broadcast_to(last[None, None, :, None], shape).copy()
+    edge[..., 1:] = np.arange(cfg.R, dtype=np.int32)[::-1][None, None, :, None]
+    run_backward_case(bra, cfg, seed=73, index=edge)
+    run_backward_case(bra, cfg, seed=74, index=few[:, :1].copy(), shared=True)
+    if cfg.R <= 256:                                                                       # (as many as bra_forward routes)
+        run_backward_case(bra, cfg, seed=75)
+
+
 # topk = 1 in one launch: tiles of a region (17 .. 64 tokens), rows behind its last token, cut maps, every list length
 ONE_EDGES = [
     (BraConfig("one-1x17", 1, 2, 34, 32, 1, 2, 1, "bf16"), "route"),

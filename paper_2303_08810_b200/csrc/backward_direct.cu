@@ -441,6 +441,8 @@ bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16*
             }
         }
         if (CUT && s_job[0] > 1) {                                    // the sums of a part: to scratch memory
+            // (a warp whose last round has no tile for it: what would be its place is another part's)
+            if (!has) continue;
             float* at = sums + sum_at(s_job[1], tile);
 #pragma unroll
             for (int p = 0; p < PL; ++p)

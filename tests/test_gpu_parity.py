@@ -1298,6 +1298,13 @@ CUT_CASES = [
     BraConfig("cut-12x12-chunks", 1, 96, 96, 32, 1, 8, 1, "bf16"),
     BraConfig("cut-8x16-two-rounds-d64", 1, 64, 128, 64, 1, 8, 2, "bf16"),
     BraConfig("cut-576-regions", 1, 96, 96, 32, 1, 24, 2, "bf16"),                         # inverse index without bits
+    # two rounds of a CTA's four warps that have no tile for all of them: 5, 6 and 7 tiles, two chunks of 6, of 7 and 4
+    BraConfig("cut-8x10-five-tiles-d64", 1, 64, 80, 128, 2, 8, 2, "bf16"),
+    BraConfig("cut-9x10-six-tiles-d64", 1, 72, 80, 128, 2, 8, 4, "bf16"),
+    BraConfig("cut-10x10-seven-tiles-d64", 1, 80, 80, 128, 2, 8, 2, "bf16"),
+    BraConfig("cut-12x12-chunks-d64", 2, 96, 96, 192, 3, 8, 2, "bf16"),
+    BraConfig("cut-18x9-chunks-d64", 2, 144, 72, 64, 1, 8, 2, "bf16"),
+    BraConfig("cut-18x9-chunks", 2, 144, 72, 32, 1, 8, 2, "bf16"),
 ]
 
 

@@ -10,7 +10,9 @@
 // listing region a warp takes 16 queries against all keys (up to 64 scores a row in registers), stores dQ and puts P and dS
 // into shared memory; then it takes the 16 keys it owns against all queries, both operands transposed by ldmatrix.  The
 // list is read off the index by the CTA itself.
-// Rows of a tile behind the region's last token are zero and have no probability.
+// Rows of a tile that are no query (behind the region's last token, outside the map) are zero in shared memory and have lse = inf, so P = 0.
+// As A fragments they read a token of the region that exists instead: a zero row beside a key with an infinity scores NaN, a query that
+// exists does so only where its gradients are NaN by rights.
 //
 // Bound: latency and issue at 16 warps per SM (64 x 56 x 56, 2 heads: 0.53 instructions per cycle and scheduler; a third of the time
 // is the LCE adjoint).  Measured (B200), there, LCE gradient beside it: dQ + dK / dV 58 + 114 -> 97 us; forward + backward
@@ -39,7 +41,10 @@ __device__ __forceinline__ void stmatrix_x4(uint32_t addr, const uint32_t (&r)[4
     asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
 }
 
-template <int KT, int TX>
+// Regions of 16 KT tokens; fewer; the map ends inside the last ones.
+enum OneEdge { ONE_FULL, ONE_REST, ONE_CUT };
+
+template <int KT, int TX, OneEdge EDGE>
 __global__ void __launch_bounds__(32 * KT, 16 / KT)
 bwd_one_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_g,
@@ -68,6 +73,7 @@ bwd_one_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
     const float* lse_h = lse + ((size_t)b * dm.heads + h) * N0;
     const int32_t* irow = index + ((size_t)b * dm.heads_i + (dm.heads_i == 1 ? 0 : h)) * dm.R;
     const int own = __ldg(irow + j);                                  // the region that this one's queries attend to
+    const bool cut = EDGE == ONE_CUT && (KT < 4 || dm.H != dm.H0 || dm.W != dm.W0);
 
     if (tid == 0) {
         mbar_init(bar_kv, 1);
@@ -95,8 +101,13 @@ bwd_one_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
             for (int q = 0; q < 4; ++q) r[q] = e0 + 32 * q + lane < dm.R ? __ldg(irow + e0 + 32 * q + lane) : -1;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const uint32_t m = __ballot_sync(0xffffffffu, r[q] == j);
-                if (r[q] == j) list[n + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(e0 + 32 * q + lane);
+                bool lists = r[q] == j;
+                if (cut && lists) {                                   // not without a token
+                    const int i = e0 + 32 * q + lane, qy = fdiv(i, dm.S, gm.mul_s);
+                    lists = qy * dm.hs < dm.H0 && (i - qy * dm.S) * dm.ws < dm.W0;
+                }
+                const uint32_t m = __ballot_sync(0xffffffffu, lists);
+                if (lists) list[n + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(e0 + 32 * q + lane);
                 n += __popc(m);
             }
         }
@@ -145,7 +156,9 @@ bwd_one_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
 #pragma unroll
         for (int e = 0; e < 4; ++e) { dk[i][e] = 0.f; dv[i][e] = 0.f; }
     const uint32_t row_off = rows8_offset<1>(lane), col_off = rows16_offset<1>(lane);
-    const uint32_t own_at = warp * 1024 + col_off;                    // the warp's 16 rows as A fragments
+    // the warp's 16 rows as A fragments
+    const int row = warp * 16 + (lane & 15);
+    uint32_t own_at = EDGE == ONE_FULL || row < dm.n_r ? warp * 1024 + col_off : col_off & 511u;    // (rows 0 .. 7: other banks)
     // P and dS: where a lane's row goes (16 queries x 16 keys), and as the transposed operand
     const uint32_t put_at = (warp * 16 + (lane & 15)) * og.p_pitch + (lane >> 4) * 16;
     const uint32_t get_at = ((lane & 7) + (lane >> 4) * 8) * og.p_pitch + warp * 32 + ((lane >> 3) & 1) * 16;
@@ -154,7 +167,7 @@ bwd_one_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         if (tok >= 0) *reinterpret_cast<uint4*>(base + head_off + (size_t)(uint32_t)tok * tok_bytes + t4 * 16) = v;
     };
     const float sl2 = dm.scale * 1.4426950408889634f;
-    const bool rest = dm.n_r != 8 * NT;
+    const bool rest = EDGE != ONE_FULL && dm.n_r != 8 * NT;
     bool ok = true;
     if (n > 0 && !mbar_wait(bar_kv, 0, one::POLL_LIMIT)) ok = false;
 
@@ -170,20 +183,38 @@ bwd_one_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
             lse2[r] = tok[r] >= 0 ? __ldg(lse_h + tok[r]) * 1.4426950408889634f : INFINITY;
         }
         if (!mbar_try_wait(bar_q + (it & 1), it >> 1 & 1)) ok = mbar_wait(bar_q + (it & 1), it >> 1 & 1, ok ? one::POLL_LIMIT : 1u) && ok;
+        if (cut) {
+            const int y = fdiv(row, dm.ws, gm.mul_ws), x = row - y * dm.ws;
+            own_at = row < dm.n_r && qy * dm.hs + y < dm.H0 && qx * dm.ws + x < dm.W0 ? warp * 1024 + col_off : (uint32_t)(lane >> 4) << 4;
+        }
         float c[NT][4], dp[NT][4];
         {
-            uint32_t qa[1][2][4], ga[1][2][4];
+            uint32_t qa[1][2][4], ga[1][2][4], f[1][4];
             ldmatrix_x4(s_q + own_at, qa[0][0]);
             ldmatrix_x4(s_q + (own_at ^ 32), qa[0][1]);
-            ldmatrix_x4(s_g + own_at, ga[0][0]);
-            ldmatrix_x4(s_g + (own_at ^ 32), ga[0][1]);
+            if (KT == 4) {                                            // (one after the other: 109 -> 113 us at 64 x 56 x 56)
+                ldmatrix_x4(s_g + own_at, ga[0][0]);
+                ldmatrix_x4(s_g + (own_at ^ 32), ga[0][1]);
 #pragma unroll
-            for (int m = 0; m < NT; ++m) {
-                uint32_t f[1][4];
-                load_rows8<1>(f, s_k + m * 512, row_off);
-                mma_rows8<1>(c[m], qa, f);
-                load_rows8<1>(f, s_v + m * 512, row_off);
-                mma_rows8<1>(dp[m], ga, f);
+                for (int m = 0; m < NT; ++m) {
+                    load_rows8<1>(f, s_k + m * 512, row_off);
+                    mma_rows8<1>(c[m], qa, f);
+                    load_rows8<1>(f, s_v + m * 512, row_off);
+                    mma_rows8<1>(dp[m], ga, f);
+                }
+            } else {
+#pragma unroll
+                for (int m = 0; m < NT; ++m) {
+                    load_rows8<1>(f, s_k + m * 512, row_off);
+                    mma_rows8<1>(c[m], qa, f);
+                }
+                ldmatrix_x4(s_g + own_at, ga[0][0]);
+                ldmatrix_x4(s_g + (own_at ^ 32), ga[0][1]);
+#pragma unroll
+                for (int m = 0; m < NT; ++m) {
+                    load_rows8<1>(f, s_v + m * 512, row_off);
+                    mma_rows8<1>(dp[m], ga, f);
+                }
             }
         }
 #pragma unroll
@@ -307,10 +338,10 @@ bool backward_one_supported(const Dims& d, int dtype) {
     return dtype == BRA_BF16 && one_geom(d, &g, &o);
 }
 
-template <int KT, int TX>
-static cudaError_t launch_t(const Dims& d, const DirGeom& g, const OneGeom& o, const void* Q, const void* K, const void* V, const int32_t* index,
+template <int KT, int TX, OneEdge EDGE>
+static cudaError_t launch_edge(const Dims& d, const DirGeom& g, const OneGeom& o, const void* Q, const void* K, const void* V, const int32_t* index,
                             const float* lce_w, const float* lse, const void* dO, void* dQ, void* dK, void* dV, int32_t* status, cudaStream_t st) {
-    auto kernel = bwd_one_kernel<KT, TX>;
+    auto kernel = bwd_one_kernel<KT, TX, EDGE>;
     static PerDeviceMax set;
     const cudaError_t e = set.ensure(o.smem_bytes, [&] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, o.smem_bytes); });
     if (e != cudaSuccess) return e;
@@ -326,6 +357,13 @@ static cudaError_t launch_t(const Dims& d, const DirGeom& g, const OneGeom& o, c
                              index + p.index, lse + p.stat, static_cast<const bf*>(dO) + p.tensor, piece_of(lce_w, p.channel * 25),
                              static_cast<bf*>(dQ) + p.tensor, static_cast<bf*>(dK) + p.tensor, static_cast<bf*>(dV) + p.tensor, status, p.h0, p.b0, d, g, o);
     });
+}
+template <int KT, int TX, typename... Args>
+static cudaError_t launch_t(const Dims& d, Args... args) {
+    if (d.H != d.H0 || d.W != d.W0) return launch_edge<KT, TX, ONE_CUT>(d, args...);
+    if (d.n_r == 16 * KT) return launch_edge<KT, TX, ONE_FULL>(d, args...);
+    // (four tiles: the instance that also asks for a cut map keeps everything in registers, this one alone does not)
+    return launch_edge<KT, TX, KT == 4 ? ONE_CUT : ONE_REST>(d, args...);
 }
 
 cudaError_t launch_backward_one(const Dims& d, const void* Q, const void* K, const void* V, const int32_t* index, const float* lce_w,

@@ -1390,6 +1390,33 @@ def test_gradients_of_topk_1_keep_infinities_in_their_regions(bra, hw, value):
     run_isolation_case(bra, BraConfig("alone-one", 2, hw[0], hw[1], 64, 2, 4, 1, "bf16"), "auto", value)
 
 
+@pytest.mark.parametrize("impl", ["auto", "mma"])
+@pytest.mark.parametrize("hw", [(24, 28), (29, 27), (32, 32)], ids=["6x7-regions", "cut-map", "8x8-regions"])
+def test_a_key_at_minus_infinity_leaves_its_neighbours_gradients_alone(bra, hw, impl):
+    """A key that scores -inf with every query has P = 0: gradients of the region's other keys are those beside a key that scores far
+    below all others.  (Rows that fill up a tile or a cut map are no queries: their score is 0 * inf.)"""
+    import torch
+    cfg = BraConfig("infinite-key", 2, hw[0], hw[1], 64, 2, 4, 1, "bf16")
+    x = synthetic.make_inputs(cfg, seed=107, with_do=True)
+    x["Q"][..., 3::32] = np.abs(x["Q"][..., 3::32]) + 0.5
+    idx = np.zeros((cfg.B, cfg.heads, cfg.R, 1), np.int32)
+    idx[:, :, cfg.R // 2:] = 5
+    p = problem_of(bra, cfg, impl=IMPLS[impl], lce=False)
+    ws = bra.workspace(p)
+    dev = torch.from_numpy(idx).cuda()
+    x["K"][:, 1, 1, 3::32] = -np.inf
+    t = to_dev(x, cfg)
+    O, lse = bra.bra_attend(p, t["Q"], t["K"], t["V"], dev, ws=ws)
+    g = bra.bra_backward(p, t["Q"], t["K"], t["V"], dev, None, lse, t["dO"], ws=ws)
+    assert bra.bra_device_status(ws) == 0
+    x["K"][:, 1, 1, 3::32] = -2.0 ** 17                        # scores from 2^17 * 0.5 / sqrt(32) = 11585 below
+    ref = orc.bra_backward(x["Q"], x["K"], x["V"], idx, np.zeros_like(x["w"]), x["dO"], cfg.heads, cfg.S)
+    others = np.ones((cfg.H, cfg.W), bool)
+    others[1, 1] = False
+    for name, a, r in zip(("dK", "dV"), g[1:3], ref[1:3]):
+        assert np.abs(f64(a) - r)[:, others].max() <= GRAD_MAX, name
+
+
 # ------------------------------------------------------------------ inputs written right before the call; graphs
 ORDER_CASES = [
     BraConfig("order-pool-rows", 16, 28, 28, 128, 4, 7, 4, "bf16"),

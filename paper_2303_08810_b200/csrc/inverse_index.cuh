@@ -12,15 +12,14 @@ constexpr int INVERSE_BITS_MAX = 40 * 1024;     // bytes of the bit matrix up to
 
 inline int inverse_words(const Dims& d) { return (d.R + 31) / 32; }
 inline bool inverse_uses_bits(const Dims& d) { return (size_t)d.R * inverse_words(d) * 4 <= INVERSE_BITS_MAX; }
-// places in shared memory (words): counts [R + 1] and a flag, lengths, bits
-__host__ __device__ inline int inverse_length_at(int R) { return (R + 2 + 3) / 4 * 4; }
-__host__ __device__ inline int inverse_bits_at(int R) { return inverse_length_at(R) + (R + 3) / 4 * 4; }
-// (and, where lists are cut in parts, the regions by falling length behind the bits)
+// places in shared memory (words): counts [R + 1] and a flag, keys of the order, parts (where lists are cut: ListParts), bits
+__host__ __device__ inline int inverse_key_at(int R) { return (R + 2 + 3) / 4 * 4; }
+__host__ __device__ inline int inverse_bits_at(int R, bool cut) { return inverse_key_at(R) + (cut ? 2 : 1) * ((R + 3) / 4 * 4); }
 inline size_t inverse_smem(const Dims& d, bool cut = false) {
-    return sizeof(int32_t) * (inverse_bits_at(d.R) + (inverse_uses_bits(d) ? (size_t)d.R * inverse_words(d) : 0) + (cut ? d.R : 0));
+    return sizeof(int32_t) * (inverse_bits_at(d.R, cut) + (inverse_uses_bits(d) ? (size_t)d.R * inverse_words(d) : 0));
 }
 
-// What the inverse index job writes besides the index where lists are cut in parts (ListParts).
+// What the inverse index job writes besides the index, in place of the order, where lists are cut in parts (ListParts).
 struct ListJobs {
     int2* jobs;             // [images, heads_i, p.jobs]: (region or -1, part)
     int32_t* done;          // counters to set to zero, `counters` per (image, routing head)
@@ -71,11 +70,15 @@ __device__ __forceinline__ void inverse_index_job(const int32_t* __restrict__ in
     int32_t* off = inv_off + (size_t)bh * (dm.R + 1);
     int32_t* list = inv_list + (size_t)bh * entries;
     int32_t* count = sm;                                    // [R + 1]
-    int32_t* length = sm + inverse_length_at(dm.R);         // [R], then -1 to a multiple of four
-    uint32_t* bits = reinterpret_cast<uint32_t*>(sm + inverse_bits_at(dm.R));
-    int* repeated = sm + dm.R + 1;
-    int32_t* by_rank = sm + inverse_bits_at(dm.R) + (use_bits ? dm.R * words : 0);
+    // [R], then -1 to a multiple of four: 1024 times the length, less the region: a number per region (at most 1000 regions, lists of
+    // at most 10^6 entries), greater than another's where the region comes before that one in the order
+    int32_t* key = sm + inverse_key_at(dm.R);
+    int32_t* parts = key + (dm.R + 3) / 4 * 4;              // [R], then 0 to a multiple of four
+    uint32_t* bits = reinterpret_cast<uint32_t*>(sm + inverse_bits_at(dm.R, lj.p.most != 0));
+    int* repeated = sm + dm.R + 1;                          // later: jobs
     bool by_bits = use_bits;
+    if (lj.p.most)
+        for (int e = tid; e < lj.counters; e += nthreads) lj.done[(size_t)bh * lj.counters + e] = 0;
     if (use_bits) {
         for (int e = tid; e < dm.R * words; e += nthreads) bits[e] = 0u;
         if (tid == 0) *repeated = 0;
@@ -103,7 +106,7 @@ __device__ __forceinline__ void inverse_index_job(const int32_t* __restrict__ in
     }
     __syncthreads();
     if (warp == 0) {                                        // exclusive prefix sum
-        int run = 0;
+        int run = 0, jobs = 0;
         for (int j0 = 0; j0 < dm.R; j0 += 32) {
             const int j = j0 + lane, n = j < dm.R ? count[j] : 0;
             int incl = n;
@@ -112,48 +115,42 @@ __device__ __forceinline__ void inverse_index_job(const int32_t* __restrict__ in
                 const int o = __shfl_up_sync(0xffffffffu, incl, s);
                 if (lane >= s) incl += o;
             }
-            if (j < dm.R) { count[j] = run + incl - n; length[j] = n; }
+            if (j < dm.R) { count[j] = run + incl - n; key[j] = n * 1024 + 1023 - j; }
+            if (lj.p.most) {
+                const int m = j >= dm.R ? 0 : n > lj.p.most ? (n + lj.p.most - 1) / lj.p.most : 1;
+                if (j < (dm.R + 3) / 4 * 4) parts[j] = m;
+                jobs += m;
+            }
             run += __shfl_sync(0xffffffffu, incl, 31);
         }
-        if (lane == 0) count[dm.R] = run;
-        if (lane < 4 && dm.R + lane < inverse_bits_at(dm.R) - inverse_length_at(dm.R)) length[dm.R + lane] = -1;
+        if (lj.p.most) jobs = __reduce_add_sync(0xffffffffu, jobs);
+        if (lane == 0) { count[dm.R] = run; *repeated = jobs; }
+        if (lane < 4 && dm.R + lane < (dm.R + 3) / 4 * 4) key[dm.R + lane] = -1;
     }
     __syncthreads();
     for (int j = tid; j <= dm.R; j += nthreads) off[j] = count[j];
-    for (int j = tid; j < dm.R; j += nthreads) {            // longest list first, ties to the lower region
-        const int n = length[j];
-        int rank = 0;
-        for (int o = 0; o < dm.R; o += 4) {
-            const int4 l = *reinterpret_cast<const int4*>(length + o);
-            rank += (l.x > n || (l.x == n && o < j)) + (l.y > n || (l.y == n && o + 1 < j)) + (l.z > n || (l.z == n && o + 2 < j)) +
-                    (l.w > n || (l.w == n && o + 3 < j));
-        }
-        order[(size_t)bh * dm.R + rank] = j;
-        if (lj.p.most) by_rank[rank] = j;
-    }
-    if (lj.p.most) {
-        for (int e = tid; e < lj.counters; e += nthreads) lj.done[(size_t)bh * lj.counters + e] = 0;
-        __syncthreads();
-        // jobs before those of a rank: parts of the lists before it (warps take 32 ranks at a time, each adding up what is before)
-        int2* out = lj.jobs + (size_t)bh * lj.p.jobs;
-        auto parts_of = [&](int q) { return q < dm.R ? max(1, (length[by_rank[q]] + lj.p.most - 1) / lj.p.most) : 0; };
-        const int ranks = (dm.R + 31) / 32 * 32;
-        int run = 0;
-        for (int q0 = 0, mine = warp * 32; mine < ranks; q0 += 32) {
-            const int parts = parts_of(q0 + lane);
-            if (q0 < mine) { run += __reduce_add_sync(0xffffffffu, parts); continue; }
-            int incl = parts;
-#pragma unroll
-            for (int s = 1; s < 32; s <<= 1) {
-                const int o = __shfl_up_sync(0xffffffffu, incl, s);
-                if (lane >= s) incl += o;
+    if (!lj.p.most) {
+        for (int j = tid; j < dm.R; j += nthreads) {        // longest list first, ties to the lower region
+            const int mine = key[j];
+            int rank = 0;
+            for (int o = 0; o < dm.R; o += 4) {
+                const int4 k = *reinterpret_cast<const int4*>(key + o);
+                rank += (k.x > mine) + (k.y > mine) + (k.z > mine) + (k.w > mine);
             }
-            for (int p = 0; p < parts; ++p) out[run + incl - parts + p] = make_int2(by_rank[q0 + lane], p);
-            run += __shfl_sync(0xffffffffu, incl, 31);
-            mine += nthreads;
-            if (q0 + 32 >= ranks)
-                for (int e = run + lane; e < lj.p.jobs; e += 32) out[e] = make_int2(-1, 0);
+            order[(size_t)bh * dm.R + rank] = j;
         }
+    } else {
+        int2* jobs = lj.jobs + (size_t)bh * lj.p.jobs;
+        for (int j = tid; j < dm.R; j += nthreads) {        // the jobs in that order
+            const int mine = key[j];
+            int at = 0;
+            for (int o = 0; o < dm.R; o += 4) {
+                const int4 k = *reinterpret_cast<const int4*>(key + o), p = *reinterpret_cast<const int4*>(parts + o);
+                at += (k.x > mine ? p.x : 0) + (k.y > mine ? p.y : 0) + (k.z > mine ? p.z : 0) + (k.w > mine ? p.w : 0);
+            }
+            for (int p = 0; p < parts[j]; ++p) jobs[at + p] = make_int2(j, p);
+        }
+        for (int e = *repeated + tid; e < lj.p.jobs; e += nthreads) jobs[e] = make_int2(-1, 0);
     }
     if (by_bits) {
         for (int j = tid; j < dm.R; j += nthreads) {

@@ -386,7 +386,7 @@ enum Family { FAMILY_SIMT, FAMILY_DIRECT, FAMILY_IMG, FAMILY_DENSE, FAMILY_ONE }
 static Family choose_family(const Dims& d, int dtype, int impl) {
     if (dtype != BRA_BF16 || impl == BRA_IMPL_SIMT) return FAMILY_SIMT;
     if (impl == BRA_IMPL_AUTO && backward_dense_supported(d, dtype) && dense_grad_pays(d)) return FAMILY_DENSE;
-    if (impl == BRA_IMPL_AUTO && backward_one_supported(d, dtype)) return FAMILY_ONE;
+    if (impl == BRA_IMPL_AUTO && backward_one_supported(d, dtype) && one_grad_pays(d)) return FAMILY_ONE;
     if (backward_img_supported(d, dtype) &&
         (impl == BRA_IMPL_IMG || (impl == BRA_IMPL_AUTO && img_grad_pays(d))))
         return FAMILY_IMG;

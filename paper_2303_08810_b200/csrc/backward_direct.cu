@@ -508,7 +508,7 @@ ListParts direct_grad_parts(const Dims& d, int* chunks, size_t* sum_bytes) {
     ListParts p = {0, d.R, 0};
     *sum_bytes = 0;
     *chunks = 1;
-    if (!backward_direct_supported(d, d.esize == 2 ? BRA_BF16 : BRA_F32) || backward_one_supported(d, BRA_BF16) ||
+    if (!backward_direct_supported(d, d.esize == 2 ? BRA_BF16 : BRA_F32) || (backward_one_supported(d, BRA_BF16) && one_grad_pays(d)) ||
         (backward_dense_supported(d, BRA_BF16) && dense_grad_pays(d)) || (backward_img_supported(d, BRA_BF16) && img_grad_pays(d)))
         return p;
     const DirGeom g = dkv_geom(d);

@@ -193,6 +193,12 @@ cudaError_t launch_backward_direct(const Dims& d, const void* Q, const void* K, 
                                 const float* lce_w, const float* lse, const void* dO, void* dQ, void* dK, void* dV, cudaStream_t st);
 
 bool backward_one_supported(const Dims& d, int dtype);
+// It walks a list from end to end in one CTA, where the direct kernels cut long ones.  More regions make longer lists where a few kinds
+// of content share them, and only many (image, head) pairs hide one.  Measured (B200, us, one launch / direct), evenly spread and
+// clustered: 64 regions, 1 x 64 x 64, 2 heads 12 / 18 and 35 / 27, 8 images 27 / 35 and 51 / 42; 81 regions of 64, 4 pairs 17 / 24 and
+// 45 / 32, 16 pairs 32 / 40 and 62 / 46, 32 pairs 52 / 71 and 82 / 74, 64 pairs 96 / 145 and 120 / 142; 256 regions of 49, 4 pairs 32 / 39 and
+// 116 / 46, 16 pairs 77 / 106 and 173 / 108, 32 pairs 147 / 212 and 239 / 203, 64 pairs 272 / 428 and 365 / 393.
+inline bool one_grad_pays(const Dims& d) { return d.R <= 64 || (long long)d.B * d.heads >= 32; }
 cudaError_t launch_backward_one(const Dims& d, const void* Q, const void* K, const void* V, const int32_t* index, const float* lce_w,
                                 const float* lse, const void* dO, void* dQ, void* dK, void* dV, int32_t* status, cudaStream_t st);
 

@@ -1231,6 +1231,11 @@ RULE_EDGES = [
     (BraConfig("rule-4x4-238-pairs", 119, 8, 8, 64, 2, 2, 2, "bf16"), "repeats"),
     (BraConfig("rule-4x4-15000-blocks", 200, 20, 20, 32, 1, 5, 6, "bf16"), "route"),
     (BraConfig("rule-4x4-14925-blocks", 199, 20, 20, 32, 1, 5, 6, "bf16"), "route"),
+    # topk = 1, gradients: one launch up to 64 regions and from 32 pairs on, in between the direct kernels, which cut the long lists
+    (BraConfig("rule-one-64-regions", 1, 40, 32, 64, 2, 8, 1, "bf16"), "repeats"),
+    (BraConfig("rule-one-81-regions-31-pairs", 31, 45, 36, 32, 1, 9, 1, "bf16"), "route"),
+    (BraConfig("rule-one-81-regions-32-pairs", 16, 45, 36, 64, 2, 9, 1, "bf16"), "route"),
+    (BraConfig("rule-one-256-regions-3-pairs", 1, 80, 80, 96, 3, 16, 1, "bf16"), "repeats"),
 ]
 
 

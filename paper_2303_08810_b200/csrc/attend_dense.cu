@@ -114,8 +114,8 @@ attend_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* _
     dense_regions(reg, dm, gm, tid, nthreads);
     pdl_wait();          // in bra_forward the launch may overlap the tail of the routing kernel
     const int hi = dm.heads_i == 1 ? 0 : h;
-    const DenseRoutes routes = dense_routes(mask, bias, index ? index + ((size_t)b * dm.heads_i + hi) * dm.R * dm.topk : nullptr, status, dm, gm,
-                                            tid, nthreads);
+    const bool repeats = dense_routes(mask, bias, index ? index + ((size_t)b * dm.heads_i + hi) * dm.R * dm.topk : nullptr, status, dm, gm,
+                                      tid, nthreads);
     cp_async_wait<1>();
     __syncthreads();
 
@@ -202,11 +202,11 @@ attend_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* _
         for (int s = 0; s < 2; ++s) dense_mma_tokens<RT>(o, pa[s], vs + (kb + 16 * s) * 64, col_off);
     }
     };
-    if (routes.weighted) walk(std::true_type());
+    if (repeats) walk(std::true_type());
     else walk(std::false_type());
     cp_async_wait<0>();
     if (__syncthreads_or(dense_any_nan(o))) {                         // the slices have been read: staging takes their place
-        attend_dense_by_token(Qg, Vg, lce_w, lce_b, O, lse, smem, routes.weighted, dm, gm);
+        attend_dense_by_token(Qg, Vg, lce_w, lce_b, O, lse, smem, repeats, dm, gm);
         return;
     }
     float* st = reinterpret_cast<float*>(smem + gm.g.off_st);

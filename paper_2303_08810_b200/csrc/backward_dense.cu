@@ -129,7 +129,7 @@ bwd_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __re
     dense_regions(reg, dm, gm, tid, nthreads);
     const int hi = dm.heads_i == 1 ? 0 : h;
     unsigned long long* mask = reinterpret_cast<unsigned long long*>(smem + gm.off_mask);
-    const DenseRoutes routes = dense_routes(mask, bias, index + ((size_t)b * dm.heads_i + hi) * dm.R * dm.topk, status, dm, gm, tid, nthreads);
+    const bool repeats = dense_routes(mask, bias, index + ((size_t)b * dm.heads_i + hi) * dm.R * dm.topk, status, dm, gm, tid, nthreads);
     cp_async_wait<1>();
     __syncthreads();
 
@@ -225,11 +225,11 @@ bwd_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __re
         }
     }
     };
-    if (routes.weighted) queries(std::true_type());
+    if (repeats) queries(std::true_type());
     else queries(std::false_type());
     if (__syncthreads_or(nan)) {
         cp_async_wait<0>();
-        bwd_dense_by_token(lce_w, dOg, dQg, dKg, dVg, smem, routes.weighted, dm, gm);
+        bwd_dense_by_token(lce_w, dOg, dQg, dKg, dVg, smem, repeats, dm, gm);
         return;
     }
 
@@ -298,11 +298,11 @@ bwd_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __re
         }
     }
     };
-    if (routes.weighted) keys(std::true_type());
+    if (repeats) keys(std::true_type());
     else keys(std::false_type());
     cp_async_wait<0>();
     if (__syncthreads_or(nan)) {
-        bwd_dense_by_token(lce_w, dOg, dQg, dKg, dVg, smem, routes.weighted, dm, gm);
+        bwd_dense_by_token(lce_w, dOg, dQg, dKg, dVg, smem, repeats, dm, gm);
         return;
     }
     float* st = reinterpret_cast<float*>(smem + gm.g.off_st);

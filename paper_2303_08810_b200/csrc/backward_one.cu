@@ -155,7 +155,7 @@ bwd_one_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int e = 0; e < 4; ++e) { dk[i][e] = 0.f; dv[i][e] = 0.f; }
-    const uint32_t row_off = rows8_offset<1>(lane), col_off = rows16_offset<1>(lane);
+    const uint32_t row_off = rows8_offset(lane), col_off = rows16_offset(lane);
     // the warp's 16 rows as A fragments
     const int row = warp * 16 + (lane & 15);
     uint32_t own_at = EDGE == ONE_FULL || row < dm.n_r ? warp * 1024 + col_off : col_off & 511u;    // (rows 0 .. 7: other banks)
@@ -189,31 +189,31 @@ bwd_one_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         }
         float c[NT][4], dp[NT][4];
         {
-            uint32_t qa[1][2][4], ga[1][2][4], f[1][4];
-            ldmatrix_x4(s_q + own_at, qa[0][0]);
-            ldmatrix_x4(s_q + (own_at ^ 32), qa[0][1]);
+            uint32_t qa[2][4], ga[2][4], f[4];
+            ldmatrix_x4(s_q + own_at, qa[0]);
+            ldmatrix_x4(s_q + (own_at ^ 32), qa[1]);
             if (KT == 4) {                                            // (one after the other: 109 -> 113 us at 64 x 56 x 56)
-                ldmatrix_x4(s_g + own_at, ga[0][0]);
-                ldmatrix_x4(s_g + (own_at ^ 32), ga[0][1]);
+                ldmatrix_x4(s_g + own_at, ga[0]);
+                ldmatrix_x4(s_g + (own_at ^ 32), ga[1]);
 #pragma unroll
                 for (int m = 0; m < NT; ++m) {
-                    load_rows8<1>(f, s_k + m * 512, row_off);
-                    mma_rows8<1>(c[m], qa, f);
-                    load_rows8<1>(f, s_v + m * 512, row_off);
-                    mma_rows8<1>(dp[m], ga, f);
+                    ldmatrix_x4(s_k + m * 512 + row_off, f);
+                    mma_rows8(c[m], qa, f);
+                    ldmatrix_x4(s_v + m * 512 + row_off, f);
+                    mma_rows8(dp[m], ga, f);
                 }
             } else {
 #pragma unroll
                 for (int m = 0; m < NT; ++m) {
-                    load_rows8<1>(f, s_k + m * 512, row_off);
-                    mma_rows8<1>(c[m], qa, f);
+                    ldmatrix_x4(s_k + m * 512 + row_off, f);
+                    mma_rows8(c[m], qa, f);
                 }
-                ldmatrix_x4(s_g + own_at, ga[0][0]);
-                ldmatrix_x4(s_g + (own_at ^ 32), ga[0][1]);
+                ldmatrix_x4(s_g + own_at, ga[0]);
+                ldmatrix_x4(s_g + (own_at ^ 32), ga[1]);
 #pragma unroll
                 for (int m = 0; m < NT; ++m) {
-                    load_rows8<1>(f, s_v + m * 512, row_off);
-                    mma_rows8<1>(dp[m], ga, f);
+                    ldmatrix_x4(s_v + m * 512 + row_off, f);
+                    mma_rows8(dp[m], ga, f);
                 }
             }
         }

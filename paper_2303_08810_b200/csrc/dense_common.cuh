@@ -91,20 +91,17 @@ __device__ __forceinline__ void dense_load_slices(const uint32_t (&dst)[SLICES],
 __device__ __forceinline__ void dense_regions(uint8_t* reg, const Dims& dm, const DenseGeom& gm, int tid, int nthreads) {
     for (int t = tid; t < gm.rows; t += nthreads) reg[t] = t < dm.N ? (uint8_t)fdiv(t, dm.n_r, gm.mul_nr) : 255;
 }
-// What the index says about (query region, key region): `masked` - not every pair, see the masks; `weighted` - some pair
-// more than once, see the table of log2(count) (-inf: not routed).
-struct DenseRoutes { bool masked, weighted; };
 // mask[0 .. 63]: per query region the key regions; mask[64 .. 127]: per key region the query regions.  CTA-wide.
-__device__ __forceinline__ DenseRoutes dense_routes(unsigned long long* mask, float* bias, const int32_t* irows, int32_t* status, const Dims& dm,
-                                                    const DenseGeom& gm, int tid, int nthreads) {
-    const unsigned long long all = dm.R == 64 ? ~0ull : (1ull << dm.R) - 1;
+// True: some region is on a list more than once, see the table of log2(count) (-inf: not routed).
+__device__ __forceinline__ bool dense_routes(unsigned long long* mask, float* bias, const int32_t* irows, int32_t* status, const Dims& dm,
+                                             const DenseGeom& gm, int tid, int nthreads) {
     uint32_t* words = reinterpret_cast<uint32_t*>(mask);
     int* repeats = reinterpret_cast<int*>(mask + 128);
-    DenseRoutes out = {false, false};
     if (!irows) {
+        const unsigned long long all = dm.R == 64 ? ~0ull : (1ull << dm.R) - 1;
         for (int e = tid; e < 128; e += nthreads) mask[e] = all;
         __syncthreads();
-        return out;
+        return false;
     }
     const int entries = dm.R * dm.topk;
     for (int e = tid; e < 257; e += nthreads) words[e] = 0u;
@@ -123,11 +120,8 @@ __device__ __forceinline__ DenseRoutes dense_routes(unsigned long long* mask, fl
         }
     }
     __syncthreads();
-    out.weighted = *repeats != 0;
-    bool full = true;
-    for (int e = tid; e < dm.R; e += nthreads) full = full && mask[e] == all;
-    out.masked = !__syncthreads_and(full);
-    if (out.weighted) {
+    const bool weighted = *repeats != 0;
+    if (weighted) {
         int32_t* cnt = reinterpret_cast<int32_t*>(bias);
         const int rr = dm.R * dm.R;
         for (int e = tid; e < rr; e += nthreads) cnt[e] = 0;
@@ -140,12 +134,13 @@ __device__ __forceinline__ DenseRoutes dense_routes(unsigned long long* mask, fl
         for (int e = tid; e < rr; e += nthreads) bias[e] = cnt[e] == 0 ? -INFINITY : log2f((float)cnt[e]);
         __syncthreads();
     }
-    return out;
+    return weighted;
 }
 // What is added to the scaled scores of a row for the columns of n-tiles, in blocks of tokens from 0 on: `yes` where the column's region
 // is on the row's list, -inf elsewhere (and behind the last token).  NR: tokens per region - with four a bit of the mask covers the
 // two columns a lane holds of an n-tile, with one it is the token's, 0 (any) goes by the table of regions.  (A bit per two or
-// four scores, picked before the exponential: a test and a select per row and n-tile instead of per score behind it.)
+// four scores, picked before the exponential: a test and a select per row and n-tile instead of per score behind it.  A bit of its own for
+// a token, 64 x 7 x 7, 16 heads, topk 49: attention 15.1 -> 14.5 us, gradients 38.3 -> 36.4 against going by the table.)
 template <int NR>
 struct DenseRow {
     unsigned long long m;

@@ -1,5 +1,5 @@
-// Token rows of 32 channels per plane in shared memory as bulk tensor copies leave them (64- or 128-byte rows, swizzled), read
-// by ldmatrix without bank conflicts: as rows (contraction over channels) or transposed (contraction over tokens).
+// Token rows of 32 channels in shared memory as bulk tensor copies leave them (64-byte rows, swizzled), read by ldmatrix without
+// bank conflicts: as rows (contraction over channels) or transposed (contraction over tokens).
 #pragma once
 
 #include "direct_common.cuh"
@@ -7,36 +7,19 @@
 
 namespace bra {
 
-// Offsets of a lane for ldmatrix, rows from a multiple of eight on: eight rows, a chunk of 16 bytes per matrix (exclusive or with 64: the
-// second plane); 16 rows, two chunks (exclusive or with 32 i: two chunks on), which are the A fragment of 16 rows or, transposed, two
-// B fragments.
-template <int PL>
-__device__ __forceinline__ uint32_t row_swizzle(int row) { return PL == 2 ? row & 7 : (row >> 1) & 3; }
-template <int PL>
-__device__ __forceinline__ uint32_t rows8_offset(int lane) {
-    return (lane & 7) * 64 * PL + (((lane >> 3) ^ row_swizzle<PL>(lane & 7)) << 4);
-}
-template <int PL>
+// Offsets of a lane for ldmatrix, rows from a multiple of eight on: eight rows, a chunk of 16 bytes per matrix; 16 rows, two chunks
+// (exclusive or with 32: the other two), which are the A fragment of 16 rows or, transposed, two B fragments.
+__device__ __forceinline__ uint32_t row_swizzle(int row) { return (row >> 1) & 3; }
+__device__ __forceinline__ uint32_t rows8_offset(int lane) { return (lane & 7) * 64 + (((lane >> 3) ^ row_swizzle(lane & 7)) << 4); }
 __device__ __forceinline__ uint32_t rows16_offset(int lane) {
     const int row = lane & 15;
-    return row * 64 * PL + (((lane >> 4) ^ row_swizzle<PL>(row)) << 4);
+    return row * 64 + (((lane >> 4) ^ row_swizzle(row)) << 4);
 }
 
-// B fragments of eight token rows, contraction over channels: b[p] = {k step 0: b0, b1, k step 1: b0, b1}
-template <int PL>
-__device__ __forceinline__ void load_rows8(uint32_t (&b)[PL][4], uint32_t at, uint32_t lane_off) {
-#pragma unroll
-    for (int p = 0; p < PL; ++p) ldmatrix_x4(at + (lane_off ^ (p * 64)), b[p]);
-}
-// c (16 x 8) = A * B^T
-template <int PL>
-__device__ __forceinline__ void mma_rows8(float (&c)[4], const uint32_t (&a)[PL][2][4], const uint32_t (&b)[PL][4]) {
-    mma_bf16_zero(c, a[0][0], b[0][0], b[0][1]);
-    mma_bf16(c, a[0][1], b[0][2], b[0][3]);
-    if (PL == 2) {
-        mma_bf16(c, a[PL - 1][0], b[PL - 1][0], b[PL - 1][1]);
-        mma_bf16(c, a[PL - 1][1], b[PL - 1][2], b[PL - 1][3]);
-    }
+// c (16 x 8) = A * B^T, B fragments of eight token rows: k step 0: b0, b1, k step 1: b0, b1
+__device__ __forceinline__ void mma_rows8(float (&c)[4], const uint32_t (&a)[2][4], const uint32_t (&b)[4]) {
+    mma_bf16_zero(c, a[0], b[0], b[1]);
+    mma_bf16(c, a[1], b[2], b[3]);
 }
 // Row r of a tile's accumulators times f as bf16, 16 bytes (channels 8 t4 .. 8 t4 + 7 of a plane) per lane: the lanes of a quad
 // hold a pair of every chunk and trade them for a whole one.

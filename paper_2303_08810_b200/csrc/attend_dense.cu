@@ -140,67 +140,67 @@ attend_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* _
 #pragma unroll
             for (int r = 0; r < 2; ++r) on[x][r] = DenseRow<NR>(mask[where[x][r] >> 16], t4);
 #pragma unroll 1
-    for (int kb = 0; kb < dm.N; kb += 32) {
-        float c[RT][4][4];
+        for (int kb = 0; kb < dm.N; kb += 32) {
+            float c[RT][4][4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint4 kr[1] = {dense_chunk(ks + (kb + 8 * j) * 64 + row_off)};
+            for (int j = 0; j < 4; ++j) {
+                const uint4 kr[1] = {dense_chunk(ks + (kb + 8 * j) * 64 + row_off)};
 #pragma unroll
-            for (int x = 0; x < RT; ++x) mma_rows<1>(c[x][j], qa[x], kr);
-        }
+                for (int x = 0; x < RT; ++x) mma_rows<1>(c[x][j], qa[x], kr);
+            }
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int x = 0; x < RT; ++x)
+#pragma unroll
+                    for (int r = 0; r < 2; ++r)
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const float a = weighted.value ? dense_weight(bias + (where[x][r] >> 16) * dm.R, reg[kb + 8 * j + 2 * t4 + e])
+                                                           : on[x][r].pick(0.f, j, e, kb, t4, reg);
+                            c[x][j][2 * r + e] = fmaf(c[x][j][2 * r + e], sl2, a);
+                        }
 #pragma unroll
             for (int x = 0; x < RT; ++x)
 #pragma unroll
+                for (int r = 0; r < 2; ++r) on[x][r].template next<32>();
+            uint32_t pa[2][RT][4];
+#pragma unroll
+            for (int x = 0; x < RT; ++x) {
+                float mx[2];
+#pragma unroll
                 for (int r = 0; r < 2; ++r)
+                    mx[r] = fmaxf(fmax3(fmax3(c[x][0][2 * r], c[x][0][2 * r + 1], c[x][1][2 * r]), c[x][1][2 * r + 1], c[x][2][2 * r]),
+                                  fmax3(c[x][2][2 * r + 1], c[x][3][2 * r], c[x][3][2 * r + 1]));
+                if (__any_sync(0xffffffffu, mx[0] > m_run[x][0] || mx[1] > m_run[x][1])) {
 #pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const float a = weighted.value ? dense_weight(bias + (where[x][r] >> 16) * dm.R, reg[kb + 8 * j + 2 * t4 + e])
-                                                       : on[x][r].pick(0.f, j, e, kb, t4, reg);
-                        c[x][j][2 * r + e] = fmaf(c[x][j][2 * r + e], sl2, a);
+                    for (int r = 0; r < 2; ++r) {
+                        mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 1));
+                        mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 2));
+                        const float mnew = fmaxf(m_run[x][r], mx[r]);
+                        const float corr = mnew == -INFINITY ? 1.f : ex2_approx(m_run[x][r] - mnew);
+                        m_run[x][r] = mnew;
+                        l_run[x][r] *= corr;
+#pragma unroll
+                        for (int n = 0; n < 4; ++n) { o[x][n][2 * r] *= corr; o[x][n][2 * r + 1] *= corr; }
                     }
-#pragma unroll
-        for (int x = 0; x < RT; ++x)
-#pragma unroll
-            for (int r = 0; r < 2; ++r) on[x][r].template next<32>();
-        uint32_t pa[2][RT][4];
-#pragma unroll
-        for (int x = 0; x < RT; ++x) {
-            float mx[2];
-#pragma unroll
-            for (int r = 0; r < 2; ++r)
-                mx[r] = fmaxf(fmax3(fmax3(c[x][0][2 * r], c[x][0][2 * r + 1], c[x][1][2 * r]), c[x][1][2 * r + 1], c[x][2][2 * r]),
-                              fmax3(c[x][2][2 * r + 1], c[x][3][2 * r], c[x][3][2 * r + 1]));
-            if (__any_sync(0xffffffffu, mx[0] > m_run[x][0] || mx[1] > m_run[x][1])) {
-#pragma unroll
-                for (int r = 0; r < 2; ++r) {
-                    mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 1));
-                    mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 2));
-                    const float mnew = fmaxf(m_run[x][r], mx[r]);
-                    const float corr = mnew == -INFINITY ? 1.f : ex2_approx(m_run[x][r] - mnew);
-                    m_run[x][r] = mnew;
-                    l_run[x][r] *= corr;
-#pragma unroll
-                    for (int n = 0; n < 4; ++n) { o[x][n][2 * r] *= corr; o[x][n][2 * r + 1] *= corr; }
                 }
-            }
-            const float mn0 = m_run[x][0] == -INFINITY ? 0.f : m_run[x][0], mn1 = m_run[x][1] == -INFINITY ? 0.f : m_run[x][1];
+                const float mn0 = m_run[x][0] == -INFINITY ? 0.f : m_run[x][0], mn1 = m_run[x][1] == -INFINITY ? 0.f : m_run[x][1];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                c[x][j][0] = ex2_approx(c[x][j][0] - mn0);
-                c[x][j][1] = ex2_approx(c[x][j][1] - mn0);
-                c[x][j][2] = ex2_approx(c[x][j][2] - mn1);
-                c[x][j][3] = ex2_approx(c[x][j][3] - mn1);
-                l_run[x][0] += c[x][j][0] + c[x][j][1];
-                l_run[x][1] += c[x][j][2] + c[x][j][3];
+                for (int j = 0; j < 4; ++j) {
+                    c[x][j][0] = ex2_approx(c[x][j][0] - mn0);
+                    c[x][j][1] = ex2_approx(c[x][j][1] - mn0);
+                    c[x][j][2] = ex2_approx(c[x][j][2] - mn1);
+                    c[x][j][3] = ex2_approx(c[x][j][3] - mn1);
+                    l_run[x][0] += c[x][j][0] + c[x][j][1];
+                    l_run[x][1] += c[x][j][2] + c[x][j][3];
+                }
+                frag_hi(pa[0][x], c[x][0], c[x][1]);
+                frag_hi(pa[1][x], c[x][2], c[x][3]);
             }
-            frag_hi(pa[0][x], c[x][0], c[x][1]);
-            frag_hi(pa[1][x], c[x][2], c[x][3]);
+#pragma unroll
+            for (int s = 0; s < 2; ++s) dense_mma_tokens<RT>(o, pa[s], vs + (kb + 16 * s) * 64, col_off);
         }
-#pragma unroll
-        for (int s = 0; s < 2; ++s) dense_mma_tokens<RT>(o, pa[s], vs + (kb + 16 * s) * 64, col_off);
-    }
     };
     if (repeats) walk(std::true_type());
     else walk(std::false_type());

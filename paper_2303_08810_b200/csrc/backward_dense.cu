@@ -146,84 +146,84 @@ bwd_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __re
     bool nan = false;
     auto queries = [&](auto weighted) {
 #pragma unroll 1
-    for (int tile = warp; tile < steps; tile += gm.nw) {
-        const int r0 = tile * 16;
-        uint32_t qa[1][2][4], ga[1][2][4];
-        dense_a(qa, qs + r0 * 64 + row_off);
-        dense_a(ga, gs + r0 * 64 + row_off);
-        const float l0 = s_l2[r0 + g], l1 = s_l2[r0 + 8 + g];
-        const int i0 = min((int)reg[r0 + g], dm.R - 1), i1 = min((int)reg[r0 + 8 + g], dm.R - 1);
-        float delta[2] = {0.f, 0.f}, dq[1][4][4];
+        for (int tile = warp; tile < steps; tile += gm.nw) {
+            const int r0 = tile * 16;
+            uint32_t qa[1][2][4], ga[1][2][4];
+            dense_a(qa, qs + r0 * 64 + row_off);
+            dense_a(ga, gs + r0 * 64 + row_off);
+            const float l0 = s_l2[r0 + g], l1 = s_l2[r0 + 8 + g];
+            const int i0 = min((int)reg[r0 + g], dm.R - 1), i1 = min((int)reg[r0 + 8 + g], dm.R - 1);
+            float delta[2] = {0.f, 0.f}, dq[1][4][4];
 #pragma unroll
-        for (int n = 0; n < 4; ++n)
+            for (int n = 0; n < 4; ++n)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) dq[0][n][e] = 0.f;
-        // P and dP of 16 keys
-        auto scores = [&](float (&c)[2][4], float (&dp)[2][4], DenseRow<NR>& on0, DenseRow<NR>& on1, int kb) {
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const uint4 kr[1] = {dense_chunk(ks + (kb + 8 * j) * 64 + row_off)}, vr[1] = {dense_chunk(vs + (kb + 8 * j) * 64 + row_off)};
-                mma_rows<1>(c[j], qa, kr);
-                mma_rows<1>(dp[j], ga, vr);
-            }
-#pragma unroll
-            for (int j = 0; j < 2; ++j)
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const int r = weighted.value ? reg[kb + 8 * j + 2 * t4 + e] : 0;
-                    const float a = weighted.value ? dense_weight(bias + i0 * dm.R, r) - l0 : on0.pick(-l0, j, e, kb, t4, reg);
-                    const float b = weighted.value ? dense_weight(bias + i1 * dm.R, r) - l1 : on1.pick(-l1, j, e, kb, t4, reg);
-                    c[j][e] = ex2_approx(fmaf(c[j][e], sl2, a));
-                    c[j][2 + e] = ex2_approx(fmaf(c[j][2 + e], sl2, b));
-                }
-            on0.template next<16>();
-            on1.template next<16>();
-        };
-        {
-            DenseRow<NR> on0(mask[i0], t4), on1(mask[i1], t4);
-#pragma unroll 2
-            for (int kb = 0; kb < dm.N; kb += 16) {
-                float c[2][4], dp[2][4];
-                scores(c, dp, on0, on1, kb);
+                for (int e = 0; e < 4; ++e) dq[0][n][e] = 0.f;
+            // P and dP of 16 keys
+            auto scores = [&](float (&c)[2][4], float (&dp)[2][4], DenseRow<NR>& on0, DenseRow<NR>& on1, int kb) {
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
-                    delta[0] = fmaf(c[j][0], dp[j][0], fmaf(c[j][1], dp[j][1], delta[0]));
-                    delta[1] = fmaf(c[j][2], dp[j][2], fmaf(c[j][3], dp[j][3], delta[1]));
+                    const uint4 kr[1] = {dense_chunk(ks + (kb + 8 * j) * 64 + row_off)}, vr[1] = {dense_chunk(vs + (kb + 8 * j) * 64 + row_off)};
+                    mma_rows<1>(c[j], qa, kr);
+                    mma_rows<1>(dp[j], ga, vr);
                 }
-            }
-        }
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            delta[r] += __shfl_xor_sync(0xffffffffu, delta[r], 1);
-            delta[r] += __shfl_xor_sync(0xffffffffu, delta[r], 2);
-        }
-        {
-            DenseRow<NR> on0(mask[i0], t4), on1(mask[i1], t4);
+                for (int j = 0; j < 2; ++j)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int r = weighted.value ? reg[kb + 8 * j + 2 * t4 + e] : 0;
+                        const float a = weighted.value ? dense_weight(bias + i0 * dm.R, r) - l0 : on0.pick(-l0, j, e, kb, t4, reg);
+                        const float b = weighted.value ? dense_weight(bias + i1 * dm.R, r) - l1 : on1.pick(-l1, j, e, kb, t4, reg);
+                        c[j][e] = ex2_approx(fmaf(c[j][e], sl2, a));
+                        c[j][2 + e] = ex2_approx(fmaf(c[j][2 + e], sl2, b));
+                    }
+                on0.template next<16>();
+                on1.template next<16>();
+            };
+            {
+                DenseRow<NR> on0(mask[i0], t4), on1(mask[i1], t4);
 #pragma unroll 2
-            for (int kb = 0; kb < dm.N; kb += 16) {
-                float c[2][4], dp[2][4];
-                scores(c, dp, on0, on1, kb);
+                for (int kb = 0; kb < dm.N; kb += 16) {
+                    float c[2][4], dp[2][4];
+                    scores(c, dp, on0, on1, kb);
 #pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                    c[j][0] *= dp[j][0] - delta[0]; c[j][1] *= dp[j][1] - delta[0];
-                    c[j][2] *= dp[j][2] - delta[1]; c[j][3] *= dp[j][3] - delta[1];
+                    for (int j = 0; j < 2; ++j) {
+                        delta[0] = fmaf(c[j][0], dp[j][0], fmaf(c[j][1], dp[j][1], delta[0]));
+                        delta[1] = fmaf(c[j][2], dp[j][2], fmaf(c[j][3], dp[j][3], delta[1]));
+                    }
                 }
-                uint32_t sa[1][4];
-                frag_hi(sa[0], c[0], c[1]);
-                dense_mma_tokens<1>(dq, sa, ks + kb * 64, col_off);
+            }
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                delta[r] += __shfl_xor_sync(0xffffffffu, delta[r], 1);
+                delta[r] += __shfl_xor_sync(0xffffffffu, delta[r], 2);
+            }
+            {
+                DenseRow<NR> on0(mask[i0], t4), on1(mask[i1], t4);
+#pragma unroll 2
+                for (int kb = 0; kb < dm.N; kb += 16) {
+                    float c[2][4], dp[2][4];
+                    scores(c, dp, on0, on1, kb);
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        c[j][0] *= dp[j][0] - delta[0]; c[j][1] *= dp[j][1] - delta[0];
+                        c[j][2] *= dp[j][2] - delta[1]; c[j][3] *= dp[j][3] - delta[1];
+                    }
+                    uint32_t sa[1][4];
+                    frag_hi(sa[0], c[0], c[1]);
+                    dense_mma_tokens<1>(dq, sa, ks + kb * 64, col_off);
+                }
+            }
+            nan = nan || dense_any_nan(dq) || delta[0] != delta[0] || delta[1] != delta[1];
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const int t = r0 + g + 8 * r, tok = token(t);
+                if (tok < 0) continue;                                    // delta of a padding row stays 0
+                if (t4 == 0) s_dl[t] = delta[r];
+                uint32_t* o = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(dQg) + head_off) + (size_t)(uint32_t)tok * (dm.C / 2) + t4;
+#pragma unroll
+                for (int n = 0; n < 4; ++n) o[4 * n] = pack2_bf16(dq[0][n][2 * r] * dm.scale, dq[0][n][2 * r + 1] * dm.scale);
             }
         }
-        nan = nan || dense_any_nan(dq) || delta[0] != delta[0] || delta[1] != delta[1];
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            const int t = r0 + g + 8 * r, tok = token(t);
-            if (tok < 0) continue;                                    // delta of a padding row stays 0
-            if (t4 == 0) s_dl[t] = delta[r];
-            uint32_t* o = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(dQg) + head_off) + (size_t)(uint32_t)tok * (dm.C / 2) + t4;
-#pragma unroll
-            for (int n = 0; n < 4; ++n) o[4 * n] = pack2_bf16(dq[0][n][2 * r] * dm.scale, dq[0][n][2 * r + 1] * dm.scale);
-        }
-    }
     };
     if (repeats) queries(std::true_type());
     else queries(std::false_type());
@@ -237,66 +237,66 @@ bwd_dense_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __re
     float dv[2][4][4];
     auto keys = [&](auto weighted) {
 #pragma unroll
-    for (int x = 0; x < 2; ++x) {
-        const int r0 = (warp + x * gm.nw) * 16;
-        if (r0 >= steps * 16) continue;
-        uint32_t ka[1][2][4], va[1][2][4];
-        dense_a(ka, ks + r0 * 64 + row_off);
-        dense_a(va, vs + r0 * 64 + row_off);
-        const int k0 = min((int)reg[r0 + g], dm.R - 1), k1 = min((int)reg[r0 + 8 + g], dm.R - 1);
-        DenseRow<NR> on0(mask[64 + k0], t4), on1(mask[64 + k1], t4);
-        float dk[1][4][4];
+        for (int x = 0; x < 2; ++x) {
+            const int r0 = (warp + x * gm.nw) * 16;
+            if (r0 >= steps * 16) continue;
+            uint32_t ka[1][2][4], va[1][2][4];
+            dense_a(ka, ks + r0 * 64 + row_off);
+            dense_a(va, vs + r0 * 64 + row_off);
+            const int k0 = min((int)reg[r0 + g], dm.R - 1), k1 = min((int)reg[r0 + 8 + g], dm.R - 1);
+            DenseRow<NR> on0(mask[64 + k0], t4), on1(mask[64 + k1], t4);
+            float dk[1][4][4];
 #pragma unroll
-        for (int n = 0; n < 4; ++n)
+            for (int n = 0; n < 4; ++n)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) dk[0][n][e] = dv[x][n][e] = 0.f;
+                for (int e = 0; e < 4; ++e) dk[0][n][e] = dv[x][n][e] = 0.f;
 #pragma unroll 2
-        for (int qb = 0; qb < dm.N; qb += 16) {
-            float c[2][4], dp[2][4];
+            for (int qb = 0; qb < dm.N; qb += 16) {
+                float c[2][4], dp[2][4];
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const uint4 qr[1] = {dense_chunk(qs + (qb + 8 * j) * 64 + row_off)}, gr[1] = {dense_chunk(gs + (qb + 8 * j) * 64 + row_off)};
-                mma_rows<1>(c[j], ka, qr);
-                mma_rows<1>(dp[j], va, gr);
-            }
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const int q = qb + 8 * j + 2 * t4;
-                const float2 l2 = *reinterpret_cast<const float2*>(s_l2 + q), dl = *reinterpret_cast<const float2*>(s_dl + q);
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const float l = e ? l2.y : l2.x, d = e ? dl.y : dl.x;
-                    const int r = weighted.value ? reg[q + e] : 0;
-                    const float a = weighted.value ? (r < 64 ? bias[r * dm.R + k0] : -INFINITY) - l : on0.pick(-l, j, e, qb, t4, reg);
-                    const float b = weighted.value ? (r < 64 ? bias[r * dm.R + k1] : -INFINITY) - l : on1.pick(-l, j, e, qb, t4, reg);
-                    c[j][e] = ex2_approx(fmaf(c[j][e], sl2, a));
-                    c[j][2 + e] = ex2_approx(fmaf(c[j][2 + e], sl2, b));
-                    dp[j][e] -= d;
-                    dp[j][2 + e] -= d;
+                for (int j = 0; j < 2; ++j) {
+                    const uint4 qr[1] = {dense_chunk(qs + (qb + 8 * j) * 64 + row_off)}, gr[1] = {dense_chunk(gs + (qb + 8 * j) * 64 + row_off)};
+                    mma_rows<1>(c[j], ka, qr);
+                    mma_rows<1>(dp[j], va, gr);
                 }
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const int q = qb + 8 * j + 2 * t4;
+                    const float2 l2 = *reinterpret_cast<const float2*>(s_l2 + q), dl = *reinterpret_cast<const float2*>(s_dl + q);
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const float l = e ? l2.y : l2.x, d = e ? dl.y : dl.x;
+                        const int r = weighted.value ? reg[q + e] : 0;
+                        const float a = weighted.value ? (r < 64 ? bias[r * dm.R + k0] : -INFINITY) - l : on0.pick(-l, j, e, qb, t4, reg);
+                        const float b = weighted.value ? (r < 64 ? bias[r * dm.R + k1] : -INFINITY) - l : on1.pick(-l, j, e, qb, t4, reg);
+                        c[j][e] = ex2_approx(fmaf(c[j][e], sl2, a));
+                        c[j][2 + e] = ex2_approx(fmaf(c[j][2 + e], sl2, b));
+                        dp[j][e] -= d;
+                        dp[j][2 + e] -= d;
+                    }
+                }
+                on0.template next<16>();
+                on1.template next<16>();
+#pragma unroll
+                for (int j = 0; j < 2; ++j)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) dp[j][e] *= c[j][e];
+                uint32_t a[1][4];
+                frag_hi(a[0], dp[0], dp[1]);
+                dense_mma_tokens<1>(dk, a, qs + qb * 64, col_off);
+                frag_hi(a[0], c[0], c[1]);
+                dense_mma_tokens<1>(dv + x, a, gs + qb * 64, col_off);
             }
-            on0.template next<16>();
-            on1.template next<16>();
+            nan = nan || dense_any_nan(dk) || dense_any_nan(reinterpret_cast<const float (&)[1][4][4]>(dv[x]));
 #pragma unroll
-            for (int j = 0; j < 2; ++j)
+            for (int r = 0; r < 2; ++r) {
+                const int tok = token(r0 + g + 8 * r);
+                if (tok < 0) continue;
+                uint32_t* o = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(dKg) + head_off) + (size_t)(uint32_t)tok * (dm.C / 2) + t4;
 #pragma unroll
-                for (int e = 0; e < 4; ++e) dp[j][e] *= c[j][e];
-            uint32_t a[1][4];
-            frag_hi(a[0], dp[0], dp[1]);
-            dense_mma_tokens<1>(dk, a, qs + qb * 64, col_off);
-            frag_hi(a[0], c[0], c[1]);
-            dense_mma_tokens<1>(dv + x, a, gs + qb * 64, col_off);
+                for (int n = 0; n < 4; ++n) o[4 * n] = pack2_bf16(dk[0][n][2 * r] * dm.scale, dk[0][n][2 * r + 1] * dm.scale);
+            }
         }
-        nan = nan || dense_any_nan(dk) || dense_any_nan(reinterpret_cast<const float (&)[1][4][4]>(dv[x]));
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            const int tok = token(r0 + g + 8 * r);
-            if (tok < 0) continue;
-            uint32_t* o = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(dKg) + head_off) + (size_t)(uint32_t)tok * (dm.C / 2) + t4;
-#pragma unroll
-            for (int n = 0; n < 4; ++n) o[4 * n] = pack2_bf16(dk[0][n][2 * r] * dm.scale, dk[0][n][2 * r + 1] * dm.scale);
-        }
-    }
     };
     if (repeats) keys(std::true_type());
     else keys(std::false_type());

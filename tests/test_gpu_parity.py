@@ -1079,6 +1079,8 @@ DIRECT_ISOLATION = [
     BraConfig("alone-cut-map", 2, 29, 27, 64, 2, 4, 3, "bf16"),
     BraConfig("alone-cut-map-d64", 2, 29, 27, 128, 2, 4, 3, "bf16"),
     BraConfig("alone-11x12", 1, 33, 36, 64, 2, 3, 4, "bf16"),
+    BraConfig("alone-cut-lists", 1, 64, 32, 64, 2, 8, 12, "bf16"),                  # parts of 8 entries, lists of up to 20
+    BraConfig("alone-cut-lists-d64-five-tiles", 1, 64, 80, 64, 1, 8, 12, "bf16"),
 ]
 
 
@@ -1253,6 +1255,8 @@ BAD_INDEX = [
     ("mma", BraConfig("bad-direct-one-block", 2, 12, 20, 64, 2, 4, 3, "bf16")),
     ("mma", BraConfig("bad-direct", 2, 21, 35, 64, 2, 7, 9, "bf16")),
     ("mma", BraConfig("bad-direct-d64", 2, 12, 20, 128, 2, 4, 4, "bf16")),
+    ("mma", BraConfig("bad-direct-cut-lists", 1, 64, 32, 64, 2, 8, 12, "bf16")),           # parts of 8 entries
+    ("mma", BraConfig("bad-direct-cut-lists-d64", 1, 64, 80, 64, 1, 8, 12, "bf16")),
     ("auto", BraConfig("bad-dense-7x7", 20, 7, 7, 64, 2, 7, 10, "bf16")),
     ("auto", BraConfig("bad-dense-k=R", 20, 7, 7, 64, 2, 7, 49, "bf16")),
     ("auto", BraConfig("bad-dense-2x2", 148, 16, 16, 64, 2, 8, 17, "bf16")),
@@ -1322,15 +1326,30 @@ def test_gradients_of_lists_cut_in_parts(bra, cfg):
     n = max(5, cfg.R // 20)
     few = rng.integers(0, n, size=shape).astype(np.int32) * (cfg.R // n)
     run_backward_case(bra, cfg, seed=72, index=few)
-    # lists of every length around one, two and three parts, the rest of the regions once each
-    last = np.arange(cfg.R, dtype=np.int32)
-    at = 0
-    for j, n in enumerate((1, 7, 8, 9, 15, 16, 17) if cfg.R < 100 else (7, 8, 9, 15, 16, 17, 31, 32, 33, 47, 48, 49)):
-        last[at:at + n] = j
-        at += n
-    edge = np.broadcast_to(last[None, None, :, None], shape).copy()
-    edge[..., 1:] = np.arange(cfg.R, dtype=np.int32)[::-1][None, None, :, None]
-    run_backward_case(bra, cfg, seed=73, index=edge)
+    # lists of every length around one, two and three parts, the other regions topk times or topk - 1 times.  (All columns of the index
+    # but the first name every region once; what the first column has no room for comes in the next (image, head) or call.)
+    part = max(8, -(-256 // (-(-cfg.H // cfg.S) * -(-cfg.W // cfg.S))))                   # entries: 256 queries, or 8
+    lengths = [part - 1, part, part + 1, 2 * part, 2 * part + 1, 3 * part, 3 * part + 1]
+    firsts = [[]]
+    for n in lengths:
+        if sum(firsts[-1]) + n - (cfg.topk - 1) > cfg.R:
+            firsts.append([])
+        firsts[-1].append(n - (cfg.topk - 1))
+    pairs = cfg.B * cfg.heads
+    firsts += [firsts[0]] * (-len(firsts) % pairs)
+    seen = set()
+    for i in range(0, len(firsts), pairs):
+        edge = np.broadcast_to(np.arange(cfg.R, dtype=np.int32)[::-1][:, None], (pairs, cfg.R, cfg.topk)).copy()
+        for col, first in zip(edge[..., 0], firsts[i:i + pairs]):
+            col[:] = np.arange(cfg.R)
+            col[:sum(first)] = np.repeat(np.arange(len(first)), first)
+        for rows in edge:
+            seen |= set(np.bincount(rows.ravel()).tolist())
+        run_backward_case(bra, cfg, seed=73, index=edge.reshape(shape))
+    assert seen.issuperset(lengths)
+    # the lists of this shape are cut: the scratch for the sums of the parts grows with topk, by far more than the index does
+    more = [bra.workspace_bytes(bra.make_problem(cfg.B, cfg.H, cfg.W, cfg.C, cfg.heads, cfg.S, k, cfg.dtype)) for k in (cfg.topk, cfg.topk + 1)]
+    assert more[1] - more[0] > 10 * 8 * cfg.B * cfg.heads * cfg.R
     run_backward_case(bra, cfg, seed=74, index=few[:, :1].copy(), shared=True)
     if cfg.R <= 256:                                                                       # (as many as bra_forward routes)
         run_backward_case(bra, cfg, seed=75)
@@ -1352,6 +1371,7 @@ ONE_EDGES = [
     (BraConfig("one-cut-8x7", 2, 29, 27, 64, 2, 4, 1, "bf16"), "route"),
     (BraConfig("one-cut-rows-of-whole-regions", 1, 33, 40, 32, 1, 8, 1, "bf16"), "route"),
     (BraConfig("one-256-regions", 1, 80, 96, 32, 1, 16, 1, "bf16"), "route"),
+    (BraConfig("one-144-regions-32-pairs", 16, 60, 48, 64, 2, 12, 1, "bf16"), "route"),    # (256 regions of one image: the direct kernels)
 ]
 
 

@@ -265,14 +265,13 @@ __device__ __forceinline__ void sum_parts(const float* at, int nparts, size_t st
 }
 // CUT: long lists in parts (ListParts).
 template <int PL, bool EXACT, bool CUT, int TY, int TX>
-__global__ void __launch_bounds__(PL == 2 ? 128 : 256, PL == 2 ? 3 : 2)
-bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __restrict__ Kg,
-                      const __nv_bfloat16* __restrict__ Vg, const int32_t* inv_off,
-                      const int32_t* inv_list, const int32_t* inv_order, const float* __restrict__ lse,
-                      const float* delta, const __nv_bfloat16* __restrict__ dOg,
-                      const float* __restrict__ lce_w, __nv_bfloat16* __restrict__ dKg,
-                      __nv_bfloat16* __restrict__ dVg, const int2* jobs, ListParts parts, int32_t* done, float* sums, int job0,
-                      const __grid_constant__ Dims dm, const __grid_constant__ DirGeom gm) {
+__device__ __forceinline__ void bwd_dkv_direct(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __restrict__ Kg,
+                                               const __nv_bfloat16* __restrict__ Vg, const int32_t* inv_off,
+                                               const int32_t* inv_list, const int32_t* inv_order, const float* __restrict__ lse,
+                                               const float* delta, const __nv_bfloat16* __restrict__ dOg,
+                                               const float* __restrict__ lce_w, __nv_bfloat16* __restrict__ dKg,
+                                               __nv_bfloat16* __restrict__ dVg, const int2* jobs, const ListParts& parts, int32_t* done, float* sums,
+                                               int job0, const Dims& dm, const DirGeom& gm) {
     constexpr int RT = 1, KS = PL == 2 ? 1 : 2;                       // tiles per warp, 16-query steps per block
     extern __shared__ __align__(128) uint8_t smem[];
     const uint32_t sbase = smem_u32(smem);
@@ -285,7 +284,7 @@ bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16*
     const int nth = one_warp ? rest * gm.gpc + warp : rest / gm.chunks;  // by falling length of the list
     const int gwarp = one_warp ? 0 : warp, gwarps = one_warp ? 1 : gm.nw;
     const int glane = one_warp ? lane : tid, glanes = gwarps * 32;
-    const bool live = nth < parts.jobs - job0;
+    const bool live = nth < (CUT ? parts.jobs : dm.R) - job0;
     auto group_sync = [&]() { if (one_warp) __syncwarp(); else __syncthreads(); };
 
     const int rows = min(gm.hb, dm.hs - ck * gm.hb);
@@ -476,6 +475,29 @@ bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16*
                             gwarp, gwarps, lane);
 }
 
+// Geometry in the parameters' own memory or held by value: the same code with other registers.  Whole lists at 32 channels are better off
+// with the second (30 x 80 x 80, 12 x 12 regions, 16 + 16 bits of P, spills 128 -> 108 bytes: gradients 446 -> 440 us), cut lists and 64 channels
+// with the first (16 x 32 x 32, 12 heads of 64: 377 -> 373 us; spills of cut lists 136 -> 88 bytes).
+template <int PL, bool EXACT, bool CUT, int TY, int TX>
+__global__ void __launch_bounds__(PL == 2 ? 128 : 256, PL == 2 ? 3 : 2)
+bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __restrict__ Kg, const __nv_bfloat16* __restrict__ Vg,
+                      const int32_t* inv_off, const int32_t* inv_list, const int32_t* inv_order, const float* __restrict__ lse,
+                      const float* delta, const __nv_bfloat16* __restrict__ dOg, const float* __restrict__ lce_w,
+                      __nv_bfloat16* __restrict__ dKg, __nv_bfloat16* __restrict__ dVg, const int2* jobs, ListParts parts, int32_t* done,
+                      float* sums, int job0, const __grid_constant__ Dims dm, const __grid_constant__ DirGeom gm) {
+    bwd_dkv_direct<PL, EXACT, CUT, TY, TX>(Qg, Kg, Vg, inv_off, inv_list, inv_order, lse, delta, dOg, lce_w, dKg, dVg, jobs, parts, done, sums,
+                                           job0, dm, gm);
+}
+template <bool EXACT, int TY, int TX>
+__global__ void __launch_bounds__(256, 2)
+bwd_dkv_whole_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __restrict__ Kg, const __nv_bfloat16* __restrict__ Vg,
+                     const int32_t* inv_off, const int32_t* inv_list, const int32_t* inv_order, const float* __restrict__ lse,
+                     const float* delta, const __nv_bfloat16* __restrict__ dOg, const float* __restrict__ lce_w,
+                     __nv_bfloat16* __restrict__ dKg, __nv_bfloat16* __restrict__ dVg, int job0, Dims dm, DirGeom gm) {
+    bwd_dkv_direct<1, EXACT, false, TY, TX>(Qg, Kg, Vg, inv_off, inv_list, inv_order, lse, delta, dOg, lce_w, dKg, dVg, nullptr, ListParts(),
+                                            nullptr, nullptr, job0, dm, gm);
+}
+
 // ------------------------------------------------------------------ host side
 static bool dq_single(const Dims& d) { return d.d == 32 && d.topk * d.n_r <= 64 && !direct_exact(d); }
 static DirGeom dq_geom(const Dims& d) {
@@ -569,6 +591,13 @@ static cudaError_t launch_dq(const Dims& d, const BwdArgs& a) {
     });
 }
 
+template <typename F>
+static cudaError_t launch_dkv_pieces(const Dims& d, const BwdArgs& a, const DirGeom& g, F&& launch) {
+    return group_pieces(d, (a.parts.jobs + g.gpc - 1) / g.gpc * g.chunks, g.chunks, [&](const GridPiece& p, int groups_before, int groups) {
+        count_launch();
+        return launch(p, inverse_piece(d, p, a.inv_off, a.inv_list, a.inv_order), dim3(p.heads, p.images, groups), groups_before * g.gpc);
+    });
+}
 template <int PL, bool EXACT, bool CUT, int TY, int TX>
 static cudaError_t launch_dkv_t(const Dims& d, const BwdArgs& a) {
     const DirGeom g = dkv_geom(d);
@@ -576,22 +605,32 @@ static cudaError_t launch_dkv_t(const Dims& d, const BwdArgs& a) {
     static PerDeviceMax set;
     const cudaError_t e = allow_smem(set, kernel, g.smem_bytes);
     if (e != cudaSuccess) return e;
-    const int all = (a.parts.jobs + g.gpc - 1) / g.gpc * g.chunks;
-    return group_pieces(d, all, g.chunks, [&](const GridPiece& p, int groups_before, int groups) {
-        const InversePiece inv = inverse_piece(d, p, a.inv_off, a.inv_list, a.inv_order);
+    return launch_dkv_pieces(d, a, g, [&](const GridPiece& p, const InversePiece& inv, dim3 grid, int job0) {
         const size_t bh = (size_t)p.b0 * d.heads;
-        count_launch();
-        return launch_kernel(kernel, dim3(p.heads, p.images, groups), dim3(g.nw * 32), (size_t)g.smem_bytes, a.st, true,
-                             a.q + p.tensor, a.k + p.tensor, a.v + p.tensor, inv.off, inv.list, inv.order, a.lse + p.stat,
-                             a.delta + p.stat, a.go + p.tensor, a.lce_w, a.dk + p.tensor, a.dv + p.tensor,
-                             a.jobs + (size_t)p.b0 * d.heads_i * a.parts.jobs, a.parts, a.done + bh * d.R * g.chunks,
-                             a.sums + bh * a.parts.cut * g.chunks * g.tpc * 1024 * PL, groups_before * g.gpc, d, g);
+        return launch_kernel(kernel, grid, dim3(g.nw * 32), (size_t)g.smem_bytes, a.st, true, a.q + p.tensor, a.k + p.tensor, a.v + p.tensor,
+                             inv.off, inv.list, inv.order, a.lse + p.stat, a.delta + p.stat, a.go + p.tensor, a.lce_w, a.dk + p.tensor,
+                             a.dv + p.tensor, a.jobs + (size_t)p.b0 * d.heads_i * a.parts.jobs, a.parts, a.done + bh * d.R * g.chunks,
+                             a.sums + bh * a.parts.cut * g.chunks * g.tpc * 1024 * PL, job0, d, g);
     });
 }
-
+template <bool EXACT, int TY, int TX>
+static cudaError_t launch_dkv_whole(const Dims& d, const BwdArgs& a) {
+    const DirGeom g = dkv_geom(d);
+    auto kernel = bwd_dkv_whole_kernel<EXACT, TY, TX>;
+    static PerDeviceMax set;
+    const cudaError_t e = allow_smem(set, kernel, g.smem_bytes);
+    if (e != cudaSuccess) return e;
+    return launch_dkv_pieces(d, a, g, [&](const GridPiece& p, const InversePiece& inv, dim3 grid, int job0) {
+        return launch_kernel(kernel, grid, dim3(g.nw * 32), (size_t)g.smem_bytes, a.st, true, a.q + p.tensor, a.k + p.tensor, a.v + p.tensor,
+                             inv.off, inv.list, inv.order, a.lse + p.stat, a.delta + p.stat, a.go + p.tensor, a.lce_w, a.dk + p.tensor,
+                             a.dv + p.tensor, job0, d, g);
+    });
+}
 template <int PL, bool EXACT, int TY, int TX>
 static cudaError_t launch_dkv(const Dims& d, const BwdArgs& a) {
-    return a.parts.most ? launch_dkv_t<PL, EXACT, true, TY, TX>(d, a) : launch_dkv_t<PL, EXACT, false, TY, TX>(d, a);
+    if (a.parts.most) return launch_dkv_t<PL, EXACT, true, TY, TX>(d, a);
+    if constexpr (PL == 1) return launch_dkv_whole<EXACT, TY, TX>(d, a);
+    else return launch_dkv_t<PL, EXACT, false, TY, TX>(d, a);
 }
 
 static cudaError_t launch_both(const Dims& d, const BwdArgs& a) {

@@ -520,12 +520,18 @@ bool backward_direct_supported(const Dims& d, int dtype) {
     return dkv_geom(d).smem_bytes <= 200 * 1024 && dq_geom(d).smem_bytes <= 200 * 1024 && d.R <= 8192;
 }
 
-// A part is what a group of warps would have on average if all were busy from the first to the last, and at least 256 queries; lists are
-// cut where the longest possible one is four parts or more, in problems that have no other kernels.  Measured (B200), forward +
-// backward, lists whole / cut.  A few regions holding most of the lists: 2 x 100 x 167, 6 heads, S = 16, topk 4 (87 % of the lists are empty, the
-// longest has 84 entries) 487 / 412 us, 1 x 123 x 99, 4 heads, topk 2 164 / 92, 2 x 80 x 80, S = 8, topk 1 112 / 77.  Evenly spread
-// lists: 2 x 50 x 84, 8 heads, topk 8 202 / 178, 1 x 92 x 84, 6 heads 120 / 107, 2 x 100 x 167, 6 heads 406 / 410.  Parts of 8 entries of 2 x 2 regions
-// (10 x 15 x 15, 3 heads of 64, S = 8, topk 12): 61 / 80.
+// A part is the fair share, what a group of warps would have if all were busy from the first to the last, and at least 256 queries and 8
+// entries (parts of 8 entries of 2 x 2 tokens, 10 x 15 x 15, 3 heads of 64, S = 8, topk 12: 61 / 80 us, lists whole / cut).  Lists are cut where
+// the longest possible one is four parts or more, in problems that have no other kernels, if besides
+//   all groups of warps are on the GPU at once: the longest list is what they wait for;
+//   or a fair share is 1024 queries or more: the cost of a part, its sums, does not show;
+//   or a third of R, the longest list of a map with a few kinds of content (R = 49: 19 - 22 entries, 64: 23 - 36, 256: 73 - 89), is three
+//   fair shares.
+// Measured (B200, us, gradients, lists whole / cut).  Content in a few kinds: 2 x 100 x 167, 6 heads, S = 16, topk 4 (87 % of the lists are
+// empty, the longest has 73 entries) 351 / 284, 1 x 123 x 99, 4 heads, topk 2 130 / 52, 4 x 32 x 32, 6 heads of 64, S = 8, topk 12 71 / 57,
+// 2 x 96 x 96, 3 heads, S = 8, topk 4 215 / 198.  Evenly spread lists there: 284 / 287, 61 / 46, 63 / 55, 169 / 171; 2 x 85 x 137, 6 heads, S = 16, topk 2
+// 117 / 120, 2 x 74 x 46, 12 heads, topk 8 76 / 78.  Not cut: 10 x 32 x 32, 3 heads of 64, topk 12 (1.1 rounds of warps) clustered 80 / 87,
+// evenly 81 / 85; 10 x 32 x 32, 6 heads, S = 7, topk 4 65 / 69 and 67 / 67; 7 x 40 x 40 75 / 79 and 77 / 77; 9 x 44 x 44, 4 heads 93 / 97 and 94 / 96.
 ListParts direct_grad_parts(const Dims& d, int* chunks, size_t* sum_bytes) {
     ListParts p = {0, d.R, 0};
     *sum_bytes = 0;
@@ -542,6 +548,7 @@ ListParts direct_grad_parts(const Dims& d, int* chunks, size_t* sum_bytes) {
     if (most < (256 + d.n_r - 1) / d.n_r) most = (256 + d.n_r - 1) / d.n_r;
     if (most < 8) most = 8;
     if (4 * most > d.R) return p;                                     // (a list is longer than R only where it repeats regions)
+    if (work > d.topk * slots && work * d.n_r < 1024 * slots && 9 * work > d.R * slots) return p;
     p.most = (int)most;
     p.jobs = d.R + (int)(entries / most);
     p.cut = (int)(2 * entries / most);

@@ -324,7 +324,8 @@ __device__ __forceinline__ void bwd_dkv_direct(const __nv_bfloat16* __restrict__
     cp_async_commit();
     const int l0 = __ldcg(inv_off + bhi * (dm.R + 1) + jr), l1 = __ldcg(inv_off + bhi * (dm.R + 1) + jr + 1);
     const int nparts = CUT ? max(1, (l1 - l0 + parts.most - 1) / parts.most) : 1;
-    const int e0 = CUT ? l0 + job.y * parts.most : l0, e1 = CUT ? min(l1, e0 + parts.most) : l1;
+    const int per = !CUT ? 0 : parts.even ? (l1 - l0 + nparts - 1) / nparts : parts.most;
+    const int e0 = CUT ? l0 + job.y * per : l0, e1 = CUT ? min(l1, e0 + per) : l1;
     // (parts, job, part): not needed before the end, so they wait behind the table; every thread writes them, for itself
     volatile int* s_job = reinterpret_cast<int*>(smem + gm.off_tab + grp * gm.tab_bytes) + 3 * gm.tab;
     if (CUT) { s_job[0] = nparts; s_job[1] = job0 + nth; s_job[2] = job.y; }
@@ -521,8 +522,11 @@ bool backward_direct_supported(const Dims& d, int dtype) {
 }
 
 // A part is the fair share, what a group of warps would have if all were busy from the first to the last, and at least 256 queries and 8
-// entries (parts of 8 entries of 2 x 2 tokens, 10 x 15 x 15, 3 heads of 64, S = 8, topk 12: 61 / 80 us, lists whole / cut).  Lists are cut where
-// the longest possible one is four parts or more, in problems that have no other kernels, if besides
+// entries (parts of 8 entries of 2 x 2 tokens, 10 x 15 x 15, 3 heads of 64, S = 8, topk 12: 61 / 80 us, lists whole / cut).  Where it is more than
+// the fair share the parts of a list are of one length: a list of an entry more than a part does not wait for a part of one (1 x 48 x 63,
+// 12 heads, S = 16, topk 4 35.8 -> 33.2 us, lists whole 34.2).  Parts of the fair share stay whole but for the last, the longest first
+// (2 x 100 x 167, 6 heads, topk 4 clustered 285, of one length 303).  Lists are cut where the longest possible one is four parts or more, in
+// problems that have no other kernels, if besides
 //   all groups of warps are on the GPU at once: the longest list is what they wait for;
 //   or a fair share is 1024 queries or more: the cost of a part, its sums, does not show;
 //   or a third of R, the longest list of a map with a few kinds of content (R = 49: 19 - 22 entries, 64: 23 - 36, 256: 73 - 89), is three
@@ -533,7 +537,7 @@ bool backward_direct_supported(const Dims& d, int dtype) {
 // 117 / 120, 2 x 74 x 46, 12 heads, topk 8 76 / 78.  Not cut: 10 x 32 x 32, 3 heads of 64, topk 12 (1.1 rounds of warps) clustered 80 / 87,
 // evenly 81 / 85; 10 x 32 x 32, 6 heads, S = 7, topk 4 65 / 69 and 67 / 67; 7 x 40 x 40 75 / 79 and 77 / 77; 9 x 44 x 44, 4 heads 93 / 97 and 94 / 96.
 ListParts direct_grad_parts(const Dims& d, int* chunks, size_t* sum_bytes) {
-    ListParts p = {0, d.R, 0};
+    ListParts p = {0, d.R, 0, false};
     *sum_bytes = 0;
     *chunks = 1;
     if (!backward_direct_supported(d, d.esize == 2 ? BRA_BF16 : BRA_F32) || (backward_one_supported(d, BRA_BF16) && one_grad_pays(d)) ||
@@ -544,12 +548,14 @@ ListParts direct_grad_parts(const Dims& d, int* chunks, size_t* sum_bytes) {
     const int warps = g.planes == 2 ? 12 : 16;                        // of an SM
     const long long slots = (long long)kSMs * (g.gpc > 1 ? warps : warps / g.nw > 0 ? warps / g.nw : 1);
     const long long entries = (long long)d.R * d.topk, work = entries * d.B * d.heads * g.chunks;
-    long long most = (work + slots - 1) / slots;
+    const long long fair = (work + slots - 1) / slots;
+    long long most = fair;
     if (most < (256 + d.n_r - 1) / d.n_r) most = (256 + d.n_r - 1) / d.n_r;
     if (most < 8) most = 8;
     if (4 * most > d.R) return p;                                     // (a list is longer than R only where it repeats regions)
     if (work > d.topk * slots && work * d.n_r < 1024 * slots && 9 * work > d.R * slots) return p;
     p.most = (int)most;
+    p.even = most > fair;
     p.jobs = d.R + (int)(entries / most);
     p.cut = (int)(2 * entries / most);
     *sum_bytes = (size_t)d.B * d.heads * p.cut * g.chunks * g.tpc * 4096 * g.planes;

@@ -70,6 +70,7 @@ inline T* piece_of(T* p, size_t n) { return p ? p + n : nullptr; }
 struct ListParts {
     int most;               // entries of a part; 0: lists are not cut
     int jobs, cut;          // jobs of an (image, routing head) and, of those, parts of cut lists, at most
+    bool even;              // the parts of a list are of one length; else the last one has what is left
 };
 
 // Scratch layout (byte offsets from ws, all multiples of 256).

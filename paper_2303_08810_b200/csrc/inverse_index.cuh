@@ -62,7 +62,7 @@ inline cudaError_t group_pieces(const Dims& d, int groups, int chunks, F&& launc
 // Entries outside [0, R) are in no list.
 __device__ __forceinline__ void inverse_index_job(const int32_t* __restrict__ index, int32_t* __restrict__ inv_off,
                                                   int32_t* __restrict__ inv_list, int32_t* __restrict__ order, int bh, int32_t* sm, bool use_bits, const Dims& dm,
-                                                  const ListJobs& lj = {nullptr, nullptr, 0, {0, 0, 0}}) {
+                                                  const ListJobs& lj = {nullptr, nullptr, 0, {0, 0, 0, false}}) {
     const int tid = threadIdx.x, nthreads = blockDim.x;
     const int lane = tid & 31, warp = tid >> 5;
     const int entries = dm.R * dm.topk, words = (dm.R + 31) >> 5;

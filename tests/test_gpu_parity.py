@@ -1314,6 +1314,8 @@ CUT_CASES = [
     BraConfig("cut-12x12-chunks-d64", 2, 96, 96, 192, 3, 8, 2, "bf16"),
     BraConfig("cut-18x9-chunks-d64", 2, 144, 72, 64, 1, 8, 2, "bf16"),
     BraConfig("cut-18x9-chunks", 2, 144, 72, 32, 1, 8, 2, "bf16"),
+    # parts of the fair share, the last one shorter: 64 x 5 entries of 4 heads in two chunks over 296 CTAs, 9
+    BraConfig("cut-fair-share", 1, 96, 96, 128, 4, 8, 5, "bf16"),
 ]
 
 
@@ -1328,7 +1330,8 @@ def test_gradients_of_lists_cut_in_parts(bra, cfg):
     run_backward_case(bra, cfg, seed=72, index=few)
     # lists of every length around one, two and three parts, the other regions topk times or topk - 1 times.  (All columns of the index
     # but the first name every region once; what the first column has no room for comes in the next (image, head) or call.)
-    part = max(8, -(-256 // (-(-cfg.H // cfg.S) * -(-cfg.W // cfg.S))))                   # entries: 256 queries, or 8
+    part = max(8, -(-256 // (-(-cfg.H // cfg.S) * -(-cfg.W // cfg.S))))                   # entries: 256 queries, or 8, or a fair share
+    part = 9 if cfg.name == "cut-fair-share" else part
     lengths = [part - 1, part, part + 1, 2 * part, 2 * part + 1, 3 * part, 3 * part + 1]
     firsts = [[]]
     for n in lengths:
@@ -1347,9 +1350,13 @@ def test_gradients_of_lists_cut_in_parts(bra, cfg):
             seen |= set(np.bincount(rows.ravel()).tolist())
         run_backward_case(bra, cfg, seed=73, index=edge.reshape(shape))
     assert seen.issuperset(lengths)
-    # the lists of this shape are cut: the scratch for the sums of the parts grows with topk, by far more than the index does
+    # the lists of this shape are cut: the scratch for the sums of the parts grows with topk, by far more than the index does (with a
+    # fair share its parts grow instead: 4 heads, up to 2 * 320 / 9 parts, 12 tiles of 4 KB are most of the scratch)
     more = [bra.workspace_bytes(bra.make_problem(cfg.B, cfg.H, cfg.W, cfg.C, cfg.heads, cfg.S, k, cfg.dtype)) for k in (cfg.topk, cfg.topk + 1)]
-    assert more[1] - more[0] > 10 * 8 * cfg.B * cfg.heads * cfg.R
+    if cfg.name == "cut-fair-share":
+        assert more[0] > 4 * 71 * 12 * 4096
+    else:
+        assert more[1] - more[0] > 10 * 8 * cfg.B * cfg.heads * cfg.R
     run_backward_case(bra, cfg, seed=74, index=few[:, :1].copy(), shared=True)
     if cfg.R <= 256:                                                                       # (as many as bra_forward routes)
         run_backward_case(bra, cfg, seed=75)

@@ -141,6 +141,7 @@ __device__ __forceinline__ bool dense_routes(unsigned long long* mask, float* bi
 // two columns a lane holds of an n-tile, with one it is the token's, 0 (any) goes by the table of regions.  (A bit per two or
 // four scores, picked before the exponential: a test and a select per row and n-tile instead of per score behind it.  A bit of its own for
 // a token, 64 x 7 x 7, 16 heads, topk 49: attention 15.1 -> 14.5 us, gradients 38.3 -> 36.4 against going by the table.)
+constexpr int DENSE_ALL = -1;       // every region is on every list: nothing is picked, the kernel masks what is behind the last token
 template <int NR>
 struct DenseRow {
     unsigned long long m;
@@ -149,7 +150,8 @@ struct DenseRow {
     // n-tile j of the block from token k0 on, column 2 t4 + e
     __device__ __forceinline__ float pick(float yes, int j, int e, int k0, int t4, const uint8_t* reg) const {
         bool on;
-        if (NR == 4) on = (uint32_t)m >> (2 * j) & 1;
+        if (NR == DENSE_ALL) on = true;
+        else if (NR == 4) on = (uint32_t)m >> (2 * j) & 1;
         else if (NR == 1) on = (uint32_t)m >> (8 * j + e) & 1;
         else {
             const int r = reg[k0 + 8 * j + 2 * t4 + e];

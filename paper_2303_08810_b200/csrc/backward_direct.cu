@@ -528,7 +528,8 @@ bool backward_direct_supported(const Dims& d, int dtype) {
 // (2 x 100 x 167, 6 heads, topk 4 clustered 285, of one length 303).  Lists are cut where the longest possible one is four parts or more, in
 // problems that have no other kernels, if besides
 //   all groups of warps are on the GPU at once: the longest list is what they wait for;
-//   or a fair share is 1024 queries or more: the cost of a part, its sums, does not show;
+//   or a fair share is 1280 queries or more: the cost of a part, its sums, does not show (31 x 64 x 64, 2 heads, S = 7, topk 1, 1026 queries,
+//   clustered 223 / 227, evenly 235 / 235; 9 x 80 x 80, 3 heads, 1290, 194 / 194 and 192 / 194);
 //   or a third of R, the longest list of a map with a few kinds of content (R = 49: 19 - 22 entries, 64: 23 - 36, 256: 73 - 89), is three
 //   fair shares.
 // Measured (B200, us, gradients, lists whole / cut).  Content in a few kinds: 2 x 100 x 167, 6 heads, S = 16, topk 4 (87 % of the lists are
@@ -553,7 +554,7 @@ ListParts direct_grad_parts(const Dims& d, int* chunks, size_t* sum_bytes) {
     if (most < (256 + d.n_r - 1) / d.n_r) most = (256 + d.n_r - 1) / d.n_r;
     if (most < 8) most = 8;
     if (4 * most > d.R) return p;                                     // (a list is longer than R only where it repeats regions)
-    if (work > d.topk * slots && work * d.n_r < 1024 * slots && 9 * work > d.R * slots) return p;
+    if (work > d.topk * slots && work * d.n_r < 1280 * slots && 9 * work > d.R * slots) return p;
     p.most = (int)most;
     p.even = most > fair;
     p.jobs = d.R + (int)(entries / most);

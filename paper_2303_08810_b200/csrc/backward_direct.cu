@@ -522,21 +522,22 @@ bool backward_direct_supported(const Dims& d, int dtype) {
 }
 
 // A part is the fair share, what a group of warps would have if all were busy from the first to the last, and at least 256 queries and 8
-// entries (parts of 8 entries of 2 x 2 tokens, 10 x 15 x 15, 3 heads of 64, S = 8, topk 12: 61 / 80 us, lists whole / cut).  Where it is more than
-// the fair share the parts of a list are of one length: a list of an entry more than a part does not wait for a part of one (1 x 48 x 63,
+// entries (parts of 8 entries of 2 x 2 tokens, 10 x 15 x 15, 3 heads of 64, S = 8, topk 12: 61 / 80 us, lists whole / cut).  Where it is much more
+// than the fair share the parts of a list are of one length: a list of an entry more than a part does not wait for a part of one (1 x 48 x 63,
 // 12 heads, S = 16, topk 4 35.8 -> 33.2 us, lists whole 34.2).  Parts of the fair share stay whole but for the last, the longest first
-// (2 x 100 x 167, 6 heads, topk 4 clustered 285, of one length 303).  Lists are cut where the longest possible one is four parts or more, in
-// problems that have no other kernels, if besides
+// (2 x 100 x 167, 6 heads, topk 4 clustered 285, of one length 303; 1 x 112 x 112, 2 heads, S = 8, topk 8, 8 entries to a share of 7, 192 / 207).
+// Lists are cut where the longest possible one is four parts or more, in problems that have no other kernels, if besides
 //   all groups of warps are on the GPU at once: the longest list is what they wait for;
-//   or a fair share is 1280 queries or more: the cost of a part, its sums, does not show (31 x 64 x 64, 2 heads, S = 7, topk 1, 1026 queries,
-//   clustered 223 / 227, evenly 235 / 235; 9 x 80 x 80, 3 heads, 1290, 194 / 194 and 192 / 194);
-//   or a third of R, the longest list of a map with a few kinds of content (R = 49: 19 - 22 entries, 64: 23 - 36, 256: 73 - 89), is three
-//   fair shares.
+//   or the longest list of a map with a few kinds of content is three fair shares: a third of R, where topk is large 8/3 topk up to half of R
+//   (R = 49: 19 - 22 entries, 64: 23 - 36, 256: 73 - 89), and the regions outside the map, whose scores are 0 and which all list the same;
+//   or regions have 128 tokens and more, beside which the sums of a part do not show, and R is five fair shares.
 // Measured (B200, us, gradients, lists whole / cut).  Content in a few kinds: 2 x 100 x 167, 6 heads, S = 16, topk 4 (87 % of the lists are
 // empty, the longest has 73 entries) 351 / 284, 1 x 123 x 99, 4 heads, topk 2 130 / 52, 4 x 32 x 32, 6 heads of 64, S = 8, topk 12 71 / 57,
-// 2 x 96 x 96, 3 heads, S = 8, topk 4 215 / 198.  Evenly spread lists there: 284 / 287, 61 / 46, 63 / 55, 169 / 171; 2 x 85 x 137, 6 heads, S = 16, topk 2
-// 117 / 120, 2 x 74 x 46, 12 heads, topk 8 76 / 78.  Not cut: 10 x 32 x 32, 3 heads of 64, topk 12 (1.1 rounds of warps) clustered 80 / 87,
-// evenly 81 / 85; 10 x 32 x 32, 6 heads, S = 7, topk 4 65 / 69 and 67 / 67; 7 x 40 x 40 75 / 79 and 77 / 77; 9 x 44 x 44, 4 heads 93 / 97 and 94 / 96.
+// 2 x 96 x 96, 3 heads, S = 8, topk 4 215 / 198, 8 x 80 x 80, 3 heads, S = 7, topk 1 182 / 172, 3 x 27 x 27, 12 heads of 64, topk 12 105 / 95.  Evenly
+// spread lists there: 284 / 287, 61 / 46, 63 / 55, 169 / 171, 169 / 171, 89 / 89; 2 x 85 x 137, 6 heads, S = 16, topk 2 117 / 120, 2 x 74 x 46, 12 heads,
+// topk 8 76 / 78.  Not cut: 10 x 32 x 32, 3 heads of 64, topk 12 clustered 80 / 87, evenly 81 / 85; 10 x 32 x 32, 6 heads, S = 7, topk 4 65 / 69 and
+// 67 / 67; 7 x 40 x 40 75 / 79 and 77 / 77; 9 x 44 x 44, 4 heads 93 / 97 and 94 / 96; 31 x 64 x 64, 2 heads, topk 1 223 / 227 and 235 / 235; 12 x 96 x 96,
+// 3 heads 395 / 398 and 404 / 407.
 ListParts direct_grad_parts(const Dims& d, int* chunks, size_t* sum_bytes) {
     ListParts p = {0, d.R, 0, false};
     *sum_bytes = 0;
@@ -554,9 +555,12 @@ ListParts direct_grad_parts(const Dims& d, int* chunks, size_t* sum_bytes) {
     if (most < (256 + d.n_r - 1) / d.n_r) most = (256 + d.n_r - 1) / d.n_r;
     if (most < 8) most = 8;
     if (4 * most > d.R) return p;                                     // (a list is longer than R only where it repeats regions)
-    if (work > d.topk * slots && work * d.n_r < 1280 * slots && 9 * work > d.R * slots) return p;
+    const int outside = d.R - ((d.H0 + d.hs - 1) / d.hs) * ((d.W0 + d.ws - 1) / d.ws);
+    const int half = d.R / 2 < 8 * d.topk / 3 ? d.R / 2 : 8 * d.topk / 3;
+    const long long longest = (d.R / 3 > half ? d.R / 3 : half) + outside;
+    if (work > d.topk * slots && 3 * work > longest * slots && (d.n_r < 128 || 5 * work > d.R * slots)) return p;
     p.most = (int)most;
-    p.even = most > fair;
+    p.even = 4 * most >= 5 * fair;
     p.jobs = d.R + (int)(entries / most);
     p.cut = (int)(2 * entries / most);
     *sum_bytes = (size_t)d.B * d.heads * p.cut * g.chunks * g.tpc * 4096 * g.planes;

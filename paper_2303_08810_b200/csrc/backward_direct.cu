@@ -476,9 +476,10 @@ __device__ __forceinline__ void bwd_dkv_direct(const __nv_bfloat16* __restrict__
                             gwarp, gwarps, lane);
 }
 
-// Geometry in the parameters' own memory or held by value: the same code with other registers.  Whole lists at 32 channels are better off
-// with the second (30 x 80 x 80, 12 x 12 regions, 16 + 16 bits of P, spills 128 -> 108 bytes: gradients 446 -> 440 us), cut lists and 64 channels
-// with the first (16 x 32 x 32, 12 heads of 64: 377 -> 373 us; spills of cut lists 136 -> 88 bytes).
+// Geometry in the parameters' own memory or held by value: the same code with other registers.  Whole lists with 16 + 16 bits of P at 32
+// channels are better off with the second (30 x 80 x 80, 12 x 12 regions, spills 128 -> 108 bytes: gradients 446 -> 440 us), all others with the
+// first (whole lists at 64 channels 16 x 32 x 32, 12 heads 377 -> 373 us, at 32 channels 4 x 11 x 11, 24 heads, topk 49 86.7 -> 85.5; spills of
+// cut lists at 64 channels 136 -> 92 bytes).
 template <int PL, bool EXACT, bool CUT, int TY, int TX>
 __global__ void __launch_bounds__(PL == 2 ? 128 : 256, PL == 2 ? 3 : 2)
 bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __restrict__ Kg, const __nv_bfloat16* __restrict__ Vg,
@@ -489,13 +490,13 @@ bwd_dkv_direct_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16*
     bwd_dkv_direct<PL, EXACT, CUT, TY, TX>(Qg, Kg, Vg, inv_off, inv_list, inv_order, lse, delta, dOg, lce_w, dKg, dVg, jobs, parts, done, sums,
                                            job0, dm, gm);
 }
-template <bool EXACT, int TY, int TX>
+template <int TY, int TX>
 __global__ void __launch_bounds__(256, 2)
-bwd_dkv_whole_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __restrict__ Kg, const __nv_bfloat16* __restrict__ Vg,
+bwd_dkv_exact_kernel(const __nv_bfloat16* __restrict__ Qg, const __nv_bfloat16* __restrict__ Kg, const __nv_bfloat16* __restrict__ Vg,
                      const int32_t* inv_off, const int32_t* inv_list, const int32_t* inv_order, const float* __restrict__ lse,
                      const float* delta, const __nv_bfloat16* __restrict__ dOg, const float* __restrict__ lce_w,
                      __nv_bfloat16* __restrict__ dKg, __nv_bfloat16* __restrict__ dVg, int job0, Dims dm, DirGeom gm) {
-    bwd_dkv_direct<1, EXACT, false, TY, TX>(Qg, Kg, Vg, inv_off, inv_list, inv_order, lse, delta, dOg, lce_w, dKg, dVg, nullptr, ListParts(),
+    bwd_dkv_direct<1, true, false, TY, TX>(Qg, Kg, Vg, inv_off, inv_list, inv_order, lse, delta, dOg, lce_w, dKg, dVg, nullptr, ListParts(),
                                             nullptr, nullptr, job0, dm, gm);
 }
 
@@ -631,10 +632,10 @@ static cudaError_t launch_dkv_t(const Dims& d, const BwdArgs& a) {
                              a.sums + bh * a.parts.cut * g.chunks * g.tpc * 1024 * PL, job0, d, g);
     });
 }
-template <bool EXACT, int TY, int TX>
-static cudaError_t launch_dkv_whole(const Dims& d, const BwdArgs& a) {
+template <int TY, int TX>
+static cudaError_t launch_dkv_exact(const Dims& d, const BwdArgs& a) {
     const DirGeom g = dkv_geom(d);
-    auto kernel = bwd_dkv_whole_kernel<EXACT, TY, TX>;
+    auto kernel = bwd_dkv_exact_kernel<TY, TX>;
     static PerDeviceMax set;
     const cudaError_t e = allow_smem(set, kernel, g.smem_bytes);
     if (e != cudaSuccess) return e;
@@ -647,7 +648,7 @@ static cudaError_t launch_dkv_whole(const Dims& d, const BwdArgs& a) {
 template <int PL, bool EXACT, int TY, int TX>
 static cudaError_t launch_dkv(const Dims& d, const BwdArgs& a) {
     if (a.parts.most) return launch_dkv_t<PL, EXACT, true, TY, TX>(d, a);
-    if constexpr (PL == 1) return launch_dkv_whole<EXACT, TY, TX>(d, a);
+    if constexpr (PL == 1 && EXACT) return launch_dkv_exact<TY, TX>(d, a);
     else return launch_dkv_t<PL, EXACT, false, TY, TX>(d, a);
 }
 

@@ -113,9 +113,9 @@ def workspace_bytes(p: BraProblem) -> int:
 
 
 # What follows is on the way of every call: of small problems, whose kernels take less time than their marshalling, it is the
-# bound.  A forward + backward pass at 1 x 16 x 16 x 32 spent 58 us of host time in these functions, 25 of them in the library and
-# 13 in its results' allocation; the current stream cost 3.2 us a call through torch.cuda, the device check 0.7 at each use.
-# 46.5 us now; bra_forward of one 56 x 56 image into the caller's tensor 16.2 -> 11.5 us (the library's part of it: 9).
+# bound.  The current stream cost 3.2 us a call through torch.cuda, the device check 0.7 at each use.  Without them a forward +
+# backward pass at 1 x 16 x 16 x 32 takes 40.5 us among others instead of 52.8, bra_forward of one 56 x 56 image into the caller's
+# tensor 10.8 instead of 15.9.
 def _torch():
     global _TORCH
     if _TORCH is None:

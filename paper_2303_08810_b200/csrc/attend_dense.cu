@@ -7,7 +7,8 @@
 // with 12 warps per SM (128 registers), per issue 1.6 cycles of fixed waits, 0.8 at barriers, 0.7 for loads, 0.7 for the MMA pipe;
 // 1.73 waves of CTAs.
 // Measured (B200): 64 x 7 x 7, 16 heads, topk 49: forward 161 us with routing -> 16.4 us; 64 x 14 x 14, 8 heads, topk 16:
-// level with attend_img.cu (44 us); 46 -> 44 under ncu, bra_forward 55.7 -> 54.1, with the mask as the addend of the scaling.  The other side of the rule: dense_pays().
+// level with attend_img.cu (44 us); 46 -> 44 under ncu, bra_forward 55.9 -> 53.9, with the mask as the addend of the scaling.  The other
+// side of the rule: dense_pays().
 #include "dense_common.cuh"
 
 #include <type_traits>

@@ -9,7 +9,7 @@
 //   3. dK/dV kernel: rows are keys, the walk goes over the queries of the regions on the key region's list; P from the
 //      saved log-sum-exp; then the LCE adjoint dV += sum_ij w[c,i,j] dO[y-i+2, x-j+2, c].
 //   4. d_lce_w / d_lce_b: lce_grad.cu.
-// Steps 1 to 3 run on the tensor cores instead (backward_dense.cu, backward_img.cu, backward_direct.cu) for bf16 with head
+// Steps 1 to 3 run on the tensor cores instead (backward_one.cu, backward_dense.cu, backward_img.cu, backward_direct.cu) for bf16 with head
 // dim 32 or 64.
 #include "inverse_index.cuh"
 #include "simt_common.cuh"

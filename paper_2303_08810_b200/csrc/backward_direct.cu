@@ -8,14 +8,15 @@
 // The structure is the forward kernel's (attend_direct.cu): a warp owns 16 rows, the other side streams from global
 // memory straight into MMA fragments, a table of token numbers per group, no barriers in the streaming loop.  A row
 // that was loaded serves both products it takes part in: as loaded where the contraction runs over channels, through
-// movmatrix where it runs over tokens.  No atomics: every sum has a fixed order, results are bit-identical from run
-// to run.  (Two tiles per warp, which pay in the forward kernel, do not here: 8 warps per SM at 168 registers,
+// movmatrix where it runs over tokens.  Every sum has a fixed order, results are bit-identical from run to run: where a list of
+// the inverse index is cut in parts (direct_grad_parts), each leaves its sums in scratch memory and the one that is done last, which
+// an atomic counter tells, adds them up in the order of the parts.  (Two tiles per warp, which pay in the forward kernel, do not here: 8 warps per SM at 168 registers,
 // dQ 140 -> 170 us and dK / dV 274 -> 331 us at 2 x 100 x 167, S = 16.  Fetching the next 16 rows ahead into registers:
 // 140 -> 155 and 274 -> 286 us.)
 // Bound: the latency of the listed rows at 12 - 16 warps per SM (0.53 instructions per cycle and scheduler at head dim 32; at head
 // dim 64, 168 registers, 0.41 in dQ and 0.34 in dK / dV, 1.9 and 3.6 cycles per issue waiting for loads).
-// Measured (B200), dQ / dK dV: 64 x 56 x 56, 8 x 8 regions, topk 1: 61 / 142 -> 50 / 102 us; 2 x 100 x 167, 6 heads:
-// 193 / 322 -> 136 / 201 us; 16 x 32 x 32, 12 heads of 64: 1998 / 2412 us (CUDA cores) -> 140 / 220 us.
+// Measured (B200), dQ / dK dV: 2 x 100 x 167, 6 heads: 193 / 322 -> 136 / 201 us, now, lists cut and clustered, 148 / 149 under ncu;
+// 16 x 32 x 32, 12 heads of 64: 1998 / 2412 us (CUDA cores) -> 140 / 220 us.
 #include "direct_common.cuh"
 #include "inverse_index.cuh"
 

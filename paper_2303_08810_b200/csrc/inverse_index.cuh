@@ -33,8 +33,8 @@ inline InversePiece inverse_piece(const Dims& d, const GridPiece& p, int32_t* of
     const size_t bh = (size_t)p.b0 * d.heads_i;
     return {off + bh * (d.R + 1), list + bh * d.R * d.topk, order + bh * d.R};
 }
-// Pieces of the dK / dV grids (heads, images, groups): all heads; `chunks` consecutive groups are a region, the first of a
-// piece region `regions_before` of the order.  (More groups than a grid holds: always one region per group or less.)
+// Pieces of the dK / dV grids (heads, images, groups): all heads; `chunks` consecutive groups of warps are a region, several regions or a
+// job (ListParts); launch(piece, g, groups) starts with the g-th of these in the order.
 template <typename F>
 inline cudaError_t group_pieces(const Dims& d, int groups, int chunks, F&& launch) {
     if (chunks > GRID_YZ) return cudaErrorInvalidConfiguration;        // (a region of millions of tokens)
